@@ -44,7 +44,11 @@ extern "C" const char *harp_status_string(harp_status_t s) {
     return "unknown status";
 }
 
-extern "C" int32_t harp_plan_error_word(const harp_plan_t *plan) { return plan ? harp_tm_error_word(plan) : -1; }
+extern "C" int32_t harp_plan_error_word(const harp_plan_t *plan) {
+    if (!plan) return -1;
+    const int32_t w = harp_tm_error_word(plan);
+    return w != 0 ? w : harp_f32_error_word(plan);
+}
 
 extern "C" int64_t harp_launch_count(void) { return g_harp_launches.load(std::memory_order_relaxed); }
 
@@ -160,6 +164,10 @@ extern "C" harp_status_t harp_plan_create(harp_plan_t **out, int64_t d, int32_t 
         harp_status_t fs = harp_col_build(p);
         if (fs != HARP_OK && fs != HARP_ERR_UNSUPPORTED) st = fs;
     }
+    if (st == HARP_OK) {
+        harp_status_t fs = harp_f32_build(p);
+        if (fs != HARP_OK && fs != HARP_ERR_UNSUPPORTED) st = fs;
+    }
     if (st != HARP_OK) {
         cudaGetLastError();
         harp_plan_destroy(p);
@@ -177,6 +185,7 @@ extern "C" void harp_plan_destroy(harp_plan_t *p) {
         harp_split_destroy(p);
         harp_col_destroy(p);
         harp_tm_destroy(p);
+        harp_f32_destroy(p);
         for (int i = 0; i < harp_plan::kStages; ++i) {
             if (p->stage_stream[i]) { cudaStreamSynchronize(p->stage_stream[i]); cudaStreamDestroy(p->stage_stream[i]); }
             if (p->stage_buf[i]) cudaFree(p->stage_buf[i]);
@@ -221,6 +230,12 @@ extern "C" harp_status_t harp_apply_ex(const harp_plan_t *plan, void *x, int64_t
     if (st != HARP_ERR_UNSUPPORTED) return st;
     st = harp_split_apply(plan, x, n_rows, dtype, transpose, s);
     if (st != HARP_ERR_UNSUPPORTED) return st;
+    // fp32 rows: up to d = 4096 the whole-row CUDA-core kernels of radices up to 8 hold enough rows of a tile to be the faster
+    // ones (4096 rows of d = 4096, radix 8: 100 us against 128); beyond, and for larger radices, passes over column groups
+    if (dtype == HARP_F32 && (plan->d > 4096 || harp_generic_max_radix(plan) > 8)) {
+        st = harp_f32_apply(plan, x, n_rows, dtype, transpose, s);
+        if (st != HARP_ERR_UNSUPPORTED) return st;
+    }
     return harp_generic_apply(plan, x, n_rows, dtype, transpose, s);
 }
 
@@ -270,7 +285,7 @@ extern "C" harp_status_t harp_apply_two_sided(void *W, harp_dtype_t dtype, const
     if (st != HARP_OK) return st;
     // column side: every column of W through Q_out -- in place with the column kernels when the
     // plan has them (no scratch needed), otherwise as rows of W^T (transpose, apply, transpose back)
-    st = harp_col_apply(plan_out, W, d_in, d_in, dtype, s);
+    st = dtype == HARP_F32 ? harp_f32_col_apply(plan_out, W, d_in, d_in, dtype, s) : harp_col_apply(plan_out, W, d_in, d_in, dtype, s);
     if (st != HARP_ERR_UNSUPPORTED) return st;
     bool own = false;
     if (!scratch) {

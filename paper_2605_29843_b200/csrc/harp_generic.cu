@@ -733,6 +733,13 @@ harp_status_t harp_generic_build(harp_plan *plan) {
     return max_fb <= 8 ? upload_element_major(ft, fb.data()) : HARP_OK;
 }
 
+int harp_generic_max_radix(const harp_plan *plan) {
+    const StageTable &st = plan->fused.m > 0 && plan->d_fused_blocks ? plan->fused : plan->st;
+    int b = 0;
+    for (int t = 0; t < st.m; ++t) b = std::max(b, (int)st.b[t]);
+    return b;
+}
+
 harp_status_t harp_generic_supported(const harp_plan *plan, harp_dtype_t dtype) {
     (void)dtype;
     if (plan->d > (int64_t)kThreads * kMaxItems) return HARP_ERR_UNSUPPORTED;

@@ -23,6 +23,7 @@ struct StageTable {
 struct FastPlan;   // tensor-core path data, whole rows per CTA (harp_fast.cu)
 struct SplitPlan;  // tensor-core path data, two passes over column groups (harp_split.cu)
 struct TmPlan;    // tensor-memory path data: tcgen05.mma, rows as the M dimension (harp_tm.cu)
+struct F32Plan;    // CUDA-core passes over column groups for fp32 rows and matrices (harp_f32.cu)
 struct ColPlan;    // tensor-core path data for applying the plan down the columns of a matrix (harp_col.cu)
 
 struct harp_plan {
@@ -50,6 +51,7 @@ struct harp_plan {
     SplitPlan *split = nullptr;
     ColPlan *col = nullptr;
     TmPlan *tm = nullptr;
+    F32Plan *f32 = nullptr;
     // test-only switch, read from the environment once, when the plan is built (HARP_NO_ROWVEC=1: the
     // CUDA-core kernels keep their tile row-major)
     bool opt_no_rowvec = false;
@@ -64,6 +66,7 @@ extern std::atomic<int64_t> g_harp_launches;
 
 // generic CUDA-core path (harp_generic.cu)
 harp_status_t harp_generic_build(harp_plan *plan);   // fused stage table for the block-owner kernel
+int harp_generic_max_radix(const harp_plan *plan);   // of the stage table its kernels run
 harp_status_t harp_generic_supported(const harp_plan *plan, harp_dtype_t dtype);
 harp_status_t harp_generic_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype,
                                  int transpose, cudaStream_t stream);
@@ -85,6 +88,8 @@ harp_status_t harp_tm_build(harp_plan *plan);
 void harp_tm_destroy(harp_plan *plan);
 harp_status_t harp_tm_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype,
                             int transpose, cudaStream_t stream);
+// cuTensorMapEncodeTiled of the driver (null if it has none)
+void *harp_tensor_map_encoder();
 int32_t harp_tm_error_word(const harp_plan *plan);
 // the stages below stride 256 alone (lower pass of the two-pass paths); 0 stages = not available
 int harp_tm_slab_stages(const harp_plan *plan);
@@ -97,6 +102,15 @@ harp_status_t harp_col_build(harp_plan *plan);
 void harp_col_destroy(harp_plan *plan);
 harp_status_t harp_col_apply(const harp_plan *plan, void *W, int64_t n_cols, int64_t ld, harp_dtype_t dtype,
                              cudaStream_t stream);
+
+// fp32 passes over column groups (harp_f32.cu): rows, and down the columns of a row-major matrix
+harp_status_t harp_f32_build(harp_plan *plan);
+void harp_f32_destroy(harp_plan *plan);
+int32_t harp_f32_error_word(const harp_plan *plan);
+harp_status_t harp_f32_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose,
+                             cudaStream_t stream);
+harp_status_t harp_f32_col_apply(const harp_plan *plan, void *W, int64_t n_cols, int64_t ld, harp_dtype_t dtype,
+                                 cudaStream_t stream);
 
 // out-of-place matrix transpose, rows x cols -> cols x rows (harp_two_sided.cu)
 harp_status_t harp_transpose_matrix(const void *src, void *dst, int64_t rows, int64_t cols,

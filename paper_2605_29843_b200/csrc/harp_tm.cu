@@ -740,6 +740,12 @@ harp_status_t harp_tm_build(harp_plan *plan) {
 
 namespace {
 
+}  // namespace
+
+void *harp_tensor_map_encoder() { return reinterpret_cast<void *>(encode_fn()); }
+
+namespace {
+
 // tensor maps of one call: rows as 2-D boxes of 64 columns, and (d > 256) as 16 runs of 16 per row
 harp_status_t encode_maps(void *x, int64_t n_rows, int64_t d, bool need_s, CUtensorMap *map_c, CUtensorMap *map_s) {
     EncodeTiledFn enc = encode_fn();

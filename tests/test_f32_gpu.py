@@ -1,0 +1,52 @@
+"""The fp32 passes over column groups (rows wider than 4096 or with a radix above 8) and the fp32 column passes of the
+two-sided product, against the oracle: every tile layout and phase form, row counts around the 32- and 64-row tiles."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2605_29843_b200 as harp
+from oracle import harp_oracle as orc
+from paper_2605_29843_b200 import workloads as wl
+from harp_testlib import TOL, gpu_apply, host_rows, promote, to_device, to_host_f64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("radices,perm", [
+    ((16, 16, 8), "identity"),            # contiguous and strided sixteen-wide blocks, an upper pass
+    ((16, 16, 8), "random"),              # permutation and signs in a kernel of their own
+    ((2, 16, 9, 4), "identity"),          # strides 1 and 2 that no 16-byte access fits
+    ((4, 4, 4, 43), "identity"),          # radix above 16 in the upper pass
+    ((8, 8, 8, 8, 2), "identity"),
+    ((8, 8, 5, 3, 11), "identity"),
+    ((4, 4, 4, 4, 4, 4, 2), "identity"),  # pairs of radix-4 stages
+    ((32, 16), "identity"),               # a first pass these kernels do not take
+])
+@pytest.mark.parametrize("n_rows", [1, 33, 64, 127])
+def test_rows_match_the_oracle(radices, perm, n_rows):
+    spec = wl.tiny_plan(61, radices, kind="qr", perm=perm, signs=True)
+    plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
+    xh = host_rows(np.random.default_rng(62).standard_normal((n_rows, spec.d)), "f32")
+    for tr, fn in ((False, orc.forward), (True, orc.transpose)):
+        got, guards = gpu_apply(plan, xh, "f32", tr)
+        assert guards
+        assert orc.rel_err_rows(got, fn(oplan, promote(xh, "f32"))) <= TOL["f32"]
+    assert harp.harp_plan_error_word(plan) == 0
+
+
+@pytest.mark.parametrize("r_out,r_in", [((8, 8, 8), (4, 3, 5)), ((16, 16, 2), (7, 4)), ((2, 2, 2, 2, 3), (4, 4, 4, 4, 4)),
+                                        ((43, 4), (4, 17)), ((64,), (2, 2)), ((8, 8, 8, 8), (8, 9))])
+def test_two_sided_fp32(r_out, r_in):
+    p_out = wl.tiny_plan(63, r_out, kind="qr", perm="identity", signs=True)
+    p_in = wl.tiny_plan(64, r_in, kind="qr", perm="identity", signs=True)
+    wh = host_rows(np.random.default_rng(65).standard_normal((p_out.d, p_in.d)), "f32")
+    wd = to_device(wh, "f32")
+    plan_out, plan_in = harp.plan_from_spec(p_out), harp.plan_from_spec(p_in)
+    harp.two_sided_(wd, plan_out, plan_in)
+    torch.cuda.synchronize()
+    want = orc.two_sided(orc.OraclePlan.from_spec(p_out), orc.OraclePlan.from_spec(p_in), promote(wh, "f32"))
+    # two sides, each within the one-sided tolerance of the row (column) norm
+    err = np.abs(to_host_f64(wd) - want)
+    scale = np.minimum(np.linalg.norm(want, axis=1, keepdims=True), np.linalg.norm(want, axis=0, keepdims=True))
+    assert np.max(err / scale) <= 2 * TOL["f32"]
+    assert harp.harp_plan_error_word(plan_out) == 0
