@@ -368,29 +368,52 @@ def shard_rows(n_rows: int, rank: int, world: int):
 
 
 # ---- torch conveniences (device memory and streams only) ----
+#
+# A decode step spends as long in this call as on the GPU (a small apply: 7 us on the device, 5.3 us here before torch and
+# the library's function were looked up once instead of in every call), so the path below is flat.
+
+_dtype_codes = {}                  # torch dtype -> harp_dtype_t
+_current_device = _raw_stream = _apply_ex = None
+
+
+def _bind_torch() -> None:
+    global _current_device, _raw_stream, _apply_ex
+    import torch
+    _dtype_codes.update({torch.float32: HARP_F32, torch.bfloat16: HARP_BF16})
+    _apply_ex = lib().harp_apply_ex
+    torch.cuda.init()
+    if hasattr(torch._C, "_cuda_getCurrentRawStream"):
+        _current_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+    else:
+        _current_device, _raw_stream = torch.cuda.current_device, lambda dev: torch.cuda.current_stream(dev).cuda_stream
+
 
 def _torch_dtype_code(t) -> int:
-    import torch
-    if t.dtype == torch.float32:
-        return HARP_F32
-    if t.dtype == torch.bfloat16:
-        return HARP_BF16
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    code = _dtype_codes.get(t.dtype)
+    if code is None:
+        raise TypeError(f"unsupported dtype {t.dtype}")
+    return code
 
 
 def apply_(plan: Plan, x, transpose: bool = False, kernel: int = KERNEL_AUTO):
     """In-place apply to a contiguous CUDA tensor [n_rows, d] on torch's current stream."""
-    import torch
-    assert x.is_cuda and x.is_contiguous() and x.dim() == 2 and x.shape[1] == plan.d
-    harp_apply(plan, x.data_ptr(), x.shape[0], _torch_dtype_code(x), transpose,
-               torch.cuda.current_stream().cuda_stream, kernel)
+    if _apply_ex is None:
+        _bind_torch()
+    shape = x.shape
+    assert x.is_cuda and x.is_contiguous() and len(shape) == 2 and shape[1] == plan.d
+    code = _dtype_codes.get(x.dtype)
+    if code is None:
+        raise TypeError(f"unsupported dtype {x.dtype}")
+    st = _apply_ex(plan.handle, x.data_ptr(), shape[0], code, 1 if transpose else 0, kernel, _raw_stream(_current_device()))
+    if st != HARP_OK:
+        raise HarpError(st, "harp_apply")
     return x
 
 
 def two_sided_(w, plan_out: Plan, plan_in: Plan, scratch=None):
-    import torch
+    if _apply_ex is None:
+        _bind_torch()
     assert w.is_cuda and w.is_contiguous() and w.shape == (plan_out.d, plan_in.d)
     harp_apply_two_sided(w.data_ptr(), _torch_dtype_code(w), plan_out, plan_in,
-                         0 if scratch is None else scratch.data_ptr(),
-                         torch.cuda.current_stream().cuda_stream)
+                         0 if scratch is None else scratch.data_ptr(), _raw_stream(_current_device()))
     return w
