@@ -1101,8 +1101,13 @@ cudaError_t launch_pass(void (*kern)(__nv_bfloat16 *, int64_t, int64_t, PassT), 
     return cudaLaunchKernelEx(&cfg, kern, x, r0, r1, P);
 }
 
-constexpr int64_t kOverlapMaxRows = 64;
-constexpr int64_t kTmSlabMinRows = 1024;
+// (measured over 96 .. 8192 rows, d = 5120 .. 28672: with the attribute a call gains 3-5 us up to about this many elements --
+// passes of some 20 us --, e.g. 512 rows of d = 8192 20.5 -> 18.5 us, and loses 1-4 % on larger batches, where CTAs that
+// wait for the kernel before them hold shared memory its last CTAs could use)
+constexpr int64_t kOverlapMaxElems = (int64_t)16 << 20;
+// (400 rows of d = 14336: 21.1 us with the mma.sync slab pass, 18.6 with the tensor-memory one; at 256 rows its 128-row tiles
+// leave a third of the SMs idle and it is the slower one)
+constexpr int64_t kTmSlabMinRows = 384;
 
 harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose,
                                cudaStream_t stream) {
@@ -1111,9 +1116,7 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
     if ((reinterpret_cast<uintptr_t>(x) & 15u) != 0) return HARP_ERR_UNSUPPORTED;
     __nv_bfloat16 *xb = static_cast<__nv_bfloat16 *>(x);
     const bool two = sp->pass[1].present || sp->dense_upper;
-    // (with the attribute on for every batch size an apply of 32768 rows at d = 14336 took 940 us instead of 907,
-    // 65536 rows at d = 28672 5.2 ms instead of 4.8: large batches are launched plainly)
-    const bool overlap = n_rows <= kOverlapMaxRows;
+    const bool overlap = n_rows * plan->d <= kOverlapMaxElems;
     auto gather = [&](int dir) -> harp_status_t {
         const int64_t n_groups = (n_rows + sp->gather_rows - 1) / sp->gather_rows;
         const unsigned grid = (unsigned)std::min<int64_t>(n_groups, sp->sms);
