@@ -6,16 +6,18 @@
 // y = v_m.  With G = dL/dy:   g_m = G,   g_t = g_{t+1} M_t^T,
 //     dL/dK_t[c][i][j] = sum over rows of  v_t[base_c + i s_t] * g_{t+1}[base_c + j s_t].
 //
-// The rows are processed in chunks; for a chunk all forward states v_0..v_{m-1} are kept in global
-// scratch (fp32) and the gradient state is walked back stage by stage.  Every sum over rows is
-// taken in fp64 in a fixed order -- no atomics, so the result does not depend on scheduling.
+// The rows are processed in chunks; for a chunk the forward states between steps are kept in global scratch (fp32) and the
+// gradient state is walked back step by step.  Every sum over rows is taken in fp64 in a fixed order -- no atomics, so the
+// result does not depend on scheduling.
 //
-// Stages of radix 2 to 8 run in "block owner" kernels: a thread owns one block c of the stage,
-// keeps K_t[c] in registers and walks the rows of its slice of the chunk, so neighbouring lanes
-// read neighbouring coordinates (or one vector when s_t = 1) and K is read once.  The backward
-// kernel of such a stage does both jobs in one sweep over v_t and g_{t+1}: it writes g_t and adds
-// v_t[i] g_{t+1}[j] into its B x B fp64 accumulators; the per-slice sums are then added slice by
-// slice.  Other radices use the plain one-thread-per-element kernels below them.
+// A step is one stage or two: what crosses memory per step is a state forward, and a state, a gradient state and the next
+// gradient state backward, so two radix-4 stages (four threads hold sixteen coordinates and transpose 4 x 4 by
+// shuffles) or two radix-2 stages (one thread holds four coordinates) in one step halve the traffic that bounds these
+// kernels.  Threads own blocks, keep their kernels in registers (read element-major, so that neighbouring threads read
+// neighbouring words) and walk over the rows of a slice; the backward kernels write the gradient state and add the
+// outer products into fp64 registers in one sweep.  Blocks too large for one thread's registers are shared by threads that
+// own some of the results (forward) or some of the rows of the gradient block (backward).  The first step reads x and the
+// last dL/dy in their own type.  Radices with no such kernel use the plain one-thread-per-element kernels.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -56,324 +58,573 @@ template <typename T> __device__ __forceinline__ float to_f32(T v);
 template <> __device__ __forceinline__ float to_f32<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-constexpr int kOwnThreads = 128;   // block-owner kernels: blocks per CTA
-constexpr int kFwdSliceRows = 8;   //                      rows per CTA, forward
-constexpr int kBwdSliceRows = 32;  //                      rows per CTA (one set of partial sums), backward
-constexpr int kRowBatch = 4;       //                      rows whose loads are issued together
+constexpr int kOwnThreads = 128;   // threads per CTA of the block-owner kernels
+constexpr int kFwdRows = 32;       // rows per CTA, forward
+constexpr int kSubs = 4;           // backward: warps that share the blocks of a warp and split the rows; their sums are added
+                                   // in shared memory, which leaves a quarter of the partial sums to write and read back
 
-template <int B> __device__ __forceinline__ void load_block(const float *p, int64_t s, float (&v)[B]) {
-    if (s == 1 && (B == 2 || B % 4 == 0)) {
-        if constexpr (B == 2) {
-            const float2 a = *reinterpret_cast<const float2 *>(p);
-            v[0] = a.x; v[1] = a.y;
-        } else {
+// B values s apart; vec: s == 1 and the row is aligned for 16-byte (8-byte bf16) accesses of four
+template <int B, typename T> __device__ __forceinline__ void load_block(const T *p, int64_t s, bool vec, float (&v)[B]) {
+    if (B % 4 == 0 && vec) {
 #pragma unroll
-            for (int q = 0; q < B / 4; ++q) {
-                const float4 a = reinterpret_cast<const float4 *>(p)[q];
-                v[4 * q] = a.x; v[4 * q + 1] = a.y; v[4 * q + 2] = a.z; v[4 * q + 3] = a.w;
+        for (int q = 0; q + 3 < B; q += 4) {
+            if constexpr (sizeof(T) == 4) {
+                const float4 a = *reinterpret_cast<const float4 *>(p + q);
+                v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
+            } else {
+                const uint2 a = *reinterpret_cast<const uint2 *>(p + q);
+                v[q] = __uint_as_float(a.x << 16); v[q + 1] = __uint_as_float(a.x & 0xffff0000u);
+                v[q + 2] = __uint_as_float(a.y << 16); v[q + 3] = __uint_as_float(a.y & 0xffff0000u);
             }
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < B; ++i) v[i] = p[(int64_t)i * s];
+        for (int i = 0; i < B; ++i) v[i] = to_f32<T>(p[(int64_t)i * s]);
     }
 }
-
-template <int B> __device__ __forceinline__ void store_block(float *p, int64_t s, const float (&v)[B]) {
-    if (s == 1 && (B == 2 || B % 4 == 0)) {
-        if constexpr (B == 2) {
-            *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
-        } else {
+template <int B> __device__ __forceinline__ void store_block(float *p, int64_t s, bool vec, const float (&v)[B]) {
+    if (B % 4 == 0 && vec) {
 #pragma unroll
-            for (int q = 0; q < B / 4; ++q)
-                reinterpret_cast<float4 *>(p)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        }
+        for (int q = 0; q + 3 < B; q += 4) *reinterpret_cast<float4 *>(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
     } else {
 #pragma unroll
         for (int i = 0; i < B; ++i) p[(int64_t)i * s] = v[i];
     }
 }
+__device__ __forceinline__ float sign_of(const int8_t *signs, int64_t i) { return signs && signs[i] < 0 ? -1.f : 1.f; }
 
-// forward stage, block owner: out[r][base_c + j s] = sum_i in[r][base_c + i s] K[c][i][j]
-template <int B>
+// ---- one stage, forward: out[r][base_c + j s] = sum_i in[r][base_c + i s] K[c][i][j]; a thread owns OUT results of block c
+template <int B, int OUT, typename TI>
 __global__ void __launch_bounds__(kOwnThreads)
-fwd_owner_kernel(const float *__restrict__ in, float *__restrict__ out, int64_t rows, int64_t d, int64_t s,
-                 const float *__restrict__ K) {
-    const int64_t c = (int64_t)blockIdx.x * kOwnThreads + threadIdx.x;
-    if (c >= d / B) return;
-    float k[B][B];
-#pragma unroll
-    for (int i = 0; i < B; ++i)
-#pragma unroll
-        for (int j = 0; j < B; ++j) k[i][j] = K[c * (B * B) + i * B + j];
-    prior_kernel_done();
+fwd_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int vec, float *__restrict__ out, int64_t rows, int64_t d, int64_t s,
+           const float *__restrict__ em) {
+    constexpr int PARTS = B / OUT, PER = kOwnThreads / PARTS;
+    const int64_t nblk = d / B, c = (int64_t)blockIdx.x * PER + threadIdx.x % PER;
+    const int o0 = (threadIdx.x / PER) * OUT;
+    if (c >= nblk) return;
     const int64_t alpha = c / s, base = alpha * B * s + (c - alpha * s);
-    const int64_t r0 = (int64_t)blockIdx.y * kFwdSliceRows, r1 = min(rows, r0 + kFwdSliceRows);
-    for (int64_t r = r0; r < r1; r += kRowBatch) {
-        float v[kRowBatch][B];
+    float k[B][OUT];
 #pragma unroll
-        for (int u = 0; u < kRowBatch; ++u)
-            if (r + u < r1) load_block<B>(in + (r + u) * d + base, s, v[u]);
+    for (int i = 0; i < B; ++i) {
+        const float sg = sign_of(signs, base + (int64_t)i * s);
 #pragma unroll
-        for (int u = 0; u < kRowBatch; ++u) {
+        for (int j = 0; j < OUT; ++j) k[i][j] = sg * em[(int64_t)(i * B + o0 + j) * nblk + c];
+    }
+    prior_kernel_done();
+    constexpr int U = B >= 8 ? 2 : 4;
+    const int64_t r0 = (int64_t)blockIdx.y * kFwdRows, r1 = min(rows, r0 + kFwdRows);
+    for (int64_t r = r0; r < r1; r += U) {
+        float v[U][B];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (r + u < r1) load_block<B, TI>(in + (r + u) * d + base, s, vec, v[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
             if (r + u >= r1) break;
-            float o[B];
+            float o[OUT];
 #pragma unroll
-            for (int j = 0; j < B; ++j) {
+            for (int j = 0; j < OUT; ++j) {
                 float acc = 0.f;
 #pragma unroll
                 for (int i = 0; i < B; ++i) acc = fmaf(v[u][i], k[i][j], acc);
                 o[j] = acc;
             }
-            store_block<B>(out + (r + u) * d + base, s, o);
+            store_block<OUT>(out + (r + u) * d + base + (int64_t)o0 * s, s, s == 1, o);
         }
     }
 }
 
-// backward stage, block owner: g_out[r][base_c + i s] = sum_j g[r][base_c + j s] K[c][i][j] (when
-// g_out is given) and part[slice][i B + j][c] = sum over the slice's rows of v[..i..] g[..j..].
-template <int B>
-__global__ void __launch_bounds__(kOwnThreads)
-bwd_owner_kernel(const float *__restrict__ v, const float *__restrict__ g, float *__restrict__ g_out, int64_t rows,
-                 int64_t d, int64_t s, const float *__restrict__ K, double *__restrict__ part) {
-    const int64_t nblk = d / B;
-    const int64_t c = (int64_t)blockIdx.x * kOwnThreads + threadIdx.x;
-    if (c >= nblk) return;
-    float k[B][B];
-    double acc[B][B];
+// CTAs per SM of the backward kernels (registers: 168 per thread from radix 5 to 8, else 128)
+constexpr int k44PerSm = 3;
+__host__ __device__ constexpr int bwd_per_sm(int b, int bi, int subs) { return (b >= 5 && b <= 8 ? 12 : 16) / (((b + bi - 1) / bi) * subs); }
+
+// sums of the warps that split the rows, added in the order of the warps; sum k of a lane goes to dst(k)
+template <int N, int SUBS, typename Dst>
+__device__ __forceinline__ void combine(const double (&acc)[N], double (*sh)[SUBS][32], int sub, int lane, Dst dst) {
+    if constexpr (SUBS > 1) {
 #pragma unroll
-    for (int i = 0; i < B; ++i)
+        for (int k = 0; k < N; ++k) sh[k][sub][lane] = acc[k];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (k % SUBS == sub) {
+                double a = sh[k][0][lane];
+#pragma unroll
+                for (int w = 1; w < SUBS; ++w) a += sh[k][w][lane];
+                if (double *p = dst(k)) *p = a;
+            }
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (double *p = dst(k)) *p = acc[k];
+    }
+}
+
+// ---- one stage, backward: g_out[r][base_c + i s] = sum_j g[r][base_c + j s] K[c][i][j] (when g_out is given) and
+// part[slice][i B + j][c] = sum over the slice's rows of v[..i..] g[..j..]; a thread owns BI values of i of block c
+template <int B, int BI, int SUBS, typename TV, typename TG>
+__global__ void __launch_bounds__(32 * ((B + BI - 1) / BI) * SUBS, bwd_per_sm(B, BI, SUBS))
+bwd_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v, const TG *__restrict__ g, int vec_g, float *__restrict__ g_out,
+           int64_t rows, int64_t d, int64_t s, int slice, const float *__restrict__ em, double *__restrict__ part) {
+    constexpr int PARTS = (B + BI - 1) / BI;
+    __shared__ double sh[SUBS > 1 ? PARTS : 1][SUBS > 1 ? BI * B : 1][SUBS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, pt = w / SUBS, sub = w - pt * SUBS, i0 = pt * BI;
+    const int64_t nblk = d / B, cc = (int64_t)blockIdx.x * 32 + lane;
+    const bool have = cc < nblk;
+    const int64_t c = have ? cc : nblk - 1;
+    const int64_t alpha = c / s, base = alpha * B * s + (c - alpha * s);
+    float k[BI][B], sg[BI];
+    double acc[BI * B];
+#pragma unroll
+    for (int i = 0; i < BI; ++i) {
+        sg[i] = i0 + i < B ? sign_of(signs, base + (int64_t)(i0 + i) * s) : 0.f;
 #pragma unroll
         for (int j = 0; j < B; ++j) {
-            k[i][j] = K[c * (B * B) + i * B + j];
-            acc[i][j] = 0.0;
+            k[i][j] = i0 + i < B ? em[(int64_t)((i0 + i) * B + j) * nblk + c] : 0.f;
+            acc[i * B + j] = 0.0;
         }
+    }
     prior_kernel_done();
-    const int64_t alpha = c / s, base = alpha * B * s + (c - alpha * s);
-    constexpr int U = B >= 7 ? 2 : kRowBatch;         // radices 7 and 8 already fill the register file
-    const int64_t r0 = (int64_t)blockIdx.y * kBwdSliceRows, r1 = min(rows, r0 + kBwdSliceRows);
-    for (int64_t r = r0; r < r1; r += U) {
-        float vv[U][B], gg[U][B];
+    const int64_t r0 = (int64_t)blockIdx.y * slice, r1 = min(rows, r0 + slice);
+    constexpr bool kWhole = B % BI == 0;
+    const bool vec_o = s == 1 && kWhole;
+#pragma unroll (B >= 7 ? 1 : 2)
+    for (int64_t r = r0 + sub; r < r1; r += SUBS) {
+        float vv[BI], gg[B];
+        if constexpr (kWhole) {
+            load_block<BI, TV>(v + r * d + base + (int64_t)i0 * s, s, vec_v, vv);
+        } else {
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (r + u < r1) {
-                load_block<B>(v + (r + u) * d + base, s, vv[u]);
-                load_block<B>(g + (r + u) * d + base, s, gg[u]);
+            for (int i = 0; i < BI; ++i) vv[i] = i0 + i < B ? to_f32<TV>(v[r * d + base + (int64_t)(i0 + i) * s]) : 0.f;
+        }
+        load_block<B, TG>(g + r * d + base, s, vec_g, gg);
+        double gd[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) gd[j] = (double)gg[j];
+#pragma unroll
+        for (int i = 0; i < BI; ++i) {
+            const double vd = (double)(sg[i] * vv[i]);
+#pragma unroll
+            for (int j = 0; j < B; ++j) acc[i * B + j] += vd * gd[j];
+        }
+        if (g_out && have) {
+            float o[BI];
+#pragma unroll
+            for (int i = 0; i < BI; ++i) {
+                float a = 0.f;
+#pragma unroll
+                for (int j = 0; j < B; ++j) a = fmaf(gg[j], k[i][j], a);
+                o[i] = a;
             }
+            float *dst = g_out + r * d + base + (int64_t)i0 * s;
+            if constexpr (kWhole) {
+                store_block<BI>(dst, s, vec_o, o);
+            } else {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (r + u >= r1) break;
-#pragma unroll
-            for (int i = 0; i < B; ++i)
-#pragma unroll
-                for (int j = 0; j < B; ++j) acc[i][j] += (double)vv[u][i] * (double)gg[u][j];
-            if (g_out) {
-                float o[B];
-#pragma unroll
-                for (int i = 0; i < B; ++i) {
-                    float a = 0.f;
-#pragma unroll
-                    for (int j = 0; j < B; ++j) a = fmaf(gg[u][j], k[i][j], a);
-                    o[i] = a;
-                }
-                store_block<B>(g_out + (r + u) * d + base, s, o);
+                for (int i = 0; i < BI; ++i)
+                    if (i0 + i < B) dst[(int64_t)i * s] = o[i];
             }
         }
     }
     double *dst = part + (int64_t)blockIdx.y * (B * B) * nblk + c;
-#pragma unroll
-    for (int i = 0; i < B; ++i)
-#pragma unroll
-        for (int j = 0; j < B; ++j) dst[(int64_t)(i * B + j) * nblk] = acc[i][j];
+    combine<BI * B, SUBS>(acc, SUBS > 1 ? sh[pt] : nullptr, sub, lane, [&](int e) -> double * {
+        const int ij = i0 * B + e;
+        return have && ij < B * B ? dst + (int64_t)ij * nblk : nullptr;
+    });
 }
 
-// Radix 16: a block kernel does not fit one thread's registers, so a thread owns block c and four
-// of its sixteen outputs (forward: columns j0..j0+3 of K[c]; backward: rows i0..i0+3, i.e. the
-// transposed product), with the four threads of a block in the same CTA so that they share the
-// sixteen inputs through L1.
-constexpr int kTileRows16 = 32;    // rows per CTA of the radix-16 kernels (one set of partial sums)
+// ---- two radix-4 stages of strides s and 4 s.  A unit is sixteen coordinates base + (i1 + 4 i2) s; its four threads q hold,
+// in the first stage's order, block i2 = q (coordinates base + 4 q s + i s) and, in the second stage's, block i1 = q
+// (base + q s + 4 j s).  S1 (s == 1): the threads of a unit are neighbouring lanes, a row's sixteen values are loaded as
+// four 16-byte pieces; otherwise eight neighbouring units share a quarter-warp each, so that accesses are whole sectors.
+template <bool S1>
+struct Pair44 {
+    int q;
+    int64_t base, c1, c2;              // first coordinate; block numbers of this thread's two blocks
+    bool have;
+    __device__ __forceinline__ Pair44(int64_t d, int64_t s, int64_t first_unit) {
+        const int lane = threadIdx.x & 31;
+        q = S1 ? lane & 3 : lane >> 3;
+        const int64_t u = first_unit + (S1 ? lane >> 2 : lane & 7);
+        have = u < d / 16;
+        const int64_t uu = have ? u : 0, alpha = uu / s, beta = uu - alpha * s;
+        base = alpha * 16 * s + beta;
+        c1 = (4 * alpha + q) * s + beta;
+        c2 = alpha * 4 * s + beta + q * s;
+    }
+    // x[i] of thread q becomes x[q] of thread i
+    __device__ __forceinline__ void transpose(float (&x)[4]) const {
+        constexpr int M1 = S1 ? 1 : 8, M2 = S1 ? 2 : 16;
+        const bool b0 = q & 1, b1 = q & 2;
+#pragma unroll
+        for (int h = 0; h < 4; h += 2) {
+            const float r = __shfl_xor_sync(0xffffffffu, b0 ? x[h] : x[h + 1], M1);
+            if (b0) x[h] = r; else x[h + 1] = r;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float r = __shfl_xor_sync(0xffffffffu, b1 ? x[h] : x[h + 2], M2);
+            if (b1) x[h] = r; else x[h + 2] = r;
+        }
+    }
+};
+__device__ __forceinline__ void mul4(const float (&x)[4], const float (&k)[4][4], float (&y)[4]) {        // y_j = sum_i x_i k[i][j]
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float a = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a = fmaf(x[i], k[i][j], a);
+        y[j] = a;
+    }
+}
+__device__ __forceinline__ void mul4t(const float (&x)[4], const float (&k)[4][4], float (&y)[4]) {       // y_i = sum_j x_j k[i][j]
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float a = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a = fmaf(x[j], k[i][j], a);
+        y[i] = a;
+    }
+}
 
-__global__ void __launch_bounds__(128)
-stage16_kernel(const float *__restrict__ in, float *__restrict__ out, int64_t rows, int64_t d, int64_t s,
-               const float *__restrict__ K, int transpose) {
-    const int64_t c = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
-    const int t0 = 4 * (threadIdx.x >> 5);
-    if (c >= d / 16) return;
-    float k[16][4];
+template <bool S1, typename TI>
+__global__ void __launch_bounds__(kOwnThreads)
+fwd44_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int vec, float *__restrict__ out, int64_t rows, int64_t d, int64_t s,
+             const float *__restrict__ em1, const float *__restrict__ em2) {
+    const Pair44<S1> u(d, s, ((int64_t)blockIdx.x * (kOwnThreads / 32) + (threadIdx.x >> 5)) * 8);
+    const int64_t nblk = d / 4, in0 = u.base + 4 * u.q * s, out0 = S1 ? in0 : u.base + u.q * s, os = S1 ? 1 : 4 * s;
+    float k1[4][4], k2[4][4];
 #pragma unroll
-    for (int q = 0; q < 16; ++q)
+    for (int i = 0; i < 4; ++i) {
+        const float sg = sign_of(signs, in0 + i * s);
 #pragma unroll
-        for (int t = 0; t < 4; ++t) k[q][t] = K[c * 256 + (transpose ? (t0 + t) * 16 + q : q * 16 + t0 + t)];
+        for (int j = 0; j < 4; ++j) {
+            k1[i][j] = sg * em1[(int64_t)(i * 4 + j) * nblk + u.c1];
+            k2[i][j] = em2[(int64_t)(i * 4 + j) * nblk + u.c2];
+        }
+    }
     prior_kernel_done();
-    const int64_t alpha = c / s, base = alpha * 16 * s + (c - alpha * s);
-    const int64_t r0 = (int64_t)blockIdx.y * kFwdSliceRows, r1 = min(rows, r0 + kFwdSliceRows);
-#pragma unroll 2
-    for (int64_t r = r0; r < r1; ++r) {
-        float v[16];
-        load_block<16>(in + r * d + base, s, v);
-        float o[4] = {0.f, 0.f, 0.f, 0.f};
+    const int64_t r0 = (int64_t)blockIdx.y * kFwdRows, r1 = min(rows, r0 + kFwdRows);
+    const TI *p = in + r0 * d + in0;
+    float *w = out + r0 * d + out0;
+    float x[4][4];
+    for (int64_t r = r0; r < r1; r += 4, p += 4 * d, w += 4 * d) {
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
+        for (int n = 0; n < 4; ++n)
+            if (r + n < r1) load_block<4, TI>(p + n * d, s, vec, x[n]);
 #pragma unroll
-            for (int t = 0; t < 4; ++t) o[t] = fmaf(v[q], k[q][t], o[t]);
-        float *dst = out + r * d + base + (int64_t)t0 * s;
-        if (s == 1) {
-            *reinterpret_cast<float4 *>(dst) = make_float4(o[0], o[1], o[2], o[3]);
-        } else {
-#pragma unroll
-            for (int t = 0; t < 4; ++t) dst[(int64_t)t * s] = o[t];
+        for (int n = 0; n < 4; ++n) {
+            if (r + n >= r1) break;
+            float y[4], z[4];
+            mul4(x[n], k1, y);
+            u.transpose(y);
+            mul4(y, k2, z);
+            if (S1) u.transpose(z);
+            if (u.have) store_block<4>(w + n * d, os, S1, z);
         }
     }
 }
 
-// part[slice][i 16 + j][c] = sum over the slice's rows of v[base_c + i s] g[base_c + j s]; a thread
-// owns block c and a 4 x 4 tile of (i, j); the sixteen tiles of a block sit in the same CTA.
-__global__ void __launch_bounds__(512)
-outer16_kernel(const float *__restrict__ v, const float *__restrict__ g, int64_t rows, int64_t d, int64_t s,
-               double *__restrict__ part) {
-    const int64_t nblk = d / 16;
-    const int64_t c = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
-    const int tile = threadIdx.x >> 5, i0 = 4 * (tile >> 2), j0 = 4 * (tile & 3);
-    if (c >= nblk) return;
-    double acc[4][4];
+template <bool S1, typename TV, typename TG>
+__global__ void __launch_bounds__(32 * kSubs, k44PerSm)
+bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v, const TG *__restrict__ g, int vec_g, float *__restrict__ g_out,
+             int64_t rows, int64_t d, int64_t s, int slice, const float *__restrict__ em1, const float *__restrict__ em2, double *__restrict__ part1,
+             double *__restrict__ part2) {
+    __shared__ double sh[32][kSubs][32];
+    const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
+    const Pair44<S1> u(d, s, (int64_t)blockIdx.x * 8);
+    const int64_t nblk = d / 4, first = u.base + 4 * u.q * s, second = S1 ? first : u.base + u.q * s, gs = S1 ? 1 : 4 * s;
+    float k1[4][4], k2[4][4], sg[4];
+    double acc[32];                            // first stage's sums, second stage's
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i) {
+        sg[i] = sign_of(signs, first + i * s);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+        for (int j = 0; j < 4; ++j) {
+            k1[i][j] = em1[(int64_t)(i * 4 + j) * nblk + u.c1];
+            k2[i][j] = em2[(int64_t)(i * 4 + j) * nblk + u.c2];
+            acc[i * 4 + j] = acc[16 + i * 4 + j] = 0.0;
+        }
+    }
     prior_kernel_done();
-    const int64_t alpha = c / s, base = alpha * 16 * s + (c - alpha * s);
-    const int64_t r0 = (int64_t)blockIdx.y * kTileRows16, r1 = min(rows, r0 + kTileRows16);
-    for (int64_t r = r0; r < r1; r += 2) {
-        float vv[2][4], gg[2][4];
+    const int64_t r0 = (int64_t)blockIdx.y * slice + sub, r1 = min(rows, (int64_t)(blockIdx.y + 1) * slice);
+    const TV *pv = v + r0 * d + first;
+    const TG *pg = g + r0 * d + second;
+    float *w = g_out ? g_out + r0 * d + first : nullptr;
+    float nv[4], ng[4];
+    if (r0 < r1) {
+        load_block<4, TV>(pv, s, vec_v, nv);
+        load_block<4, TG>(pg, gs, vec_g, ng);
+    }
+    for (int64_t r = r0; r < r1; r += kSubs) {
+        float x[4], y[4], gy[4], h[4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
-            if (r + u < r1) {
-                load_block<4>(v + (r + u) * d + base + (int64_t)i0 * s, s, vv[u]);
-                load_block<4>(g + (r + u) * d + base + (int64_t)j0 * s, s, gg[u]);
+        for (int i = 0; i < 4; ++i) { x[i] = sg[i] * nv[i]; gy[i] = ng[i]; }
+        pv += kSubs * d;
+        pg += kSubs * d;
+        if (r + kSubs < r1) {                  // the next row's values are on their way
+            load_block<4, TV>(pv, s, vec_v, nv);
+            load_block<4, TG>(pg, gs, vec_g, ng);
+        }
+        if (S1) u.transpose(gy);
+        mul4(x, k1, y);
+        u.transpose(y);
+        {
+            double gd[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) gd[j] = (double)gy[j];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const double vd = (double)y[i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[16 + i * 4 + j] += vd * gd[j];
+            }
+        }
+        mul4t(gy, k2, h);
+        u.transpose(h);
+        {
+            double gd[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) gd[j] = (double)h[j];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const double vd = (double)x[i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i * 4 + j] += vd * gd[j];
+            }
+        }
+        if (w) {
+            float o[4];
+            mul4t(h, k1, o);
+            if (u.have) store_block<4>(w, s, S1, o);
+            w += kSubs * d;
+        }
+    }
+    double *d1 = part1 + (int64_t)blockIdx.y * 16 * nblk + u.c1, *d2 = part2 + (int64_t)blockIdx.y * 16 * nblk + u.c2;
+    combine<32, kSubs>(acc, sh, sub, lane, [&](int e) -> double * {
+        return !u.have ? nullptr : e < 16 ? d1 + (int64_t)e * nblk : d2 + (int64_t)(e - 16) * nblk;
+    });
+}
+
+// ---- two radix-2 stages of strides s and 2 s: a thread holds the four coordinates base + (i1 + 2 i2) s
+struct Pair22 {
+    int64_t base, c1[2], c2[2];        // block numbers: first stage at i2 = 0, 1, second stage at i1 = 0, 1
+    bool have;
+    __device__ __forceinline__ Pair22(int64_t d, int64_t s, int64_t unit) {
+        have = unit < d / 4;
+        const int64_t u = have ? unit : 0;
+        const int64_t alpha = u / s, beta = u - alpha * s;
+        base = alpha * 4 * s + beta;
+        c1[0] = 2 * alpha * s + beta;
+        c1[1] = c1[0] + s;
+        c2[0] = 2 * alpha * s + beta;
+        c2[1] = c2[0] + s;
+    }
+};
+
+template <typename TI>
+__global__ void __launch_bounds__(kOwnThreads)
+fwd22_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int vec, float *__restrict__ out, int64_t rows, int64_t d, int64_t s,
+             const float *__restrict__ em1, const float *__restrict__ em2) {
+    const Pair22 u(d, s, (int64_t)blockIdx.x * kOwnThreads + threadIdx.x);
+    if (!u.have) return;
+    const int64_t nblk = d / 2;
+    float k1[2][2][2], k2[2][2][2];
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float sg = sign_of(signs, u.base + (i + 2 * b) * s);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                k1[b][i][j] = sg * em1[(int64_t)(i * 2 + j) * nblk + u.c1[b]];
+                k2[b][i][j] = em2[(int64_t)(i * 2 + j) * nblk + u.c2[b]];
+            }
+        }
+    prior_kernel_done();
+    const int64_t r0 = (int64_t)blockIdx.y * kFwdRows, r1 = min(rows, r0 + kFwdRows);
+    const TI *p = in + r0 * d + u.base;
+    float *w = out + r0 * d + u.base;
+    for (int64_t r = r0; r < r1; r += 4, p += 4 * d, w += 4 * d) {
+        float x[4][4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+            if (r + n < r1) load_block<4, TI>(p + n * d, s, vec, x[n]);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            if (r + n >= r1) break;
+            float y[4], z[4];
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) y[j + 2 * b] = fmaf(x[n][1 + 2 * b], k1[b][1][j], fmaf(x[n][2 * b], k1[b][0][j], 0.f));
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) z[b + 2 * j] = fmaf(y[b + 2], k2[b][1][j], fmaf(y[b], k2[b][0][j], 0.f));
+            store_block<4>(w + n * d, s, s == 1, z);
+        }
+    }
+}
+
+template <typename TV, typename TG>
+__global__ void __launch_bounds__(32 * kSubs, 4)
+bwd22_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v, const TG *__restrict__ g, int vec_g, float *__restrict__ g_out,
+             int64_t rows, int64_t d, int64_t s, int slice, const float *__restrict__ em1, const float *__restrict__ em2, double *__restrict__ part1,
+             double *__restrict__ part2) {
+    __shared__ double sh[16][kSubs][32];
+    const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
+    const Pair22 u(d, s, (int64_t)blockIdx.x * 32 + lane);
+    const int64_t nblk = d / 2;
+    float k1[2][2][2], k2[2][2][2], sg[4];
+    double acc[16];                            // first stage's sums [i2][i][j], second stage's [i1][i][j]
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            sg[i + 2 * b] = sign_of(signs, u.base + (i + 2 * b) * s);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                k1[b][i][j] = em1[(int64_t)(i * 2 + j) * nblk + u.c1[b]];
+                k2[b][i][j] = em2[(int64_t)(i * 2 + j) * nblk + u.c2[b]];
+                acc[b * 4 + i * 2 + j] = acc[8 + b * 4 + i * 2 + j] = 0.0;
+            }
+        }
+    prior_kernel_done();
+    const int64_t r0 = (int64_t)blockIdx.y * slice + sub, r1 = min(rows, (int64_t)(blockIdx.y + 1) * slice);
+    constexpr int U = 2;
+    for (int64_t r = r0; r < r1; r += U * kSubs) {
+        float xx[U][4], gg[U][4];
+#pragma unroll
+        for (int n = 0; n < U; ++n)
+            if (r + n * kSubs < r1) {
+                load_block<4, TV>(v + (r + n * kSubs) * d + u.base, s, vec_v, xx[n]);
+                load_block<4, TG>(g + (r + n * kSubs) * d + u.base, s, vec_g, gg[n]);
             }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (r + u >= r1) break;
+        for (int n = 0; n < U; ++n) {
+            if (r + n * kSubs >= r1) break;
+            float x[4], y[4], h[4], o[4];
+            double xd[4], yd[4], gd[4], hd[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 4; ++i) x[i] = sg[i] * xx[n][i];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += (double)vv[u][i] * (double)gg[u][j];
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    y[j + 2 * b] = fmaf(x[1 + 2 * b], k1[b][1][j], fmaf(x[2 * b], k1[b][0][j], 0.f));
+                    // gradient behind the first stage: sum over the second stage's results
+                    h[b + 2 * j] = fmaf(gg[n][b + 2], k2[b][j][1], fmaf(gg[n][b], k2[b][j][0], 0.f));
+                }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { xd[i] = (double)x[i]; yd[i] = (double)y[i]; gd[i] = (double)gg[n][i]; hd[i] = (double)h[i]; }
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        acc[8 + b * 4 + i * 2 + j] += yd[b + 2 * i] * gd[b + 2 * j];
+                        acc[b * 4 + i * 2 + j] += xd[i + 2 * b] * hd[j + 2 * b];
+                    }
+            if (g_out && u.have) {
+#pragma unroll
+                for (int b = 0; b < 2; ++b)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) o[i + 2 * b] = fmaf(h[1 + 2 * b], k1[b][i][1], fmaf(h[2 * b], k1[b][i][0], 0.f));
+                store_block<4>(g_out + (r + n * kSubs) * d + u.base, s, s == 1, o);
+            }
         }
     }
-    double *dst = part + (int64_t)blockIdx.y * 256 * nblk + c;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) dst[(int64_t)((i0 + i) * 16 + j0 + j) * nblk] = acc[i][j];
+    double *d1 = part1 + (int64_t)blockIdx.y * 4 * nblk, *d2 = part2 + (int64_t)blockIdx.y * 4 * nblk;
+    combine<16, kSubs>(acc, sh, sub, lane, [&](int e) -> double * {
+        if (!u.have) return nullptr;
+        const int b = (e >> 2) & 1, ij = e & 3;
+        return e < 8 ? d1 + (int64_t)ij * nblk + u.c1[b] : d2 + (int64_t)ij * nblk + u.c2[b];
+    });
 }
 
-// grad[c][i][j] (+)= sum over slices of part[slice][i b + j][c].  A CTA owns 32 neighbouring
-// entries (one per lane); warp w adds the slices w, w + 8, ... and the eight sums are added in
-// the order of w, so the result does not depend on scheduling.
+// ---- sums over slices of all stages that keep partial sums: grad[c][i][j] (+)= sum over slices of part[slice][i b + j][c],
+// slices in order, eight warps taking every eighth slice and their sums added in the order of the warps
+struct ReduceStage { int64_t off, part_off, n_blk, total; int32_t bb, rows, n_slices; };
+struct ReduceTable { int32_t m; int64_t total; ReduceStage st[HARP_MAX_STAGES]; };
+
 __global__ void __launch_bounds__(kThreads)
-reduce_slices_kernel(const double *__restrict__ part, int64_t n_slices, int64_t nblk, int bb, float *__restrict__ grad,
-                     int accumulate) {
+reduce_kernel(const double *__restrict__ part, float *__restrict__ grad, int accumulate, const ReduceTable tab) {
     prior_kernel_done();
     __shared__ double warp_sum[kThreads / 32][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t total = nblk * bb;
-    for (int64_t q0 = (int64_t)blockIdx.x * 32; q0 < total; q0 += (int64_t)gridDim.x * 32) {
-        const int64_t q = q0 + lane;
+    for (int64_t q0 = (int64_t)blockIdx.x * 32; q0 < tab.total; q0 += (int64_t)gridDim.x * 32) {
+        int64_t q = q0 + lane;
+        const bool have = q < tab.total;
+        int t = 0;
+        while (t + 1 < tab.m && q >= tab.st[t].total) { q -= tab.st[t].total; ++t; }
+        const ReduceStage &s = tab.st[t];
         double sum = 0.0;
-        if (q < total) {
+        if (have) {
+            const double *p = part + s.part_off + q;
 #pragma unroll 4
-            for (int64_t sl = w; sl < n_slices; sl += kThreads / 32) sum += part[sl * total + q];
+            for (int sl = w; sl < s.n_slices; sl += kThreads / 32) sum += p[(int64_t)sl * s.total];
         }
         warp_sum[w][lane] = sum;
         __syncthreads();
-        if (w == 0 && q < total) {
+        if (w == 0 && have) {
             double all = warp_sum[0][lane];
             for (int k = 1; k < kThreads / 32; ++k) all += warp_sum[k][lane];
-            const int64_t ij = q / nblk, c = q - ij * nblk;
-            float *dst = grad + c * bb + ij;
+            const int64_t ij = q / s.n_blk, c = q - ij * s.n_blk;
+            float *dst = grad + s.off + c * s.bb + ij;
             *dst = accumulate ? *dst + (float)all : (float)all;
         }
         __syncthreads();
     }
 }
 
-// position of element i in the staged row of load_rows_kernel: two elements of padding per 64,
-// so that a digit-reversal gather (strides of 64 elements and more) spreads over the banks
-__device__ __forceinline__ int64_t staged_pos(int64_t i) { return i + 2 * (i >> 6); }
-
-// as load_kernel, one CTA per row: the row of x is read in order into shared memory and gathered
-// from there, so the permutation costs no scattered global reads
+// ---- x with the permutation and the signs of the plan, rows of the same type: out[r][i] = s[perm[i]] x[r][perm[i]].  A row at
+// a time through shared memory (two elements of padding per 64 keep a digit reversal off the same banks); staged = 0: rows
+// too long for that are gathered from global memory
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-load_rows_kernel(const T *__restrict__ x, const T *__restrict__ gy, int64_t rows, int64_t d, const int32_t *__restrict__ perm,
-                 const int8_t *__restrict__ signs, float *__restrict__ v0, float *__restrict__ g) {
+permute_kernel(const T *__restrict__ x, int vec, T *__restrict__ out, int64_t rows, int64_t d, const int32_t *__restrict__ perm,
+               const int8_t *__restrict__ signs, int staged) {
     prior_kernel_done();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *row = reinterpret_cast<T *>(smem_raw);
-    constexpr int V = 16 / (int)sizeof(T);                 // elements per 16-byte access
-    // 16-byte accesses when every row starts on a 16-byte boundary; V divides 64, so the V elements
-    // of one access stay next to each other in the staged row
-    const bool vec = d % V == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(gy)) & 15) == 0;
+    constexpr int V = 16 / (int)sizeof(T);
     for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
-        if (vec) {
-            for (int64_t i = (int64_t)threadIdx.x * V; i < d; i += (int64_t)kThreads * V) {
-                const uint4 raw = *reinterpret_cast<const uint4 *>(x + r * d + i);
-                const uint32_t *w = reinterpret_cast<const uint32_t *>(&raw);
-                uint32_t *dst = reinterpret_cast<uint32_t *>(row + staged_pos(i));   // 4-byte aligned: staged_pos(i) is even
-#pragma unroll
-                for (int k = 0; k < 4; ++k) dst[k] = w[k];
-                const uint4 rg = *reinterpret_cast<const uint4 *>(gy + r * d + i);
-                const T *tg = reinterpret_cast<const T *>(&rg);
-                float *gd = g + r * d + i;
-#pragma unroll
-                for (int k = 0; k < V; k += 4)
-                    *reinterpret_cast<float4 *>(gd + k) =
-                        make_float4(to_f32<T>(tg[k]), to_f32<T>(tg[k + 1]), to_f32<T>(tg[k + 2]), to_f32<T>(tg[k + 3]));
+        if (staged) {
+            if (vec) {
+#pragma unroll 2
+                for (int64_t i = (int64_t)threadIdx.x * V; i < d; i += kThreads * V) {
+                    const uint4 q = *reinterpret_cast<const uint4 *>(x + r * d + i);
+                    uint32_t *dst = reinterpret_cast<uint32_t *>(row + i + 2 * (i >> 6));     // 4-byte aligned: the index is even
+                    dst[0] = q.x; dst[1] = q.y; dst[2] = q.z; dst[3] = q.w;
+                }
+            } else {
+                for (int64_t i = threadIdx.x; i < d; i += kThreads) row[i + 2 * (i >> 6)] = x[r * d + i];
             }
-        } else {
-            for (int64_t i = threadIdx.x; i < d; i += kThreads) {
-                row[staged_pos(i)] = x[r * d + i];
-                g[r * d + i] = to_f32<T>(gy[r * d + i]);
-            }
+            __syncthreads();
         }
-        __syncthreads();
         if (d % 4 == 0) {
-            for (int64_t i = (int64_t)threadIdx.x * 4; i < d; i += (int64_t)kThreads * 4) {
-                const int4 src = *reinterpret_cast<const int4 *>(perm + i);
-                const int sidx[4] = {src.x, src.y, src.z, src.w};
-                float o[4];
+            for (int64_t i = (int64_t)threadIdx.x * 4; i < d; i += kThreads * 4) {
+                const int4 s4 = *reinterpret_cast<const int4 *>(perm + i);
+                const int src[4] = {s4.x, s4.y, s4.z, s4.w};
+                __align__(16) T o[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const float sg = (signs && signs[sidx[k]] < 0) ? -1.f : 1.f;
-                    o[k] = sg * to_f32<T>(row[staged_pos(sidx[k])]);
+                    const T v = staged ? row[src[k] + 2 * (src[k] >> 6)] : x[r * d + src[k]];
+                    o[k] = signs && signs[src[k]] < 0 ? (T)-v : v;
                 }
-                *reinterpret_cast<float4 *>(v0 + r * d + i) = make_float4(o[0], o[1], o[2], o[3]);
+                if constexpr (sizeof(T) == 2) *reinterpret_cast<uint2 *>(out + r * d + i) = *reinterpret_cast<const uint2 *>(o);
+                else *reinterpret_cast<uint4 *>(out + r * d + i) = *reinterpret_cast<const uint4 *>(o);
             }
         } else {
             for (int64_t i = threadIdx.x; i < d; i += kThreads) {
-                const int64_t src = perm[i];
-                const float sg = (signs && signs[src] < 0) ? -1.f : 1.f;
-                v0[r * d + i] = sg * to_f32<T>(row[staged_pos(src)]);
+                const int src = perm[i];
+                const T v = staged ? row[src + 2 * (src >> 6)] : x[r * d + src];
+                out[r * d + i] = signs && signs[src] < 0 ? (T)-v : v;
             }
         }
         __syncthreads();
-    }
-}
-
-// v0[r][i] = s[perm[i]] * x[r][perm[i]],  g[r][i] = gy[r][i]   (both fp32)
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-load_kernel(const T *__restrict__ x, const T *__restrict__ gy, int64_t rows, int64_t d, const int32_t *__restrict__ perm,
-            const int8_t *__restrict__ signs, float *__restrict__ v0, float *__restrict__ g) {
-    prior_kernel_done();
-    // a thread keeps its coordinate and walks over rows (blockIdx.y, then in steps of gridDim.y)
-    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (i >= d) return;
-    const int64_t src = perm ? perm[i] : i;
-    const float sg = (signs && signs[src] < 0) ? -1.f : 1.f;
-    for (int64_t r = blockIdx.y; r < rows; r += gridDim.y) {
-        v0[r * d + i] = sg * to_f32<T>(x[r * d + src]);
-        g[r * d + i] = to_f32<T>(gy[r * d + i]);
     }
 }
 
@@ -381,8 +632,9 @@ load_kernel(const T *__restrict__ x, const T *__restrict__ gy, int64_t rows, int
 // Neighbouring lanes hold neighbouring positions: inside one block when s is small, in neighbouring
 // blocks otherwise -- so K is read block-major (entry k of block c at c b^2 + k) for s < 8 and
 // element-major (at k D + c) from s = 8 on; kc_step / kk_step are the two strides of that choice.
+template <typename TI>
 __global__ void __launch_bounds__(kThreads)
-stage_kernel(const float *__restrict__ in, float *__restrict__ out, int64_t rows, int64_t d, int b, int64_t s,
+stage_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, float *__restrict__ out, int64_t rows, int64_t d, int b, int64_t s,
              const float *__restrict__ K, int64_t kc_step, int64_t kk_step, int transpose) {
     prior_kernel_done();
     // a thread keeps its position (the index arithmetic is done once) and walks over rows
@@ -394,9 +646,12 @@ stage_kernel(const float *__restrict__ in, float *__restrict__ out, int64_t rows
     const float *Kc = K + (alpha * s + beta) * kc_step + (transpose ? j * b : j) * kk_step;
     const int64_t k_step = (transpose ? 1 : (int64_t)b) * kk_step;     // from K[..][i][j] to K[..][i+1][j] (or [j][i+1])
     for (int64_t r = blockIdx.y; r < rows; r += gridDim.y) {
-        const float *row = in + r * d + base;
+        const TI *row = in + r * d + base;
         float acc = 0.f;
-        for (int i = 0; i < b; ++i) acc = fmaf(row[(int64_t)i * s], Kc[(int64_t)i * k_step], acc);
+        for (int i = 0; i < b; ++i) {
+            const float v = to_f32<TI>(row[(int64_t)i * s]);
+            acc = fmaf(signs && signs[base + (int64_t)i * s] < 0 ? -v : v, Kc[(int64_t)i * k_step], acc);
+        }
         out[r * d + pos] = acc;
     }
 }
@@ -406,8 +661,9 @@ stage_kernel(const float *__restrict__ in, float *__restrict__ out, int64_t rows
 // are added in a fixed order, so the result does not depend on scheduling.
 // The 32 entries are neighbours within a block for s < 8 and the same entry of 32 neighbouring
 // blocks from s = 8 on (by_block = 0), so that the lanes read neighbouring coordinates either way.
+template <typename TV, typename TG>
 __global__ void __launch_bounds__(kThreads)
-outer_kernel(const float *__restrict__ v, const float *__restrict__ g, int64_t rows, int64_t d, int b, int64_t s,
+outer_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const TG *__restrict__ g, int64_t rows, int64_t d, int b, int64_t s,
              float *__restrict__ grad, int accumulate, int by_block) {
     prior_kernel_done();
     __shared__ double part[kThreads / 32][32];
@@ -424,8 +680,10 @@ outer_kernel(const float *__restrict__ v, const float *__restrict__ g, int64_t r
             const int64_t i = ij / b, j = ij - i * b;
             const int64_t alpha = c / s, beta = c - alpha * s;
             const int64_t base = alpha * b * s + beta;
-            const float *pv = v + base + i * s, *pg = g + base + j * s;
-            for (int64_t r = w; r < rows; r += kThreads / 32) acc += (double)pv[r * d] * (double)pg[r * d];
+            const TV *pv = v + base + i * s;
+            const TG *pg = g + base + j * s;
+            for (int64_t r = w; r < rows; r += kThreads / 32) acc += (double)to_f32<TV>(pv[r * d]) * (double)to_f32<TG>(pg[r * d]);
+            if (signs && signs[base + i * s] < 0) acc = -acc;
         }
         part[w][lane] = acc;
         __syncthreads();
@@ -472,54 +730,194 @@ dim3 column_grid(int64_t d, int64_t rows) {
     return dim3((unsigned)gx, (unsigned)gy);
 }
 
-bool owner_radix(int b) { return b >= 2 && b <= 8; }
+// ---- steps of a plan
 
-dim3 owner_grid16(int64_t d, int64_t rows, int slice_rows) {
-    return dim3((unsigned)((d / 16 + 31) / 32), (unsigned)((rows + slice_rows - 1) / slice_rows));
+struct Step { int t, n; };             // stages [t, t + n): one stage, or two of radix 4 or of radix 2
+
+std::vector<Step> make_steps(const StageTable &st) {
+    std::vector<Step> steps;
+    for (int t = 0; t < st.m;) {
+        const int b = st.b[t];
+        const bool two = t + 1 < st.m && st.b[t + 1] == b && (b == 4 || b == 2);
+        steps.push_back({t, two ? 2 : 1});
+        t += two ? 2 : 1;
+    }
+    return steps;
 }
 
-dim3 owner_grid(int64_t d, int b, int64_t rows, int slice_rows) {
-    return dim3((unsigned)((d / b + kOwnThreads - 1) / kOwnThreads), (unsigned)((rows + slice_rows - 1) / slice_rows));
-}
-
-void launch_fwd_owner(int b, const float *in, float *out, int64_t rows, int64_t d, int64_t s, const float *K, cudaStream_t st) {
-    const dim3 grid = owner_grid(d, b, rows, kFwdSliceRows);
+bool owner_radix(int b) { return (b >= 2 && b <= 8) || b == 16; }
+// A backward kernel runs as one wave of CTAs, each with the largest number of rows that needs (a wave and a sixth takes as
+// long as two: 2048 rows of d = 4096, 52 us with 128 rows per CTA): columns of CTAs, CTAs per SM -> rows per CTA
+struct Shape { int64_t x; int per_sm; };
+Shape bwd_shape(const harp_plan *plan, const Step &sp) {
+    const int64_t d = plan->d;
+    const int b = plan->st.b[sp.t];
+    if (sp.n == 2) return b == 4 ? Shape{(d / 16 + 7) / 8, k44PerSm} : Shape{(d / 4 + 31) / 32, 4};
+    const int64_t x = (d / b + 31) / 32;
     switch (b) {
-        case 2: launch_dep(fwd_owner_kernel<2>, dim3(grid), dim3(kOwnThreads), 0, st, in, out, rows, d, s, K); break;
-        case 3: launch_dep(fwd_owner_kernel<3>, dim3(grid), dim3(kOwnThreads), 0, st, in, out, rows, d, s, K); break;
-        case 4: launch_dep(fwd_owner_kernel<4>, dim3(grid), dim3(kOwnThreads), 0, st, in, out, rows, d, s, K); break;
-        case 5: launch_dep(fwd_owner_kernel<5>, dim3(grid), dim3(kOwnThreads), 0, st, in, out, rows, d, s, K); break;
-        case 6: launch_dep(fwd_owner_kernel<6>, dim3(grid), dim3(kOwnThreads), 0, st, in, out, rows, d, s, K); break;
-        case 7: launch_dep(fwd_owner_kernel<7>, dim3(grid), dim3(kOwnThreads), 0, st, in, out, rows, d, s, K); break;
-        default: launch_dep(fwd_owner_kernel<8>, dim3(grid), dim3(kOwnThreads), 0, st, in, out, rows, d, s, K); break;
+        case 7: case 8: return {x, bwd_per_sm(b, 4, 2)};
+        case 16: return {x, bwd_per_sm(16, 2, 1)};
+        case 5: return {x, bwd_per_sm(5, 5, kSubs)};
+        case 6: return {x, bwd_per_sm(6, 3, kSubs)};
+        default: return {x, bwd_per_sm(b, b, kSubs)};
     }
 }
+int slice_rows(const harp_plan *plan, const Step &sp, int64_t rows, int sms) {
+    const Shape sh = bwd_shape(plan, sp);
+    const int64_t y = std::max<int64_t>(1, sms * (int64_t)sh.per_sm / sh.x);
+    return (int)std::max<int64_t>(8, (rows + y - 1) / y);
+}
+bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+dim3 grid2(int64_t x, int per_x, int64_t rows, int per_y) { return dim3((unsigned)((x + per_x - 1) / per_x), (unsigned)((rows + per_y - 1) / per_y)); }
 
-void launch_bwd_owner(int b, const float *v, const float *g, float *g_out, int64_t rows, int64_t d, int64_t s, const float *K,
-                      double *part, cudaStream_t st) {
-    const dim3 grid = owner_grid(d, b, rows, kBwdSliceRows);
-    switch (b) {
-        case 2: launch_dep(bwd_owner_kernel<2>, dim3(grid), dim3(kOwnThreads), 0, st, v, g, g_out, rows, d, s, K, part); break;
-        case 3: launch_dep(bwd_owner_kernel<3>, dim3(grid), dim3(kOwnThreads), 0, st, v, g, g_out, rows, d, s, K, part); break;
-        case 4: launch_dep(bwd_owner_kernel<4>, dim3(grid), dim3(kOwnThreads), 0, st, v, g, g_out, rows, d, s, K, part); break;
-        case 5: launch_dep(bwd_owner_kernel<5>, dim3(grid), dim3(kOwnThreads), 0, st, v, g, g_out, rows, d, s, K, part); break;
-        case 6: launch_dep(bwd_owner_kernel<6>, dim3(grid), dim3(kOwnThreads), 0, st, v, g, g_out, rows, d, s, K, part); break;
-        case 7: launch_dep(bwd_owner_kernel<7>, dim3(grid), dim3(kOwnThreads), 0, st, v, g, g_out, rows, d, s, K, part); break;
-        default: launch_dep(bwd_owner_kernel<8>, dim3(grid), dim3(kOwnThreads), 0, st, v, g, g_out, rows, d, s, K, part); break;
+// one step forward: out = in through the step's stages
+template <typename TI>
+void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int8_t *signs, float *out, int64_t rows, cudaStream_t st) {
+    const int64_t d = plan->d, s = plan->st.s[sp.t];
+    const int b = plan->st.b[sp.t];
+    const float *em = plan->d_blocks_em + plan->st.off[sp.t];
+    const float *em2 = sp.n == 2 ? plan->d_blocks_em + plan->st.off[sp.t + 1] : nullptr;
+    const int vec = s == 1 && d % 4 == 0 && aligned16(in);
+    if (sp.n == 2 && b == 4) {
+        const dim3 grid = grid2(d / 16, 8 * (kOwnThreads / 32), rows, kFwdRows);
+        if (s == 1) launch_dep(fwd44_kernel<true, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, em, em2);
+        else launch_dep(fwd44_kernel<false, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, em, em2);
+        return;
     }
+    if (sp.n == 2) {
+        launch_dep(fwd22_kernel<TI>, grid2(d / 4, kOwnThreads, rows, kFwdRows), dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, em, em2);
+        return;
+    }
+#define HARP_FWD(B, OUT) case B: launch_dep(fwd_kernel<B, OUT, TI>, grid2(d / B, kOwnThreads / (B / OUT), rows, kFwdRows), dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, em); return
+    switch (b) {
+        HARP_FWD(2, 2); HARP_FWD(3, 3); HARP_FWD(4, 4); HARP_FWD(5, 5); HARP_FWD(6, 6); HARP_FWD(7, 7); HARP_FWD(8, 4); HARP_FWD(16, 4);
+        default: break;
+    }
+#undef HARP_FWD
+    const bool by_em = s >= 8;                     // see stage_kernel
+    launch_dep(stage_kernel<TI>, column_grid(d, rows), dim3(kThreads), 0, st, in, signs, out, rows, d, b, s, by_em ? em : plan->d_blocks + plan->st.off[sp.t],
+               by_em ? 1 : (int64_t)b * b, by_em ? d / b : 1, 0);
+}
+
+// one step backward: g_out (unless null) from g, sums of the step's outer products into part (or, radices without owner
+// kernels, into grad)
+template <typename TV, typename TG>
+int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8_t *signs, const TG *g, float *g_out, int64_t rows, double *part, double *part2,
+                  int slice, float *grad, int acc, cudaStream_t st) {
+    const int64_t d = plan->d, s = plan->st.s[sp.t];
+    const int b = plan->st.b[sp.t];
+    const float *em = plan->d_blocks_em + plan->st.off[sp.t];
+    const float *em2 = sp.n == 2 ? plan->d_blocks_em + plan->st.off[sp.t + 1] : nullptr;
+    const int vec_v = s == 1 && d % 4 == 0 && aligned16(v), vec_g = s == 1 && d % 4 == 0 && aligned16(g);
+    if (sp.n == 2 && b == 4) {
+        const dim3 grid = grid2(d / 16, 8, rows, slice);
+        if (s == 1) launch_dep(bwd44_kernel<true, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, em2, part, part2);
+        else launch_dep(bwd44_kernel<false, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, em2, part, part2);
+        return 1;
+    }
+    if (sp.n == 2) {
+        launch_dep(bwd22_kernel<TV, TG>, grid2(d / 4, 32, rows, slice), dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, em2, part, part2);
+        return 1;
+    }
+#define HARP_BWD(B, BI, SUBS) case B: launch_dep(bwd_kernel<B, BI, SUBS, TV, TG>, grid2(d / B, 32, rows, slice), dim3(32 * ((B + BI - 1) / BI) * SUBS), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, part); return 1
+    switch (b) {
+        HARP_BWD(2, 2, kSubs); HARP_BWD(3, 3, kSubs); HARP_BWD(4, 4, kSubs); HARP_BWD(5, 5, kSubs); HARP_BWD(6, 3, kSubs); HARP_BWD(7, 4, 2);
+        HARP_BWD(8, 4, 2); HARP_BWD(16, 2, 1);
+        default: break;
+    }
+#undef HARP_BWD
+    const bool by_em = s >= 8;
+    launch_dep(outer_kernel<TV, TG>, dim3((unsigned)std::min<int64_t>((d * b + 31) / 32, 148 * 64)), dim3(kThreads), 0, st, v, signs, g, rows, d, b, s,
+               grad + plan->st.off[sp.t], acc, by_em ? 0 : 1);
+    if (!g_out) return 1;
+    launch_dep(stage_kernel<TG>, column_grid(d, rows), dim3(kThreads), 0, st, g, (const int8_t *)nullptr, g_out, rows, d, b, s,
+               by_em ? em : plan->d_blocks + plan->st.off[sp.t], by_em ? 1 : (int64_t)b * b, by_em ? d / b : 1, 1);
+    return 2;
 }
 
 template <typename T>
-void launch_load(const T *x, const T *gy, int64_t rows, int64_t d, const harp_plan_t *plan, float *v0, float *g, cudaStream_t st) {
-    const size_t smem = (size_t)(d + 2 * (d >> 6) + 2) * sizeof(T);
-    // per call: the attribute belongs to the current device's copy of the kernel
-    const bool big_ok = smem > 48 * 1024 &&
-        cudaFuncSetAttribute(load_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess;
-    if (plan->d_perm && (smem <= 48 * 1024 || (big_ok && smem <= 200 * 1024)))
-        launch_dep(load_rows_kernel<T>, dim3((unsigned)std::min<int64_t>(rows, 148 * 8)), dim3(kThreads), smem, st, x, gy, rows, d,
-                   plan->d_perm, plan->d_signs, v0, g);
-    else
-        launch_dep(load_kernel<T>, column_grid(d, rows), dim3(kThreads), 0, st, x, gy, rows, d, plan->d_perm, plan->d_signs, v0, g);
+harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_t n_rows, float *grad, int accumulate, cudaStream_t st) {
+    const int64_t d = plan->d;
+    const StageTable &tab = plan->st;
+    const std::vector<Step> steps = make_steps(tab);
+    const int n = (int)steps.size(), n_g = std::min(n - 1, 2), ring = std::max(1, n_g);
+    const bool permuted = plan->d_perm != nullptr;
+    // chunk of rows whose forward states, gradient states and permuted rows fit about 200 MB; the partial sums of a wave of
+    // CTAs come on top
+    const int64_t per_row = std::max<int64_t>(1, d * (4 * (int64_t)(n - 1 + n_g) + (permuted ? (int64_t)sizeof(T) : 0)));
+    const int64_t most = std::max<int64_t>(16, (200ll << 20) / per_row), n_chunks = (n_rows + most - 1) / most;
+    const int64_t chunk = (n_rows + n_chunks - 1) / n_chunks;
+    int sms = 148;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device);
+    int64_t part_len = 0, part_off[HARP_MAX_STAGES] = {};
+    ReduceTable red{};
+    for (const Step &sp : steps) {
+        const int b = tab.b[sp.t];
+        if (!owner_radix(b)) continue;
+        const int slice = slice_rows(plan, sp, chunk, sms);
+        for (int t = sp.t; t < sp.t + sp.n; ++t) {
+            part_off[t] = part_len;
+            red.st[red.m++] = ReduceStage{tab.off[t], part_len, d / b, d * b, b * b, slice, 0};
+            red.total += d * b;
+            part_len += ((chunk + slice - 1) / slice) * d * b;
+        }
+    }
+    const int64_t plane = (chunk * d + 3) / 4 * 4;
+    const size_t bytes = (size_t)(part_len * 8 + 16 + plane * 4 * (n - 1 + n_g) + (permuted ? plane * (int64_t)sizeof(T) : 0));
+    double *part = nullptr;
+    cudaMemPool_t pool = scratch_pool(plan->device);
+    const cudaError_t ae = pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&part), bytes, pool, st) : cudaMallocAsync(reinterpret_cast<void **>(&part), bytes, st);
+    if (ae != cudaSuccess) {
+        cudaGetLastError();
+        return HARP_ERR_ALLOC;
+    }
+    float *vp = reinterpret_cast<float *>(part + (part_len + 1) / 2 * 2), *gp = vp + (n - 1) * plane;      // state planes on 16-byte boundaries
+    T *xp = reinterpret_cast<T *>(gp + n_g * plane);
+    const int8_t *signs = permuted ? nullptr : plan->d_signs;       // the permutation kernel carries the signs
+    harp_status_t rc = HARP_OK;
+    for (int64_t r0 = 0; r0 < n_rows && rc == HARP_OK; r0 += chunk) {
+        const int64_t rows = std::min(chunk, n_rows - r0);
+        const int acc = accumulate || r0 > 0 ? 1 : 0;
+        const T *xc = x + r0 * d, *gc = gy + r0 * d;
+        int launches = 0;
+        if (permuted) {
+            size_t smem = (size_t)(d + 2 * (d >> 6) + 2) * sizeof(T);
+            // per call: the attribute belongs to the current device's copy of the kernel
+            const int staged = smem <= 48 * 1024 || (smem <= 200 * 1024 && cudaFuncSetAttribute(permute_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess);
+            if (!staged) smem = 0;
+            launch_dep(permute_kernel<T>, dim3((unsigned)std::min<int64_t>(rows, 148 * 8)), dim3(kThreads), smem, st, xc, (int)(aligned16(xc) && d % (16 / (int64_t)sizeof(T)) == 0), xp,
+                       rows, d, plan->d_perm, plan->d_signs, staged);
+            xc = xp;
+            ++launches;
+        }
+        for (int k = 0; k + 1 < n; ++k, ++launches) {
+            if (k == 0) step_forward<T>(plan, steps[0], xc, signs, vp, rows, st);
+            else step_forward<float>(plan, steps[(size_t)k], vp + (k - 1) * plane, nullptr, vp + k * plane, rows, st);
+        }
+        for (int k = n - 1; k >= 0; --k) {
+            const Step &sp = steps[(size_t)k];
+            const float *v_in = vp + (k - 1) * plane, *g_in = gp + ((k + 1) % ring) * plane;
+            float *out = k > 0 ? gp + (k % ring) * plane : nullptr;
+            const int slice = slice_rows(plan, sp, chunk, sms);
+            double *p1 = part + part_off[sp.t], *p2 = sp.n == 2 ? part + part_off[sp.t + 1] : nullptr;
+            if (k == 0 && k == n - 1) launches += step_backward<T, T>(plan, sp, xc, signs, gc, out, rows, p1, p2, slice, grad, acc, st);
+            else if (k == n - 1) launches += step_backward<float, T>(plan, sp, v_in, nullptr, gc, out, rows, p1, p2, slice, grad, acc, st);
+            else if (k == 0) launches += step_backward<T, float>(plan, sp, xc, signs, g_in, out, rows, p1, p2, slice, grad, acc, st);
+            else launches += step_backward<float, float>(plan, sp, v_in, nullptr, g_in, out, rows, p1, p2, slice, grad, acc, st);
+        }
+        if (red.m > 0) {
+            for (int k = 0; k < red.m; ++k) {
+                const int per = red.st[k].rows;
+                red.st[k].n_slices = (int32_t)((rows + per - 1) / per);
+            }
+            launch_dep(reduce_kernel, dim3((unsigned)std::min<int64_t>((red.total + 31) / 32, 148 * 16)), dim3(kThreads), 0, st, part, grad, acc, red);
+            ++launches;
+        }
+        g_harp_launches.fetch_add(launches, std::memory_order_relaxed);
+        if (cudaGetLastError() != cudaSuccess) rc = HARP_ERR_CUDA;
+    }
+    cudaFreeAsync(part, st);
+    return rc;
 }
 
 }  // namespace
@@ -541,97 +939,10 @@ extern "C" harp_status_t harp_grad_blocks(const harp_plan_t *plan, const void *x
     if (reinterpret_cast<uintptr_t>(x) % es || reinterpret_cast<uintptr_t>(gy) % es || reinterpret_cast<uintptr_t>(grad) % 4)
         return HARP_ERR_BAD_DIM;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int64_t d = plan->d;
-    const int m = plan->st.m;
     if (n_rows == 0) {
         if (!accumulate && cudaMemsetAsync(grad, 0, sizeof(float) * (size_t)plan->n_params, st) != cudaSuccess) return HARP_ERR_CUDA;
         return HARP_OK;
     }
-    // chunk of rows whose m forward states, two gradient states and the per-slice sums of the
-    // block-owner stages (at most one state: 8 bytes x d b / 32 per row, b <= 16) fit ~256 MB
-    const int64_t per_row = (int64_t)(m + 3) * d * (int64_t)sizeof(float);
-    const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(n_rows, 1 << 18), (256ll << 20) / per_row));
-    int64_t part_bytes = 0;                          // per-slice sums of the stage that needs most
-    for (int t = 0; t < m; ++t) {
-        const int b = plan->st.b[t];
-        const int slice = owner_radix(b) ? kBwdSliceRows : (b == 16 ? kTileRows16 : 0);
-        if (slice) part_bytes = std::max<int64_t>(part_bytes, ((chunk + slice - 1) / slice) * d * b * (int64_t)sizeof(double));
-    }
-    const int64_t state_bytes = (int64_t)(m + 2) * chunk * d * (int64_t)sizeof(float);
-    float *scratch = nullptr;
-    const size_t scratch_bytes = (size_t)(state_bytes + 256 + part_bytes);
-    cudaMemPool_t pool = scratch_pool(plan->device);
-    const cudaError_t alloc_err = pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&scratch), scratch_bytes, pool, st)
-                                       : cudaMallocAsync(reinterpret_cast<void **>(&scratch), scratch_bytes, st);
-    if (alloc_err != cudaSuccess) {
-        cudaGetLastError();
-        return HARP_ERR_ALLOC;
-    }
-    const int64_t plane = chunk * d;                  // floats per state
-    float *ga = scratch + (int64_t)m * plane, *gb = ga + plane;
-    // fp64 per-slice sums of the block-owner stages, behind the states, on the next 256-byte boundary
-    double *part = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(gb + plane) + 255) & ~(uintptr_t)255);
-    harp_status_t rc = HARP_OK;
-    for (int64_t r0 = 0; r0 < n_rows && rc == HARP_OK; r0 += chunk) {
-        const int64_t rows = std::min(chunk, n_rows - r0);
-        if (dtype == HARP_F32)
-            launch_load<float>((const float *)x + r0 * d, (const float *)gy + r0 * d, rows, d, plan, scratch, ga, st);
-        else
-            launch_load<__nv_bfloat16>((const __nv_bfloat16 *)x + r0 * d, (const __nv_bfloat16 *)gy + r0 * d, rows, d, plan, scratch,
-                                       ga, st);
-        int launches = 1;
-        // forward states v_1 .. v_{m-1} (v_t in plane t)
-        for (int t = 0; t + 1 < m; ++t, ++launches) {
-            const int b = plan->st.b[t];
-            const float *K = plan->d_blocks + plan->st.off[t];
-            const int64_t s = plan->st.s[t];
-            const bool em = s >= 8;                          // see stage_kernel
-            const float *v_in = scratch + t * plane;
-            float *v_out = scratch + (t + 1) * plane;
-            if (owner_radix(b))
-                launch_fwd_owner(b, v_in, v_out, rows, d, s, K, st);
-            else if (b == 16)
-                launch_dep(stage16_kernel, owner_grid16(d, rows, kFwdSliceRows), dim3(128), 0, st, v_in, v_out, rows, d, s, K, 0);
-            else
-                launch_dep(stage_kernel, column_grid(d, rows), dim3(kThreads), 0, st, v_in, v_out, rows, d, b, s,
-                           em ? plan->d_blocks_em + plan->st.off[t] : K, em ? 1 : (int64_t)b * b, em ? d / b : 1, 0);
-        }
-        // backward: entry sums, and the gradient state one stage back
-        float *g_cur = ga, *g_nxt = gb;
-        const int acc = (accumulate || r0 > 0) ? 1 : 0;
-        for (int t = m - 1; t >= 0; --t) {
-            const int b = plan->st.b[t];
-            const int64_t s = plan->st.s[t];
-            const float *K = plan->d_blocks + plan->st.off[t];
-            const float *v_t = scratch + t * plane;
-            float *grad_t = grad + plan->st.off[t];
-            const dim3 reduce_grid((unsigned)std::min<int64_t>((d * b + 31) / 32, 148 * 16));
-            if (owner_radix(b)) {
-                launch_bwd_owner(b, v_t, g_cur, t > 0 ? g_nxt : nullptr, rows, d, s, K, part, st);
-                launch_dep(reduce_slices_kernel, reduce_grid, dim3(kThreads), 0, st, part, (rows + kBwdSliceRows - 1) / kBwdSliceRows,
-                           d / b, b * b, grad_t, acc);
-                launches += 2;
-            } else if (b == 16) {
-                launch_dep(outer16_kernel, owner_grid16(d, rows, kTileRows16), dim3(512), 0, st, v_t, g_cur, rows, d, s, part);
-                launch_dep(reduce_slices_kernel, reduce_grid, dim3(kThreads), 0, st, part, (rows + kTileRows16 - 1) / kTileRows16,
-                           d / b, b * b, grad_t, acc);
-                if (t > 0)
-                    launch_dep(stage16_kernel, owner_grid16(d, rows, kFwdSliceRows), dim3(128), 0, st, g_cur, g_nxt, rows, d, s, K, 1);
-                launches += t > 0 ? 3 : 2;
-            } else {
-                const bool em = s >= 8;
-                launch_dep(outer_kernel, dim3((unsigned)std::min<int64_t>((d * b + 31) / 32, 148 * 64)), dim3(kThreads), 0, st, v_t,
-                           g_cur, rows, d, b, s, grad_t, acc, em ? 0 : 1);
-                if (t > 0)
-                    launch_dep(stage_kernel, column_grid(d, rows), dim3(kThreads), 0, st, g_cur, g_nxt, rows, d, b, s,
-                               em ? plan->d_blocks_em + plan->st.off[t] : K, em ? 1 : (int64_t)b * b, em ? d / b : 1, 1);
-                launches += t > 0 ? 2 : 1;
-            }
-            if (t > 0) std::swap(g_cur, g_nxt);
-        }
-        g_harp_launches.fetch_add(launches, std::memory_order_relaxed);
-        if (cudaGetLastError() != cudaSuccess) rc = HARP_ERR_CUDA;
-    }
-    cudaFreeAsync(scratch, st);
-    return rc;
+    return dtype == HARP_F32 ? grad_blocks<float>(plan, (const float *)x, (const float *)gy, n_rows, grad, accumulate, st)
+                             : grad_blocks<__nv_bfloat16>(plan, (const __nv_bfloat16 *)x, (const __nv_bfloat16 *)gy, n_rows, grad, accumulate, st);
 }
