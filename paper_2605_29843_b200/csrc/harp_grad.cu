@@ -136,7 +136,7 @@ fwd_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int vec,
 
 // CTAs per SM of the backward kernels (registers: 168 per thread from radix 5 to 8, else 128)
 constexpr int k44PerSm = 3;
-__host__ __device__ constexpr int bwd_per_sm(int b, int bi, int subs) { return (b >= 5 && b <= 8 ? 12 : 16) / (((b + bi - 1) / bi) * subs); }
+__host__ __device__ constexpr int bwd_per_sm(int b, int bi, int subs) { return (b >= 5 && b <= 6 ? 12 : 16) / (((b + bi - 1) / bi) * subs); }
 
 // sums of the warps that split the rows, added in the order of the warps; sum k of a lane goes to dst(k)
 template <int N, int SUBS, typename Dst>
@@ -755,7 +755,8 @@ Shape bwd_shape(const harp_plan *plan, const Step &sp) {
     if (sp.n == 2) return b == 4 ? Shape{(d / 16 + 7) / 8, k44PerSm} : Shape{(d / 4 + 31) / 32, 4};
     const int64_t x = (d / b + 31) / 32;
     switch (b) {
-        case 7: case 8: return {x, bwd_per_sm(b, 4, 2)};
+        case 7: return {x, bwd_per_sm(7, 4, 2)};
+        case 8: return {x, bwd_per_sm(8, 2, 2)};
         case 16: return {x, bwd_per_sm(16, 2, 1)};
         case 5: return {x, bwd_per_sm(5, 5, kSubs)};
         case 6: return {x, bwd_per_sm(6, 3, kSubs)};
@@ -822,7 +823,7 @@ int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8
 #define HARP_BWD(B, BI, SUBS) case B: launch_dep(bwd_kernel<B, BI, SUBS, TV, TG>, grid2(d / B, 32, rows, slice), dim3(32 * ((B + BI - 1) / BI) * SUBS), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, part); return 1
     switch (b) {
         HARP_BWD(2, 2, kSubs); HARP_BWD(3, 3, kSubs); HARP_BWD(4, 4, kSubs); HARP_BWD(5, 5, kSubs); HARP_BWD(6, 3, kSubs); HARP_BWD(7, 4, 2);
-        HARP_BWD(8, 4, 2); HARP_BWD(16, 2, 1);
+        HARP_BWD(8, 2, 2); HARP_BWD(16, 2, 1);
         default: break;
     }
 #undef HARP_BWD
