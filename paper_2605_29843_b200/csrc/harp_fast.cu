@@ -64,6 +64,8 @@ struct PhaseDesc {
     int32_t B;                 // 8 or 16
     int32_t lane_step;         // element offset between the slots of lanes q and q+1
     int32_t j_off[4];          // element offsets of a lane's slots
+    int32_t lm, jr[4];         // local index of slot j of lane q is lm * q + jr[j]
+    int32_t order;             // cluster variant: offset of the item order inside ctab
 };
 
 struct FastParams {
@@ -79,6 +81,11 @@ struct FastParams {
     // phases whose block fragments a CTA keeps in tensor memory for all its tiles (bit p = phase p):
     // warp w reads the fragments of its own items w and w + 16 from its 32 lanes, 32 columns per item
     uint32_t tm_mask;
+    // cluster variant: chunk numbers of a row in the order of the CTA that loads / stores them, item numbers of every phase in
+    // the order of the CTA that runs them, and the phases after which the results move to another CTA (bit p = phase p)
+    const int32_t *ctab;
+    int32_t ctab_len, order_in, order_out;
+    uint32_t xchg_mask;
     PhaseDesc ph[kMaxPhases];
 };
 
@@ -144,6 +151,27 @@ __device__ __forceinline__ void ss16_store(const TileCtx &c, const PhaseDesc &ph
         sts128(a1 + 2u * ph.j_off[j], raw[j][1]);
     }
 }
+// The same store in the cluster variant after an exchange phase: slot j of lane q goes to the CTA that owns the phase's local
+// index of that slot from here on, at the same place of its tile.
+__device__ __forceinline__ void st_cluster128(uint32_t addr, uint32_t rank, const uint4 &v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("st.shared::cluster.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(remote), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+template <int NJ>
+__device__ __forceinline__ void store_to_owner(const TileCtx &c, const PhaseDesc &ph, int it, const uint4 (&raw)[NJ][2], int cs) {
+    const uint32_t a0 = c.sbase + 2u * (uint32_t)(c.g * c.pitch + c.q * ph.lane_step + c.tab[ph.items_off + it]);
+    const uint32_t a1 = a0 + 2u * (uint32_t)(8 * c.pitch);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const uint32_t rank = (uint32_t)((ph.lm * c.q + ph.jr[j]) * cs / ph.B);
+        st_cluster128(a0 + 2u * ph.j_off[j], rank, raw[j][0]);
+        st_cluster128(a1 + 2u * ph.j_off[j], rank, raw[j][1]);
+    }
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 // ---- MODE_GS: operands from global memory
 __device__ __forceinline__ void gs_load(const TileCtx &c, const PhaseDesc &ph, int it, uint4 (&raw)[4][2], uint4 (&bf)[8],
                                         int tm_slot) {
@@ -170,11 +198,17 @@ __device__ __forceinline__ void gs_store(const TileCtx &c, const PhaseDesc &ph, 
 // scheme does not pay for the others.
 __host__ __device__ constexpr uint32_t bit(int mode) { return 1u << mode; }
 constexpr uint32_t kModesGeneral = bit(MODE_CC) | bit(MODE_SS) | bit(MODE_GS) | bit(MODE_CG);
+constexpr uint32_t kModesInPlace = bit(MODE_CC) | bit(MODE_SS);                 // identity permutation
 constexpr uint32_t kModesReorderOut = bit(MODE_SS) | bit(MODE_PO);   // the digit-reversal scheme, both directions
 
-template <int NT, uint32_t MODES>
+// CL: a cluster of cs CTAs works on one tile (batches whose tiles would leave most SMs idle).  Every CTA keeps the tile's layout
+// and holds the part of it that it owns: the blocks of a phase are dealt out by the value of a digit that the phase does
+// not mix, and where the next phase needs another digit the phase's results are written to their new owner through
+// distributed shared memory.  What bounds a lone tile is one SM fetching the block kernels of a whole row (393 KB at
+// d = 4096) and running their items one after the other; cs SMs share both.
+template <int NT, uint32_t MODES, bool CL>
 __global__ void __launch_bounds__(NT, 1)
-harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles, int stagger, FastParams P) {
+harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles, int stagger, int cs, FastParams P) {
     constexpr int NW = NT / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileCtx c;
@@ -188,15 +222,20 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
     int32_t *tab_s = reinterpret_cast<int32_t *>(smem_raw + (size_t)kTileRows * pitch * 2);
     for (int i = threadIdx.x; i < P.tables_len; i += NT) tab_s[i] = __ldg(P.tables + i);
     c.tab = tab_s;
+    // cluster variant: rank, and the chunk and item orders behind the tables
+    const int rank = CL ? (int)(blockIdx.x % (unsigned)cs) : 0;
+    const int32_t *ord = tab_s + P.tables_len;
+    if (CL)
+        for (int i = threadIdx.x; i < P.ctab_len; i += NT) tab_s[P.tables_len + i] = __ldg(P.ctab + i);
     // ---- block fragments of up to two phases into tensor memory, once per CTA ----
     uint32_t &tm_base_s = *reinterpret_cast<uint32_t *>(tab_s + P.tables_len);   // one word after the tables
-    if (P.tm_mask) {
+    if (!CL && P.tm_mask) {
         if (c.warp == 0) harp_tm::tmem_alloc(smem_u32(&tm_base_s), 512);
         harp_tm::tc_fence_before();
     }
     __syncthreads();
     c.tm_warp = 0;
-    if (P.tm_mask) {
+    if (!CL && P.tm_mask) {
         harp_tm::tc_fence_after();
         c.tm_warp = tm_base_s + ((uint32_t)((c.warp & 3) * 32) << 16) + (uint32_t)((c.warp >> 2) * 128);
         int slot = 0;
@@ -221,7 +260,7 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
     // HBM bandwidth at those moments while it idles during the phases.  Three classes of CTAs
     // start a quarter of a tile period apart (a bounded wait on the clock; only used when every
     // CTA has several tiles, so the delay is small against the run).
-    if (stagger > 0) {
+    if (!CL && stagger > 0) {
         const long long wait = (long long)(blockIdx.x % 3) * stagger, t0 = clock64();
         while (clock64() - t0 < wait) { }
     }
@@ -231,10 +270,11 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
     // that kernel has completed.  The kernel after this one may start its own preamble as SMs become free.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (CL) cluster_sync();                        // every CTA of the cluster is running before anybody writes to its shared memory
 #ifdef HARP_FAST_TIMING
     long long tacc[16] = {0}, tlast = clock64();
 #endif
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    for (int64_t tile = CL ? blockIdx.x / (unsigned)cs : blockIdx.x; tile < n_tiles; tile += CL ? n_tiles : gridDim.x) {
         const int64_t row0 = tile * kTileRows;
 #ifdef HARP_FAST_TIMING
         if (threadIdx.x == 0) { tacc[0] += 1; tlast = clock64(); }
@@ -250,12 +290,16 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
             // a thread owns the same 16-byte chunks of every row; no index arithmetic per chunk
             const int32_t *cmap = tab_s + P.copy_in;
             const int chunks = d >> 3;
-            for (int ch = threadIdx.x; ch < chunks; ch += NT) {
+            const int per_in = CL ? chunks / cs : chunks, first_in = CL ? rank * per_in : 0;
+            const int rsteps = CL ? max(1, NT / per_in) : 1, r_first = CL && rsteps > 1 ? threadIdx.x / per_in : 0;     // few chunks: threads share the rows
+            if (r_first < rsteps)
+            for (int cj = CL && rsteps > 1 ? threadIdx.x - r_first * per_in : threadIdx.x; cj < per_in; cj += NT) {
+                const int ch = CL ? ord[P.order_in + first_in + cj] : cj;
                 const uint32_t dst = c.sbase + 2u * (uint32_t)cmap[ch];
                 const __nv_bfloat16 *src = x + row0 * d + 8 * ch;
                 const __nv_bfloat16 *last_src = x + last * d + 8 * ch;
 #pragma unroll 4
-                for (int r = 0; r < kTileRows; ++r)
+                for (int r = r_first; r < kTileRows; r += rsteps)
                     cp_async16(dst + 2u * (uint32_t)(r * pitch), row0 + r <= last ? src + (int64_t)r * d : last_src);
             }
             cp_async_wait_all();
@@ -265,14 +309,18 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
 
         for (int p = 0; p < P.n_phases; ++p) {
             const PhaseDesc &ph = P.ph[p];
-            const int n = ph.n_items;
-            const int tm_slot = ((P.tm_mask >> p) & 1u) ? __popc(P.tm_mask & ((1u << p) - 1u)) : -1;
+            // items [0, n) of the phase, or this CTA's share of them in its order
+            const int n = CL ? ph.n_items / cs : ph.n_items;
+            const int32_t *item = ord + ph.order + rank * n;
+            const bool xchg = CL && ((P.xchg_mask >> p) & 1u);
+            const int tm_slot = !CL && ((P.tm_mask >> p) & 1u) ? __popc(P.tm_mask & ((1u << p) - 1u)) : -1;
             if ((MODES & bit(MODE_CC)) && ph.mode == MODE_CC) {
                 // lane -> (matrix row, 8-column half) of the 16x16 (or 16x8) operand tile
                 const int mrow = (lane & 7) + ((lane >> 3) & 1) * 8, mcol = (lane >> 4) * 8;
                 if (ph.B == 16) {
 #pragma unroll 4
-                    for (int it = warp; it < n; it += NW) {
+                    for (int k = warp; k < n; k += NW) {
+                        const int it = CL ? item[k] : k;
                         const uint32_t addr = c.sbase + 2u * (uint32_t)(mrow * pitch + tab_s[ph.items_off + it] + mcol);
                         const uint4 bf = __ldg(ph.bfrag + (size_t)it * 32 + lane);
                         uint32_t a[4];
@@ -287,7 +335,8 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                     const uint32_t *bf8 = reinterpret_cast<const uint32_t *>(ph.bfrag);
                     const int mrow2 = (lane & 15);
 #pragma unroll 4
-                    for (int it = warp; it < n; it += NW) {
+                    for (int k = warp; k < n; k += NW) {
+                        const int it = CL ? item[k] : k;
                         const uint32_t addr = c.sbase + 2u * (uint32_t)(mrow2 * pitch + tab_s[ph.items_off + it]);
                         const uint32_t bf = __ldg(bf8 + (size_t)it * 32 + lane);
                         uint32_t a[2];
@@ -302,14 +351,17 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                 // kernel sits at the register limit and every variant that holds more spills)
                 uint4 raw[4][2], bf[8];
                 uint32_t unused[8][4];
-                for (int it = warp; it < n; it += NW) {
+                for (int k = warp; k < n; k += NW) {
+                    const int it = CL ? item[k] : k;
                     ss16_load(c, ph, it, raw, bf, tm_slot);
                     octet_mma16<true>(raw, bf, unused);
-                    ss16_store(c, ph, it, raw);
+                    if (xchg) store_to_owner<4>(c, ph, it, raw, cs);
+                    else ss16_store(c, ph, it, raw);
                 }
             } else if ((MODES & bit(MODE_SS)) && ph.mode == MODE_SS) {
                 const uint32_t *bf8 = reinterpret_cast<const uint32_t *>(ph.bfrag);
-                for (int it = warp; it < n; it += NW) {
+                for (int k = warp; k < n; k += NW) {
+                        const int it = CL ? item[k] : k;
                     const uint32_t a0 = c.sbase + 2u * (uint32_t)(c.g * pitch + c.q * ph.lane_step + tab_s[ph.items_off + it]);
                     const uint32_t a1 = a0 + 2u * (uint32_t)(8 * pitch);
                     uint4 raw[2][2];
@@ -322,6 +374,10 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                         raw[j][1] = lds128(a1 + 2u * ph.j_off[j]);
                     }
                     octet_mma8(raw, bf);
+                    if (xchg) {
+                        store_to_owner<2>(c, ph, it, raw, cs);
+                        continue;
+                    }
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         sts128(a0 + 2u * ph.j_off[j], raw[j][0]);
@@ -331,7 +387,8 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
             } else if ((MODES & bit(MODE_GS)) && ph.mode == MODE_GS) {
                 uint4 raw[4][2], bf[8];
                 uint32_t mats[8][4];
-                for (int it = warp; it < n; it += NW) {
+                for (int k = warp; k < n; k += NW) {
+                        const int it = CL ? item[k] : k;
                     gs_load(c, ph, it, raw, bf, tm_slot);
                     octet_mma16<false>(raw, bf, mats);
                     gs_store(c, ph, it, mats);
@@ -340,7 +397,8 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                 // contiguous blocks in (ldmatrix), eight-block runs out to the same sixteen 16-byte
                 // slots the item read (a per-item table names them): in place, no barrier
                 const int mrow = (lane & 7) + ((lane >> 3) & 1) * 8, mcol = (lane >> 4) * 8;
-                for (int it = warp; it < n; it += NW) {
+                for (int k = warp; k < n; k += NW) {
+                        const int it = CL ? item[k] : k;
                     const int32_t *tab = tab_s + ph.items_off + it * 24;
                     uint4 bf[8], out[4][2];
                     load_frag8(bf, ph.bfrag + (size_t)it * 256 + lane, tm_slot >= 0, tm_item(c, tm_slot, it));
@@ -406,7 +464,8 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                     }
                 }
             }
-            __syncthreads();
+            if (xchg) cluster_sync();
+            else __syncthreads();
             FAST_MARK(2 + p);
         }
 
@@ -414,11 +473,15 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
             const int32_t *cmap = tab_s + P.copy_out;
             const int chunks = d >> 3;
             const int rows = (int)min((int64_t)kTileRows, n_rows - row0);
-            for (int ch = threadIdx.x; ch < chunks; ch += NT) {
+            const int per_out = CL ? chunks / cs : chunks, first_out = CL ? rank * per_out : 0;
+            const int rsteps = CL ? max(1, NT / per_out) : 1, r_first = CL && rsteps > 1 ? threadIdx.x / per_out : 0;
+            if (r_first < rsteps)
+            for (int cj = CL && rsteps > 1 ? threadIdx.x - r_first * per_out : threadIdx.x; cj < per_out; cj += NT) {
+                const int ch = CL ? ord[P.order_out + first_out + cj] : cj;
                 const uint32_t src = c.sbase + 2u * (uint32_t)cmap[ch];
                 __nv_bfloat16 *dst = x + row0 * d + 8 * ch;
 #pragma unroll 4
-                for (int r = 0; r < rows; ++r) stg128(dst + (int64_t)r * d, lds128(src + 2u * (uint32_t)(r * pitch)));
+                for (int r = r_first; r < rows; r += rsteps) stg128(dst + (int64_t)r * d, lds128(src + 2u * (uint32_t)(r * pitch)));
             }
             __syncthreads();
         }
@@ -429,7 +492,7 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
         for (int k = 0; k < 16; ++k)
             if (tacc[k]) atomicAdd((unsigned long long *)&g_fast_timing[k], (unsigned long long)tacc[k]);
 #endif
-    if (P.tm_mask) {
+    if (!CL && P.tm_mask) {
         harp_tm::tc_fence_before();
         __syncthreads();
         if (c.warp == 0) harp_tm::tmem_dealloc(tm_base_s, 512);
@@ -446,6 +509,9 @@ struct FastPlan {
     int variant_fwd = 0, variant_bwd = 0;     // which compiled set of phase modes each direction needs
     std::vector<void *> dev_allocs;
     int max_ctas = 0;
+    int max_cluster = 1;                      // CTAs that may share a tile (1: no cluster variant)
+    size_t cl_smem_bytes = 0;
+    int clusters[4] = {0, 0, 0, 0};           // clusters of 1, 2, 4, 8 CTAs the device holds at once
 };
 
 namespace {
@@ -795,6 +861,10 @@ harp_status_t harp_fast_build(harp_plan *plan) {
     // the eight blocks' values: a run of eight neighbouring output coordinates.
     // reorder_slots[dir][item][r] is that slot's offset and chunk_out[dir] the chunk map of the
     // copy to global memory that follows from it.
+    // Cluster variant: digit T has the largest stride of the direction's layout, V is the middle phase; a phase is dealt out by
+    // T, the phase that mixes T by V, and the reordering phase (whose items span eight values of T) by V too.
+    const bool clustered = np >= 3 && (identity || (digitrev && np == 3));
+    std::vector<int32_t> out_owner[2];             // digit reversal: value of V of the chunk's place before the copy out
     std::vector<int32_t> reorder_slots[2], chunk_out[2];
     for (int dir = 0; dir < 2 && digitrev; ++dir) {
         const Layout &L = dir == 0 ? Lsrc : Lnat;
@@ -808,12 +878,15 @@ harp_status_t harp_fast_build(harp_plan *plan) {
             fprintf(stderr, " pitch %lld\n", (long long)pitch);
         }
         chunk_out[dir].assign((size_t)(d / 8), 0);
+        out_owner[dir].assign((size_t)(d / 8), 0);
         for (int64_t hi = 0; hi < d; hi += span)
             for (int64_t lo = 0; lo < So; lo += 8)
                 for (int r = 0; r < 16; ++r) {
                     const int32_t off = (int32_t)reorder_off(L, dir, hi, lo, slot_of[r]);
                     reorder_slots[dir].push_back(off);
                     chunk_out[dir][(size_t)((hi + lo + (int64_t)r * So) / 8)] = off;
+                    const int64_t co = hi + lo + (slot_of[r] & 7), pos = dir == 0 ? (int64_t)plan->h_perm[(size_t)co] : inv[(size_t)co];
+                    out_owner[dir][(size_t)((hi + lo + (int64_t)r * So) / 8)] = (int32_t)((pos / L.S[1]) % phases[1].B);
                 }
     }
 
@@ -848,6 +921,40 @@ harp_status_t harp_fast_build(harp_plan *plan) {
             P.copy_in = dir == 0 ? -1 : off_nat;
             P.copy_out = dir == 0 ? off_nat : -1;
         }
+        // cluster variant: orders of chunks and items by the owner's digit value
+        std::vector<int32_t> ctab;
+        const bool src_layout = digitrev && dir == 0;
+        const Layout &Lc = src_layout ? Lsrc : Lnat;
+        const int pT = src_layout ? 0 : np - 1, pV = digitrev ? 1 : np - 2;
+        auto by_digit = [&](const std::vector<int32_t> &value) {         // positions sorted by value, stable
+            std::vector<int32_t> o(value.size());
+            for (size_t i = 0; i < o.size(); ++i) o[i] = (int32_t)i;
+            std::stable_sort(o.begin(), o.end(), [&](int32_t a, int32_t b) { return value[(size_t)a] < value[(size_t)b]; });
+            const int32_t at = (int32_t)ctab.size();
+            ctab.insert(ctab.end(), o.begin(), o.end());
+            return at;
+        };
+        auto digit_of = [&](int p, int64_t pos) { return (int32_t)((pos / Lc.S[(size_t)p]) % phases[(size_t)p].B); };
+        auto owner_phase = [&](int p) { return p == pT || (digitrev && p == (dir == 0 ? np - 1 : 0)) ? pV : pT; };
+        if (clustered) {
+            const int p_first = dir == 0 ? 0 : np - 1, p_last = dir == 0 ? np - 1 : 0;
+            std::vector<int32_t> vin((size_t)(d / 8)), vout((size_t)(d / 8));
+            for (int64_t c = 0; c < d / 8; ++c) {
+                vin[(size_t)c] = digit_of(owner_phase(p_first), 8 * c);
+                vout[(size_t)c] = digitrev ? out_owner[dir][(size_t)c] : digit_of(owner_phase(p_last), 8 * c);
+            }
+            P.order_in = by_digit(vin);
+            P.order_out = by_digit(vout);
+            P.xchg_mask = 0;
+            for (int k = 0; k + 1 < np; ++k) {
+                const int p = dir == 0 ? k : np - 1 - k, next = dir == 0 ? k + 1 : np - 2 - k;
+                // the new owner's digit is the one this phase mixes (checked below)
+                if (owner_phase(p) != owner_phase(next)) {
+                    P.xchg_mask |= 1u << k;
+                    if (owner_phase(next) != p) st = HARP_ERR_CUDA;
+                }
+            }
+        }
         for (int k = 0; k < np && st == HARP_OK; ++k) {
             const int p = dir == 0 ? k : np - 1 - k;     // phase executed k-th
             const HostPhase &hp = phases[(size_t)p];
@@ -866,7 +973,9 @@ harp_status_t harp_fast_build(harp_plan *plan) {
             const Layout &L = src_side ? Lsrc : Lnat;
             const int lm = (mode == MODE_GS || mode == MODE_CG || mode == MODE_CC || mode == MODE_PO)
                                ? 1 : L.lm[(size_t)p];   // table-indexed slots use the plain map
+            D.lm = lm;
             const int *jo = B == 16 ? (lm == 1 ? joff1_16 : lm == 2 ? joff2_16 : joff4_16) : (lm == 1 ? joff1_8 : joff2_8);
+            for (int j = 0; j < 4; ++j) D.jr[j] = jo[j];
             if (mode == MODE_GS || mode == MODE_CG) {    // these index the item table by slot
                 D.lane_step = lm;
                 for (int j = 0; j < 4; ++j) D.j_off[j] = jo[j];
@@ -888,11 +997,13 @@ harp_status_t harp_fast_build(harp_plan *plan) {
             };
             // enumerate items and the natural base coordinate of every block
             std::vector<int32_t> items;
+            std::vector<int32_t> item_owner;             // value of the digit by which the cluster variant deals the items out
             std::vector<int64_t> block_base;             // natural coordinate of local index 0, per block in item order
             int ints_per_item = 1;
             if (mode == MODE_CC) {
                 for (int64_t c = 0; c < nblk0; ++c) {
                     items.push_back((int32_t)phys_nat(c * B0));
+                    item_owner.push_back(digit_of(owner_phase(p), c * B0));
                     block_base.push_back(c * B0);
                 }
             } else if (mode == MODE_SS && !src_side) {
@@ -900,6 +1011,7 @@ harp_status_t harp_fast_build(harp_plan *plan) {
                 for (int64_t hi = 0; hi < d; hi += span)
                     for (int64_t lo = 0; lo < hp.S; lo += 8) {
                         items.push_back((int32_t)phys_nat(hi + lo));
+                        item_owner.push_back(digit_of(owner_phase(p), hi + lo));
                         for (int e = 0; e < 8; ++e) block_base.push_back(hi + lo + e);
                     }
             } else if (mode == MODE_SS) {
@@ -908,6 +1020,7 @@ harp_status_t harp_fast_build(harp_plan *plan) {
                 for (int64_t hi = 0; hi < d; hi += span)
                     for (int64_t lo = 0; lo < Ss; lo += 8) {
                         items.push_back((int32_t)phys_src(hi + lo));
+                        item_owner.push_back(digit_of(owner_phase(p), hi + lo));
                         for (int e = 0; e < 8; ++e) block_base.push_back(inv[(size_t)(hi + lo + e)]);
                     }
             } else if (mode == MODE_PO) {
@@ -922,6 +1035,7 @@ harp_status_t harp_fast_build(harp_plan *plan) {
                             // natural coordinate of the block's local index 0
                             const int64_t nb = dir == 0 ? hi + lo + e : inv[(size_t)(hi + lo + e)];
                             items.push_back((int32_t)(dir == 0 ? phys_src(plan->h_perm[(size_t)nb]) : phys_nat(nb)));
+                            if (e == 0) item_owner.push_back(digit_of(owner_phase(p), dir == 0 ? (int64_t)plan->h_perm[(size_t)nb] : nb));
                             block_base.push_back(nb);
                         }
                         for (int r = 0; r < 16; ++r) items.push_back(reorder_slots[dir][item_no * 16 + (size_t)r]);
@@ -969,6 +1083,7 @@ harp_status_t harp_fast_build(harp_plan *plan) {
                 }
                 if (!ok) { st = HARP_ERR_UNSUPPORTED; break; }
             }
+            if (clustered) D.order = by_digit(item_owner);
             D.items_off = (int32_t)tables.size();
             tables.insert(tables.end(), items.begin(), items.end());
             // fragments: B[k-slot][n-slot] = G[local index of the k-slot][local index of the n-slot]
@@ -1020,12 +1135,17 @@ harp_status_t harp_fast_build(harp_plan *plan) {
         }
         P.tables = upload(fp, tables, st);
         P.tables_len = (int32_t)tables.size();
+        P.ctab = upload(fp, ctab, st);
+        P.ctab_len = (int32_t)ctab.size();
+        fp->cl_smem_bytes = std::max(fp->cl_smem_bytes, tile_bytes + (tables.size() + ctab.size()) * sizeof(int32_t) + 16);
         fp->smem_bytes = std::max(fp->smem_bytes, tile_bytes + tables.size() * sizeof(int32_t) + 16);
     }
     if (st == HARP_OK && fp->smem_bytes > 227u * 1024u) st = HARP_ERR_UNSUPPORTED;
     if (st == HARP_OK) {
-        if (cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesGeneral>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-            cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesReorderOut>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+        if (cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesGeneral, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesReorderOut, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesInPlace, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesReorderOut, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
             st = HARP_ERR_CUDA;
         fp->variant_fwd = digitrev ? 1 : 0;
         fp->variant_bwd = digitrev ? 1 : 0;
@@ -1033,6 +1153,26 @@ harp_status_t harp_fast_build(harp_plan *plan) {
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         fp->max_ctas = sms > 0 ? sms : 148;
+        if (clustered && fp->cl_smem_bytes <= 227u * 1024u) {
+            fp->max_cluster = std::min(phases[(size_t)(np - 1)].B, std::min(phases[(size_t)(np - 2)].B, phases[0].B)) >= 8 ? 8 : 1;
+            for (int lg = 1; lg < 4; ++lg) {
+                cudaLaunchConfig_t cfg = {};
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = 1u << lg;
+                at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+                cfg.gridDim = dim3((unsigned)fp->max_ctas / (1u << lg) * (1u << lg));
+                cfg.blockDim = dim3(kThreads);
+                cfg.dynamicSmemBytes = fp->cl_smem_bytes;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                int nc = 0;
+                const cudaError_t e = digitrev ? cudaOccupancyMaxActiveClusters(&nc, harp_fast_kernel<kThreads, kModesReorderOut, true>, &cfg)
+                                               : cudaOccupancyMaxActiveClusters(&nc, harp_fast_kernel<kThreads, kModesInPlace, true>, &cfg);
+                if (e != cudaSuccess) { cudaGetLastError(); nc = 0; }
+                fp->clusters[lg] = nc;
+            }
+        }
     }
     plan->fast = fp;
     if (st != HARP_OK) {
@@ -1076,21 +1216,29 @@ harp_status_t harp_fast_apply(const harp_plan *plan, void *x, int64_t n_rows, ha
     // a quarter of a tile period, estimated from the measured 28 k cycles per tile of d = 4096 with
     // three phases (the gain is flat between half and the full value)
     const int stagger = n_tiles >= 4 * (int64_t)grid ? (int)(0.57 * (double)P.d * P.n_phases) : 0;
+    // clusters while all tiles are in flight at once: the more CTAs share a tile the better
+    int cs = 1;
+    for (int lg = 3; lg >= 1 && cs == 1; --lg)
+        if ((1 << lg) <= fp->max_cluster && n_tiles <= fp->clusters[lg]) cs = 1 << lg;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = dim3((unsigned)(cs > 1 ? (int)n_tiles * cs : grid));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = fp->smem_bytes;
+    cfg.dynamicSmemBytes = cs > 1 ? fp->cl_smem_bytes : fp->smem_bytes;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cs;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cs > 1 ? 2 : 1;
     cudaError_t err;
-    switch (transpose ? fp->variant_bwd : fp->variant_fwd) {
-        case 1: err = cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesReorderOut>, xb, n_rows, n_tiles, stagger, P); break;
-        default: err = cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesGeneral>, xb, n_rows, n_tiles, stagger, P); break;
-    }
+    const bool reorder = (transpose ? fp->variant_bwd : fp->variant_fwd) == 1;
+    if (cs > 1) err = reorder ? cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesReorderOut, true>, xb, n_rows, n_tiles, 0, cs, P)
+                              : cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesInPlace, true>, xb, n_rows, n_tiles, 0, cs, P);
+    else err = reorder ? cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesReorderOut, false>, xb, n_rows, n_tiles, stagger, cs, P)
+                       : cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesGeneral, false>, xb, n_rows, n_tiles, stagger, cs, P);
     g_harp_launches.fetch_add(1, std::memory_order_relaxed);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? HARP_OK : HARP_ERR_CUDA;
 }
