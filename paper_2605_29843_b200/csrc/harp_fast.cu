@@ -268,9 +268,9 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
     // attribute, a CTA gets here while the kernel before it in the stream is still running on other SMs
     // (tables, tensor-memory fill and the start delay then cost nothing); the rows are touched only after
     // that kernel has completed.  The kernel after this one may start its own preamble as SMs become free.
+    if (CL) cluster_sync();                        // every CTA of the cluster is running before anybody writes to its shared memory
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (CL) cluster_sync();                        // every CTA of the cluster is running before anybody writes to its shared memory
 #ifdef HARP_FAST_TIMING
     long long tacc[16] = {0}, tlast = clock64();
 #endif
@@ -934,7 +934,7 @@ harp_status_t harp_fast_build(harp_plan *plan) {
             ctab.insert(ctab.end(), o.begin(), o.end());
             return at;
         };
-        auto digit_of = [&](int p, int64_t pos) { return (int32_t)((pos / Lc.S[(size_t)p]) % phases[(size_t)p].B); };
+        auto digit_of = [&](int p, int64_t pos) { return !clustered ? 0 : (int32_t)((pos / Lc.S[(size_t)p]) % phases[(size_t)p].B); };
         auto owner_phase = [&](int p) { return p == pT || (digitrev && p == (dir == 0 ? np - 1 : 0)) ? pV : pT; };
         if (clustered) {
             const int p_first = dir == 0 ? 0 : np - 1, p_last = dir == 0 ? np - 1 : 0;
@@ -1216,10 +1216,14 @@ harp_status_t harp_fast_apply(const harp_plan *plan, void *x, int64_t n_rows, ha
     // a quarter of a tile period, estimated from the measured 28 k cycles per tile of d = 4096 with
     // three phases (the gain is flat between half and the full value)
     const int stagger = n_tiles >= 4 * (int64_t)grid ? (int)(0.57 * (double)P.d * P.n_phases) : 0;
-    // clusters while all tiles are in flight at once: the more CTAs share a tile the better
+    // Clusters while all tiles are in flight at once.  Measured (16 to 1100 rows, radices 8 and 16): eight CTAs gain from d = 2048 on
+    // (16 rows of d = 4096: 12.3 -> 7.8 us, radix 8 15.5 -> 6.9), four from 4096 on (500 rows: 12.7 -> 11.9, radix 8 15.8 ->
+    // 10.5), two only where four phases are run (1100 rows, radix 8: 15.9 -> 14.6; radix 16 13.0 -> 13.5)
     int cs = 1;
-    for (int lg = 3; lg >= 1 && cs == 1; --lg)
-        if ((1 << lg) <= fp->max_cluster && n_tiles <= fp->clusters[lg]) cs = 1 << lg;
+    if (n_tiles <= fp->clusters[3] && P.d >= 2048) cs = 8;
+    else if (n_tiles <= fp->clusters[2] && P.d >= 4096) cs = 4;
+    else if (n_tiles <= fp->clusters[1] && P.d >= 4096 && P.n_phases >= 4) cs = 2;
+    if (cs > fp->max_cluster) cs = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(cs > 1 ? (int)n_tiles * cs : grid));
     cfg.blockDim = dim3(kThreads);
