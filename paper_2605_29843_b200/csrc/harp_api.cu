@@ -47,7 +47,9 @@ extern "C" const char *harp_status_string(harp_status_t s) {
 extern "C" int32_t harp_plan_error_word(const harp_plan_t *plan) {
     if (!plan) return -1;
     const int32_t w = harp_tm_error_word(plan);
-    return w != 0 ? w : harp_f32_error_word(plan);
+    if (w != 0) return w;
+    const int32_t s = harp_split_error_word(plan);
+    return s != 0 ? s : harp_f32_error_word(plan);
 }
 
 extern "C" int64_t harp_launch_count(void) { return g_harp_launches.load(std::memory_order_relaxed); }

@@ -66,5 +66,45 @@ inline int strided_slot(int kappa, int B, int lane_mult) {
     return lane_mult * qq + (lane_mult == 1 ? joff1[j] : joff2[j]);
 }
 
+// a fused group of stages [t0, t1): operand width, real coordinates of a block, natural stride
+struct GPhase {
+    int t0, t1;
+    int B, B_real;
+    int64_t S;
+};
+
+// Fragment words of one block of a pass (mma.sync B operand, zero-padded), signs folded into the first stage:
+// lane i's words (four for B = 16, one for B = 8) go to dst + i * lane_words.
+template <typename Slot>
+inline void block_fragment(const harp_plan *plan, const GPhase &gp, int64_t base, int dir, const Slot &slot, uint32_t *dst, int lane_words,
+                           std::vector<double> &F) {
+    const int Br = gp.B_real;
+    fused_block(plan, HostPhase{gp.t0, gp.t1, Br, gp.S, 0, 1}, base, F);
+    auto G = [&](int rin, int rout) -> double {
+        if (rin >= Br || rout >= Br) return 0.0;
+        double v = dir == 0 ? F[(size_t)rin * Br + rout] : F[(size_t)rout * Br + rin];
+        if (gp.t0 == 0 && !plan->h_signs.empty()) {
+            const int64_t pos = base + (int64_t)(dir == 0 ? rin : rout) * gp.S;
+            v *= (double)plan->h_signs[(size_t)(plan->h_perm.empty() ? pos : plan->h_perm[(size_t)pos])];
+        }
+        return v;
+    };
+    for (int lane = 0; lane < 32; ++lane, dst += lane_words) {
+        const int gg = lane >> 2, qq = lane & 3;
+        for (int nt = 0; nt < gp.B / 8; ++nt) {
+            const int n = slot(8 * nt + gg);
+            for (int h = 0; h < gp.B / 8; ++h)
+                dst[gp.B / 8 * nt + h] = f2bf(G(slot(8 * h + 2 * qq), n)) | ((uint32_t)f2bf(G(slot(8 * h + 2 * qq + 1), n)) << 16);
+        }
+    }
+}
 
 }  // namespace harp_fuse
+
+// passes fed by the copy engine (harp_pipe.cu)
+struct PipePlan;
+harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<harp_fuse::GPhase> &phs, bool lower, int64_t S_mid, int64_t U,
+                              PipePlan **out);
+void harp_pipe_destroy(PipePlan *pp);
+harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int transpose, bool overlap, cudaStream_t stream);
+int32_t harp_pipe_error_word(const PipePlan *pp);

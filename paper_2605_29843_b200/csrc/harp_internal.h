@@ -80,6 +80,7 @@ harp_status_t harp_fast_apply(const harp_plan *plan, void *x, int64_t n_rows, ha
 // tensor-core path for wide rows (harp_split.cu)
 harp_status_t harp_split_build(harp_plan *plan);
 void harp_split_destroy(harp_plan *plan);
+int32_t harp_split_error_word(const harp_plan *plan);
 harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype,
                                int transpose, cudaStream_t stream);
 

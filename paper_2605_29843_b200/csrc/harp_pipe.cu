@@ -1,0 +1,521 @@
+// The two passes of the wide-row path (see harp_split.cu) fed by the copy engine, for batches that fill it.
+//
+// The mma.sync passes of harp_split.cu spend 60 % of a tile's time on moving it: cp.async in and 16-byte stores out hold the
+// issuing warps at the rate at which the load/store unit takes 32-byte runs.  Bulk tensor copies move the same boxes
+// without a warp: 16 rows x 56 runs of 32 bytes in 1.4 cycles a run one way, 3.3 both ways (4.6 TB/s on 144 SMs), 64-byte
+// runs and longer at the HBM rate.  Here three teams of eight warps (two where blocks are 16 wide) share the fragments of the
+// CTA's column group; every team has two tile buffers and multiplies one while the other is stored and refilled.
+//
+// The tile's layout is what the copy engine writes, chosen so that the 16-byte accesses of a quarter-warp (two rows, four
+// local indices) hit eight bank groups:
+//   lower pass  [box of 64 coordinates][row][128 bytes], 128-byte swizzle, boxes 128 bytes apart beyond their size: an index
+//               step of one chunk or one box moves the swizzle by one, lanes hold the local indices 2q, 2q+1;
+//   upper pass  [half of the rows][row][outer digit][inner digit][32 bytes], 32-byte swizzle.  The inner digit's radix is odd
+//               (or there is one digit), so a step of either digit is an odd number of 32-byte columns; the two rows of a
+//               quarter-warp come from the two halves, which lie an odd number of 128 bytes apart, so that the swizzle
+//               gives them different 16-byte halves of a column.
+#include <algorithm>
+#include <new>
+#include <vector>
+
+#include "harp_fuse.h"
+#include "harp_internal.h"
+#include "harp_mma.cuh"
+#include "harp_tm_ptx.cuh"
+
+namespace {
+
+using namespace harp_fuse;
+using harp_tm::mbar_expect_tx;
+using harp_tm::mbar_init;
+using harp_tm::mbar_try;
+
+constexpr int kTeamWarps = 8, kTeamThreads = 32 * kTeamWarps;
+constexpr int kMaxPipePhases = 3, kMaxPipeBufs = 4;
+constexpr uint32_t kPipeSpin = 1u << 22;      // limit of every wait for a bulk copy
+
+struct PipePhase {
+    int32_t mode;              // 0 = contiguous blocks of eight, two at a time; 1 = strided blocks, eight per item
+    int32_t B, B_real;
+    int32_t n_items, items_off;
+    int32_t bfrag_off;         // word offset of the phase's fragments inside a column group's block
+    int32_t lm;                // local index of slot j of lane q: lm * q + jr[j]
+    int32_t jr[4];
+    int32_t step[2];           // byte offset of local index r: (r * unit >> shift) * step[1] + (r * unit & mask) * step[0]
+    int32_t unit, shift;
+};
+
+struct PipePass {
+    int32_t n_phases, n_cg, MT, mt_shift;
+    int32_t n_box, box_bytes, box_pitch;      // bulk copies of a tile, their size, their distance in shared memory
+    int32_t row_bytes;                        // upper: distance of neighbouring rows of a half
+    int32_t tile_bytes, n_buf;                // distance of a team's buffers, their number
+    int32_t n_tiles, n_parts;                 // n_parts > 0: a CTA keeps its column group and takes every n_parts-th tile; 0: equal shares of the list
+    const int32_t *tables;                    // byte offsets of the items
+    int32_t tables_len;
+    const uint32_t *bfrag;                    // [column group][bfrag_words]
+    int32_t bfrag_words;
+    PipePhase ph[kMaxPipePhases];
+};
+
+__device__ __forceinline__ uint32_t lds32p(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int a, int b, int c, int d, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+                 ::"r"(dst), "l"(map), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, int a, int b, int c, int d, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];"
+                 ::"l"(map), "r"(a), "r"(b), "r"(c), "r"(d), "r"(src) : "memory");
+}
+
+template <bool LOWER> __device__ __forceinline__ uint32_t swz(uint32_t a) {
+    return LOWER ? a ^ (((a >> 7) & 7u) << 4) : a ^ (((a >> 7) & 1u) << 4);
+}
+__device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
+    const int e = r * ph.unit;
+    return (uint32_t)((e >> ph.shift) * ph.step[1] + (e & ((1 << ph.shift) - 1)) * ph.step[0]);
+}
+
+// A team: eight warps with n_buf tile buffers of their own.  Tiles of the CTA's column group go to its teams in turn; a team's
+// thread 0 issues its bulk copies.  Sixteen-wide blocks need 128 registers: one team, two CTAs per SM.
+template <bool LOWER, bool B16>
+__global__ void __launch_bounds__(kTeamThreads * (B16 ? 1 : 3), B16 ? 2 : 1)
+harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const PipePass P) {
+    constexpr int TEAMS = B16 ? 1 : 3;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[TEAMS * kMaxPipeBufs];
+    __shared__ int dead;
+    const uint32_t smem0 = (smem_u32(smem_raw) + 127u) & ~127u;
+    const int team = threadIdx.x / kTeamThreads, tid = threadIdx.x - team * kTeamThreads;
+    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
+    const int NB = P.n_buf;
+    const uint32_t bufs = smem0 + (uint32_t)(team * NB * P.tile_bytes);
+    const uint32_t bf_s = smem0 + (uint32_t)(TEAMS * NB * P.tile_bytes);
+    const uint32_t tab_s = bf_s + 4u * (uint32_t)P.bfrag_words;
+    for (int i = threadIdx.x; i < P.tables_len; i += TEAMS * kTeamThreads)
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(tab_s + 4u * i), "r"(__ldg(P.tables + i)) : "memory");
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < TEAMS * kMaxPipeBufs; ++b) mbar_init(smem_u32(&full_bar[b]), 1);
+        dead = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+
+    // rows of a lane: LOWER g and g + 8 of a 16-row group; upper: g / 2 and g / 2 + 4 of the half g & 1
+    const uint32_t row0_off = LOWER ? 128u * (uint32_t)g : (uint32_t)((g & 1) * P.box_pitch + (g >> 1) * P.row_bytes);
+    const uint32_t row8_off = LOWER ? 1024u : 4u * (uint32_t)P.row_bytes;
+    const uint32_t mt_step = LOWER ? 2048u : 8u * (uint32_t)P.row_bytes;
+
+    // Rows past the end of the batch arrive as zeros and are not written.
+    auto load = [&](int cg, int tile, int b) {
+        const uint32_t bar = smem_u32(&full_bar[team * kMaxPipeBufs + b]), dst = bufs + (uint32_t)(b * P.tile_bytes);
+        mbar_expect_tx(bar, (uint32_t)(P.n_box * P.box_bytes));
+        for (int k = 0; k < P.n_box; ++k) {
+            if constexpr (LOWER) harp_tm::tma_load_2d(dst + (uint32_t)(k * P.box_pitch), &tmap, 64 * (cg * P.n_box + k), tile * 16 * P.MT, bar);
+            else tma_load_4d(dst + (uint32_t)(k * P.box_pitch), &tmap, 16 * cg, 0, 0, tile * 16 * P.MT + 8 * P.MT * k, bar);
+        }
+    };
+    auto store = [&](int cg, int tile, int b) {
+        const uint32_t src = bufs + (uint32_t)(b * P.tile_bytes);
+        for (int k = 0; k < P.n_box; ++k) {
+            if constexpr (LOWER) harp_tm::tma_store_2d(&tmap, 64 * (cg * P.n_box + k), tile * 16 * P.MT, src + (uint32_t)(k * P.box_pitch));
+            else tma_store_4d(&tmap, 16 * cg, 0, 0, tile * 16 * P.MT + 8 * P.MT * k, src + (uint32_t)(k * P.box_pitch));
+        }
+        harp_tm::bulk_commit();
+    };
+    auto team_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory"); };
+
+    // segments of this CTA: a column group and its tiles
+    int64_t at = 0, end = 1;
+    if (P.n_parts == 0) {
+        const int64_t all = (int64_t)P.n_cg * P.n_tiles, per = all / gridDim.x, extra = all % gridDim.x;
+        at = blockIdx.x * per + min((int64_t)blockIdx.x, extra);
+        end = at + per + ((int64_t)blockIdx.x < extra ? 1 : 0);
+    }
+    uint32_t parity = 0;
+    bool waited = false;
+    while (at < end) {
+        int cg, first, step, count;
+        if (P.n_parts > 0) {
+            cg = blockIdx.x % P.n_cg;
+            first = blockIdx.x / P.n_cg;
+            step = P.n_parts;
+            count = first < P.n_tiles ? (P.n_tiles - first + step - 1) / step : 0;
+            at = end;
+        } else {
+            cg = (int)(at / P.n_tiles);
+            first = (int)(at - (int64_t)cg * P.n_tiles);
+            step = 1;
+            count = (int)min((int64_t)(P.n_tiles - first), end - at);
+            at += count;
+        }
+        // fragments of the column group (plan data); every team is through with the ones before
+        __syncthreads();
+        const uint32_t *src = P.bfrag + (size_t)cg * P.bfrag_words;
+        for (int i = threadIdx.x * 4; i < P.bfrag_words; i += TEAMS * kTeamThreads * 4) cp_async16(bf_s + 4u * i, src + i);
+        cp_async_wait_all();
+        __syncthreads();
+        if (!waited) {                               // the rows only once the kernel before has completed
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            waited = true;
+        }
+        if (tid == 0 && !*(volatile int *)&dead)
+            for (int k = 0; k < NB; ++k)
+                if (team + k * TEAMS < count) load(cg, first + (team + k * TEAMS) * step, k);
+        int b = 0;
+        for (int t = team; t < count; t += TEAMS, b = b + 1 == NB ? 0 : b + 1) {
+            const uint32_t bar = smem_u32(&full_bar[team * kMaxPipeBufs + b]), sbase = bufs + (uint32_t)(b * P.tile_bytes);
+            uint32_t it = 0;
+            while (!mbar_try(bar, (parity >> b) & 1u)) {
+                if (++it > kPipeSpin || ((it & 63) == 63 && *(volatile int *)&dead)) {
+                    *(volatile int *)&dead = 1;       // from here on nothing is copied any more
+                    atomicExch(err, 301);
+                    break;
+                }
+            }
+            parity ^= 1u << b;
+            for (int p = 0; p < P.n_phases; ++p) {
+                const PipePhase &ph = P.ph[p];
+                if (p > 0) team_sync();
+                if (LOWER && ph.mode == 0) {
+                    // two neighbouring 8-wide blocks per ldmatrix.x4 / stmatrix.x4
+                    const uint32_t lrow = 128u * (uint32_t)((lane & 7) + ((lane >> 3) & 1) * 8), lcol = 16u * (uint32_t)(lane >> 4);
+                    for (int i2 = 2 * warp; i2 < ph.n_items; i2 += 2 * kTeamWarps) {
+                        const uint32_t bfa = bf_s + 4u * (uint32_t)(ph.bfrag_off + i2 * 32 + lane);
+                        const uint32_t bf0 = lds32p(bfa), bf1 = lds32p(bfa + 128);
+                        uint32_t addr = sbase + lds32p(tab_s + 4u * (uint32_t)(ph.items_off + i2)) + lrow + lcol;
+                        addr = swz<LOWER>(addr);             // 16 rows further is the same swizzle
+                        for (int mt = 0; mt < P.MT; ++mt, addr += mt_step) {
+                            uint32_t a[4];
+                            ldmatrix_x4(a, addr);
+                            const uint32_t a_lo[2] = {a[0], a[1]}, a_hi[2] = {a[2], a[3]};
+                            float c0[4], c1[4];
+                            mma_k8(c0, a_lo, bf0);
+                            mma_k8(c1, a_hi, bf1);
+                            stmatrix_x4(addr, pack_bf16(c0[0], c0[1]), pack_bf16(c0[2], c0[3]), pack_bf16(c1[0], c1[1]), pack_bf16(c1[2], c1[3]));
+                        }
+                    }
+                } else if (B16 && ph.B == 16) {
+                    uint32_t so[4];
+                    bool ok[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        ok[j] = ph.lm * q + ph.jr[j] < ph.B_real;
+                        so[j] = ok[j] ? local_off(ph, ph.lm * q + ph.jr[j]) : 0u;      // padded slots read slot 0 and are not stored
+                    }
+                    const int n_work = ph.n_items * P.MT;
+                    for (int w = warp; w < n_work; w += kTeamWarps) {
+                        const int i1 = w >> P.mt_shift, mt = w & (P.MT - 1);
+                        const uint32_t a0 = sbase + lds32p(tab_s + 4u * (uint32_t)(ph.items_off + i1)) + row0_off + (uint32_t)mt * mt_step;
+                        const uint32_t bfa = bf_s + 4u * (uint32_t)(ph.bfrag_off + (i1 * 256 + lane) * 4);
+                        uint4 raw[4][2], bf[8];
+                        uint32_t unused[8][4];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) bf[e] = lds128(bfa + e * 512);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            raw[j][0] = lds128(swz<LOWER>(a0 + so[j]));
+                            raw[j][1] = lds128(swz<LOWER>(a0 + so[j] + row8_off));
+                        }
+                        octet_mma16<true>(raw, bf, unused);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (ok[j]) {
+                                sts128(swz<LOWER>(a0 + so[j]), raw[j][0]);
+                                sts128(swz<LOWER>(a0 + so[j] + row8_off), raw[j][1]);
+                            }
+                    }
+                } else {
+                    uint32_t so[2];
+                    bool ok[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        ok[j] = ph.lm * q + ph.jr[j] < ph.B_real;
+                        so[j] = ok[j] ? local_off(ph, ph.lm * q + ph.jr[j]) : 0u;
+                    }
+                    const int n_work = ph.n_items * P.MT;
+                    for (int w = warp; w < n_work; w += kTeamWarps) {
+                        const int i1 = w >> P.mt_shift, mt = w & (P.MT - 1);
+                        const uint32_t a0 = sbase + lds32p(tab_s + 4u * (uint32_t)(ph.items_off + i1)) + row0_off + (uint32_t)mt * mt_step;
+                        const uint32_t bfa = bf_s + 4u * (uint32_t)(ph.bfrag_off + i1 * 256 + lane * 4);
+                        uint4 raw[2][2];
+                        uint32_t bf[8], ad[2][2];
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            ad[j][0] = swz<LOWER>(a0 + so[j]);
+                            ad[j][1] = swz<LOWER>(a0 + so[j] + row8_off);
+                            raw[j][0] = lds128(ad[j][0]);
+                            raw[j][1] = lds128(ad[j][1]);
+                        }
+                        {
+                            const uint4 f0 = lds128(bfa), f1 = lds128(bfa + 512);
+                            bf[0] = f0.x; bf[1] = f0.y; bf[2] = f0.z; bf[3] = f0.w;
+                            bf[4] = f1.x; bf[5] = f1.y; bf[6] = f1.z; bf[7] = f1.w;
+                        }
+                        octet_mma8(raw, bf);
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            if (ok[j]) {
+                                sts128(ad[j][0], raw[j][0]);
+                                sts128(ad[j][1], raw[j][1]);
+                            }
+                    }
+                }
+                // the store of the tile before has had a phase's time to be read: refill its buffer
+                if (p == 0 && tid == 0 && t > team && t + (NB - 1) * TEAMS < count && !*(volatile int *)&dead) {
+                    harp_tm::bulk_wait_read0();
+                    load(cg, first + (t + (NB - 1) * TEAMS) * step, b == 0 ? NB - 1 : b - 1);
+                }
+            }
+            harp_tm::fence_async_smem();             // results before the copy engine reads them
+            team_sync();
+            if (tid == 0 && !*(volatile int *)&dead) store(cg, first + t * step, b);
+        }
+        if (tid == 0) harp_tm::bulk_wait_read0();
+    }
+    if (tid == 0) {
+        harp_tm::bulk_wait0();
+        if (*(volatile int *)&dead)                  // a load that came late must not land in the next CTA's memory
+            for (int k = 0; k < NB; ++k)
+                for (uint32_t it = 0; it < kPipeSpin && !mbar_try(smem_u32(&full_bar[team * kMaxPipeBufs + k]), (parity >> k) & 1u); ++it) {}
+    }
+}
+
+// ------------------------------------------------------------------------------- host
+
+typedef CUresult (*EncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
+                                const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+template <bool LOWER, bool B16>
+cudaError_t launch_pipe(const CUtensorMap &tmap, int32_t *err, const PipePass &P, unsigned grid, size_t smem, bool overlap, cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kTeamThreads * (B16 ? 1 : 3));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, harp_pipe_kernel<LOWER, B16>, tmap, err, P);
+}
+
+}  // namespace
+
+struct PipePlan {
+    PipePass dir[2];           // forward, transpose
+    bool lower = false, b16 = false;
+    int64_t d = 0, S_mid = 1;
+    int r_in = 1, r_out = 1;   // upper: radices of the inner and the outer digit of a tile
+    int64_t s_in = 0, s_out = 0;   // ... and their strides in coordinates
+    size_t smem = 0;
+    int sms = 148;
+    int32_t *d_err = nullptr;
+    std::vector<void *> dev_allocs;
+};
+
+void harp_pipe_destroy(PipePlan *pp) {
+    if (!pp) return;
+    for (void *p : pp->dev_allocs) cudaFree(p);
+    delete pp;
+}
+
+int32_t harp_pipe_error_word(const PipePlan *pp) {
+    if (!pp || !pp->d_err) return 0;
+    int32_t v = 0;
+    return cudaMemcpy(&v, pp->d_err, sizeof(v), cudaMemcpyDeviceToHost) == cudaSuccess ? v : -1;
+}
+
+// The pass over `phs` (lower: slabs of S_mid coordinates; upper: sixteen neighbouring positions of all U slabs).
+// HARP_ERR_UNSUPPORTED: a shape for which the layouts above are not free of conflicts, or whose tiles do not fit.
+harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &phs, bool lower, int64_t S_mid, int64_t U, PipePlan **out) {
+    *out = nullptr;
+    const int np = (int)phs.size();
+    if (np < 1 || np > kMaxPipePhases || !harp_tensor_map_encoder()) return HARP_ERR_UNSUPPORTED;
+    bool any16 = false;
+    for (const GPhase &gp : phs) any16 = any16 || gp.B == 16;
+    PipePass P{};
+    PipePlan pl;
+    P.n_phases = np;
+    if (lower) {
+        // boxes of 64 coordinates; the first phase in pairs of neighbouring blocks, the others by octets
+        if (any16 || S_mid % 64 != 0 || S_mid > 512 || phs[0].S != 1 || phs[0].B_real != 8) return HARP_ERR_UNSUPPORTED;
+        for (int p = 1; p < np; ++p)
+            if (phs[(size_t)p].S % 8 != 0) return HARP_ERR_UNSUPPORTED;
+        P.n_cg = (int)U;
+        P.n_box = (int)(S_mid / 64);
+    } else {
+        // the digit of odd radix inside, so that a step of either digit is an odd number of columns
+        if (np > 2 || S_mid % 16 != 0 || U > 64) return HARP_ERR_UNSUPPORTED;
+        const int in = np == 2 && phs[1].B_real % 2 != 0 ? 1 : 0;
+        if (np == 2 && phs[(size_t)in].B_real % 2 == 0) return HARP_ERR_UNSUPPORTED;
+        pl.r_in = phs[(size_t)in].B_real;
+        pl.s_in = phs[(size_t)in].S;
+        if (np == 2) { pl.r_out = phs[(size_t)(1 - in)].B_real; pl.s_out = phs[(size_t)(1 - in)].S; }
+        P.n_cg = (int)(S_mid / 16);
+        P.n_box = 2;
+        P.row_bytes = (int32_t)(32 * U);
+    }
+    auto place = [&](int64_t c) -> int64_t {             // byte offset of an octet; c: coordinate within the slab (lower) or natural coordinate
+        if (lower) return (c / 64) * P.box_pitch + (c % 64) * 2;
+        const int64_t i = (c / pl.s_in) % pl.r_in, o = np == 2 ? (c / pl.s_out) % pl.r_out : 0;
+        return (o * pl.r_in + i) * 32 + (c % 16) * 2;
+    };
+    int words = 0, items = 0;
+    for (const GPhase &gp : phs) {
+        const int n_blk = (int)((lower ? S_mid : U * 16) / gp.B_real);
+        words += n_blk * 32 * (gp.B == 16 ? 4 : 1);
+        items += lower && gp.S == 1 ? n_blk : n_blk / 8;
+    }
+    // the largest tile that fits; a pass of one phase refills a buffer while two others are full
+    const int teams = any16 ? 1 : 3;
+    const size_t most = any16 ? 112u * 1024u : 226u * 1024u;
+    P.n_buf = np == 1 ? 3 : 2;
+    for (P.MT = 4, P.mt_shift = 2;; P.MT /= 2, --P.mt_shift) {
+        P.box_bytes = lower ? 128 * 16 * P.MT : 8 * P.MT * P.row_bytes;
+        P.box_pitch = P.box_bytes + 128;                 // an odd number of 128 bytes: P.box_bytes is a multiple of 256
+        P.tile_bytes = P.n_box * P.box_pitch;
+        pl.smem = (size_t)teams * P.n_buf * P.tile_bytes + (size_t)words * 4 + (size_t)items * 4 + 128;
+        if (pl.smem <= most) break;
+        if (P.MT == 1) return HARP_ERR_UNSUPPORTED;
+    }
+    pl.lower = lower;
+    pl.b16 = any16;
+    pl.d = plan->d;
+    pl.S_mid = S_mid;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (sms > 0) pl.sms = sms;
+
+    static const int jo16[4] = {0, 4, 8, 12}, jo8[2][2] = {{0, 4}, {0, 1}};
+    harp_status_t st = HARP_OK;
+    auto upload = [&](const void *src, size_t bytes) -> void * {
+        void *p = nullptr;
+        if (st != HARP_OK) return nullptr;
+        if (cudaMalloc(&p, std::max<size_t>(16, bytes)) != cudaSuccess) { st = HARP_ERR_ALLOC; return nullptr; }
+        pl.dev_allocs.push_back(p);
+        if (cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) st = HARP_ERR_CUDA;
+        return p;
+    };
+    const int32_t zero = 0;
+    pl.d_err = static_cast<int32_t *>(upload(&zero, sizeof(zero)));
+    for (int dir = 0; dir < 2 && st == HARP_OK; ++dir) {
+        std::vector<int32_t> tab;
+        std::vector<uint32_t> frag((size_t)P.n_cg * words, 0u);
+        std::vector<double> F;
+        int at = 0;
+        for (int k = 0; k < np; ++k) {
+            const GPhase &gp = phs[(size_t)(dir == 0 ? k : np - 1 - k)];
+            PipePhase &D = P.ph[k];
+            D = PipePhase{};
+            D.mode = lower && gp.S == 1 ? 0 : 1;
+            D.B = gp.B;
+            D.B_real = gp.B_real;
+            D.lm = lower && D.mode == 1 ? 2 : 1;
+            for (int j = 0; j < 4; ++j) D.jr[j] = gp.B == 16 ? jo16[j] : j < 2 ? jo8[D.lm - 1][j] : 0;
+            D.items_off = (int32_t)tab.size();
+            D.bfrag_off = at;
+            if (lower) {                                 // in octets: eight to a box
+                D.unit = (int32_t)(gp.S / 8);
+                D.shift = 3;
+                D.step[0] = 16;
+                D.step[1] = P.box_pitch;
+            } else {
+                D.unit = 1;
+                D.step[1] = gp.S == pl.s_in ? 32 : 32 * pl.r_in;
+            }
+            // first coordinates of the blocks (lower: within the slab; upper: within position group 0)
+            std::vector<int64_t> first;
+            if (D.mode == 0) {
+                for (int64_t c = 0; c < S_mid; c += 8) { first.push_back(c); tab.push_back((int32_t)place(c)); }
+            } else {
+                const int64_t span = gp.S * gp.B_real, all = lower ? S_mid : plan->d, lo_step = lower ? 8 : S_mid;
+                for (int64_t hi = 0; hi < all; hi += span)
+                    for (int64_t lo = 0; lo < gp.S; lo += lo_step)
+                        for (int64_t l8 = 0; l8 < (lower ? 8 : 16); l8 += 8) {
+                            const int64_t c = hi + lo + l8;
+                            for (int r = 0; r < gp.B_real; ++r) {       // every octet that the kernel reaches
+                                const int e = r * D.unit;
+                                const int64_t a = place(c) + (e >> D.shift) * D.step[1] + (e & ((1 << D.shift) - 1)) * D.step[0];
+                                if (a != place(c + r * gp.S) || a < 0 || a + 16 > (lower ? P.tile_bytes : P.row_bytes)) return HARP_ERR_UNSUPPORTED;
+                            }
+                            tab.push_back((int32_t)place(c));
+                            for (int e = 0; e < 8; ++e) first.push_back(c + e);
+                        }
+            }
+            D.n_items = (int32_t)tab.size() - D.items_off;
+            auto slot = [&](int s) { return D.mode == 0 ? s : strided_slot(s, gp.B, D.lm); };
+            const int wpl = gp.B == 16 ? 4 : 1;
+            const bool grouped = D.mode == 1 && gp.B == 8;       // [item][blocks 0-3 | 4-7][lane][4 words]
+            for (int cg = 0; cg < P.n_cg; ++cg)
+                for (size_t i = 0; i < first.size(); ++i) {
+                    const int64_t base = (lower ? cg * S_mid : cg * 16) + first[i];
+                    uint32_t *dst = frag.data() + (size_t)cg * words + at + (grouped ? (i / 8) * 256 + ((i % 8) / 4) * 128 + i % 4 : i * 32 * wpl);
+                    block_fragment(plan, gp, base, dir, slot, dst, grouped ? 4 : wpl, F);
+                }
+            at += (int)first.size() * 32 * wpl;
+        }
+        if (at != words || (int)tab.size() != items || words % 4 != 0) return HARP_ERR_UNSUPPORTED;
+        P.tables_len = items;
+        P.bfrag_words = words;
+        P.tables = static_cast<const int32_t *>(upload(tab.data(), tab.size() * 4));
+        P.bfrag = static_cast<const uint32_t *>(upload(frag.data(), frag.size() * 4));
+        pl.dir[dir] = P;
+    }
+    PipePlan *pp = st == HARP_OK ? new (std::nothrow) PipePlan(pl) : nullptr;
+    if (!pp) {
+        for (void *p : pl.dev_allocs) cudaFree(p);
+        return st == HARP_OK ? HARP_ERR_ALLOC : st;
+    }
+    *out = pp;
+    if (cudaFuncSetAttribute(harp_pipe_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess ||
+        cudaFuncSetAttribute(harp_pipe_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess ||
+        cudaFuncSetAttribute(harp_pipe_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024) != cudaSuccess)
+        return HARP_ERR_CUDA;
+    return HARP_OK;
+}
+
+// x: n_rows contiguous rows, 16-byte aligned.
+harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int transpose, bool overlap, cudaStream_t stream) {
+    if (!pp || n_rows > ((int64_t)1 << 30)) return HARP_ERR_UNSUPPORTED;
+    PipePass P = pp->dir[transpose ? 1 : 0];
+    P.n_tiles = (int32_t)((n_rows + 16 * P.MT - 1) / (16 * P.MT));
+    const int64_t slots = (int64_t)pp->sms * (pp->b16 ? 2 : 1);
+    // A column group per CTA keeps its fragments, and the CTAs at the same rows: neighbouring 32-byte runs meet in L2.  Where
+    // the groups leave more than a tenth of the SMs without work, lower passes (whole lines) share the list out evenly.
+    P.n_parts = (int32_t)std::min<int64_t>(P.n_tiles, std::max<int64_t>(1, slots / P.n_cg));
+    if (pp->lower && (P.n_cg > slots || slots % P.n_cg * 10 > slots)) P.n_parts = 0;
+    const unsigned grid = (unsigned)(P.n_parts > 0 ? (int64_t)P.n_parts * P.n_cg : std::min<int64_t>((int64_t)P.n_tiles * P.n_cg, slots));
+    const auto enc = reinterpret_cast<EncodeTiled>(harp_tensor_map_encoder());
+    CUtensorMap tmap = {};
+    const cuuint32_t ones[4] = {1, 1, 1, 1};
+    const cuuint64_t n = (cuuint64_t)n_rows, pitch = (cuuint64_t)pp->d * 2;
+    CUresult r;
+    if (pp->lower) {
+        const cuuint64_t gdim[2] = {(cuuint64_t)pp->d, n}, gstr[1] = {pitch};
+        const cuuint32_t box[2] = {64, (cuuint32_t)(16 * P.MT)};
+        r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    } else {
+        // (position, inner digit, outer digit, row)
+        const cuuint64_t gdim[4] = {(cuuint64_t)pp->S_mid, (cuuint64_t)pp->r_in, (cuuint64_t)pp->r_out, n};
+        const cuuint64_t gstr[3] = {(cuuint64_t)pp->s_in * 2, (cuuint64_t)(pp->r_out > 1 ? pp->s_out : pp->s_in) * 2, pitch};
+        const cuuint32_t box[4] = {16, (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
+        r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    }
+    if (r != CUDA_SUCCESS) return HARP_ERR_CUDA;
+    const cudaError_t err = pp->lower ? launch_pipe<true, false>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream)
+                            : pp->b16 ? launch_pipe<false, true>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream)
+                                      : launch_pipe<false, false>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream);
+    g_harp_launches.fetch_add(1, std::memory_order_relaxed);
+    return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? HARP_OK : HARP_ERR_CUDA;
+}

@@ -683,6 +683,7 @@ struct SplitPlan {
     const uint16_t *gather[2] = {nullptr, nullptr};
     int gather_rows = 1;       // rows per buffer of the gather kernel
     size_t gather_smem = 0;
+    PipePlan *pipe[2] = {nullptr, nullptr};   // the passes fed by the copy engine (harp_pipe.cu), where the shape allows them
     // dense upper pass (replaces pass[1] when set)
     bool dense_upper = false;
     bool up_in_regs = false;   // fragments in registers (harp_upper_reg_kernel)
@@ -692,12 +693,6 @@ struct SplitPlan {
 };
 
 namespace {
-
-struct GPhase {                // a fused group of stages
-    int t0, t1;
-    int B, B_real;
-    int64_t S;                 // natural stride
-};
 
 template <typename T>
 T *upload_s(SplitPlan *sp, const std::vector<T> &v, harp_status_t &st) {
@@ -868,42 +863,16 @@ harp_status_t build_pass(const harp_plan *plan, SplitPlan *sp, PassHost &ph_out,
             for (int p = 0; p < np; ++p) {
                 const GPhase &gp = phs[(size_t)p];
                 const ItemSet &is = sets[(size_t)p];
-                const int B = gp.B, Br = gp.B_real;
                 const int l = is.mode == 0 ? 1 : lm[(size_t)p];
-                HostPhase hp{gp.t0, gp.t1, Br, gp.S, 0, 1};
-                const int wpl = B == 16 ? 4 : 1;
+                const int wpl = gp.B == 16 ? 4 : 1;
+                auto slot = [&](int s) { return is.mode == 0 ? s : strided_slot(s, gp.B, l); };
+                // 8-wide strided phases: the words of an item's eight blocks sit together per lane,
+                // [item][blocks 0-3 | 4-7][lane][4 words], so that a lane fetches them with two 16-byte loads
+                const bool grouped = is.mode == 1 && gp.B == 8;
                 for (size_t bi = 0; bi < is.block_rel.size(); ++bi) {
-                    const int64_t base = cg_base + is.block_rel[bi];
-                    fused_block(plan, hp, base, F);
-                    auto G = [&](int rin, int rout) -> double {
-                        if (rin >= Br || rout >= Br) return 0.0;
-                        double v = dir == 0 ? F[(size_t)rin * Br + rout] : F[(size_t)rout * Br + rin];
-                        if (gp.t0 == 0 && !plan->h_signs.empty()) {
-                            const int64_t pos = base + (int64_t)(dir == 0 ? rin : rout) * gp.S;
-                            v *= (double)plan->h_signs[(size_t)(plan->h_perm.empty() ? pos : plan->h_perm[(size_t)pos])];
-                        }
-                        return v;
-                    };
-                    auto slot = [&](int s) { return is.mode == 0 ? s : strided_slot(s, B, l); };
-                    uint32_t *dst0 = frag.data() + (size_t)cgi * words + frag_off[(size_t)p] + bi * 32 * wpl;
-                    // 8-wide strided phases: the words of an item's eight blocks sit together per lane,
-                    // [item][blocks 0-3 | 4-7][lane][4 words], so that a lane fetches them with two 16-byte loads
-                    const bool grouped = is.mode == 1 && B == 8;
-                    uint32_t *grp0 = frag.data() + (size_t)cgi * words + frag_off[(size_t)p] + (bi / 8) * 256 + ((bi % 8) / 4) * 128 + (bi % 4);
-                    for (int lane = 0; lane < 32; ++lane) {
-                        const int gg = lane >> 2, qq = lane & 3;
-                        uint32_t *dst = grouped ? grp0 + lane * 4 : dst0 + lane * wpl;
-                        if (B == 16) {
-                            for (int nt = 0; nt < 2; ++nt) {
-                                const int n = slot(8 * nt + gg);
-                                dst[2 * nt] = f2bf(G(slot(2 * qq), n)) | ((uint32_t)f2bf(G(slot(2 * qq + 1), n)) << 16);
-                                dst[2 * nt + 1] = f2bf(G(slot(2 * qq + 8), n)) | ((uint32_t)f2bf(G(slot(2 * qq + 9), n)) << 16);
-                            }
-                        } else {
-                            const int n = slot(gg);
-                            dst[0] = f2bf(G(slot(2 * qq), n)) | ((uint32_t)f2bf(G(slot(2 * qq + 1), n)) << 16);
-                        }
-                    }
+                    uint32_t *dst = frag.data() + (size_t)cgi * words + frag_off[(size_t)p] +
+                                    (grouped ? (bi / 8) * 256 + ((bi % 8) / 4) * 128 + bi % 4 : bi * 32 * wpl);
+                    block_fragment(plan, gp, cg_base + is.block_rel[bi], dir, slot, dst, grouped ? 4 : wpl, F);
                 }
             }
         }
@@ -1023,6 +992,11 @@ harp_status_t harp_split_build(harp_plan *plan) {
     harp_status_t st = build_pass(plan, sp, sp->pass[0], lower, true, S_mid, U, 1);
     if (st == HARP_OK && want_dense) st = build_dense_upper(plan, sp, lower.back().t1, S_mid, U);
     else if (st == HARP_OK && !upper.empty()) st = build_pass(plan, sp, sp->pass[1], upper, false, S_mid, U, Lw);
+    for (int s = 0; s < 2 && st == HARP_OK; ++s) {
+        if (!sp->pass[s].present) continue;
+        st = harp_pipe_build(plan, s == 0 ? lower : upper, s == 0, S_mid, U, &sp->pipe[s]);
+        if (st == HARP_ERR_UNSUPPORTED) st = HARP_OK;
+    }
     if (st == HARP_OK &&
         (cudaFuncSetAttribute(harp_split_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024) != cudaSuccess ||
          cudaFuncSetAttribute(harp_split_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024) != cudaSuccess ||
@@ -1078,6 +1052,7 @@ harp_status_t harp_split_build(harp_plan *plan) {
 void harp_split_destroy(harp_plan *plan) {
     if (!plan->split) return;
     for (void *p : plan->split->dev_allocs) cudaFree(p);
+    for (PipePlan *pp : plan->split->pipe) harp_pipe_destroy(pp);
     delete plan->split;
     plan->split = nullptr;
 }
@@ -1108,6 +1083,14 @@ constexpr int64_t kOverlapMaxElems = (int64_t)16 << 20;
 // (400 rows of d = 14336: 21.1 us with the mma.sync slab pass, 18.6 with the tensor-memory one; at 256 rows its 128-row tiles
 // leave a third of the SMs idle and it is the slower one)
 constexpr int64_t kTmSlabMinRows = 384;
+
+static int64_t pipe_min_rows() { const char *e = getenv("HARP_PIPE_ROWS"); return e ? atoll(e) : 1024; }
+int32_t harp_split_error_word(const harp_plan *plan) {
+    int32_t w = 0;
+    if (plan->split)
+        for (const PipePlan *pp : plan->split->pipe) w = w != 0 ? w : harp_pipe_error_word(pp);
+    return w;
+}
 
 harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose,
                                cudaStream_t stream) {
@@ -1165,6 +1148,11 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
                 const harp_status_t ts = harp_tm_slab_apply(plan, xb + r0 * plan->d, r1 - r0, dtype, transpose, stream);
                 if (ts == HARP_OK) continue;
                 if (ts != HARP_ERR_UNSUPPORTED) return ts;
+            }
+            if (sp->pipe[pi] && r1 - r0 >= pipe_min_rows()) {
+                const harp_status_t ps = harp_pipe_apply(sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
+                if (ps != HARP_OK) return ps;
+                continue;
             }
             const PassHost &ph = sp->pass[pi];
             SplitPass P = transpose ? ph.bwd : ph.fwd;
