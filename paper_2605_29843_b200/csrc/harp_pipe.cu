@@ -30,7 +30,6 @@ using harp_tm::mbar_expect_tx;
 using harp_tm::mbar_init;
 using harp_tm::mbar_try;
 
-constexpr int kTeamWarps = 8, kTeamThreads = 32 * kTeamWarps;
 constexpr int kMaxPipePhases = 3, kMaxPipeBufs = 4;
 constexpr uint32_t kPipeSpin = 1u << 22;      // limit of every wait for a bulk copy
 
@@ -80,12 +79,87 @@ __device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
     return (uint32_t)((e >> ph.shift) * ph.step[1] + (e & ((1 << ph.shift) - 1)) * ph.step[0]);
 }
 
-// A team: eight warps with n_buf tile buffers of their own.  Tiles of the CTA's column group go to its teams in turn; a team's
-// thread 0 issues its bulk copies.  Sixteen-wide blocks need 128 registers: one team, two CTAs per SM.
-template <bool LOWER, bool B16>
-__global__ void __launch_bounds__(kTeamThreads * (B16 ? 1 : 3), B16 ? 2 : 1)
+// The kinds of pass.  A team is a few warps with n_buf tile buffers of their own; tiles of the CTA's column group go to its
+// teams in turn and a team's thread 0 issues its bulk copies.
+//   lower8, upper8   three teams of eight warps, at most 85 registers; the teams share the fragments
+//   upper16          sixteen-wide blocks need 128 registers: one team, two CTAs per SM
+//   dense32, dense48 all upper stages as one block of up to 32 or 48: a warp holds sixteen rows of eight positions, the two octets of a
+//                    tile make a team of two warps
+enum Kind { kLower8, kUpper8, kUpper16, kDense32, kDense48 };
+template <int K> struct KindOf {
+    static constexpr bool lower = K == kLower8, b16 = K == kUpper16;
+    static constexpr int ks = K == kDense32 ? 2 : K == kDense48 ? 3 : 0;
+    static constexpr int team_warps = ks ? 2 : 8, team_threads = 32 * team_warps, teams = b16 ? 1 : 3, threads = teams * team_threads;
+    static constexpr int ctas = b16 ? 2 : 1;
+};
+
+// Eight positions of sixteen rows through one dense block each (U <= 16 KS).  raw: slot s of this lane is coordinate
+// 16 (s / 4) + q + 4 (s % 4); results replace the operands word by word.
+// Fragments: [pair of positions][pair of column tiles][position of the pair][KS][lane][4 words].
+template <int KS, typename Mid>
+__device__ __forceinline__ void dense_octet(uint32_t a0, uint32_t row8_off, int q, int U, uint32_t bfa, const Mid &mid) {
+    uint4 raw[4 * KS][2];
+#pragma unroll
+    for (int s = 0; s < 4 * KS; ++s) {
+        const int u = 16 * (s / 4) + q + 4 * (s % 4);
+        const uint32_t o = a0 + 32u * (uint32_t)u;
+        raw[s][0] = u < U ? lds128(swz<false>(o)) : make_uint4(0u, 0u, 0u, 0u);
+        raw[s][1] = u < U ? lds128(swz<false>(o + row8_off)) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        uint32_t a[2][KS][4];
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const uint32_t x = word_of(raw[4 * ks + 2 * (m >> 1)][m & 1], w), y = word_of(raw[4 * ks + 2 * (m >> 1) + 1][m & 1], w);
+                a[0][ks][m] = pair_lo(x, y);
+                a[1][ks][m] = pair_hi(x, y);
+            }
+#pragma unroll
+        for (int c = 0; c < KS; ++c) {
+            uint4 f[2][KS];
+#pragma unroll
+            for (int ee = 0; ee < 2; ++ee)
+#pragma unroll
+                for (int t = 0; t < KS; ++t) f[ee][t] = lds128(bfa + 512u * (uint32_t)(((w * KS + c) * 2 + ee) * KS + t));
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                float acc[2][4];
+#pragma unroll
+                for (int ee = 0; ee < 2; ++ee)
+#pragma unroll
+                    for (int ks = 0; ks < KS; ++ks) {
+                        const int at = 2 * (k * KS + ks);
+                        const uint32_t b0 = word_of(f[ee][at / 4], at % 4), b1 = word_of(f[ee][at / 4], at % 4 + 1);
+                        if (ks == 0) mma_k16(acc[ee], a[ee][ks], b0, b1);
+                        else mma_k16_acc(acc[ee], a[ee][ks], b0, b1);
+                    }
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) set_word(raw[4 * c + i + 2 * k][h], w, pack_bf16(acc[0][i + 2 * h], acc[1][i + 2 * h]));
+            }
+        }
+        if (w == 1) mid();
+    }
+#pragma unroll
+    for (int s = 0; s < 4 * KS; ++s) {
+        const int u = 16 * (s / 4) + q + 4 * (s % 4);
+        const uint32_t o = a0 + 32u * (uint32_t)u;
+        if (u < U) {
+            sts128(swz<false>(o), raw[s][0]);
+            sts128(swz<false>(o + row8_off), raw[s][1]);
+        }
+    }
+}
+
+template <int K>
+__global__ void __launch_bounds__(KindOf<K>::threads, KindOf<K>::ctas)
 harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const PipePass P) {
-    constexpr int TEAMS = B16 ? 1 : 3;
+    constexpr bool LOWER = KindOf<K>::lower, B16 = KindOf<K>::b16;
+    constexpr int KS = KindOf<K>::ks, TEAMS = KindOf<K>::teams, kTeamWarps = KindOf<K>::team_warps, kTeamThreads = KindOf<K>::team_threads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[TEAMS * kMaxPipeBufs];
     __shared__ int dead;
@@ -97,7 +171,7 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
     const uint32_t bf_s = smem0 + (uint32_t)(TEAMS * NB * P.tile_bytes);
     const uint32_t tab_s = bf_s + 4u * (uint32_t)P.bfrag_words;
     for (int i = threadIdx.x; i < P.tables_len; i += TEAMS * kTeamThreads)
-        asm volatile("st.shared.u32 [%0], %1;" ::"r"(tab_s + 4u * i), "r"(__ldg(P.tables + i)) : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(tab_s + 4u * i), "l"(P.tables + i) : "memory");
     if (threadIdx.x == 0) {
         for (int b = 0; b < TEAMS * kMaxPipeBufs; ++b) mbar_init(smem_u32(&full_bar[b]), 1);
         dead = 0;
@@ -157,8 +231,6 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
         __syncthreads();
         const uint32_t *src = P.bfrag + (size_t)cg * P.bfrag_words;
         for (int i = threadIdx.x * 4; i < P.bfrag_words; i += TEAMS * kTeamThreads * 4) cp_async16(bf_s + 4u * i, src + i);
-        cp_async_wait_all();
-        __syncthreads();
         if (!waited) {                               // the rows only once the kernel before has completed
             asm volatile("griddepcontrol.wait;" ::: "memory");
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -167,6 +239,8 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
         if (tid == 0 && !*(volatile int *)&dead)
             for (int k = 0; k < NB; ++k)
                 if (team + k * TEAMS < count) load(cg, first + (team + k * TEAMS) * step, k);
+        cp_async_wait_all();
+        __syncthreads();
         int b = 0;
         for (int t = team; t < count; t += TEAMS, b = b + 1 == NB ? 0 : b + 1) {
             const uint32_t bar = smem_u32(&full_bar[team * kMaxPipeBufs + b]), sbase = bufs + (uint32_t)(b * P.tile_bytes);
@@ -179,6 +253,17 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
                 }
             }
             parity ^= 1u << b;
+            // the store of the tile before has had a phase's time to be read: refill its buffer
+            auto refill = [&]() {
+                if (tid == 0 && t > team && t + (NB - 1) * TEAMS < count && !*(volatile int *)&dead) {
+                    harp_tm::bulk_wait_read0();
+                    load(cg, first + (t + (NB - 1) * TEAMS) * step, b == 0 ? NB - 1 : b - 1);
+                }
+            };
+            if constexpr (KS > 0) {
+                dense_octet<KS>(sbase + 16u * (uint32_t)warp + row0_off, row8_off, q, P.ph[0].B_real,
+                                bf_s + 16u * (uint32_t)(warp * 8 * KS * KS * 32 + lane), refill);
+            } else
             for (int p = 0; p < P.n_phases; ++p) {
                 const PipePhase &ph = P.ph[p];
                 if (p > 0) team_sync();
@@ -266,11 +351,7 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
                             }
                     }
                 }
-                // the store of the tile before has had a phase's time to be read: refill its buffer
-                if (p == 0 && tid == 0 && t > team && t + (NB - 1) * TEAMS < count && !*(volatile int *)&dead) {
-                    harp_tm::bulk_wait_read0();
-                    load(cg, first + (t + (NB - 1) * TEAMS) * step, b == 0 ? NB - 1 : b - 1);
-                }
+                if (p == 0) refill();
             }
             harp_tm::fence_async_smem();             // results before the copy engine reads them
             team_sync();
@@ -292,11 +373,15 @@ typedef CUresult (*EncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, 
                                 const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-template <bool LOWER, bool B16>
+constexpr int smem_most(int kind) { return kind == kUpper16 ? 112 * 1024 : 226 * 1024; }
+
+template <int K>
 cudaError_t launch_pipe(const CUtensorMap &tmap, int32_t *err, const PipePass &P, unsigned grid, size_t smem, bool overlap, cudaStream_t stream) {
+    const cudaError_t ae = cudaFuncSetAttribute(harp_pipe_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_most(K));
+    if (ae != cudaSuccess) return ae;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kTeamThreads * (B16 ? 1 : 3));
+    cfg.blockDim = dim3(KindOf<K>::threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -304,14 +389,40 @@ cudaError_t launch_pipe(const CUtensorMap &tmap, int32_t *err, const PipePass &P
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, harp_pipe_kernel<LOWER, B16>, tmap, err, P);
+    return cudaLaunchKernelEx(&cfg, harp_pipe_kernel<K>, tmap, err, P);
+}
+
+// Fragments of the dense blocks (see dense_octet), sixteen positions per column group.
+void dense_fragments(const harp_plan *plan, const GPhase &gp, int n_cg, int ks, int dir, std::vector<uint32_t> &frag) {
+    const int U = gp.B_real;
+    std::vector<double> F;
+    auto coord = [&](int slot) { return 16 * (slot / 16) + strided_slot(slot % 16, 16, 1); };
+    for (int l = 0; l < 16 * n_cg; ++l) {
+        fused_block(plan, HostPhase{gp.t0, gp.t1, U, gp.S, 0, 1}, l, F);
+        auto G = [&](int slot_in, int slot_out) -> double {
+            const int i = coord(slot_in), o = coord(slot_out);
+            return i >= U || o >= U ? 0.0 : dir == 0 ? F[(size_t)i * U + o] : F[(size_t)o * U + i];
+        };
+        for (int c = 0; c < ks; ++c)
+            for (int k = 0; k < 2; ++k)
+                for (int s = 0; s < ks; ++s)
+                    for (int h = 0; h < 2; ++h) {
+                        const int f = 2 * (k * ks + s) + h;
+                        // [octet][pair of positions][c][position of the pair][f / 4][lane][f % 4]
+                        uint32_t *dst = frag.data() + ((size_t)(((l / 2) * ks + c) * 2 + l % 2) * ks + f / 4) * 128 + f % 4;
+                        for (int lane = 0; lane < 32; ++lane) {
+                            const int n = 16 * c + 8 * k + (lane >> 2), kk = 16 * s + 8 * h + 2 * (lane & 3);
+                            dst[lane * 4] = f2bf(G(kk, n)) | ((uint32_t)f2bf(G(kk + 1, n)) << 16);
+                        }
+                    }
+    }
 }
 
 }  // namespace
 
 struct PipePlan {
     PipePass dir[2];           // forward, transpose
-    bool lower = false, b16 = false;
+    int kind = kLower8;
     int64_t d = 0, S_mid = 1;
     int r_in = 1, r_out = 1;   // upper: radices of the inner and the outer digit of a tile
     int64_t s_in = 0, s_out = 0;   // ... and their strides in coordinates
@@ -339,21 +450,23 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
     *out = nullptr;
     const int np = (int)phs.size();
     if (np < 1 || np > kMaxPipePhases || !harp_tensor_map_encoder()) return HARP_ERR_UNSUPPORTED;
-    bool any16 = false;
-    for (const GPhase &gp : phs) any16 = any16 || gp.B == 16;
+    int widest = 8;
+    for (const GPhase &gp : phs) widest = std::max(widest, gp.B);
     PipePass P{};
     PipePlan pl;
+    pl.kind = lower ? kLower8 : widest == 8 ? kUpper8 : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
+    const int ks = pl.kind >= kDense32 ? widest / 16 : 0;
     P.n_phases = np;
     if (lower) {
         // boxes of 64 coordinates; the first phase in pairs of neighbouring blocks, the others by octets
-        if (any16 || S_mid % 64 != 0 || S_mid > 512 || phs[0].S != 1 || phs[0].B_real != 8) return HARP_ERR_UNSUPPORTED;
+        if (widest > 8 || S_mid % 64 != 0 || S_mid > 512 || phs[0].S != 1 || phs[0].B_real != 8) return HARP_ERR_UNSUPPORTED;
         for (int p = 1; p < np; ++p)
             if (phs[(size_t)p].S % 8 != 0) return HARP_ERR_UNSUPPORTED;
         P.n_cg = (int)U;
         P.n_box = (int)(S_mid / 64);
     } else {
         // the digit of odd radix inside, so that a step of either digit is an odd number of columns
-        if (np > 2 || S_mid % 16 != 0 || U > 64) return HARP_ERR_UNSUPPORTED;
+        if (np > (ks ? 1 : 2) || widest > 48 || S_mid % 16 != 0 || U > 64) return HARP_ERR_UNSUPPORTED;
         const int in = np == 2 && phs[1].B_real % 2 != 0 ? 1 : 0;
         if (np == 2 && phs[(size_t)in].B_real % 2 == 0) return HARP_ERR_UNSUPPORTED;
         pl.r_in = phs[(size_t)in].B_real;
@@ -371,14 +484,14 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
     int words = 0, items = 0;
     for (const GPhase &gp : phs) {
         const int n_blk = (int)((lower ? S_mid : U * 16) / gp.B_real);
-        words += n_blk * 32 * (gp.B == 16 ? 4 : 1);
-        items += lower && gp.S == 1 ? n_blk : n_blk / 8;
+        words += ks ? 16 * 4 * ks * ks * 32 : n_blk * 32 * (gp.B == 16 ? 4 : 1);
+        items += ks ? 0 : lower && gp.S == 1 ? n_blk : n_blk / 8;
     }
     // the largest tile that fits; a pass of one phase refills a buffer while two others are full
-    const int teams = any16 ? 1 : 3;
-    const size_t most = any16 ? 112u * 1024u : 226u * 1024u;
-    P.n_buf = np == 1 ? 3 : 2;
-    for (P.MT = 4, P.mt_shift = 2;; P.MT /= 2, --P.mt_shift) {
+    const int teams = pl.kind == kUpper16 ? 1 : 3;
+    const size_t most = (size_t)smem_most(pl.kind);
+    P.n_buf = np == 1 && !ks ? 3 : 2;
+    for (P.MT = ks ? 1 : 4, P.mt_shift = ks ? 0 : 2;; P.MT /= 2, --P.mt_shift) {
         P.box_bytes = lower ? 128 * 16 * P.MT : 8 * P.MT * P.row_bytes;
         P.box_pitch = P.box_bytes + 128;                 // an odd number of 128 bytes: P.box_bytes is a multiple of 256
         P.tile_bytes = P.n_box * P.box_pitch;
@@ -386,8 +499,6 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
         if (pl.smem <= most) break;
         if (P.MT == 1) return HARP_ERR_UNSUPPORTED;
     }
-    pl.lower = lower;
-    pl.b16 = any16;
     pl.d = plan->d;
     pl.S_mid = S_mid;
     int dev = 0, sms = 0;
@@ -423,6 +534,11 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
             for (int j = 0; j < 4; ++j) D.jr[j] = gp.B == 16 ? jo16[j] : j < 2 ? jo8[D.lm - 1][j] : 0;
             D.items_off = (int32_t)tab.size();
             D.bfrag_off = at;
+            if (ks) {
+                dense_fragments(plan, gp, P.n_cg, ks, dir, frag);
+                at = words;
+                continue;
+            }
             if (lower) {                                 // in octets: eight to a box
                 D.unit = (int32_t)(gp.S / 8);
                 D.shift = 3;
@@ -476,10 +592,6 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
         return st == HARP_OK ? HARP_ERR_ALLOC : st;
     }
     *out = pp;
-    if (cudaFuncSetAttribute(harp_pipe_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess ||
-        cudaFuncSetAttribute(harp_pipe_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess ||
-        cudaFuncSetAttribute(harp_pipe_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024) != cudaSuccess)
-        return HARP_ERR_CUDA;
     return HARP_OK;
 }
 
@@ -487,19 +599,25 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
 harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int transpose, bool overlap, cudaStream_t stream) {
     if (!pp || n_rows > ((int64_t)1 << 30)) return HARP_ERR_UNSUPPORTED;
     PipePass P = pp->dir[transpose ? 1 : 0];
+    const int64_t slots = (int64_t)pp->sms * (pp->kind == kUpper16 ? 2 : 1);
+    // a batch with less than half a tile per CTA is cut finer
+    while (P.MT > 1 && (n_rows + 16 * P.MT - 1) / (16 * P.MT) * P.n_cg * 2 < slots) {
+        P.MT /= 2;
+        --P.mt_shift;
+        P.box_bytes /= 2;
+    }
     P.n_tiles = (int32_t)((n_rows + 16 * P.MT - 1) / (16 * P.MT));
-    const int64_t slots = (int64_t)pp->sms * (pp->b16 ? 2 : 1);
     // A column group per CTA keeps its fragments, and the CTAs at the same rows: neighbouring 32-byte runs meet in L2.  Where
     // the groups leave more than a tenth of the SMs without work, lower passes (whole lines) share the list out evenly.
     P.n_parts = (int32_t)std::min<int64_t>(P.n_tiles, std::max<int64_t>(1, slots / P.n_cg));
-    if (pp->lower && (P.n_cg > slots || slots % P.n_cg * 10 > slots)) P.n_parts = 0;
+    if (pp->kind == kLower8 && (P.n_cg > slots || slots % P.n_cg * 10 > slots)) P.n_parts = 0;
     const unsigned grid = (unsigned)(P.n_parts > 0 ? (int64_t)P.n_parts * P.n_cg : std::min<int64_t>((int64_t)P.n_tiles * P.n_cg, slots));
     const auto enc = reinterpret_cast<EncodeTiled>(harp_tensor_map_encoder());
     CUtensorMap tmap = {};
     const cuuint32_t ones[4] = {1, 1, 1, 1};
     const cuuint64_t n = (cuuint64_t)n_rows, pitch = (cuuint64_t)pp->d * 2;
     CUresult r;
-    if (pp->lower) {
+    if (pp->kind == kLower8) {
         const cuuint64_t gdim[2] = {(cuuint64_t)pp->d, n}, gstr[1] = {pitch};
         const cuuint32_t box[2] = {64, (cuuint32_t)(16 * P.MT)};
         r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -513,9 +631,14 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
                 CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
     if (r != CUDA_SUCCESS) return HARP_ERR_CUDA;
-    const cudaError_t err = pp->lower ? launch_pipe<true, false>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream)
-                            : pp->b16 ? launch_pipe<false, true>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream)
-                                      : launch_pipe<false, false>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream);
+    cudaError_t err = cudaErrorInvalidValue;
+    switch (pp->kind) {
+        case kLower8: err = launch_pipe<kLower8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kUpper8: err = launch_pipe<kUpper8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kUpper16: err = launch_pipe<kUpper16>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kDense32: err = launch_pipe<kDense32>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kDense48: err = launch_pipe<kDense48>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+    }
     g_harp_launches.fetch_add(1, std::memory_order_relaxed);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? HARP_OK : HARP_ERR_CUDA;
 }

@@ -993,7 +993,8 @@ harp_status_t harp_split_build(harp_plan *plan) {
     if (st == HARP_OK && want_dense) st = build_dense_upper(plan, sp, lower.back().t1, S_mid, U);
     else if (st == HARP_OK && !upper.empty()) st = build_pass(plan, sp, sp->pass[1], upper, false, S_mid, U, Lw);
     for (int s = 0; s < 2 && st == HARP_OK; ++s) {
-        if (!sp->pass[s].present) continue;
+        if (s == 1 && want_dense) upper = {GPhase{lower.back().t1, m, U <= 16 ? 16 : U <= 32 ? 32 : U <= 48 ? 48 : 64, (int)U, S_mid}};
+        if (s == 1 && upper.empty()) continue;
         st = harp_pipe_build(plan, s == 0 ? lower : upper, s == 0, S_mid, U, &sp->pipe[s]);
         if (st == HARP_ERR_UNSUPPORTED) st = HARP_OK;
     }
@@ -1116,6 +1117,11 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
         const int64_t r1 = std::min(n_rows, r0 + (two ? sp->chunk_rows : n_rows));
         for (int s = 0; s < (two ? 2 : 1); ++s) {
             const int pi = transpose ? (two ? 1 - s : 0) : s;
+            if (sp->pipe[pi] && r1 - r0 >= pipe_min_rows() && !(pi == 0 && r1 - r0 >= kTmSlabMinRows && harp_tm_slab_stages(plan) == sp->lower_stages)) {
+                const harp_status_t ps = harp_pipe_apply(sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
+                if (ps != HARP_OK) return ps;
+                continue;
+            }
             if (pi == 1 && sp->dense_upper) {
                 const UpperPass &P = transpose ? sp->up_bwd : sp->up_fwd;
                 const int64_t tile_rows = 16 * P.MT;
@@ -1148,11 +1154,6 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
                 const harp_status_t ts = harp_tm_slab_apply(plan, xb + r0 * plan->d, r1 - r0, dtype, transpose, stream);
                 if (ts == HARP_OK) continue;
                 if (ts != HARP_ERR_UNSUPPORTED) return ts;
-            }
-            if (sp->pipe[pi] && r1 - r0 >= pipe_min_rows()) {
-                const harp_status_t ps = harp_pipe_apply(sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
-                if (ps != HARP_OK) return ps;
-                continue;
             }
             const PassHost &ph = sp->pass[pi];
             SplitPass P = transpose ? ph.bwd : ph.fwd;
