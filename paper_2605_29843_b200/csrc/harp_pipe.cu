@@ -38,6 +38,7 @@ struct PipePhase {
     int32_t B, B_real;
     int32_t n_items, items_off;
     int32_t bfrag_off;         // word offset of the phase's fragments inside a column group's block
+    int32_t frag_lanes;        // lanes whose words of an 8-wide octet are kept: a block of seven needs no eighth column
     int32_t lm;                // local index of slot j of lane q: lm * q + jr[j]
     int32_t jr[4];
     int32_t step[2];           // byte offset of local index r: (r * unit >> shift) * step[1] + (r * unit & mask) * step[0]
@@ -54,6 +55,7 @@ struct PipePass {
     int32_t tables_len;
     const uint32_t *bfrag;                    // [column group][bfrag_words]
     int32_t bfrag_words;
+    const uint4 *frag64;                      // lower: [column group][block of 64][8 column tiles][2][lane], see dense_phase
     PipePhase ph[kMaxPipePhases];
 };
 
@@ -71,9 +73,6 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, int a, int 
                  ::"l"(map), "r"(a), "r"(b), "r"(c), "r"(d), "r"(src) : "memory");
 }
 
-template <bool LOWER> __device__ __forceinline__ uint32_t swz(uint32_t a) {
-    return LOWER ? a ^ (((a >> 7) & 7u) << 4) : a ^ (((a >> 7) & 1u) << 4);
-}
 __device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
     const int e = r * ph.unit;
     return (uint32_t)((e >> ph.shift) * ph.step[1] + (e & ((1 << ph.shift) - 1)) * ph.step[0]);
@@ -82,29 +81,33 @@ __device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
 // The kinds of pass.  A team is a few warps with n_buf tile buffers of their own; tiles of the CTA's column group go to its
 // teams in turn and a team's thread 0 issues its bulk copies.
 //   lower8, upper8   three teams of eight warps, at most 85 registers; the teams share the fragments
-//   upper16          sixteen-wide blocks need 128 registers: one team, two CTAs per SM
+//   upper16          sixteen-wide blocks need 128 registers: two teams
 //   dense32, dense48 all upper stages as one block of up to 32 or 48: a warp holds sixteen rows of eight positions, the two octets of a
 //                    tile make a team of two warps
-enum Kind { kLower8, kUpper8, kUpper16, kDense32, kDense48 };
+enum Kind { kLower64, kUpper8, kUpper16, kUpper16Wide, kDense32, kDense48 };
+constexpr bool is_wide(int K) { return K == kUpper16Wide; }
+constexpr bool is_b16(int K) { return K == kUpper16 || K == kUpper16Wide; }
 template <int K> struct KindOf {
-    static constexpr bool lower = K == kLower8, b16 = K == kUpper16;
+    static constexpr bool lower = K == kLower64, b16 = is_b16(K), wide = is_wide(K);
     static constexpr int ks = K == kDense32 ? 2 : K == kDense48 ? 3 : 0;
-    static constexpr int team_warps = ks ? 2 : 8, team_threads = 32 * team_warps, teams = b16 ? 1 : 3, threads = teams * team_threads;
-    static constexpr int ctas = b16 ? 2 : 1;
+    static constexpr int team_warps = ks ? 2 : 8, team_threads = 32 * team_warps, teams = b16 || lower ? 2 : 3, threads = teams * team_threads;
+    static constexpr int swizzle_bits = lower ? 7 : wide ? 3 : 1;
 };
+template <int K> __device__ __forceinline__ uint32_t swz(uint32_t a) { return a ^ (((a >> 7) & (uint32_t)KindOf<K>::swizzle_bits) << 4); }
 
 // Eight positions of sixteen rows through one dense block each (U <= 16 KS).  raw: slot s of this lane is coordinate
 // 16 (s / 4) + q + 4 (s % 4); results replace the operands word by word.
 // Fragments: [pair of positions][pair of column tiles][position of the pair][KS][lane][4 words].
-template <int KS, typename Mid>
+template <int K, typename Mid>
 __device__ __forceinline__ void dense_octet(uint32_t a0, uint32_t row8_off, int q, int U, uint32_t bfa, const Mid &mid) {
+    constexpr int KS = KindOf<K>::ks;
     uint4 raw[4 * KS][2];
 #pragma unroll
     for (int s = 0; s < 4 * KS; ++s) {
         const int u = 16 * (s / 4) + q + 4 * (s % 4);
         const uint32_t o = a0 + 32u * (uint32_t)u;
-        raw[s][0] = u < U ? lds128(swz<false>(o)) : make_uint4(0u, 0u, 0u, 0u);
-        raw[s][1] = u < U ? lds128(swz<false>(o + row8_off)) : make_uint4(0u, 0u, 0u, 0u);
+        raw[s][0] = u < U ? lds128(swz<K>(o)) : make_uint4(0u, 0u, 0u, 0u);
+        raw[s][1] = u < U ? lds128(swz<K>(o + row8_off)) : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
@@ -149,16 +152,44 @@ __device__ __forceinline__ void dense_octet(uint32_t a0, uint32_t row8_off, int 
         const int u = 16 * (s / 4) + q + 4 * (s % 4);
         const uint32_t o = a0 + 32u * (uint32_t)u;
         if (u < U) {
-            sts128(swz<false>(o), raw[s][0]);
-            sts128(swz<false>(o + row8_off), raw[s][1]);
+            sts128(swz<K>(o), raw[s][0]);
+            sts128(swz<K>(o + row8_off), raw[s][1]);
+        }
+    }
+}
+
+// Blocks of 64 contiguous coordinates, fragments in registers: f[2 n + s] holds, for column tile n, the words of k-steps 2 s and
+// 2 s + 1.  box: sixteen-row groups of 128-byte rows, 128-byte swizzle; the rows of a group are rewritten by the warp that read them.
+__device__ __forceinline__ void dense_phase(const uint4 (&f)[16], uint32_t box, int lane, int MT) {
+    uint32_t row = box + 128u * (uint32_t)((lane & 7) + ((lane >> 3) & 1) * 8);
+    const uint32_t hi = (uint32_t)lane >> 4, x = (row >> 7) & 7u;             // sixteen rows further is the same swizzle
+    for (int mt = 0; mt < MT; ++mt, row += 2048u) {
+        uint32_t a[4][4];
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) ldmatrix_x4(a[ks], row + (((2u * ks + hi) ^ x) << 4));
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float acc[2][4];
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    const uint4 &w = f[2 * (2 * c + k) + ks / 2];
+                    const uint32_t b0 = ks % 2 ? w.z : w.x, b1 = ks % 2 ? w.w : w.y;
+                    if (ks == 0) mma_k16(acc[k], a[ks], b0, b1);
+                    else mma_k16_acc(acc[k], a[ks], b0, b1);
+                }
+            stmatrix_x4(row + (((2u * c + hi) ^ x) << 4), pack_bf16(acc[0][0], acc[0][1]), pack_bf16(acc[0][2], acc[0][3]),
+                        pack_bf16(acc[1][0], acc[1][1]), pack_bf16(acc[1][2], acc[1][3]));
         }
     }
 }
 
 template <int K>
-__global__ void __launch_bounds__(KindOf<K>::threads, KindOf<K>::ctas)
+__global__ void __launch_bounds__(KindOf<K>::threads, 1)
 harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const PipePass P) {
     constexpr bool LOWER = KindOf<K>::lower, B16 = KindOf<K>::b16;
+    constexpr int LW = KindOf<K>::wide ? 32 : 16;          // upper: positions of a column group
     constexpr int KS = KindOf<K>::ks, TEAMS = KindOf<K>::teams, kTeamWarps = KindOf<K>::team_warps, kTeamThreads = KindOf<K>::team_threads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[TEAMS * kMaxPipeBufs];
@@ -190,14 +221,14 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
         mbar_expect_tx(bar, (uint32_t)(P.n_box * P.box_bytes));
         for (int k = 0; k < P.n_box; ++k) {
             if constexpr (LOWER) harp_tm::tma_load_2d(dst + (uint32_t)(k * P.box_pitch), &tmap, 64 * (cg * P.n_box + k), tile * 16 * P.MT, bar);
-            else tma_load_4d(dst + (uint32_t)(k * P.box_pitch), &tmap, 16 * cg, 0, 0, tile * 16 * P.MT + 8 * P.MT * k, bar);
+            else tma_load_4d(dst + (uint32_t)(k * P.box_pitch), &tmap, LW * cg, 0, 0, tile * 16 * P.MT + 8 * P.MT * k, bar);
         }
     };
     auto store = [&](int cg, int tile, int b) {
         const uint32_t src = bufs + (uint32_t)(b * P.tile_bytes);
         for (int k = 0; k < P.n_box; ++k) {
             if constexpr (LOWER) harp_tm::tma_store_2d(&tmap, 64 * (cg * P.n_box + k), tile * 16 * P.MT, src + (uint32_t)(k * P.box_pitch));
-            else tma_store_4d(&tmap, 16 * cg, 0, 0, tile * 16 * P.MT + 8 * P.MT * k, src + (uint32_t)(k * P.box_pitch));
+            else tma_store_4d(&tmap, LW * cg, 0, 0, tile * 16 * P.MT + 8 * P.MT * k, src + (uint32_t)(k * P.box_pitch));
         }
         harp_tm::bulk_commit();
     };
@@ -236,6 +267,12 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             waited = true;
         }
+        [[maybe_unused]] uint4 f64[LOWER ? 16 : 1];
+        if constexpr (LOWER) {
+            const uint4 *f = P.frag64 + ((size_t)cg * P.n_box + min(warp, P.n_box - 1)) * 512 + lane;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) f64[i] = __ldg(f + 32 * i);
+        }
         if (tid == 0 && !*(volatile int *)&dead)
             for (int k = 0; k < NB; ++k)
                 if (team + k * TEAMS < count) load(cg, first + (team + k * TEAMS) * step, k);
@@ -261,30 +298,14 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
                 }
             };
             if constexpr (KS > 0) {
-                dense_octet<KS>(sbase + 16u * (uint32_t)warp + row0_off, row8_off, q, P.ph[0].B_real,
+                dense_octet<K>(sbase + 16u * (uint32_t)warp + row0_off, row8_off, q, P.ph[0].B_real,
                                 bf_s + 16u * (uint32_t)(warp * 8 * KS * KS * 32 + lane), refill);
             } else
             for (int p = 0; p < P.n_phases; ++p) {
                 const PipePhase &ph = P.ph[p];
                 if (p > 0) team_sync();
                 if (LOWER && ph.mode == 0) {
-                    // two neighbouring 8-wide blocks per ldmatrix.x4 / stmatrix.x4
-                    const uint32_t lrow = 128u * (uint32_t)((lane & 7) + ((lane >> 3) & 1) * 8), lcol = 16u * (uint32_t)(lane >> 4);
-                    for (int i2 = 2 * warp; i2 < ph.n_items; i2 += 2 * kTeamWarps) {
-                        const uint32_t bfa = bf_s + 4u * (uint32_t)(ph.bfrag_off + i2 * 32 + lane);
-                        const uint32_t bf0 = lds32p(bfa), bf1 = lds32p(bfa + 128);
-                        uint32_t addr = sbase + lds32p(tab_s + 4u * (uint32_t)(ph.items_off + i2)) + lrow + lcol;
-                        addr = swz<LOWER>(addr);             // 16 rows further is the same swizzle
-                        for (int mt = 0; mt < P.MT; ++mt, addr += mt_step) {
-                            uint32_t a[4];
-                            ldmatrix_x4(a, addr);
-                            const uint32_t a_lo[2] = {a[0], a[1]}, a_hi[2] = {a[2], a[3]};
-                            float c0[4], c1[4];
-                            mma_k8(c0, a_lo, bf0);
-                            mma_k8(c1, a_hi, bf1);
-                            stmatrix_x4(addr, pack_bf16(c0[0], c0[1]), pack_bf16(c0[2], c0[3]), pack_bf16(c1[0], c1[1]), pack_bf16(c1[2], c1[3]));
-                        }
-                    }
+                    if constexpr (LOWER) if (warp < P.n_box) dense_phase(f64, sbase + (uint32_t)(warp * P.box_pitch), lane, P.MT);
                 } else if (B16 && ph.B == 16) {
                     uint32_t so[4];
                     bool ok[4];
@@ -304,15 +325,15 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
                         for (int e = 0; e < 8; ++e) bf[e] = lds128(bfa + e * 512);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            raw[j][0] = lds128(swz<LOWER>(a0 + so[j]));
-                            raw[j][1] = lds128(swz<LOWER>(a0 + so[j] + row8_off));
+                            raw[j][0] = lds128(swz<K>(a0 + so[j]));
+                            raw[j][1] = lds128(swz<K>(a0 + so[j] + row8_off));
                         }
                         octet_mma16<true>(raw, bf, unused);
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
                             if (ok[j]) {
-                                sts128(swz<LOWER>(a0 + so[j]), raw[j][0]);
-                                sts128(swz<LOWER>(a0 + so[j] + row8_off), raw[j][1]);
+                                sts128(swz<K>(a0 + so[j]), raw[j][0]);
+                                sts128(swz<K>(a0 + so[j] + row8_off), raw[j][1]);
                             }
                     }
                 } else {
@@ -327,18 +348,18 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
                     for (int w = warp; w < n_work; w += kTeamWarps) {
                         const int i1 = w >> P.mt_shift, mt = w & (P.MT - 1);
                         const uint32_t a0 = sbase + lds32p(tab_s + 4u * (uint32_t)(ph.items_off + i1)) + row0_off + (uint32_t)mt * mt_step;
-                        const uint32_t bfa = bf_s + 4u * (uint32_t)(ph.bfrag_off + i1 * 256 + lane * 4);
+                        const uint32_t bfa = bf_s + 4u * (uint32_t)(ph.bfrag_off + (i1 * 2 * ph.frag_lanes + min(lane, ph.frag_lanes - 1)) * 4);
                         uint4 raw[2][2];
                         uint32_t bf[8], ad[2][2];
 #pragma unroll
                         for (int j = 0; j < 2; ++j) {
-                            ad[j][0] = swz<LOWER>(a0 + so[j]);
-                            ad[j][1] = swz<LOWER>(a0 + so[j] + row8_off);
+                            ad[j][0] = swz<K>(a0 + so[j]);
+                            ad[j][1] = swz<K>(a0 + so[j] + row8_off);
                             raw[j][0] = lds128(ad[j][0]);
                             raw[j][1] = lds128(ad[j][1]);
                         }
                         {
-                            const uint4 f0 = lds128(bfa), f1 = lds128(bfa + 512);
+                            const uint4 f0 = lds128(bfa), f1 = lds128(bfa + 16u * (uint32_t)ph.frag_lanes);
                             bf[0] = f0.x; bf[1] = f0.y; bf[2] = f0.z; bf[3] = f0.w;
                             bf[4] = f1.x; bf[5] = f1.y; bf[6] = f1.z; bf[7] = f1.w;
                         }
@@ -355,7 +376,9 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
             }
             harp_tm::fence_async_smem();             // results before the copy engine reads them
             team_sync();
-            if (tid == 0 && !*(volatile int *)&dead) store(cg, first + t * step, b);
+            if (tid == 0 && !*(volatile int *)&dead) {
+                store(cg, first + t * step, b);
+            }
         }
         if (tid == 0) harp_tm::bulk_wait_read0();
     }
@@ -373,11 +396,11 @@ typedef CUresult (*EncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, 
                                 const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-constexpr int smem_most(int kind) { return kind == kUpper16 ? 112 * 1024 : 226 * 1024; }
+constexpr int kPipeSmem = 226 * 1024;
 
 template <int K>
 cudaError_t launch_pipe(const CUtensorMap &tmap, int32_t *err, const PipePass &P, unsigned grid, size_t smem, bool overlap, cudaStream_t stream) {
-    const cudaError_t ae = cudaFuncSetAttribute(harp_pipe_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_most(K));
+    const cudaError_t ae = cudaFuncSetAttribute(harp_pipe_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPipeSmem);
     if (ae != cudaSuccess) return ae;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -418,11 +441,37 @@ void dense_fragments(const harp_plan *plan, const GPhase &gp, int n_cg, int ks, 
     }
 }
 
+// Fragments of the contiguous blocks of 64 (see dense_phase).
+std::vector<uint32_t> block64_fragments(const harp_plan *plan, const GPhase &gp, int dir) {
+    std::vector<uint32_t> frag((size_t)plan->d / 64 * 2048);
+    std::vector<double> F;
+    for (int64_t base = 0; base < plan->d; base += 64) {
+        fused_block(plan, HostPhase{gp.t0, gp.t1, 64, 1, 0, 1}, base, F);
+        auto G = [&](int i, int o) -> double {
+            double v = dir == 0 ? F[(size_t)i * 64 + o] : F[(size_t)o * 64 + i];
+            if (!plan->h_signs.empty()) {
+                const int64_t pos = base + (dir == 0 ? i : o);
+                v *= (double)plan->h_signs[(size_t)(plan->h_perm.empty() ? pos : plan->h_perm[(size_t)pos])];
+            }
+            return v;
+        };
+        for (int nt = 0; nt < 8; ++nt)
+            for (int ks = 0; ks < 4; ++ks)
+                for (int h = 0; h < 2; ++h)
+                    for (int lane = 0; lane < 32; ++lane) {
+                        const int n = 8 * nt + (lane >> 2), k = 16 * ks + 8 * h + 2 * (lane & 3);
+                        frag[(size_t)base / 64 * 2048 + (2 * nt + ks / 2) * 128 + lane * 4 + 2 * (ks % 2) + h] =
+                            f2bf(G(k, n)) | ((uint32_t)f2bf(G(k + 1, n)) << 16);
+                    }
+    }
+    return frag;
+}
+
 }  // namespace
 
 struct PipePlan {
     PipePass dir[2];           // forward, transpose
-    int kind = kLower8;
+    int kind = kLower64;
     int64_t d = 0, S_mid = 1;
     int r_in = 1, r_out = 1;   // upper: radices of the inner and the outer digit of a tile
     int64_t s_in = 0, s_out = 0;   // ... and their strides in coordinates
@@ -446,57 +495,61 @@ int32_t harp_pipe_error_word(const PipePlan *pp) {
 
 // The pass over `phs` (lower: slabs of S_mid coordinates; upper: sixteen neighbouring positions of all U slabs).
 // HARP_ERR_UNSUPPORTED: a shape for which the layouts above are not free of conflicts, or whose tiles do not fit.
-harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &phs, bool lower, int64_t S_mid, int64_t U, PipePlan **out) {
+harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bool lower, int64_t S_mid, int64_t U, bool wide, PipePlan **out) {
     *out = nullptr;
+    if (lower) {                                         // the first two phases as blocks of 64
+        if (phs.size() < 2 || phs[0].B_real * phs[1].B_real != 64) return HARP_ERR_UNSUPPORTED;
+        phs[1] = GPhase{phs[0].t0, phs[1].t1, 64, 64, phs[0].S};
+        phs.erase(phs.begin());
+    }
     const int np = (int)phs.size();
     if (np < 1 || np > kMaxPipePhases || !harp_tensor_map_encoder()) return HARP_ERR_UNSUPPORTED;
     int widest = 8;
     for (const GPhase &gp : phs) widest = std::max(widest, gp.B);
     PipePass P{};
     PipePlan pl;
-    pl.kind = lower ? kLower8 : widest == 8 ? kUpper8 : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
-    const int ks = pl.kind >= kDense32 ? widest / 16 : 0;
+    pl.kind = lower ? kLower64 : widest == 8 ? kUpper8 : widest == 16 ? (wide ? kUpper16Wide : kUpper16) : widest == 32 ? kDense32 : kDense48;
+    const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = wide ? 32 : 16;
+    if (wide && !is_wide(pl.kind)) return HARP_ERR_UNSUPPORTED;
     P.n_phases = np;
     if (lower) {
-        // boxes of 64 coordinates; the first phase in pairs of neighbouring blocks, the others by octets
-        if (widest > 8 || S_mid % 64 != 0 || S_mid > 512 || phs[0].S != 1 || phs[0].B_real != 8) return HARP_ERR_UNSUPPORTED;
+        if (S_mid > 512) return HARP_ERR_UNSUPPORTED;
         for (int p = 1; p < np; ++p)
-            if (phs[(size_t)p].S % 8 != 0) return HARP_ERR_UNSUPPORTED;
+            if (phs[(size_t)p].B != 8) return HARP_ERR_UNSUPPORTED;
         P.n_cg = (int)U;
         P.n_box = (int)(S_mid / 64);
     } else {
         // the digit of odd radix inside, so that a step of either digit is an odd number of columns
-        if (np > (ks ? 1 : 2) || widest > 48 || S_mid % 16 != 0 || U > 64) return HARP_ERR_UNSUPPORTED;
+        if (np > (ks ? 1 : 2) || widest > 48 || S_mid % Lw != 0 || U > 64) return HARP_ERR_UNSUPPORTED;
         const int in = np == 2 && phs[1].B_real % 2 != 0 ? 1 : 0;
         if (np == 2 && phs[(size_t)in].B_real % 2 == 0) return HARP_ERR_UNSUPPORTED;
         pl.r_in = phs[(size_t)in].B_real;
         pl.s_in = phs[(size_t)in].S;
         if (np == 2) { pl.r_out = phs[(size_t)(1 - in)].B_real; pl.s_out = phs[(size_t)(1 - in)].S; }
-        P.n_cg = (int)(S_mid / 16);
+        P.n_cg = (int)(S_mid / Lw);
         P.n_box = 2;
-        P.row_bytes = (int32_t)(32 * U);
+        P.row_bytes = (int32_t)(2 * Lw * U);
     }
     auto place = [&](int64_t c) -> int64_t {             // byte offset of an octet; c: coordinate within the slab (lower) or natural coordinate
         if (lower) return (c / 64) * P.box_pitch + (c % 64) * 2;
         const int64_t i = (c / pl.s_in) % pl.r_in, o = np == 2 ? (c / pl.s_out) % pl.r_out : 0;
-        return (o * pl.r_in + i) * 32 + (c % 16) * 2;
+        return (o * pl.r_in + i) * 2 * Lw + (c % Lw) * 2;
     };
     int words = 0, items = 0;
     for (const GPhase &gp : phs) {
-        const int n_blk = (int)((lower ? S_mid : U * 16) / gp.B_real);
-        words += ks ? 16 * 4 * ks * ks * 32 : n_blk * 32 * (gp.B == 16 ? 4 : 1);
-        items += ks ? 0 : lower && gp.S == 1 ? n_blk : n_blk / 8;
+        const int n_blk = (int)((lower ? S_mid : U * Lw) / gp.B_real);
+        words += lower && gp.S == 1 ? 0 : ks ? 16 * 4 * ks * ks * 32 : n_blk * (gp.B == 16 ? 128 : !lower && gp.B_real == 7 ? 28 : 32);
+        items += ks || (lower && gp.S == 1) ? 0 : n_blk / 8;
     }
     // the largest tile that fits; a pass of one phase refills a buffer while two others are full
-    const int teams = pl.kind == kUpper16 ? 1 : 3;
-    const size_t most = (size_t)smem_most(pl.kind);
-    P.n_buf = np == 1 && !ks ? 3 : 2;
+    const int teams = is_b16(pl.kind) || lower ? 2 : 3;
+    P.n_buf = lower || (np == 1 && !ks) ? 3 : 2;
     for (P.MT = ks ? 1 : 4, P.mt_shift = ks ? 0 : 2;; P.MT /= 2, --P.mt_shift) {
         P.box_bytes = lower ? 128 * 16 * P.MT : 8 * P.MT * P.row_bytes;
-        P.box_pitch = P.box_bytes + 128;                 // an odd number of 128 bytes: P.box_bytes is a multiple of 256
+        P.box_pitch = P.box_bytes + (wide ? 256 : 128);  // (P.box_bytes is a multiple of twice that)
         P.tile_bytes = P.n_box * P.box_pitch;
         pl.smem = (size_t)teams * P.n_buf * P.tile_bytes + (size_t)words * 4 + (size_t)items * 4 + 128;
-        if (pl.smem <= most) break;
+        if (pl.smem <= kPipeSmem) break;
         if (P.MT == 1) return HARP_ERR_UNSUPPORTED;
     }
     pl.d = plan->d;
@@ -508,16 +561,16 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
 
     static const int jo16[4] = {0, 4, 8, 12}, jo8[2][2] = {{0, 4}, {0, 1}};
     harp_status_t st = HARP_OK;
-    auto upload = [&](const void *src, size_t bytes) -> void * {
+    auto upload = [&](const auto &v) -> void * {
+        const size_t bytes = v.size() * sizeof(v[0]);
         void *p = nullptr;
         if (st != HARP_OK) return nullptr;
         if (cudaMalloc(&p, std::max<size_t>(16, bytes)) != cudaSuccess) { st = HARP_ERR_ALLOC; return nullptr; }
         pl.dev_allocs.push_back(p);
-        if (cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) st = HARP_ERR_CUDA;
+        if (cudaMemcpy(p, v.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) st = HARP_ERR_CUDA;
         return p;
     };
-    const int32_t zero = 0;
-    pl.d_err = static_cast<int32_t *>(upload(&zero, sizeof(zero)));
+    pl.d_err = static_cast<int32_t *>(upload(std::vector<int32_t>(1, 0)));
     for (int dir = 0; dir < 2 && st == HARP_OK; ++dir) {
         std::vector<int32_t> tab;
         std::vector<uint32_t> frag((size_t)P.n_cg * words, 0u);
@@ -531,9 +584,14 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
             D.B = gp.B;
             D.B_real = gp.B_real;
             D.lm = lower && D.mode == 1 ? 2 : 1;
+            D.frag_lanes = !lower && gp.B_real == 7 ? 28 : 32;
             for (int j = 0; j < 4; ++j) D.jr[j] = gp.B == 16 ? jo16[j] : j < 2 ? jo8[D.lm - 1][j] : 0;
             D.items_off = (int32_t)tab.size();
             D.bfrag_off = at;
+            if (D.mode == 0) {
+                P.frag64 = static_cast<const uint4 *>(upload(block64_fragments(plan, gp, dir)));
+                continue;
+            }
             if (ks) {
                 dense_fragments(plan, gp, P.n_cg, ks, dir, frag);
                 at = words;
@@ -546,17 +604,15 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
                 D.step[1] = P.box_pitch;
             } else {
                 D.unit = 1;
-                D.step[1] = gp.S == pl.s_in ? 32 : 32 * pl.r_in;
+                D.step[1] = (gp.S == pl.s_in ? 2 : 2 * pl.r_in) * Lw;
             }
             // first coordinates of the blocks (lower: within the slab; upper: within position group 0)
             std::vector<int64_t> first;
-            if (D.mode == 0) {
-                for (int64_t c = 0; c < S_mid; c += 8) { first.push_back(c); tab.push_back((int32_t)place(c)); }
-            } else {
+            {
                 const int64_t span = gp.S * gp.B_real, all = lower ? S_mid : plan->d, lo_step = lower ? 8 : S_mid;
                 for (int64_t hi = 0; hi < all; hi += span)
                     for (int64_t lo = 0; lo < gp.S; lo += lo_step)
-                        for (int64_t l8 = 0; l8 < (lower ? 8 : 16); l8 += 8) {
+                        for (int64_t l8 = 0; l8 < (lower ? 8 : Lw); l8 += 8) {
                             const int64_t c = hi + lo + l8;
                             for (int r = 0; r < gp.B_real; ++r) {       // every octet that the kernel reaches
                                 const int e = r * D.unit;
@@ -568,22 +624,25 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
                         }
             }
             D.n_items = (int32_t)tab.size() - D.items_off;
-            auto slot = [&](int s) { return D.mode == 0 ? s : strided_slot(s, gp.B, D.lm); };
+            auto slot = [&](int s) { return strided_slot(s, gp.B, D.lm); };
             const int wpl = gp.B == 16 ? 4 : 1;
-            const bool grouped = D.mode == 1 && gp.B == 8;       // [item][blocks 0-3 | 4-7][lane][4 words]
+            const bool grouped = gp.B == 8;       // [item][blocks 0-3 | 4-7][lane][4 words]
+            uint32_t one[128];
             for (int cg = 0; cg < P.n_cg; ++cg)
                 for (size_t i = 0; i < first.size(); ++i) {
-                    const int64_t base = (lower ? cg * S_mid : cg * 16) + first[i];
-                    uint32_t *dst = frag.data() + (size_t)cg * words + at + (grouped ? (i / 8) * 256 + ((i % 8) / 4) * 128 + i % 4 : i * 32 * wpl);
-                    block_fragment(plan, gp, base, dir, slot, dst, grouped ? 4 : wpl, F);
+                    uint32_t *dst = frag.data() + (size_t)cg * words + at;
+                    if (grouped) dst += (i / 8 * 2 + i % 8 / 4) * D.frag_lanes * 4 + i % 4;
+                    else dst += i * 32 * wpl;
+                    block_fragment(plan, gp, (lower ? cg * S_mid : cg * Lw) + first[i], dir, slot, one, wpl, F);
+                    for (int w = 0; w < (grouped ? D.frag_lanes : 32 * wpl); ++w) dst[grouped ? 4 * w : w] = one[w];
                 }
-            at += (int)first.size() * 32 * wpl;
+            at += (int)first.size() * (grouped ? D.frag_lanes : 32 * wpl);
         }
         if (at != words || (int)tab.size() != items || words % 4 != 0) return HARP_ERR_UNSUPPORTED;
         P.tables_len = items;
         P.bfrag_words = words;
-        P.tables = static_cast<const int32_t *>(upload(tab.data(), tab.size() * 4));
-        P.bfrag = static_cast<const uint32_t *>(upload(frag.data(), frag.size() * 4));
+        P.tables = static_cast<const int32_t *>(upload(tab));
+        P.bfrag = static_cast<const uint32_t *>(upload(frag));
         pl.dir[dir] = P;
     }
     PipePlan *pp = st == HARP_OK ? new (std::nothrow) PipePlan(pl) : nullptr;
@@ -599,7 +658,7 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
 harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int transpose, bool overlap, cudaStream_t stream) {
     if (!pp || n_rows > ((int64_t)1 << 30)) return HARP_ERR_UNSUPPORTED;
     PipePass P = pp->dir[transpose ? 1 : 0];
-    const int64_t slots = (int64_t)pp->sms * (pp->kind == kUpper16 ? 2 : 1);
+    const int64_t slots = pp->sms;
     // a batch with less than half a tile per CTA is cut finer
     while (P.MT > 1 && (n_rows + 16 * P.MT - 1) / (16 * P.MT) * P.n_cg * 2 < slots) {
         P.MT /= 2;
@@ -610,14 +669,14 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
     // A column group per CTA keeps its fragments, and the CTAs at the same rows: neighbouring 32-byte runs meet in L2.  Where
     // the groups leave more than a tenth of the SMs without work, lower passes (whole lines) share the list out evenly.
     P.n_parts = (int32_t)std::min<int64_t>(P.n_tiles, std::max<int64_t>(1, slots / P.n_cg));
-    if (pp->kind == kLower8 && (P.n_cg > slots || slots % P.n_cg * 10 > slots)) P.n_parts = 0;
+    if (pp->kind == kLower64 && (P.n_cg > slots || slots % P.n_cg * 10 > slots)) P.n_parts = 0;
     const unsigned grid = (unsigned)(P.n_parts > 0 ? (int64_t)P.n_parts * P.n_cg : std::min<int64_t>((int64_t)P.n_tiles * P.n_cg, slots));
     const auto enc = reinterpret_cast<EncodeTiled>(harp_tensor_map_encoder());
     CUtensorMap tmap = {};
     const cuuint32_t ones[4] = {1, 1, 1, 1};
     const cuuint64_t n = (cuuint64_t)n_rows, pitch = (cuuint64_t)pp->d * 2;
     CUresult r;
-    if (pp->kind == kLower8) {
+    if (pp->kind == kLower64) {
         const cuuint64_t gdim[2] = {(cuuint64_t)pp->d, n}, gstr[1] = {pitch};
         const cuuint32_t box[2] = {64, (cuuint32_t)(16 * P.MT)};
         r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -626,15 +685,16 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
         // (position, inner digit, outer digit, row)
         const cuuint64_t gdim[4] = {(cuuint64_t)pp->S_mid, (cuuint64_t)pp->r_in, (cuuint64_t)pp->r_out, n};
         const cuuint64_t gstr[3] = {(cuuint64_t)pp->s_in * 2, (cuuint64_t)(pp->r_out > 1 ? pp->s_out : pp->s_in) * 2, pitch};
-        const cuuint32_t box[4] = {16, (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
+        const cuuint32_t box[4] = {(cuuint32_t)(is_wide(pp->kind) ? 32 : 16), (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
         r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                is_wide(pp->kind) ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
     if (r != CUDA_SUCCESS) return HARP_ERR_CUDA;
     cudaError_t err = cudaErrorInvalidValue;
     switch (pp->kind) {
-        case kLower8: err = launch_pipe<kLower8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kLower64: err = launch_pipe<kLower64>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper8: err = launch_pipe<kUpper8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kUpper16Wide: err = launch_pipe<kUpper16Wide>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper16: err = launch_pipe<kUpper16>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kDense32: err = launch_pipe<kDense32>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kDense48: err = launch_pipe<kDense48>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;

@@ -683,7 +683,7 @@ struct SplitPlan {
     const uint16_t *gather[2] = {nullptr, nullptr};
     int gather_rows = 1;       // rows per buffer of the gather kernel
     size_t gather_smem = 0;
-    PipePlan *pipe[2] = {nullptr, nullptr};   // the passes fed by the copy engine (harp_pipe.cu), where the shape allows them
+    PipePlan *pipe[3] = {nullptr, nullptr, nullptr};   // the passes fed by the copy engine (harp_pipe.cu), where the shape allows them
     // dense upper pass (replaces pass[1] when set)
     bool dense_upper = false;
     bool up_in_regs = false;   // fragments in registers (harp_upper_reg_kernel)
@@ -992,10 +992,9 @@ harp_status_t harp_split_build(harp_plan *plan) {
     harp_status_t st = build_pass(plan, sp, sp->pass[0], lower, true, S_mid, U, 1);
     if (st == HARP_OK && want_dense) st = build_dense_upper(plan, sp, lower.back().t1, S_mid, U);
     else if (st == HARP_OK && !upper.empty()) st = build_pass(plan, sp, sp->pass[1], upper, false, S_mid, U, Lw);
-    for (int s = 0; s < 2 && st == HARP_OK; ++s) {
-        if (s == 1 && want_dense) upper = {GPhase{lower.back().t1, m, U <= 16 ? 16 : U <= 32 ? 32 : U <= 48 ? 48 : 64, (int)U, S_mid}};
-        if (s == 1 && upper.empty()) continue;
-        st = harp_pipe_build(plan, s == 0 ? lower : upper, s == 0, S_mid, U, &sp->pipe[s]);
+    if (want_dense) upper = {GPhase{lower.back().t1, m, (int)(U + 15) / 16 * 16, (int)U, S_mid}};
+    for (int s = 0; s < (upper.empty() ? 1 : 3) && st == HARP_OK; ++s) {
+        st = harp_pipe_build(plan, s == 0 ? lower : upper, s == 0, S_mid, U, s == 2, &sp->pipe[s]);
         if (st == HARP_ERR_UNSUPPORTED) st = HARP_OK;
     }
     if (st == HARP_OK &&
@@ -1085,6 +1084,7 @@ constexpr int64_t kOverlapMaxElems = (int64_t)16 << 20;
 // leave a third of the SMs idle and it is the slower one)
 constexpr int64_t kTmSlabMinRows = 384;
 
+static int64_t pipe_wide_rows() { const char *e = getenv("HARP_WIDE_ROWS"); return e ? atoll(e) : 512; }
 static int64_t pipe_min_rows() { const char *e = getenv("HARP_PIPE_ROWS"); return e ? atoll(e) : 1024; }
 int32_t harp_split_error_word(const harp_plan *plan) {
     int32_t w = 0;
@@ -1118,7 +1118,7 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
         for (int s = 0; s < (two ? 2 : 1); ++s) {
             const int pi = transpose ? (two ? 1 - s : 0) : s;
             if (sp->pipe[pi] && r1 - r0 >= pipe_min_rows() && !(pi == 0 && r1 - r0 >= kTmSlabMinRows && harp_tm_slab_stages(plan) == sp->lower_stages)) {
-                const harp_status_t ps = harp_pipe_apply(sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
+                const harp_status_t ps = harp_pipe_apply(pi == 1 && sp->pipe[2] && r1 - r0 >= pipe_wide_rows() ? sp->pipe[2] : sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
                 if (ps != HARP_OK) return ps;
                 continue;
             }
