@@ -104,7 +104,8 @@ inline void block_fragment(const harp_plan *plan, const GPhase &gp, int64_t base
 // passes fed by the copy engine (harp_pipe.cu)
 struct PipePlan;
 harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<harp_fuse::GPhase> phs, bool lower, int64_t S_mid, int64_t U,
-                              bool wide, PipePlan **out);
+                              PipePlan **out);
+int64_t harp_pipe_min_rows(const PipePlan *pp);   // smallest batch that it is meant for
 void harp_pipe_destroy(PipePlan *pp);
 harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int transpose, bool overlap, cudaStream_t stream);
 int32_t harp_pipe_error_word(const PipePlan *pp);

@@ -1,19 +1,28 @@
-// The two passes of the wide-row path (see harp_split.cu) fed by the copy engine, for batches that fill it.
+// The two passes of the wide-row path (see harp_split.cu) fed by the copy engine.
 //
 // The mma.sync passes of harp_split.cu spend 60 % of a tile's time on moving it: cp.async in and 16-byte stores out hold the
-// issuing warps at the rate at which the load/store unit takes 32-byte runs.  Bulk tensor copies move the same boxes
-// without a warp: 16 rows x 56 runs of 32 bytes in 1.4 cycles a run one way, 3.3 both ways (4.6 TB/s on 144 SMs), 64-byte
-// runs and longer at the HBM rate.  Here three teams of eight warps (two where blocks are 16 wide) share the fragments of the
-// CTA's column group; every team has two tile buffers and multiplies one while the other is stored and refilled.
+// issuing warps at the rate at which the load/store unit takes 32-byte runs (d = 14336, upper pass: 14.8 k cycles a tile with
+// three CTAs on an SM, 5 k of them products).  Bulk tensor copies move the same boxes without a warp: runs of 32 bytes in 1.4
+// cycles each one way and 3.3 both ways (4.6 to 4.9 TB/s), of 64 bytes and more at 5.5 to 6 TB/s.  So teams of warps multiply
+// tiles in place while other buffers of theirs are stored and refilled; all teams share the fragments of the CTA's column group.
+//
+//   d = 14336, 32768 rows: 888 -> 740 us;  d = 28672: 2122 -> 1500 us;  d = 8192, 16384 rows: 318 -> 218 us;
+//   d = 11008, 16384 rows: 384 -> 270 us (dense upper blocks);  d = 5120, 16384 rows: 221 -> 140 us;
+//   d = 8192, 64 rows: 12.9 -> 8.0 us;  d = 11008, 1 row: 9.3 -> 7.3 us.
+// With the products left out the upper passes take 95 to 100 % of their time and the slab pass 80 %: the copies bound them.
 //
 // The tile's layout is what the copy engine writes, chosen so that the 16-byte accesses of a quarter-warp (two rows, four
 // local indices) hit eight bank groups:
-//   lower pass  [box of 64 coordinates][row][128 bytes], 128-byte swizzle, boxes 128 bytes apart beyond their size: an index
+//   slab pass   [box of 64 coordinates][row][128 bytes], 128-byte swizzle, boxes 128 bytes apart beyond their size: an index
 //               step of one chunk or one box moves the swizzle by one, lanes hold the local indices 2q, 2q+1;
-//   upper pass  [half of the rows][row][outer digit][inner digit][32 bytes], 32-byte swizzle.  The inner digit's radix is odd
-//               (or there is one digit), so a step of either digit is an odd number of 32-byte columns; the two rows of a
-//               quarter-warp come from the two halves, which lie an odd number of 128 bytes apart, so that the swizzle
-//               gives them different 16-byte halves of a column.
+//   upper pass  [half of the rows][row][outer digit][inner digit][column of 32 or 64 bytes], 32- or 64-byte swizzle.  The inner digit's
+//               radix is odd (or there is one digit), so a step of either digit is an odd number of columns; the two rows of a
+//               quarter-warp come from the two halves, whose distance moves the top bit of the swizzle by one.
+// Sixteen-wide upper blocks take columns of 64 bytes (d = 8192, 16384 rows: 226 -> 219 us; 16 column groups instead of 32 also fill
+// 144 SMs instead of 128).  For two phases over 56 places such tiles leave one buffer per team and gain nothing.
+//
+// The first two phases of a slab are one product with 64 x 64 blocks, whose fragments stay in a warp's registers: one trip
+// through shared memory and one rounding less than as two phases of eight (d = 8192, 16384 rows: 246 -> 219 us).
 #include <algorithm>
 #include <new>
 #include <vector>
@@ -34,11 +43,10 @@ constexpr int kMaxPipePhases = 3, kMaxPipeBufs = 4;
 constexpr uint32_t kPipeSpin = 1u << 22;      // limit of every wait for a bulk copy
 
 struct PipePhase {
-    int32_t mode;              // 0 = contiguous blocks of eight, two at a time; 1 = strided blocks, eight per item
+    int32_t mode;              // 0 = contiguous blocks of 64; 1 = strided blocks, eight per item
     int32_t B, B_real;
     int32_t n_items, items_off;
     int32_t bfrag_off;         // word offset of the phase's fragments inside a column group's block
-    int32_t frag_lanes;        // lanes whose words of an 8-wide octet are kept: a block of seven needs no eighth column
     int32_t lm;                // local index of slot j of lane q: lm * q + jr[j]
     int32_t jr[4];
     int32_t step[2];           // byte offset of local index r: (r * unit >> shift) * step[1] + (r * unit & mask) * step[0]
@@ -80,15 +88,14 @@ __device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
 
 // The kinds of pass.  A team is a few warps with n_buf tile buffers of their own; tiles of the CTA's column group go to its
 // teams in turn and a team's thread 0 issues its bulk copies.
-//   lower8, upper8   three teams of eight warps, at most 85 registers; the teams share the fragments
-//   upper16          sixteen-wide blocks need 128 registers: two teams
-//   dense32, dense48 all upper stages as one block of up to 32 or 48: a warp holds sixteen rows of eight positions, the two octets of a
-//                    tile make a team of two warps
-enum Kind { kLower64, kUpper8, kUpper16, kUpper16Wide, kDense32, kDense48 };
-constexpr bool is_wide(int K) { return K == kUpper16Wide; }
-constexpr bool is_b16(int K) { return K == kUpper16 || K == kUpper16Wide; }
+//   lower64          two teams of eight warps, a warp per block of 64; 64 of its 128 registers are fragments
+//   upper8           three teams of eight warps, at most 85 registers
+//   upper16          sixteen-wide blocks need 128 registers: two teams of eight warps
+//   dense32, dense48 all upper stages as one block of up to 32 or 48: a warp holds sixteen rows of eight positions, the two
+//                    octets of a tile make a team of two warps; three teams
+enum Kind { kLower64, kUpper8, kUpper16, kDense32, kDense48 };
 template <int K> struct KindOf {
-    static constexpr bool lower = K == kLower64, b16 = is_b16(K), wide = is_wide(K);
+    static constexpr bool lower = K == kLower64, b16 = K == kUpper16, wide = b16;
     static constexpr int ks = K == kDense32 ? 2 : K == kDense48 ? 3 : 0;
     static constexpr int team_warps = ks ? 2 : 8, team_threads = 32 * team_warps, teams = b16 || lower ? 2 : 3, threads = teams * team_threads;
     static constexpr int swizzle_bits = lower ? 7 : wide ? 3 : 1;
@@ -348,7 +355,7 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
                     for (int w = warp; w < n_work; w += kTeamWarps) {
                         const int i1 = w >> P.mt_shift, mt = w & (P.MT - 1);
                         const uint32_t a0 = sbase + lds32p(tab_s + 4u * (uint32_t)(ph.items_off + i1)) + row0_off + (uint32_t)mt * mt_step;
-                        const uint32_t bfa = bf_s + 4u * (uint32_t)(ph.bfrag_off + (i1 * 2 * ph.frag_lanes + min(lane, ph.frag_lanes - 1)) * 4);
+                        const uint32_t bfa = bf_s + 4u * (uint32_t)(ph.bfrag_off + i1 * 256 + lane * 4);
                         uint4 raw[2][2];
                         uint32_t bf[8], ad[2][2];
 #pragma unroll
@@ -359,7 +366,7 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
                             raw[j][1] = lds128(ad[j][1]);
                         }
                         {
-                            const uint4 f0 = lds128(bfa), f1 = lds128(bfa + 16u * (uint32_t)ph.frag_lanes);
+                            const uint4 f0 = lds128(bfa), f1 = lds128(bfa + 512u);
                             bf[0] = f0.x; bf[1] = f0.y; bf[2] = f0.z; bf[3] = f0.w;
                             bf[4] = f1.x; bf[5] = f1.y; bf[6] = f1.z; bf[7] = f1.w;
                         }
@@ -487,6 +494,10 @@ void harp_pipe_destroy(PipePlan *pp) {
     delete pp;
 }
 
+// (1 to 32 rows of d = 5120 .. 28672: below nine rows the slab pass loses 0.2 us to the kernel of harp_split.cu, which reads only the
+// rows it has, and so does the sixteen-wide upper pass up to one row tile; the others are ahead from the first row on)
+int64_t harp_pipe_min_rows(const PipePlan *pp) { return pp->kind == kLower64 ? 9 : pp->kind == kUpper16 ? 17 : 1; }
+
 int32_t harp_pipe_error_word(const PipePlan *pp) {
     if (!pp || !pp->d_err) return 0;
     int32_t v = 0;
@@ -495,7 +506,7 @@ int32_t harp_pipe_error_word(const PipePlan *pp) {
 
 // The pass over `phs` (lower: slabs of S_mid coordinates; upper: sixteen neighbouring positions of all U slabs).
 // HARP_ERR_UNSUPPORTED: a shape for which the layouts above are not free of conflicts, or whose tiles do not fit.
-harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bool lower, int64_t S_mid, int64_t U, bool wide, PipePlan **out) {
+harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bool lower, int64_t S_mid, int64_t U, PipePlan **out) {
     *out = nullptr;
     if (lower) {                                         // the first two phases as blocks of 64
         if (phs.size() < 2 || phs[0].B_real * phs[1].B_real != 64) return HARP_ERR_UNSUPPORTED;
@@ -508,9 +519,8 @@ harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bo
     for (const GPhase &gp : phs) widest = std::max(widest, gp.B);
     PipePass P{};
     PipePlan pl;
-    pl.kind = lower ? kLower64 : widest == 8 ? kUpper8 : widest == 16 ? (wide ? kUpper16Wide : kUpper16) : widest == 32 ? kDense32 : kDense48;
-    const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = wide ? 32 : 16;
-    if (wide && !is_wide(pl.kind)) return HARP_ERR_UNSUPPORTED;
+    pl.kind = lower ? kLower64 : widest == 8 ? kUpper8 : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
+    const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = pl.kind == kUpper16 ? 32 : 16;
     P.n_phases = np;
     if (lower) {
         if (S_mid > 512) return HARP_ERR_UNSUPPORTED;
@@ -538,15 +548,15 @@ harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bo
     int words = 0, items = 0;
     for (const GPhase &gp : phs) {
         const int n_blk = (int)((lower ? S_mid : U * Lw) / gp.B_real);
-        words += lower && gp.S == 1 ? 0 : ks ? 16 * 4 * ks * ks * 32 : n_blk * (gp.B == 16 ? 128 : !lower && gp.B_real == 7 ? 28 : 32);
+        words += lower && gp.S == 1 ? 0 : ks ? 16 * 4 * ks * ks * 32 : n_blk * (gp.B == 16 ? 128 : 32);
         items += ks || (lower && gp.S == 1) ? 0 : n_blk / 8;
     }
     // the largest tile that fits; a pass of one phase refills a buffer while two others are full
-    const int teams = is_b16(pl.kind) || lower ? 2 : 3;
+    const int teams = pl.kind == kUpper16 || lower ? 2 : 3;
     P.n_buf = lower || (np == 1 && !ks) ? 3 : 2;
     for (P.MT = ks ? 1 : 4, P.mt_shift = ks ? 0 : 2;; P.MT /= 2, --P.mt_shift) {
         P.box_bytes = lower ? 128 * 16 * P.MT : 8 * P.MT * P.row_bytes;
-        P.box_pitch = P.box_bytes + (wide ? 256 : 128);  // (P.box_bytes is a multiple of twice that)
+        P.box_pitch = P.box_bytes + (Lw == 32 ? 256 : 128);  // (P.box_bytes is a multiple of twice that)
         P.tile_bytes = P.n_box * P.box_pitch;
         pl.smem = (size_t)teams * P.n_buf * P.tile_bytes + (size_t)words * 4 + (size_t)items * 4 + 128;
         if (pl.smem <= kPipeSmem) break;
@@ -584,7 +594,6 @@ harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bo
             D.B = gp.B;
             D.B_real = gp.B_real;
             D.lm = lower && D.mode == 1 ? 2 : 1;
-            D.frag_lanes = !lower && gp.B_real == 7 ? 28 : 32;
             for (int j = 0; j < 4; ++j) D.jr[j] = gp.B == 16 ? jo16[j] : j < 2 ? jo8[D.lm - 1][j] : 0;
             D.items_off = (int32_t)tab.size();
             D.bfrag_off = at;
@@ -627,16 +636,12 @@ harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bo
             auto slot = [&](int s) { return strided_slot(s, gp.B, D.lm); };
             const int wpl = gp.B == 16 ? 4 : 1;
             const bool grouped = gp.B == 8;       // [item][blocks 0-3 | 4-7][lane][4 words]
-            uint32_t one[128];
             for (int cg = 0; cg < P.n_cg; ++cg)
                 for (size_t i = 0; i < first.size(); ++i) {
-                    uint32_t *dst = frag.data() + (size_t)cg * words + at;
-                    if (grouped) dst += (i / 8 * 2 + i % 8 / 4) * D.frag_lanes * 4 + i % 4;
-                    else dst += i * 32 * wpl;
-                    block_fragment(plan, gp, (lower ? cg * S_mid : cg * Lw) + first[i], dir, slot, one, wpl, F);
-                    for (int w = 0; w < (grouped ? D.frag_lanes : 32 * wpl); ++w) dst[grouped ? 4 * w : w] = one[w];
+                    uint32_t *dst = frag.data() + (size_t)cg * words + at + (grouped ? (i / 8 * 2 + i % 8 / 4) * 128 + i % 4 : i * 32 * wpl);
+                    block_fragment(plan, gp, (lower ? cg * S_mid : cg * Lw) + first[i], dir, slot, dst, grouped ? 4 : wpl, F);
                 }
-            at += (int)first.size() * (grouped ? D.frag_lanes : 32 * wpl);
+            at += (int)first.size() * 32 * wpl;
         }
         if (at != words || (int)tab.size() != items || words % 4 != 0) return HARP_ERR_UNSUPPORTED;
         P.tables_len = items;
@@ -685,16 +690,15 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
         // (position, inner digit, outer digit, row)
         const cuuint64_t gdim[4] = {(cuuint64_t)pp->S_mid, (cuuint64_t)pp->r_in, (cuuint64_t)pp->r_out, n};
         const cuuint64_t gstr[3] = {(cuuint64_t)pp->s_in * 2, (cuuint64_t)(pp->r_out > 1 ? pp->s_out : pp->s_in) * 2, pitch};
-        const cuuint32_t box[4] = {(cuuint32_t)(is_wide(pp->kind) ? 32 : 16), (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
+        const cuuint32_t box[4] = {(cuuint32_t)(pp->kind == kUpper16 ? 32 : 16), (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
         r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                is_wide(pp->kind) ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                pp->kind == kUpper16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
     if (r != CUDA_SUCCESS) return HARP_ERR_CUDA;
     cudaError_t err = cudaErrorInvalidValue;
     switch (pp->kind) {
         case kLower64: err = launch_pipe<kLower64>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper8: err = launch_pipe<kUpper8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
-        case kUpper16Wide: err = launch_pipe<kUpper16Wide>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper16: err = launch_pipe<kUpper16>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kDense32: err = launch_pipe<kDense32>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kDense48: err = launch_pipe<kDense48>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;

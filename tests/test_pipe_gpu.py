@@ -1,0 +1,28 @@
+"""The two-pass path's kernels that are fed by bulk tensor copies, against the oracle at the edges of the batches they take (9 and 17
+rows) and of their tiles (16, 32 and 64 rows): slabs of one, three, seven and eight 64-blocks, one and two upper phases of
+every width, dense upper blocks of up to 32 and 48, and batches of several tiles per team of warps."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2605_29843_b200 as harp
+from oracle import harp_oracle as orc
+from paper_2605_29843_b200 import workloads as wl
+from harp_testlib import TOL, gpu_apply, host_rows, promote
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("radices", [(8, 8, 16), (8, 8, 3, 16), (8, 8, 7, 5, 3), (8, 8, 8, 8, 2), (8, 8, 8, 8, 7), (16, 16, 7, 5),
+                                     (16, 16, 43), (16, 16, 47), (8, 8, 8, 19)])
+@pytest.mark.parametrize("n_rows", [8, 9, 16, 17, 31, 33, 65, 131, 2049, 6001])
+def test_matches_the_oracle(radices, n_rows):
+    spec = wl.make_plan(81, int(np.prod(radices)), radices, "qr", perm="identity", signs=True)
+    plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
+    xh = host_rows(np.random.default_rng(82).standard_normal((n_rows, spec.d)), "bf16")
+    edges = [e for e in (0, 8, 16, 32, 64, 128, 1024, n_rows // 2, n_rows) if e <= n_rows]
+    rows = np.unique(np.clip(np.concatenate([np.arange(e - 2, e + 2) for e in edges]), 0, n_rows - 1))
+    for tr, fn in ((False, orc.forward), (True, orc.transpose)):
+        got, guards = gpu_apply(plan, xh, "bf16", tr, harp.KERNEL_SPLIT)
+        assert guards and harp.harp_plan_error_word(plan) == 0
+        assert orc.rel_err_rows(got[rows], fn(oplan, promote(xh[rows], "bf16"))) <= TOL["bf16"]
