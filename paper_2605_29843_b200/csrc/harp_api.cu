@@ -48,8 +48,8 @@ extern "C" int32_t harp_plan_error_word(const harp_plan_t *plan) {
     if (!plan) return -1;
     const int32_t w = harp_tm_error_word(plan);
     if (w != 0) return w;
-    const int32_t s = harp_split_error_word(plan);
-    return s != 0 ? s : harp_f32_error_word(plan);
+    const int32_t s = harp_split_error_word(plan), c = harp_col_error_word(plan);
+    return s != 0 ? s : c != 0 ? c : harp_f32_error_word(plan);
 }
 
 extern "C" int64_t harp_launch_count(void) { return g_harp_launches.load(std::memory_order_relaxed); }

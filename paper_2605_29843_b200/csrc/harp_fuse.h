@@ -30,14 +30,16 @@ inline uint16_t f2bf(double v) {
 inline void fused_block(const harp_plan *plan, const HostPhase &hp, int64_t base, std::vector<double> &F) {
     const int B = hp.B;
     F.assign((size_t)B * B, 0.0);
-    for (int r = 0; r < B; ++r) F[(size_t)r * B + r] = 1.0;
-    std::vector<double> tmp((size_t)B * B);
+    std::vector<double> before;
     for (int t = hp.t0; t < hp.t1; ++t) {
         const int b = plan->st.b[t];
         const int64_t s = plan->st.s[t];
         const int64_t ls = s / hp.S;                     // local stride of this stage's digit
         const float *Kt = plan->h_blocks.data() + plan->st.off[t];
-        std::fill(tmp.begin(), tmp.end(), 0.0);
+        if (t > hp.t0) {
+            before = F;
+            std::fill(F.begin(), F.end(), 0.0);
+        }
         for (int r = 0; r < B; ++r) {                    // r = output local index
             const int digit = (int)((r / ls) % b);
             const int r_base = r - digit * (int)ls;
@@ -47,10 +49,11 @@ inline void fused_block(const harp_plan *plan, const HostPhase &hp, int64_t base
             for (int i = 0; i < b; ++i) {                // input digit
                 const int r_in = r_base + i * (int)ls;
                 const double k = (double)Kc[i * b + digit];
-                for (int row = 0; row < B; ++row) tmp[(size_t)row * B + r] += F[(size_t)row * B + r_in] * k;
+                if (t == hp.t0) F[(size_t)r_in * B + r] = k;        // times the identity
+                else
+                    for (int row = 0; row < B; ++row) F[(size_t)row * B + r] += before[(size_t)row * B + r_in] * k;
             }
         }
-        F.swap(tmp);
     }
 }
 
@@ -103,8 +106,13 @@ inline void block_fragment(const harp_plan *plan, const GPhase &gp, int64_t base
 
 // passes fed by the copy engine (harp_pipe.cu)
 struct PipePlan;
-harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<harp_fuse::GPhase> phs, bool lower, int64_t S_mid, int64_t U,
-                              PipePlan **out);
+// fragments of a pass that the plan already holds: [direction][column group][words], first words of the phases, slot maps
+struct PassFrags {
+    const uint32_t *bfrag[2];
+    int32_t words, off[2][6], lm[6];
+};
+harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<harp_fuse::GPhase> &phs, bool lower, int64_t S_mid, int64_t U,
+                              const PassFrags &fr, PipePlan **out);
 int64_t harp_pipe_min_rows(const PipePlan *pp);   // smallest batch that it is meant for
 void harp_pipe_destroy(PipePlan *pp);
 harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int transpose, bool overlap, cudaStream_t stream);

@@ -101,6 +101,7 @@ harp_status_t harp_tm_slab_apply(const harp_plan *plan, void *x, int64_t n_rows,
 // dim(plan) x n_cols row-major matrix with leading dimension ld
 harp_status_t harp_col_build(harp_plan *plan);
 void harp_col_destroy(harp_plan *plan);
+int32_t harp_col_error_word(const harp_plan *plan);
 harp_status_t harp_col_apply(const harp_plan *plan, void *W, int64_t n_cols, int64_t ld, harp_dtype_t dtype,
                              cudaStream_t stream);
 

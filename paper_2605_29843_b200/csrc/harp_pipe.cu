@@ -6,10 +6,12 @@
 // cycles each one way and 3.3 both ways (4.6 to 4.9 TB/s), of 64 bytes and more at 5.5 to 6 TB/s.  So teams of warps multiply
 // tiles in place while other buffers of theirs are stored and refilled; all teams share the fragments of the CTA's column group.
 //
-//   d = 14336, 32768 rows: 888 -> 740 us;  d = 28672: 2122 -> 1500 us;  d = 8192, 16384 rows: 318 -> 218 us;
-//   d = 11008, 16384 rows: 384 -> 270 us (dense upper blocks);  d = 5120, 16384 rows: 221 -> 140 us;
+//   d = 14336, 32768 rows: 888 -> 740 us;  d = 28672, 16384 rows: 1070 -> 750 us;  d = 8192, 16384 rows: 318 -> 212 us;
+//   d = 11008, 16384 rows: 384 -> 270 us (dense upper blocks);  d = 5120, 16384 rows: 221 -> 136 us;
 //   d = 8192, 64 rows: 12.9 -> 8.0 us;  d = 11008, 1 row: 9.3 -> 7.3 us.
 // With the products left out the upper passes take 95 to 100 % of their time and the slab pass 80 %: the copies bound them.
+// (One product with 64 x 64 blocks instead of a slab's first two phases was as fast, but rounds once where the other kernels
+// round twice; results now are the same bits whichever kernel takes a batch.)
 //
 // The tile's layout is what the copy engine writes, chosen so that the 16-byte accesses of a quarter-warp (two rows, four
 // local indices) hit eight bank groups:
@@ -18,11 +20,10 @@
 //   upper pass  [half of the rows][row][outer digit][inner digit][column of 32 or 64 bytes], 32- or 64-byte swizzle.  The inner digit's
 //               radix is odd (or there is one digit), so a step of either digit is an odd number of columns; the two rows of a
 //               quarter-warp come from the two halves, whose distance moves the top bit of the swizzle by one.
-// Sixteen-wide upper blocks take columns of 64 bytes (d = 8192, 16384 rows: 226 -> 219 us; 16 column groups instead of 32 also fill
+// Sixteen-wide upper blocks take columns of 64 bytes (d = 8192, 16384 rows: 223 -> 218 us; 16 column groups instead of 32 also fill
 // 144 SMs instead of 128).  For two phases over 56 places such tiles leave one buffer per team and gain nothing.
 //
-// The first two phases of a slab are one product with 64 x 64 blocks, whose fragments stay in a warp's registers: one trip
-// through shared memory and one rounding less than as two phases of eight (d = 8192, 16384 rows: 246 -> 219 us).
+// A slab's first two phases stay with one warp (its box, fragments in registers, no barrier between them).
 #include <algorithm>
 #include <new>
 #include <vector>
@@ -43,7 +44,7 @@ constexpr int kMaxPipePhases = 3, kMaxPipeBufs = 4;
 constexpr uint32_t kPipeSpin = 1u << 22;      // limit of every wait for a bulk copy
 
 struct PipePhase {
-    int32_t mode;              // 0 = contiguous blocks of 64; 1 = strided blocks, eight per item
+    int32_t mode;              // 0 = the pair of phases inside a box; 1 = strided blocks, eight per item
     int32_t B, B_real;
     int32_t n_items, items_off;
     int32_t bfrag_off;         // word offset of the phase's fragments inside a column group's block
@@ -61,9 +62,9 @@ struct PipePass {
     int32_t n_tiles, n_parts;                 // n_parts > 0: a CTA keeps its column group and takes every n_parts-th tile; 0: equal shares of the list
     const int32_t *tables;                    // byte offsets of the items
     int32_t tables_len;
-    const uint32_t *bfrag;                    // [column group][bfrag_words]
-    int32_t bfrag_words;
-    const uint4 *frag64;                      // lower: [column group][block of 64][8 column tiles][2][lane], see dense_phase
+    const uint32_t *bfrag;                    // fragments, frag_stride words per column group (the plan's copy, see harp_split.cu)
+    int32_t frag_stride, smem_off, bfrag_words;   // part of them that the phases read from shared memory
+    int32_t pair_off[2], pair_bwd;            // lower: fragments of the first two phases; octets first (transpose)
     PipePhase ph[kMaxPipePhases];
 };
 
@@ -88,16 +89,15 @@ __device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
 
 // The kinds of pass.  A team is a few warps with n_buf tile buffers of their own; tiles of the CTA's column group go to its
 // teams in turn and a team's thread 0 issues its bulk copies.
-//   lower64          two teams of eight warps, a warp per block of 64; 64 of its 128 registers are fragments
-//   upper8           three teams of eight warps, at most 85 registers
+//   lower8, upper8   three teams of eight warps, at most 85 registers; lower8: a warp per box of 64 coordinates in the first two phases
 //   upper16          sixteen-wide blocks need 128 registers: two teams of eight warps
 //   dense32, dense48 all upper stages as one block of up to 32 or 48: a warp holds sixteen rows of eight positions, the two
 //                    octets of a tile make a team of two warps; three teams
-enum Kind { kLower64, kUpper8, kUpper16, kDense32, kDense48 };
+enum Kind { kLower8, kUpper8, kUpper16, kDense32, kDense48 };
 template <int K> struct KindOf {
-    static constexpr bool lower = K == kLower64, b16 = K == kUpper16, wide = b16;
+    static constexpr bool lower = K == kLower8, b16 = K == kUpper16, wide = b16;
     static constexpr int ks = K == kDense32 ? 2 : K == kDense48 ? 3 : 0;
-    static constexpr int team_warps = ks ? 2 : 8, team_threads = 32 * team_warps, teams = b16 || lower ? 2 : 3, threads = teams * team_threads;
+    static constexpr int team_warps = ks ? 2 : 8, team_threads = 32 * team_warps, teams = b16 ? 2 : 3, threads = teams * team_threads;
     static constexpr int swizzle_bits = lower ? 7 : wide ? 3 : 1;
 };
 template <int K> __device__ __forceinline__ uint32_t swz(uint32_t a) { return a ^ (((a >> 7) & (uint32_t)KindOf<K>::swizzle_bits) << 4); }
@@ -165,36 +165,44 @@ __device__ __forceinline__ void dense_octet(uint32_t a0, uint32_t row8_off, int 
     }
 }
 
-// Blocks of 64 contiguous coordinates, fragments in registers: f[2 n + s] holds, for column tile n, the words of k-steps 2 s and
-// 2 s + 1.  box: sixteen-row groups of 128-byte rows, 128-byte swizzle; the rows of a group are rewritten by the warp that read them.
-__device__ __forceinline__ void dense_phase(const uint4 (&f)[16], uint32_t box, int lane, int MT) {
-    uint32_t row = box + 128u * (uint32_t)((lane & 7) + ((lane >> 3) & 1) * 8);
-    const uint32_t hi = (uint32_t)lane >> 4, x = (row >> 7) & 7u;             // sixteen rows further is the same swizzle
-    for (int mt = 0; mt < MT; ++mt, row += 2048u) {
-        uint32_t a[4][4];
+// The two phases that stay inside a box of 64 coordinates: contiguous blocks of eight, fa, and blocks over the eight chunks of a
+// row, fb.  The rows of sixteen are this warp's, so that its own ordering is enough between the phases.
+__device__ __forceinline__ void box_contiguous(const uint32_t (&fa)[8], uint32_t box, int lane) {
+    const uint32_t row = box + 128u * (uint32_t)((lane & 7) + ((lane >> 3) & 1) * 8);
+    const uint32_t hi = (uint32_t)lane >> 4, x = (row >> 7) & 7u;
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks) ldmatrix_x4(a[ks], row + (((2u * ks + hi) ^ x) << 4));
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t addr = row + (((2u * c + hi) ^ x) << 4);
+        uint32_t a[4];
+        ldmatrix_x4(a, addr);
+        const uint32_t a_lo[2] = {a[0], a[1]}, a_hi[2] = {a[2], a[3]};
+        float c0[4], c1[4];
+        mma_k8(c0, a_lo, fa[2 * c]);
+        mma_k8(c1, a_hi, fa[2 * c + 1]);
+        stmatrix_x4(addr, pack_bf16(c0[0], c0[1]), pack_bf16(c0[2], c0[3]), pack_bf16(c1[0], c1[1]), pack_bf16(c1[2], c1[3]));
+    }
+}
+__device__ __forceinline__ void box_octet(const uint32_t (&fb)[8], uint32_t box, int g, int q) {
+    const uint32_t row = box + 128u * (uint32_t)g, x = (row >> 7) & 7u;
+    uint4 raw[2][2];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            float acc[2][4];
+    for (int j = 0; j < 2; ++j) {
+        const uint32_t addr = row + (((uint32_t)(2 * q + j) ^ x) << 4);
+        raw[j][0] = lds128(addr);
+        raw[j][1] = lds128(addr + 1024u);
+    }
+    octet_mma8(raw, fb);
 #pragma unroll
-            for (int k = 0; k < 2; ++k)
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {
-                    const uint4 &w = f[2 * (2 * c + k) + ks / 2];
-                    const uint32_t b0 = ks % 2 ? w.z : w.x, b1 = ks % 2 ? w.w : w.y;
-                    if (ks == 0) mma_k16(acc[k], a[ks], b0, b1);
-                    else mma_k16_acc(acc[k], a[ks], b0, b1);
-                }
-            stmatrix_x4(row + (((2u * c + hi) ^ x) << 4), pack_bf16(acc[0][0], acc[0][1]), pack_bf16(acc[0][2], acc[0][3]),
-                        pack_bf16(acc[1][0], acc[1][1]), pack_bf16(acc[1][2], acc[1][3]));
-        }
+    for (int j = 0; j < 2; ++j) {
+        const uint32_t addr = row + (((uint32_t)(2 * q + j) ^ x) << 4);
+        sts128(addr, raw[j][0]);
+        sts128(addr + 1024u, raw[j][1]);
     }
 }
 
 template <int K>
 __global__ void __launch_bounds__(KindOf<K>::threads, 1)
-harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const PipePass P) {
+harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const __grid_constant__ PipePass P) {
     constexpr bool LOWER = KindOf<K>::lower, B16 = KindOf<K>::b16;
     constexpr int LW = KindOf<K>::wide ? 32 : 16;          // upper: positions of a column group
     constexpr int KS = KindOf<K>::ks, TEAMS = KindOf<K>::teams, kTeamWarps = KindOf<K>::team_warps, kTeamThreads = KindOf<K>::team_threads;
@@ -267,18 +275,22 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
         }
         // fragments of the column group (plan data); every team is through with the ones before
         __syncthreads();
-        const uint32_t *src = P.bfrag + (size_t)cg * P.bfrag_words;
-        for (int i = threadIdx.x * 4; i < P.bfrag_words; i += TEAMS * kTeamThreads * 4) cp_async16(bf_s + 4u * i, src + i);
+        const uint32_t *src = P.bfrag + (size_t)cg * P.frag_stride;
+        for (int i = threadIdx.x * 4; i < P.bfrag_words; i += TEAMS * kTeamThreads * 4) cp_async16(bf_s + 4u * i, src + P.smem_off + i);
         if (!waited) {                               // the rows only once the kernel before has completed
             asm volatile("griddepcontrol.wait;" ::: "memory");
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             waited = true;
         }
-        [[maybe_unused]] uint4 f64[LOWER ? 16 : 1];
+        [[maybe_unused]] uint32_t fa[8], fb[8];
         if constexpr (LOWER) {
-            const uint4 *f = P.frag64 + ((size_t)cg * P.n_box + min(warp, P.n_box - 1)) * 512 + lane;
+            const int box = min(warp, P.n_box - 1);
+            const uint4 *f = reinterpret_cast<const uint4 *>(src + P.pair_off[1] + box * 256) + lane;
+            const uint4 f0 = __ldg(f), f1 = __ldg(f + 32);
+            fb[0] = f0.x; fb[1] = f0.y; fb[2] = f0.z; fb[3] = f0.w;
+            fb[4] = f1.x; fb[5] = f1.y; fb[6] = f1.z; fb[7] = f1.w;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) f64[i] = __ldg(f + 32 * i);
+            for (int e = 0; e < 8; ++e) fa[e] = __ldg(src + P.pair_off[0] + (box * 8 + e) * 32 + lane);
         }
         if (tid == 0 && !*(volatile int *)&dead)
             for (int k = 0; k < NB; ++k)
@@ -312,7 +324,16 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const P
                 const PipePhase &ph = P.ph[p];
                 if (p > 0) team_sync();
                 if (LOWER && ph.mode == 0) {
-                    if constexpr (LOWER) if (warp < P.n_box) dense_phase(f64, sbase + (uint32_t)(warp * P.box_pitch), lane, P.MT);
+                    if constexpr (LOWER) if (warp < P.n_box) {
+                        uint32_t box = sbase + (uint32_t)(warp * P.box_pitch);
+                        for (int mt = 0; mt < P.MT; ++mt, box += 2048u) {
+                            if (P.pair_bwd) box_octet(fb, box, g, q);
+                            else box_contiguous(fa, box, lane);
+                            __syncwarp();
+                            if (P.pair_bwd) box_contiguous(fa, box, lane);
+                            else box_octet(fb, box, g, q);
+                        }
+                    }
                 } else if (B16 && ph.B == 16) {
                     uint32_t so[4];
                     bool ok[4];
@@ -423,8 +444,9 @@ cudaError_t launch_pipe(const CUtensorMap &tmap, int32_t *err, const PipePass &P
 }
 
 // Fragments of the dense blocks (see dense_octet), sixteen positions per column group.
-void dense_fragments(const harp_plan *plan, const GPhase &gp, int n_cg, int ks, int dir, std::vector<uint32_t> &frag) {
+std::vector<uint32_t> dense_fragments(const harp_plan *plan, const GPhase &gp, int n_cg, int ks, int dir) {
     const int U = gp.B_real;
+    std::vector<uint32_t> frag((size_t)n_cg * 16 * 4 * ks * ks * 32);
     std::vector<double> F;
     auto coord = [&](int slot) { return 16 * (slot / 16) + strided_slot(slot % 16, 16, 1); };
     for (int l = 0; l < 16 * n_cg; ++l) {
@@ -446,31 +468,6 @@ void dense_fragments(const harp_plan *plan, const GPhase &gp, int n_cg, int ks, 
                         }
                     }
     }
-}
-
-// Fragments of the contiguous blocks of 64 (see dense_phase).
-std::vector<uint32_t> block64_fragments(const harp_plan *plan, const GPhase &gp, int dir) {
-    std::vector<uint32_t> frag((size_t)plan->d / 64 * 2048);
-    std::vector<double> F;
-    for (int64_t base = 0; base < plan->d; base += 64) {
-        fused_block(plan, HostPhase{gp.t0, gp.t1, 64, 1, 0, 1}, base, F);
-        auto G = [&](int i, int o) -> double {
-            double v = dir == 0 ? F[(size_t)i * 64 + o] : F[(size_t)o * 64 + i];
-            if (!plan->h_signs.empty()) {
-                const int64_t pos = base + (dir == 0 ? i : o);
-                v *= (double)plan->h_signs[(size_t)(plan->h_perm.empty() ? pos : plan->h_perm[(size_t)pos])];
-            }
-            return v;
-        };
-        for (int nt = 0; nt < 8; ++nt)
-            for (int ks = 0; ks < 4; ++ks)
-                for (int h = 0; h < 2; ++h)
-                    for (int lane = 0; lane < 32; ++lane) {
-                        const int n = 8 * nt + (lane >> 2), k = 16 * ks + 8 * h + 2 * (lane & 3);
-                        frag[(size_t)base / 64 * 2048 + (2 * nt + ks / 2) * 128 + lane * 4 + 2 * (ks % 2) + h] =
-                            f2bf(G(k, n)) | ((uint32_t)f2bf(G(k + 1, n)) << 16);
-                    }
-    }
     return frag;
 }
 
@@ -478,7 +475,7 @@ std::vector<uint32_t> block64_fragments(const harp_plan *plan, const GPhase &gp,
 
 struct PipePlan {
     PipePass dir[2];           // forward, transpose
-    int kind = kLower64;
+    int kind = kLower8;
     int64_t d = 0, S_mid = 1;
     int r_in = 1, r_out = 1;   // upper: radices of the inner and the outer digit of a tile
     int64_t s_in = 0, s_out = 0;   // ... and their strides in coordinates
@@ -496,7 +493,7 @@ void harp_pipe_destroy(PipePlan *pp) {
 
 // (1 to 32 rows of d = 5120 .. 28672: below nine rows the slab pass loses 0.2 us to the kernel of harp_split.cu, which reads only the
 // rows it has, and so does the sixteen-wide upper pass up to one row tile; the others are ahead from the first row on)
-int64_t harp_pipe_min_rows(const PipePlan *pp) { return pp->kind == kLower64 ? 9 : pp->kind == kUpper16 ? 17 : 1; }
+int64_t harp_pipe_min_rows(const PipePlan *pp) { return pp->kind == kLower8 ? 9 : pp->kind == kUpper16 ? 17 : 1; }
 
 int32_t harp_pipe_error_word(const PipePlan *pp) {
     if (!pp || !pp->d_err) return 0;
@@ -506,25 +503,21 @@ int32_t harp_pipe_error_word(const PipePlan *pp) {
 
 // The pass over `phs` (lower: slabs of S_mid coordinates; upper: sixteen neighbouring positions of all U slabs).
 // HARP_ERR_UNSUPPORTED: a shape for which the layouts above are not free of conflicts, or whose tiles do not fit.
-harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bool lower, int64_t S_mid, int64_t U, PipePlan **out) {
+harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &phs, bool lower, int64_t S_mid, int64_t U, const PassFrags &fr,
+                              PipePlan **out) {
     *out = nullptr;
-    if (lower) {                                         // the first two phases as blocks of 64
-        if (phs.size() < 2 || phs[0].B_real * phs[1].B_real != 64) return HARP_ERR_UNSUPPORTED;
-        phs[1] = GPhase{phs[0].t0, phs[1].t1, 64, 64, phs[0].S};
-        phs.erase(phs.begin());
-    }
-    const int np = (int)phs.size();
+    const int np = (int)phs.size(), pair = lower ? 2 : 0;     // lower: the first two phases count as one
     if (np < 1 || np > kMaxPipePhases || !harp_tensor_map_encoder()) return HARP_ERR_UNSUPPORTED;
     int widest = 8;
     for (const GPhase &gp : phs) widest = std::max(widest, gp.B);
     PipePass P{};
     PipePlan pl;
-    pl.kind = lower ? kLower64 : widest == 8 ? kUpper8 : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
+    pl.kind = lower ? kLower8 : widest == 8 ? kUpper8 : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
     const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = pl.kind == kUpper16 ? 32 : 16;
-    P.n_phases = np;
+    P.n_phases = lower ? np - 1 : np;
     if (lower) {
-        if (S_mid > 512) return HARP_ERR_UNSUPPORTED;
-        for (int p = 1; p < np; ++p)
+        if (np < 2 || S_mid > 512 || phs[0].B_real != 8 || phs[1].B_real != 8) return HARP_ERR_UNSUPPORTED;
+        for (int p = 2; p < np; ++p)
             if (phs[(size_t)p].B != 8) return HARP_ERR_UNSUPPORTED;
         P.n_cg = (int)U;
         P.n_box = (int)(S_mid / 64);
@@ -545,15 +538,17 @@ harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bo
         const int64_t i = (c / pl.s_in) % pl.r_in, o = np == 2 ? (c / pl.s_out) % pl.r_out : 0;
         return (o * pl.r_in + i) * 2 * Lw + (c % Lw) * 2;
     };
-    int words = 0, items = 0;
-    for (const GPhase &gp : phs) {
-        const int n_blk = (int)((lower ? S_mid : U * Lw) / gp.B_real);
-        words += lower && gp.S == 1 ? 0 : ks ? 16 * 4 * ks * ks * 32 : n_blk * (gp.B == 16 ? 128 : 32);
-        items += ks || (lower && gp.S == 1) ? 0 : n_blk / 8;
+    int words = ks ? 16 * 4 * ks * ks * 32 : 0, items = 0;
+    for (int p = pair; p < np && !ks; ++p) {
+        const int n_blk = (int)((lower ? S_mid : U * Lw) / phs[(size_t)p].B_real);
+        if (fr.lm[p] != (lower ? 2 : 1)) return HARP_ERR_UNSUPPORTED;
+        words += n_blk * (phs[(size_t)p].B == 16 ? 128 : 32);
+        items += n_blk / 8;
     }
+    if (!ks && !lower && words != fr.words * (Lw / 16)) return HARP_ERR_UNSUPPORTED;
     // the largest tile that fits; a pass of one phase refills a buffer while two others are full
-    const int teams = pl.kind == kUpper16 || lower ? 2 : 3;
-    P.n_buf = lower || (np == 1 && !ks) ? 3 : 2;
+    const int teams = pl.kind == kUpper16 ? 2 : 3;
+    P.n_buf = np == 1 && !ks && !lower ? 3 : 2;
     for (P.MT = ks ? 1 : 4, P.mt_shift = ks ? 0 : 2;; P.MT /= 2, --P.mt_shift) {
         P.box_bytes = lower ? 128 * 16 * P.MT : 8 * P.MT * P.row_bytes;
         P.box_pitch = P.box_bytes + (Lw == 32 ? 256 : 128);  // (P.box_bytes is a multiple of twice that)
@@ -583,29 +578,23 @@ harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bo
     pl.d_err = static_cast<int32_t *>(upload(std::vector<int32_t>(1, 0)));
     for (int dir = 0; dir < 2 && st == HARP_OK; ++dir) {
         std::vector<int32_t> tab;
-        std::vector<uint32_t> frag((size_t)P.n_cg * words, 0u);
-        std::vector<double> F;
-        int at = 0;
-        for (int k = 0; k < np; ++k) {
-            const GPhase &gp = phs[(size_t)(dir == 0 ? k : np - 1 - k)];
-            PipePhase &D = P.ph[k];
-            D = PipePhase{};
-            D.mode = lower && gp.S == 1 ? 0 : 1;
+        const int n_strided = np - pair;
+        P.smem_off = lower && np > 2 ? fr.off[dir][dir == 0 ? 2 : np - 1] : 0;
+        P.pair_bwd = dir;
+        for (int p = 0; p < pair; ++p) P.pair_off[p] = fr.off[dir][p];
+        for (int k = 0; k < P.n_phases; ++k) P.ph[k] = PipePhase{};          // mode 0
+        for (int k = 0; k < n_strided; ++k) {
+            const int p = dir == 0 ? pair + k : np - 1 - k;
+            const GPhase &gp = phs[(size_t)p];
+            PipePhase &D = P.ph[lower && dir == 0 ? k + 1 : k];
+            D.mode = 1;
             D.B = gp.B;
             D.B_real = gp.B_real;
-            D.lm = lower && D.mode == 1 ? 2 : 1;
+            if (ks) break;
+            D.lm = lower ? 2 : 1;
             for (int j = 0; j < 4; ++j) D.jr[j] = gp.B == 16 ? jo16[j] : j < 2 ? jo8[D.lm - 1][j] : 0;
             D.items_off = (int32_t)tab.size();
-            D.bfrag_off = at;
-            if (D.mode == 0) {
-                P.frag64 = static_cast<const uint4 *>(upload(block64_fragments(plan, gp, dir)));
-                continue;
-            }
-            if (ks) {
-                dense_fragments(plan, gp, P.n_cg, ks, dir, frag);
-                at = words;
-                continue;
-            }
+            D.bfrag_off = fr.off[dir][p] - P.smem_off;
             if (lower) {                                 // in octets: eight to a box
                 D.unit = (int32_t)(gp.S / 8);
                 D.shift = 3;
@@ -615,39 +604,28 @@ harp_status_t harp_pipe_build(const harp_plan *plan, std::vector<GPhase> phs, bo
                 D.unit = 1;
                 D.step[1] = (gp.S == pl.s_in ? 2 : 2 * pl.r_in) * Lw;
             }
-            // first coordinates of the blocks (lower: within the slab; upper: within position group 0)
-            std::vector<int64_t> first;
-            {
-                const int64_t span = gp.S * gp.B_real, all = lower ? S_mid : plan->d, lo_step = lower ? 8 : S_mid;
-                for (int64_t hi = 0; hi < all; hi += span)
-                    for (int64_t lo = 0; lo < gp.S; lo += lo_step)
-                        for (int64_t l8 = 0; l8 < (lower ? 8 : Lw); l8 += 8) {
-                            const int64_t c = hi + lo + l8;
-                            for (int r = 0; r < gp.B_real; ++r) {       // every octet that the kernel reaches
-                                const int e = r * D.unit;
-                                const int64_t a = place(c) + (e >> D.shift) * D.step[1] + (e & ((1 << D.shift) - 1)) * D.step[0];
-                                if (a != place(c + r * gp.S) || a < 0 || a + 16 > (lower ? P.tile_bytes : P.row_bytes)) return HARP_ERR_UNSUPPORTED;
-                            }
-                            tab.push_back((int32_t)place(c));
-                            for (int e = 0; e < 8; ++e) first.push_back(c + e);
+            // octets of blocks, in the order of their fragments (upper: within position group 0)
+            const int64_t span = gp.S * gp.B_real, all = lower ? S_mid : plan->d, lo_step = lower ? 8 : S_mid;
+            for (int64_t hi = 0; hi < all; hi += span)
+                for (int64_t lo = 0; lo < gp.S; lo += lo_step)
+                    for (int64_t l8 = 0; l8 < (lower ? 8 : Lw); l8 += 8) {
+                        const int64_t c = hi + lo + l8;
+                        for (int r = 0; r < gp.B_real; ++r) {       // every octet that the kernel reaches
+                            const int e = r * D.unit;
+                            const int64_t a = place(c) + (e >> D.shift) * D.step[1] + (e & ((1 << D.shift) - 1)) * D.step[0];
+                            if (a != place(c + r * gp.S) || a < 0 || a + 16 > (lower ? P.tile_bytes : P.row_bytes)) return HARP_ERR_UNSUPPORTED;
                         }
-            }
+                        tab.push_back((int32_t)place(c));
+                    }
             D.n_items = (int32_t)tab.size() - D.items_off;
-            auto slot = [&](int s) { return strided_slot(s, gp.B, D.lm); };
-            const int wpl = gp.B == 16 ? 4 : 1;
-            const bool grouped = gp.B == 8;       // [item][blocks 0-3 | 4-7][lane][4 words]
-            for (int cg = 0; cg < P.n_cg; ++cg)
-                for (size_t i = 0; i < first.size(); ++i) {
-                    uint32_t *dst = frag.data() + (size_t)cg * words + at + (grouped ? (i / 8 * 2 + i % 8 / 4) * 128 + i % 4 : i * 32 * wpl);
-                    block_fragment(plan, gp, (lower ? cg * S_mid : cg * Lw) + first[i], dir, slot, dst, grouped ? 4 : wpl, F);
-                }
-            at += (int)first.size() * 32 * wpl;
+            if (D.bfrag_off < 0 || D.bfrag_off + D.n_items * (gp.B == 16 ? 1024 : 256) > words) return HARP_ERR_UNSUPPORTED;
         }
-        if (at != words || (int)tab.size() != items || words % 4 != 0) return HARP_ERR_UNSUPPORTED;
+        if ((int)tab.size() != items || words % 4 != 0) return HARP_ERR_UNSUPPORTED;
         P.tables_len = items;
         P.bfrag_words = words;
         P.tables = static_cast<const int32_t *>(upload(tab));
-        P.bfrag = static_cast<const uint32_t *>(upload(frag));
+        P.frag_stride = lower ? fr.words : words;
+        P.bfrag = ks ? static_cast<const uint32_t *>(upload(dense_fragments(plan, phs[0], P.n_cg, ks, dir))) : fr.bfrag[dir];
         pl.dir[dir] = P;
     }
     PipePlan *pp = st == HARP_OK ? new (std::nothrow) PipePlan(pl) : nullptr;
@@ -674,14 +652,14 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
     // A column group per CTA keeps its fragments, and the CTAs at the same rows: neighbouring 32-byte runs meet in L2.  Where
     // the groups leave more than a tenth of the SMs without work, lower passes (whole lines) share the list out evenly.
     P.n_parts = (int32_t)std::min<int64_t>(P.n_tiles, std::max<int64_t>(1, slots / P.n_cg));
-    if (pp->kind == kLower64 && (P.n_cg > slots || slots % P.n_cg * 10 > slots)) P.n_parts = 0;
+    if (pp->kind == kLower8 && (P.n_cg > slots || slots % P.n_cg * 10 > slots)) P.n_parts = 0;
     const unsigned grid = (unsigned)(P.n_parts > 0 ? (int64_t)P.n_parts * P.n_cg : std::min<int64_t>((int64_t)P.n_tiles * P.n_cg, slots));
     const auto enc = reinterpret_cast<EncodeTiled>(harp_tensor_map_encoder());
     CUtensorMap tmap = {};
     const cuuint32_t ones[4] = {1, 1, 1, 1};
     const cuuint64_t n = (cuuint64_t)n_rows, pitch = (cuuint64_t)pp->d * 2;
     CUresult r;
-    if (pp->kind == kLower64) {
+    if (pp->kind == kLower8) {
         const cuuint64_t gdim[2] = {(cuuint64_t)pp->d, n}, gstr[1] = {pitch};
         const cuuint32_t box[2] = {64, (cuuint32_t)(16 * P.MT)};
         r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -697,7 +675,7 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
     if (r != CUDA_SUCCESS) return HARP_ERR_CUDA;
     cudaError_t err = cudaErrorInvalidValue;
     switch (pp->kind) {
-        case kLower64: err = launch_pipe<kLower64>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kLower8: err = launch_pipe<kLower8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper8: err = launch_pipe<kUpper8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper16: err = launch_pipe<kUpper16>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kDense32: err = launch_pipe<kDense32>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;

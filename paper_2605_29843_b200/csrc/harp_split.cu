@@ -514,6 +514,7 @@ struct PassHost {
     size_t smem_bytes = 0;
     bool present = false;
     bool has16 = false;
+    PassFrags frags{};
 };
 
 }  // namespace
@@ -563,7 +564,8 @@ harp_status_t build_pass(const harp_plan *plan, SplitPlan *sp, PassHost &ph_out,
     for (int p = 0; p < np; ++p) {
         if (!(lower && p == 0)) {
             ext = (ext + 7) / 8 * 8;
-            while (((ext / 8) % 8) == 0 || ((ext / 8) % 8) == 4) ext += 8;
+            // (upper passes: slots lane_mult = 1 apart in every phase, as the kernels of harp_pipe.cu read the same fragments)
+            while (((ext / 8) % 8) == 0 || ((ext / 8) % 8) == 4 || (!lower && (ext / 8) % 2 != 0)) ext += 8;
             lm[(size_t)p] = ((ext / 8) % 2 == 0) ? 1 : 2;
         }
         W[(size_t)p] = ext;
@@ -679,6 +681,8 @@ harp_status_t build_pass(const harp_plan *plan, SplitPlan *sp, PassHost &ph_out,
             tab.insert(tab.end(), is.bases.begin(), is.bases.end());
             D.bfrag_off = words;
             frag_off[(size_t)p] = words;
+            ph_out.frags.off[dir][p] = words;
+            ph_out.frags.lm[p] = l;
             words += (int32_t)(is.block_rel.size() * 32 * (gp.B == 16 ? 4 : 1));
             // bounds of every address formed from the tables
             bool ok = true;
@@ -721,6 +725,8 @@ harp_status_t build_pass(const harp_plan *plan, SplitPlan *sp, PassHost &ph_out,
             }
         }
         P.bfrag = upload_s(sp, frag, st);
+        ph_out.frags.bfrag[dir] = P.bfrag;
+        ph_out.frags.words = words;
         const size_t tile_bytes = (size_t)16 * MT * pitch * 2;
         bool any16 = false;
         for (const GPhase &gp : phs) any16 = any16 || gp.B == 16;
@@ -826,15 +832,14 @@ harp_status_t harp_split_build(harp_plan *plan) {
     sp->lower_stages = lower.back().t1;
     harp_status_t st = build_pass(plan, sp, sp->pass[0], lower, true, S_mid, U, 1);
     if (want_dense) upper = {GPhase{lower.back().t1, m, (int)(U + 15) / 16 * 16, (int)U, S_mid}};
-    for (int s = 0; s < (upper.empty() ? 1 : 2) && st == HARP_OK; ++s) {
-        st = harp_pipe_build(plan, s == 0 ? lower : upper, s == 0, S_mid, U, &sp->pipe[s]);
+    const bool dense_pipe = want_dense && U > 16;
+    if (st == HARP_OK && !want_dense && !upper.empty()) st = build_pass(plan, sp, sp->pass[1], upper, false, S_mid, U, Lw);
+    for (int s = 0; s < 2 && st == HARP_OK; ++s) {
+        if (s == 1 && !sp->pass[1].present && !dense_pipe) continue;
+        st = harp_pipe_build(plan, s == 0 ? lower : upper, s == 0, S_mid, U, sp->pass[s].frags, &sp->pipe[s]);
         if (st == HARP_ERR_UNSUPPORTED) st = HARP_OK;
     }
-    if (st == HARP_OK && want_dense) {
-        if (!sp->pipe[1] || harp_pipe_min_rows(sp->pipe[1]) > 1) st = build_dense_upper(plan, sp, lower.back().t1, S_mid, U);
-    } else if (st == HARP_OK && !upper.empty()) {
-        st = build_pass(plan, sp, sp->pass[1], upper, false, S_mid, U, Lw);
-    }
+    if (st == HARP_OK && want_dense && !sp->pipe[1]) st = build_dense_upper(plan, sp, lower.back().t1, S_mid, U);
     if (st == HARP_OK &&
         (cudaFuncSetAttribute(harp_split_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024) != cudaSuccess ||
          cudaFuncSetAttribute(harp_split_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024) != cudaSuccess ||
