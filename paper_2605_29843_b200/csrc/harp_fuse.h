@@ -112,7 +112,7 @@ struct PassFrags {
     int32_t words, off[2][6], lm[6];
 };
 harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<harp_fuse::GPhase> &phs, bool lower, int64_t S_mid, int64_t U,
-                              const PassFrags &fr, PipePlan **out);
+                              bool wide, const PassFrags &fr, PipePlan **out);
 int64_t harp_pipe_min_rows(const PipePlan *pp);   // smallest batch that it is meant for
 void harp_pipe_destroy(PipePlan *pp);
 harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int transpose, bool overlap, cudaStream_t stream);

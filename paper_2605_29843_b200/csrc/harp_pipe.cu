@@ -90,14 +90,15 @@ __device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
 // The kinds of pass.  A team is a few warps with n_buf tile buffers of their own; tiles of the CTA's column group go to its
 // teams in turn and a team's thread 0 issues its bulk copies.
 //   lower8, upper8   three teams of eight warps, at most 85 registers; lower8: a warp per box of 64 coordinates in the first two phases
+//   upper8Wide       one team of sixteen warps, two phases, a warp's two octets of each with their fragments in registers
 //   upper16          sixteen-wide blocks need 128 registers: two teams of eight warps
 //   dense32, dense48 all upper stages as one block of up to 32 or 48: a warp holds sixteen rows of eight positions, the two
 //                    octets of a tile make a team of two warps; three teams
-enum Kind { kLower8, kUpper8, kUpper16, kDense32, kDense48 };
+enum Kind { kLower8, kUpper8, kUpper8Wide, kUpper16, kDense32, kDense48 };
 template <int K> struct KindOf {
-    static constexpr bool lower = K == kLower8, b16 = K == kUpper16, wide = b16;
+    static constexpr bool lower = K == kLower8, b16 = K == kUpper16, wide = K == kUpper8Wide || b16;
     static constexpr int ks = K == kDense32 ? 2 : K == kDense48 ? 3 : 0;
-    static constexpr int team_warps = ks ? 2 : 8, team_threads = 32 * team_warps, teams = b16 ? 2 : 3, threads = teams * team_threads;
+    static constexpr int team_warps = ks ? 2 : K == kUpper8Wide ? 16 : 8, team_threads = 32 * team_warps, teams = K == kUpper8Wide ? 1 : b16 ? 2 : 3, threads = teams * team_threads;
     static constexpr int swizzle_bits = lower ? 7 : wide ? 3 : 1;
 };
 template <int K> __device__ __forceinline__ uint32_t swz(uint32_t a) { return a ^ (((a >> 7) & (uint32_t)KindOf<K>::swizzle_bits) << 4); }
@@ -282,7 +283,20 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
             asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             waited = true;
         }
-        [[maybe_unused]] uint32_t fa[8], fb[8];
+        [[maybe_unused]] uint32_t fa[8], fb[8], wf[2][2][8];
+        if constexpr (K == kUpper8Wide) {
+            // the fragments of two neighbouring groups of sixteen positions: item = (block, octet of the 32 positions)
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const int i1 = min(warp + kTeamWarps * k, P.ph[p].n_items - 1), l8 = i1 & 3;
+                    const uint4 *f = reinterpret_cast<const uint4 *>(src + (l8 >> 1) * (P.frag_stride / 2) + P.ph[p].bfrag_off + ((i1 >> 2) * 2 + (l8 & 1)) * 256) + lane;
+                    const uint4 f0 = __ldg(f), f1 = __ldg(f + 32);
+                    wf[p][k][0] = f0.x; wf[p][k][1] = f0.y; wf[p][k][2] = f0.z; wf[p][k][3] = f0.w;
+                    wf[p][k][4] = f1.x; wf[p][k][5] = f1.y; wf[p][k][6] = f1.z; wf[p][k][7] = f1.w;
+                }
+        }
         if constexpr (LOWER) {
             const int box = min(warp, P.n_box - 1);
             const uint4 *f = reinterpret_cast<const uint4 *>(src + P.pair_off[1] + box * 256) + lane;
@@ -316,7 +330,44 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
                     load(cg, first + (t + (NB - 1) * TEAMS) * step, b == 0 ? NB - 1 : b - 1);
                 }
             };
-            if constexpr (KS > 0) {
+            if constexpr (K == kUpper8Wide) {
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    const PipePhase &ph = P.ph[p];
+                    if (p > 0) team_sync();
+                    uint32_t so[2];
+                    bool ok[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        ok[j] = q + 4 * j < ph.B_real;
+                        so[j] = ok[j] ? (uint32_t)((q + 4 * j) * ph.step[1]) : 0u;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const int i1 = warp + kTeamWarps * k;
+                        if (i1 < ph.n_items) {
+                            const uint32_t a0 = sbase + lds32p(tab_s + 4u * (uint32_t)(ph.items_off + i1)) + row0_off;
+                            uint4 raw[2][2];
+                            uint32_t ad[2][2];
+#pragma unroll
+                            for (int j = 0; j < 2; ++j) {
+                                ad[j][0] = swz<K>(a0 + so[j]);
+                                ad[j][1] = swz<K>(a0 + so[j] + row8_off);
+                                raw[j][0] = lds128(ad[j][0]);
+                                raw[j][1] = lds128(ad[j][1]);
+                            }
+                            octet_mma8(raw, wf[p][k]);
+#pragma unroll
+                            for (int j = 0; j < 2; ++j)
+                                if (ok[j]) {
+                                    sts128(ad[j][0], raw[j][0]);
+                                    sts128(ad[j][1], raw[j][1]);
+                                }
+                        }
+                    }
+                    if (p == 0) refill();
+                }
+            } else if constexpr (KS > 0) {
                 dense_octet<K>(sbase + 16u * (uint32_t)warp + row0_off, row8_off, q, P.ph[0].B_real,
                                 bf_s + 16u * (uint32_t)(warp * 8 * KS * KS * 32 + lane), refill);
             } else
@@ -503,7 +554,7 @@ int32_t harp_pipe_error_word(const PipePlan *pp) {
 
 // The pass over `phs` (lower: slabs of S_mid coordinates; upper: sixteen neighbouring positions of all U slabs).
 // HARP_ERR_UNSUPPORTED: a shape for which the layouts above are not free of conflicts, or whose tiles do not fit.
-harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &phs, bool lower, int64_t S_mid, int64_t U, const PassFrags &fr,
+harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &phs, bool lower, int64_t S_mid, int64_t U, bool wide, const PassFrags &fr,
                               PipePlan **out) {
     *out = nullptr;
     const int np = (int)phs.size(), pair = lower ? 2 : 0;     // lower: the first two phases count as one
@@ -512,8 +563,9 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
     for (const GPhase &gp : phs) widest = std::max(widest, gp.B);
     PipePass P{};
     PipePlan pl;
-    pl.kind = lower ? kLower8 : widest == 8 ? kUpper8 : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
-    const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = pl.kind == kUpper16 ? 32 : 16;
+    pl.kind = lower ? kLower8 : widest == 8 ? (wide ? kUpper8Wide : kUpper8) : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
+    const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = pl.kind == kUpper16 || pl.kind == kUpper8Wide ? 32 : 16;
+    if (wide && (pl.kind != kUpper8Wide || np != 2)) return HARP_ERR_UNSUPPORTED;
     P.n_phases = lower ? np - 1 : np;
     if (lower) {
         if (np < 2 || S_mid > 512 || phs[0].B_real != 8 || phs[1].B_real != 8) return HARP_ERR_UNSUPPORTED;
@@ -547,9 +599,10 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
     }
     if (!ks && !lower && words != fr.words * (Lw / 16)) return HARP_ERR_UNSUPPORTED;
     // the largest tile that fits; a pass of one phase refills a buffer while two others are full
-    const int teams = pl.kind == kUpper16 ? 2 : 3;
-    P.n_buf = np == 1 && !ks && !lower ? 3 : 2;
-    for (P.MT = ks ? 1 : 4, P.mt_shift = ks ? 0 : 2;; P.MT /= 2, --P.mt_shift) {
+    const int teams = wide ? 1 : pl.kind == kUpper16 ? 2 : 3;
+    P.n_buf = wide || (np == 1 && !ks && !lower) ? 3 : 2;
+    if (wide) words = 0;
+    for (P.MT = ks || wide ? 1 : 4, P.mt_shift = P.MT / 2;; P.MT /= 2, --P.mt_shift) {
         P.box_bytes = lower ? 128 * 16 * P.MT : 8 * P.MT * P.row_bytes;
         P.box_pitch = P.box_bytes + (Lw == 32 ? 256 : 128);  // (P.box_bytes is a multiple of twice that)
         P.tile_bytes = P.n_box * P.box_pitch;
@@ -618,13 +671,13 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
                         tab.push_back((int32_t)place(c));
                     }
             D.n_items = (int32_t)tab.size() - D.items_off;
-            if (D.bfrag_off < 0 || D.bfrag_off + D.n_items * (gp.B == 16 ? 1024 : 256) > words) return HARP_ERR_UNSUPPORTED;
+            if (wide ? D.n_items > 32 : D.bfrag_off < 0 || D.bfrag_off + D.n_items * (gp.B == 16 ? 1024 : 256) > words) return HARP_ERR_UNSUPPORTED;
         }
         if ((int)tab.size() != items || words % 4 != 0) return HARP_ERR_UNSUPPORTED;
         P.tables_len = items;
         P.bfrag_words = words;
         P.tables = static_cast<const int32_t *>(upload(tab));
-        P.frag_stride = lower ? fr.words : words;
+        P.frag_stride = wide ? 2 * fr.words : lower ? fr.words : words;
         P.bfrag = ks ? static_cast<const uint32_t *>(upload(dense_fragments(plan, phs[0], P.n_cg, ks, dir))) : fr.bfrag[dir];
         pl.dir[dir] = P;
     }
@@ -668,15 +721,16 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
         // (position, inner digit, outer digit, row)
         const cuuint64_t gdim[4] = {(cuuint64_t)pp->S_mid, (cuuint64_t)pp->r_in, (cuuint64_t)pp->r_out, n};
         const cuuint64_t gstr[3] = {(cuuint64_t)pp->s_in * 2, (cuuint64_t)(pp->r_out > 1 ? pp->s_out : pp->s_in) * 2, pitch};
-        const cuuint32_t box[4] = {(cuuint32_t)(pp->kind == kUpper16 ? 32 : 16), (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
+        const cuuint32_t box[4] = {(cuuint32_t)(pp->kind == kUpper16 || pp->kind == kUpper8Wide ? 32 : 16), (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
         r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                pp->kind == kUpper16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                pp->kind == kUpper16 || pp->kind == kUpper8Wide ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
     if (r != CUDA_SUCCESS) return HARP_ERR_CUDA;
     cudaError_t err = cudaErrorInvalidValue;
     switch (pp->kind) {
         case kLower8: err = launch_pipe<kLower8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper8: err = launch_pipe<kUpper8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kUpper8Wide: err = launch_pipe<kUpper8Wide>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper16: err = launch_pipe<kUpper16>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kDense32: err = launch_pipe<kDense32>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kDense48: err = launch_pipe<kDense48>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;

@@ -529,7 +529,7 @@ struct SplitPlan {
     const uint16_t *gather[2] = {nullptr, nullptr};
     int gather_rows = 1;       // rows per buffer of the gather kernel
     size_t gather_smem = 0;
-    PipePlan *pipe[2] = {nullptr, nullptr};   // the passes fed by the copy engine (harp_pipe.cu), where the shape allows them
+    PipePlan *pipe[3] = {nullptr, nullptr, nullptr};   // the passes fed by the copy engine (harp_pipe.cu), where the shape allows them
     // dense upper pass (replaces pass[1] when set)
     bool dense_upper = false;
     UpperPass up_fwd{}, up_bwd{};
@@ -834,9 +834,9 @@ harp_status_t harp_split_build(harp_plan *plan) {
     if (want_dense) upper = {GPhase{lower.back().t1, m, (int)(U + 15) / 16 * 16, (int)U, S_mid}};
     const bool dense_pipe = want_dense && U > 16;
     if (st == HARP_OK && !want_dense && !upper.empty()) st = build_pass(plan, sp, sp->pass[1], upper, false, S_mid, U, Lw);
-    for (int s = 0; s < 2 && st == HARP_OK; ++s) {
-        if (s == 1 && !sp->pass[1].present && !dense_pipe) continue;
-        st = harp_pipe_build(plan, s == 0 ? lower : upper, s == 0, S_mid, U, sp->pass[s].frags, &sp->pipe[s]);
+    for (int s = 0; s < 3 && st == HARP_OK; ++s) {
+        if (s > 0 && !sp->pass[1].present && !dense_pipe) continue;
+        st = harp_pipe_build(plan, s == 0 ? lower : upper, s == 0, S_mid, U, s == 2, sp->pass[s > 0].frags, &sp->pipe[s]);
         if (st == HARP_ERR_UNSUPPORTED) st = HARP_OK;
     }
     if (st == HARP_OK && want_dense && !sp->pipe[1]) st = build_dense_upper(plan, sp, lower.back().t1, S_mid, U);
@@ -963,7 +963,7 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
                 if (ts != HARP_ERR_UNSUPPORTED) return ts;
             }
             if (sp->pipe[pi] && r1 - r0 >= harp_pipe_min_rows(sp->pipe[pi])) {
-                const harp_status_t ps = harp_pipe_apply(sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
+                const harp_status_t ps = harp_pipe_apply(pi == 1 && sp->pipe[2] && r1 - r0 >= (getenv("HARP_WIDE_ROWS") ? atoll(getenv("HARP_WIDE_ROWS")) : 1024) ? sp->pipe[2] : sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
                 if (ps != HARP_OK) return ps;
                 continue;
             }
