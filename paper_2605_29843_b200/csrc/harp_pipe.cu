@@ -20,9 +20,10 @@
 //   upper pass  [half of the rows][row][outer digit][inner digit][column of 32 or 64 bytes], 32- or 64-byte swizzle.  The inner digit's
 //               radix is odd (or there is one digit), so a step of either digit is an odd number of columns; the two rows of a
 //               quarter-warp come from the two halves, whose distance moves the top bit of the swizzle by one.
-// Sixteen-wide upper blocks take columns of 64 bytes (d = 8192, 16384 rows: 223 -> 218 us; 16 column groups instead of 32 also fill
-// 144 SMs instead of 128).  For two phases over 56 places such tiles leave one buffer per team and gain nothing.
-//
+// Columns of 64 bytes double the fragments of a column group and halve the number of groups.  Sixteen-wide blocks take them (d = 8192,
+// 16384 rows: 223 -> 218 us; 16 groups instead of 32 also fill 144 SMs instead of 128), and so do two phases of eight for
+// batches that fill the SMs, with the fragments in registers so that three buffers fit (d = 14336, 32768 rows: 750 -> 667 us;
+// d = 28672, 4096 rows: 190 -> 175 us; with the fragments in shared memory and one buffer per team it was slower than columns of 32).
 // A slab's first two phases stay with one warp (its box, fragments in registers, no barrier between them).
 #include <algorithm>
 #include <new>
@@ -543,8 +544,17 @@ void harp_pipe_destroy(PipePlan *pp) {
 }
 
 // (1 to 32 rows of d = 5120 .. 28672: below nine rows the slab pass loses 0.2 us to the kernel of harp_split.cu, which reads only the
-// rows it has, and so does the sixteen-wide upper pass up to one row tile; the others are ahead from the first row on)
-int64_t harp_pipe_min_rows(const PipePlan *pp) { return pp->kind == kLower8 ? 9 : pp->kind == kUpper16 ? 17 : 1; }
+// rows it has, and so does the sixteen-wide upper pass up to one row tile; the others are ahead from the first row on.  The
+// wide tiles of two phases pay once they give three quarters of the SMs one: 128 rows of d = 28672 14.0 -> 13.1 us, 256 of
+// d = 14336 13.3 -> 12.3; at half of that 0.3 to 0.6 us are lost.)
+int64_t harp_pipe_min_rows(const PipePlan *pp) {
+    switch (pp->kind) {
+        case kLower8: return 9;
+        case kUpper16: return 17;
+        case kUpper8Wide: return 16 * (3 * pp->sms / (4 * pp->dir[0].n_cg)) + 1;
+        default: return 1;
+    }
+}
 
 int32_t harp_pipe_error_word(const PipePlan *pp) {
     if (!pp || !pp->d_err) return 0;

@@ -529,7 +529,7 @@ struct SplitPlan {
     const uint16_t *gather[2] = {nullptr, nullptr};
     int gather_rows = 1;       // rows per buffer of the gather kernel
     size_t gather_smem = 0;
-    PipePlan *pipe[3] = {nullptr, nullptr, nullptr};   // the passes fed by the copy engine (harp_pipe.cu), where the shape allows them
+    PipePlan *pipe[3] = {nullptr, nullptr, nullptr};   // the passes fed by the copy engine (harp_pipe.cu), where the shape allows them; [2] upper, large batches
     // dense upper pass (replaces pass[1] when set)
     bool dense_upper = false;
     UpperPass up_fwd{}, up_bwd{};
@@ -963,7 +963,8 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
                 if (ts != HARP_ERR_UNSUPPORTED) return ts;
             }
             if (sp->pipe[pi] && r1 - r0 >= harp_pipe_min_rows(sp->pipe[pi])) {
-                const harp_status_t ps = harp_pipe_apply(pi == 1 && sp->pipe[2] && r1 - r0 >= (getenv("HARP_WIDE_ROWS") ? atoll(getenv("HARP_WIDE_ROWS")) : 1024) ? sp->pipe[2] : sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
+                const bool wide = pi == 1 && sp->pipe[2] && r1 - r0 >= harp_pipe_min_rows(sp->pipe[2]);
+                const harp_status_t ps = harp_pipe_apply(wide ? sp->pipe[2] : sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
                 if (ps != HARP_OK) return ps;
                 continue;
             }
