@@ -19,6 +19,7 @@
 // own some of the results (forward) or some of the rows of the gradient block (backward).  The first step reads x and the
 // last dL/dy in their own type.  Radices with no such kernel use the plain one-thread-per-element kernels.
 #include <algorithm>
+#include <type_traits>
 #include <map>
 #include <mutex>
 
@@ -140,7 +141,7 @@ __host__ __device__ constexpr int bwd_per_sm(int b, int bi, int subs) { return (
 
 // sums of the warps that split the rows, added in the order of the warps; sum k of a lane goes to dst(k)
 template <int N, int SUBS, typename Dst>
-__device__ __forceinline__ void combine(const double (&acc)[N], double (*sh)[SUBS][32], int sub, int lane, Dst dst) {
+__device__ __forceinline__ void combine(const double (&acc)[N], double (*sh)[SUBS][32], int sub, int lane, int add, Dst dst) {
     if constexpr (SUBS > 1) {
 #pragma unroll
         for (int k = 0; k < N; ++k) sh[k][sub][lane] = acc[k];
@@ -151,12 +152,12 @@ __device__ __forceinline__ void combine(const double (&acc)[N], double (*sh)[SUB
                 double a = sh[k][0][lane];
 #pragma unroll
                 for (int w = 1; w < SUBS; ++w) a += sh[k][w][lane];
-                if (double *p = dst(k)) *p = a;
+                if (double *p = dst(k)) *p = add ? *p + a : a;
             }
     } else {
 #pragma unroll
         for (int k = 0; k < N; ++k)
-            if (double *p = dst(k)) *p = acc[k];
+            if (double *p = dst(k)) *p = add ? *p + acc[k] : acc[k];
     }
 }
 
@@ -165,7 +166,7 @@ __device__ __forceinline__ void combine(const double (&acc)[N], double (*sh)[SUB
 template <int B, int BI, int SUBS, typename TV, typename TG>
 __global__ void __launch_bounds__(32 * ((B + BI - 1) / BI) * SUBS, bwd_per_sm(B, BI, SUBS))
 bwd_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v, const TG *__restrict__ g, int vec_g, float *__restrict__ g_out,
-           int64_t rows, int64_t d, int64_t s, int slice, const float *__restrict__ em, double *__restrict__ part) {
+           int64_t rows, int64_t d, int64_t s, int slice, int add, const float *__restrict__ em, double *__restrict__ part) {
     constexpr int PARTS = (B + BI - 1) / BI;
     __shared__ double sh[SUBS > 1 ? PARTS : 1][SUBS > 1 ? BI * B : 1][SUBS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, pt = w / SUBS, sub = w - pt * SUBS, i0 = pt * BI;
@@ -227,7 +228,7 @@ bwd_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v
         }
     }
     double *dst = part + (int64_t)blockIdx.y * (B * B) * nblk + c;
-    combine<BI * B, SUBS>(acc, SUBS > 1 ? sh[pt] : nullptr, sub, lane, [&](int e) -> double * {
+    combine<BI * B, SUBS>(acc, SUBS > 1 ? sh[pt] : nullptr, sub, lane, add, [&](int e) -> double * {
         const int ij = i0 * B + e;
         return have && ij < B * B ? dst + (int64_t)ij * nblk : nullptr;
     });
@@ -328,7 +329,7 @@ fwd44_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int ve
 template <bool S1, typename TV, typename TG>
 __global__ void __launch_bounds__(32 * kSubs, k44PerSm)
 bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v, const TG *__restrict__ g, int vec_g, float *__restrict__ g_out,
-             int64_t rows, int64_t d, int64_t s, int slice, const float *__restrict__ em1, const float *__restrict__ em2, double *__restrict__ part1,
+             int64_t rows, int64_t d, int64_t s, int slice, int add, const float *__restrict__ em1, const float *__restrict__ em2, double *__restrict__ part1,
              double *__restrict__ part2) {
     __shared__ double sh[32][kSubs][32];
     const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
@@ -401,7 +402,7 @@ bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
         }
     }
     double *d1 = part1 + (int64_t)blockIdx.y * 16 * nblk + u.c1, *d2 = part2 + (int64_t)blockIdx.y * 16 * nblk + u.c2;
-    combine<32, kSubs>(acc, sh, sub, lane, [&](int e) -> double * {
+    combine<32, kSubs>(acc, sh, sub, lane, add, [&](int e) -> double * {
         return !u.have ? nullptr : e < 16 ? d1 + (int64_t)e * nblk : d2 + (int64_t)(e - 16) * nblk;
     });
 }
@@ -470,7 +471,7 @@ fwd22_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int ve
 template <typename TV, typename TG>
 __global__ void __launch_bounds__(32 * kSubs, 4)
 bwd22_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v, const TG *__restrict__ g, int vec_g, float *__restrict__ g_out,
-             int64_t rows, int64_t d, int64_t s, int slice, const float *__restrict__ em1, const float *__restrict__ em2, double *__restrict__ part1,
+             int64_t rows, int64_t d, int64_t s, int slice, int add, const float *__restrict__ em1, const float *__restrict__ em2, double *__restrict__ part1,
              double *__restrict__ part2) {
     __shared__ double sh[16][kSubs][32];
     const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
@@ -537,7 +538,7 @@ bwd22_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
         }
     }
     double *d1 = part1 + (int64_t)blockIdx.y * 4 * nblk, *d2 = part2 + (int64_t)blockIdx.y * 4 * nblk;
-    combine<16, kSubs>(acc, sh, sub, lane, [&](int e) -> double * {
+    combine<16, kSubs>(acc, sh, sub, lane, add, [&](int e) -> double * {
         if (!u.have) return nullptr;
         const int b = (e >> 2) & 1, ij = e & 3;
         return e < 8 ? d1 + (int64_t)ij * nblk + u.c1[b] : d2 + (int64_t)ij * nblk + u.c2[b];
@@ -579,51 +580,70 @@ reduce_kernel(const double *__restrict__ part, float *__restrict__ grad, int acc
     }
 }
 
-// ---- x with the permutation and the signs of the plan, rows of the same type: out[r][i] = s[perm[i]] x[r][perm[i]].  A row at
-// a time through shared memory (two elements of padding per 64 keep a digit reversal off the same banks); staged = 0: rows
-// too long for that are gathered from global memory
+// ---- x with the permutation and the signs of the plan, rows of the same type: out[r][i] = s[perm[i]] x[r][perm[i]].  R rows at a
+// time through shared memory (two elements of padding per 64 keep a digit reversal off the same banks), so that an index and
+// its sign, twice the bytes of a bf16 row, are read once for all of them; staged = 0: rows too long for that are gathered from
+// global memory one by one.  T: the bits of an element.  (2731 rows of d = 4096, bf16: 26 us with one row at a time, 17 with four)
 template <typename T>
-__global__ void __launch_bounds__(kThreads)
-permute_kernel(const T *__restrict__ x, int vec, T *__restrict__ out, int64_t rows, int64_t d, const int32_t *__restrict__ perm,
-               const int8_t *__restrict__ signs, int staged) {
+__global__ void __launch_bounds__(kThreads, 5)
+permute_kernel(const T *__restrict__ x, int vec, T *__restrict__ out, int64_t rows, int d, const int32_t *__restrict__ perm,
+               const int8_t *__restrict__ signs, int staged, int R) {
     prior_kernel_done();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *row = reinterpret_cast<T *>(smem_raw);
+    T *tile = reinterpret_cast<T *>(smem_raw);
     constexpr int V = 16 / (int)sizeof(T);
-    for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+    constexpr T kSignBit = (T)((T)1 << (8 * sizeof(T) - 1));
+    const int pitch = (d + 2 * (d >> 6) + 2) / 2 * 2;
+    for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < rows; r0 += (int64_t)gridDim.x * R) {
+        const int nr = (int)min((int64_t)R, rows - r0);
+        const T *xr = x + r0 * d;
+        T *outr = out + r0 * d;
         if (staged) {
-            if (vec) {
-#pragma unroll 2
-                for (int64_t i = (int64_t)threadIdx.x * V; i < d; i += kThreads * V) {
-                    const uint4 q = *reinterpret_cast<const uint4 *>(x + r * d + i);
-                    uint32_t *dst = reinterpret_cast<uint32_t *>(row + i + 2 * (i >> 6));     // 4-byte aligned: the index is even
+            if (vec) {                                   // the rows are one run of 16-byte pieces
+#pragma unroll 4
+                for (int i = (int)threadIdx.x * V; i < nr * d; i += kThreads * V) {
+                    const uint4 q = *reinterpret_cast<const uint4 *>(xr + i);
+                    const int rr = (i >= d) + (i >= 2 * d) + (i >= 3 * d), c = i - rr * d;
+                    uint32_t *dst = reinterpret_cast<uint32_t *>(tile + rr * pitch + c + 2 * (c >> 6));     // 4-byte aligned: the index is even
                     dst[0] = q.x; dst[1] = q.y; dst[2] = q.z; dst[3] = q.w;
                 }
             } else {
-                for (int64_t i = threadIdx.x; i < d; i += kThreads) row[i + 2 * (i >> 6)] = x[r * d + i];
+                for (int rr = 0; rr < nr; ++rr)
+                    for (int i = threadIdx.x; i < d; i += kThreads) tile[rr * pitch + i + 2 * (i >> 6)] = xr[(int64_t)rr * d + i];
             }
             __syncthreads();
         }
-        if (d % 4 == 0) {
-            for (int64_t i = (int64_t)threadIdx.x * 4; i < d; i += kThreads * 4) {
-                const int4 s4 = *reinterpret_cast<const int4 *>(perm + i);
-                const int src[4] = {s4.x, s4.y, s4.z, s4.w};
-                __align__(16) T o[4];
+        auto gather = [&](const T *from, int step, bool padded) {
+            if (d % 4 == 0) {
+                for (int i = (int)threadIdx.x * 4; i < d; i += kThreads * 4) {
+                    const int4 s4 = *reinterpret_cast<const int4 *>(perm + i);
+                    int src[4] = {s4.x, s4.y, s4.z, s4.w};
+                    T flip[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const T v = staged ? row[src[k] + 2 * (src[k] >> 6)] : x[r * d + src[k]];
-                    o[k] = signs && signs[src[k]] < 0 ? (T)-v : v;
+                    for (int k = 0; k < 4; ++k) {
+                        flip[k] = signs && signs[src[k]] < 0 ? kSignBit : (T)0;
+                        if (padded) src[k] += 2 * (src[k] >> 6);
+                    }
+                    const T *f = from;
+                    T *to = outr + i;
+                    for (int rr = 0; rr < nr; ++rr, f += step, to += d) {
+                        T o[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) o[k] = f[src[k]] ^ flip[k];
+                        if constexpr (sizeof(T) == 2) *reinterpret_cast<uint2 *>(to) = make_uint2(o[0] | (uint32_t)o[1] << 16, o[2] | (uint32_t)o[3] << 16);
+                        else *reinterpret_cast<uint4 *>(to) = make_uint4(o[0], o[1], o[2], o[3]);
+                    }
                 }
-                if constexpr (sizeof(T) == 2) *reinterpret_cast<uint2 *>(out + r * d + i) = *reinterpret_cast<const uint2 *>(o);
-                else *reinterpret_cast<uint4 *>(out + r * d + i) = *reinterpret_cast<const uint4 *>(o);
+            } else {
+                for (int i = threadIdx.x; i < d; i += kThreads) {
+                    const int src = perm[i], at = padded ? src + 2 * (src >> 6) : src;
+                    const T flip = signs && signs[src] < 0 ? kSignBit : (T)0;
+                    for (int rr = 0; rr < nr; ++rr) outr[(int64_t)rr * d + i] = from[(int64_t)rr * step + at] ^ flip;
+                }
             }
-        } else {
-            for (int64_t i = threadIdx.x; i < d; i += kThreads) {
-                const int src = perm[i];
-                const T v = staged ? row[src + 2 * (src >> 6)] : x[r * d + src];
-                out[r * d + i] = signs && signs[src] < 0 ? (T)-v : v;
-            }
-        }
+        };
+        if (staged) gather(tile, pitch, true);
+        else gather(xr, d, false);
         __syncthreads();
     }
 }
@@ -804,7 +824,7 @@ void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int
 // kernels, into grad)
 template <typename TV, typename TG>
 int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8_t *signs, const TG *g, float *g_out, int64_t rows, double *part, double *part2,
-                  int slice, float *grad, int acc, cudaStream_t st) {
+                  int slice, int add, float *grad, int acc, cudaStream_t st) {
     const int64_t d = plan->d, s = plan->st.s[sp.t];
     const int b = plan->st.b[sp.t];
     const float *em = plan->d_blocks_em + plan->st.off[sp.t];
@@ -812,15 +832,15 @@ int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8
     const int vec_v = s == 1 && d % 4 == 0 && aligned16(v), vec_g = s == 1 && d % 4 == 0 && aligned16(g);
     if (sp.n == 2 && b == 4) {
         const dim3 grid = grid2(d / 16, 8, rows, slice);
-        if (s == 1) launch_dep(bwd44_kernel<true, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, em2, part, part2);
-        else launch_dep(bwd44_kernel<false, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, em2, part, part2);
+        if (s == 1) launch_dep(bwd44_kernel<true, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, em2, part, part2);
+        else launch_dep(bwd44_kernel<false, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, em2, part, part2);
         return 1;
     }
     if (sp.n == 2) {
-        launch_dep(bwd22_kernel<TV, TG>, grid2(d / 4, 32, rows, slice), dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, em2, part, part2);
+        launch_dep(bwd22_kernel<TV, TG>, grid2(d / 4, 32, rows, slice), dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, em2, part, part2);
         return 1;
     }
-#define HARP_BWD(B, BI, SUBS) case B: launch_dep(bwd_kernel<B, BI, SUBS, TV, TG>, grid2(d / B, 32, rows, slice), dim3(32 * ((B + BI - 1) / BI) * SUBS), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, em, part); return 1
+#define HARP_BWD(B, BI, SUBS) case B: launch_dep(bwd_kernel<B, BI, SUBS, TV, TG>, grid2(d / B, 32, rows, slice), dim3(32 * ((B + BI - 1) / BI) * SUBS), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, part); return 1
     switch (b) {
         HARP_BWD(2, 2, kSubs); HARP_BWD(3, 3, kSubs); HARP_BWD(4, 4, kSubs); HARP_BWD(5, 5, kSubs); HARP_BWD(6, 3, kSubs); HARP_BWD(7, 4, 2);
         HARP_BWD(8, 2, 2); HARP_BWD(16, 2, 1);
@@ -882,12 +902,16 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
         const T *xc = x + r0 * d, *gc = gy + r0 * d;
         int launches = 0;
         if (permuted) {
-            size_t smem = (size_t)(d + 2 * (d >> 6) + 2) * sizeof(T);
+            using Bits = std::conditional_t<sizeof(T) == 2, uint16_t, uint32_t>;
+            const size_t row_smem = (size_t)((d + 2 * (d >> 6) + 2) / 2 * 2) * sizeof(T);
+            int R = 4;                             // (the kernel counts on at most four)
+            while (R > 1 && R * row_smem > 100 * 1024) R /= 2;
+            size_t smem = R * row_smem;
             // per call: the attribute belongs to the current device's copy of the kernel
-            const int staged = smem <= 48 * 1024 || (smem <= 200 * 1024 && cudaFuncSetAttribute(permute_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess);
+            const int staged = smem <= 48 * 1024 || (smem <= 200 * 1024 && cudaFuncSetAttribute(permute_kernel<Bits>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess);
             if (!staged) smem = 0;
-            launch_dep(permute_kernel<T>, dim3((unsigned)std::min<int64_t>(rows, 148 * 8)), dim3(kThreads), smem, st, xc, (int)(aligned16(xc) && d % (16 / (int64_t)sizeof(T)) == 0), xp,
-                       rows, d, plan->d_perm, plan->d_signs, staged);
+            launch_dep(permute_kernel<Bits>, dim3((unsigned)std::min<int64_t>((rows + R - 1) / R, 148 * 8)), dim3(kThreads), smem, st, reinterpret_cast<const Bits *>(xc), (int)(aligned16(xc) && d % (16 / (int64_t)sizeof(T)) == 0), reinterpret_cast<Bits *>(xp),
+                       rows, (int)d, plan->d_perm, plan->d_signs, staged, R);
             xc = xp;
             ++launches;
         }
@@ -901,17 +925,14 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
             float *out = k > 0 ? gp + (k % ring) * plane : nullptr;
             const int slice = slice_rows(plan, sp, chunk, sms);
             double *p1 = part + part_off[sp.t], *p2 = sp.n == 2 ? part + part_off[sp.t + 1] : nullptr;
-            if (k == 0 && k == n - 1) launches += step_backward<T, T>(plan, sp, xc, signs, gc, out, rows, p1, p2, slice, grad, acc, st);
-            else if (k == n - 1) launches += step_backward<float, T>(plan, sp, v_in, nullptr, gc, out, rows, p1, p2, slice, grad, acc, st);
-            else if (k == 0) launches += step_backward<T, float>(plan, sp, xc, signs, g_in, out, rows, p1, p2, slice, grad, acc, st);
-            else launches += step_backward<float, float>(plan, sp, v_in, nullptr, g_in, out, rows, p1, p2, slice, grad, acc, st);
+            if (k == 0 && k == n - 1) launches += step_backward<T, T>(plan, sp, xc, signs, gc, out, rows, p1, p2, slice, r0 > 0, grad, acc, st);
+            else if (k == n - 1) launches += step_backward<float, T>(plan, sp, v_in, nullptr, gc, out, rows, p1, p2, slice, r0 > 0, grad, acc, st);
+            else if (k == 0) launches += step_backward<T, float>(plan, sp, xc, signs, g_in, out, rows, p1, p2, slice, r0 > 0, grad, acc, st);
+            else launches += step_backward<float, float>(plan, sp, v_in, nullptr, g_in, out, rows, p1, p2, slice, r0 > 0, grad, acc, st);
         }
-        if (red.m > 0) {
-            for (int k = 0; k < red.m; ++k) {
-                const int per = red.st[k].rows;
-                red.st[k].n_slices = (int32_t)((rows + per - 1) / per);
-            }
-            launch_dep(reduce_kernel, dim3((unsigned)std::min<int64_t>((red.total + 31) / 32, 148 * 16)), dim3(kThreads), 0, st, part, grad, acc, red);
+        if (red.m > 0 && r0 + chunk >= n_rows) {
+            for (int k = 0; k < red.m; ++k) red.st[k].n_slices = (int32_t)((chunk + red.st[k].rows - 1) / red.st[k].rows);
+            launch_dep(reduce_kernel, dim3((unsigned)std::min<int64_t>((red.total + 31) / 32, 148 * 16)), dim3(kThreads), 0, st, part, grad, accumulate, red);
             ++launches;
         }
         g_harp_launches.fetch_add(launches, std::memory_order_relaxed);
