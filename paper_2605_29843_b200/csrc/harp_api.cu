@@ -228,6 +228,10 @@ extern "C" harp_status_t harp_apply_ex(const harp_plan_t *plan, void *x, int64_t
         st = harp_tm_apply(plan, x, n_rows, dtype, transpose, s);
         if (st != HARP_ERR_UNSUPPORTED) return st;
     }
+    if (dtype == HARP_BF16 && harp_fast_yields(plan, n_rows)) {
+        st = harp_split_apply(plan, x, n_rows, dtype, transpose, s);
+        if (st != HARP_ERR_UNSUPPORTED) return st;
+    }
     st = harp_fast_apply(plan, x, n_rows, dtype, transpose, s);
     if (st != HARP_ERR_UNSUPPORTED) return st;
     st = harp_split_apply(plan, x, n_rows, dtype, transpose, s);

@@ -1202,6 +1202,17 @@ void harp_fast_destroy(harp_plan *plan) {
     plan->fast = nullptr;
 }
 
+// Batches that the two-pass path takes from this kernel.  With four phases (radix 8, d = 4096) a whole-row tile costs more than two
+// passes at copy rate, unless its batch is less than the clusters of eight hold (128 rows 7.7 us against 7.8) or nearly one full
+// wave of tiles (1800 to 2300 rows 17 us against 18 to 19); 256 rows 10.0 -> 8.4 us, 1024 14.8 -> 12.3, 2500 30.9 -> 20.3,
+// 16384 123 -> 111.  With three phases of sixteen (97 against 91 us, 65536 rows 366 against 396) it keeps them.
+bool harp_fast_yields(const harp_plan *plan, int64_t n_rows) {
+    const FastPlan *fp = plan->fast;
+    if (!fp || fp->fwd.n_phases < 4 || plan->d < 4096 || !plan->h_perm.empty() || !harp_split_piped(plan)) return false;
+    const int64_t n_tiles = (n_rows + kTileRows - 1) / kTileRows;
+    return n_tiles > fp->clusters[3] && (n_tiles * 4 <= fp->max_ctas * 3 || n_tiles > fp->max_ctas);
+}
+
 harp_status_t harp_fast_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose,
                               cudaStream_t stream) {
     const FastPlan *fp = plan->fast;

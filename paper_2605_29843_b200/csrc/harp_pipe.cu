@@ -24,6 +24,7 @@
 // 16384 rows: 223 -> 218 us; 16 groups instead of 32 also fill 144 SMs instead of 128), and so do two phases of eight for
 // batches that fill the SMs, with the fragments in registers so that three buffers fit (d = 14336, 32768 rows: 750 -> 667 us;
 // d = 28672, 4096 rows: 190 -> 175 us; with the fragments in shared memory and one buffer per team it was slower than columns of 32).
+// One phase of eight takes them too (d = 4096, radix 8, 16384 rows: 119 -> 111 us).
 // A slab's first two phases stay with one warp (its box, fragments in registers, no barrier between them).
 #include <algorithm>
 #include <new>
@@ -90,14 +91,16 @@ __device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
 
 // The kinds of pass.  A team is a few warps with n_buf tile buffers of their own; tiles of the CTA's column group go to its
 // teams in turn and a team's thread 0 issues its bulk copies.
-//   lower8, upper8   three teams of eight warps, at most 85 registers; lower8: a warp per box of 64 coordinates in the first two phases
+//   lower8, upper8, upper8One   three teams of eight warps, at most 85 registers; lower8: a warp per box of 64 coordinates in the first two phases
+//                    (upper8One: one phase, columns of 64 bytes)
 //   upper8Wide       one team of sixteen warps, two phases, a warp's two octets of each with their fragments in registers
 //   upper16          sixteen-wide blocks need 128 registers: two teams of eight warps
 //   dense32, dense48 all upper stages as one block of up to 32 or 48: a warp holds sixteen rows of eight positions, the two
 //                    octets of a tile make a team of two warps; three teams
-enum Kind { kLower8, kUpper8, kUpper8Wide, kUpper16, kDense32, kDense48 };
+enum Kind { kLower8, kUpper8, kUpper8One, kUpper8Wide, kUpper16, kDense32, kDense48 };
+constexpr bool is_wide(int K) { return K == kUpper8One || K == kUpper8Wide || K == kUpper16; }
 template <int K> struct KindOf {
-    static constexpr bool lower = K == kLower8, b16 = K == kUpper16, wide = K == kUpper8Wide || b16;
+    static constexpr bool lower = K == kLower8, b16 = K == kUpper16, wide = is_wide(K);
     static constexpr int ks = K == kDense32 ? 2 : K == kDense48 ? 3 : 0;
     static constexpr int team_warps = ks ? 2 : K == kUpper8Wide ? 16 : 8, team_threads = 32 * team_warps, teams = K == kUpper8Wide ? 1 : b16 ? 2 : 3, threads = teams * team_threads;
     static constexpr int swizzle_bits = lower ? 7 : wide ? 3 : 1;
@@ -573,8 +576,8 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
     for (const GPhase &gp : phs) widest = std::max(widest, gp.B);
     PipePass P{};
     PipePlan pl;
-    pl.kind = lower ? kLower8 : widest == 8 ? (wide ? kUpper8Wide : kUpper8) : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
-    const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = pl.kind == kUpper16 || pl.kind == kUpper8Wide ? 32 : 16;
+    pl.kind = lower ? kLower8 : widest == 8 ? (wide ? kUpper8Wide : np == 1 && S_mid % 32 == 0 ? kUpper8One : kUpper8) : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
+    const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = is_wide(pl.kind) ? 32 : 16;
     if (wide && (pl.kind != kUpper8Wide || np != 2)) return HARP_ERR_UNSUPPORTED;
     P.n_phases = lower ? np - 1 : np;
     if (lower) {
@@ -731,15 +734,16 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
         // (position, inner digit, outer digit, row)
         const cuuint64_t gdim[4] = {(cuuint64_t)pp->S_mid, (cuuint64_t)pp->r_in, (cuuint64_t)pp->r_out, n};
         const cuuint64_t gstr[3] = {(cuuint64_t)pp->s_in * 2, (cuuint64_t)(pp->r_out > 1 ? pp->s_out : pp->s_in) * 2, pitch};
-        const cuuint32_t box[4] = {(cuuint32_t)(pp->kind == kUpper16 || pp->kind == kUpper8Wide ? 32 : 16), (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
+        const cuuint32_t box[4] = {(cuuint32_t)(is_wide(pp->kind) ? 32 : 16), (cuuint32_t)pp->r_in, (cuuint32_t)pp->r_out, (cuuint32_t)(8 * P.MT)};
         r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, x, gdim, gstr, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                pp->kind == kUpper16 || pp->kind == kUpper8Wide ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                is_wide(pp->kind) ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
     if (r != CUDA_SUCCESS) return HARP_ERR_CUDA;
     cudaError_t err = cudaErrorInvalidValue;
     switch (pp->kind) {
         case kLower8: err = launch_pipe<kLower8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper8: err = launch_pipe<kUpper8>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
+        case kUpper8One: err = launch_pipe<kUpper8One>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper8Wide: err = launch_pipe<kUpper8Wide>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kUpper16: err = launch_pipe<kUpper16>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;
         case kDense32: err = launch_pipe<kDense32>(tmap, pp->d_err, P, grid, pp->smem, overlap, stream); break;

@@ -924,6 +924,8 @@ constexpr int64_t kOverlapMaxElems = (int64_t)16 << 20;
 // leave a third of the SMs idle and it is the slower one)
 constexpr int64_t kTmSlabMinRows = 384;
 
+bool harp_split_piped(const harp_plan *plan) { return plan->split && plan->split->pipe[0] && plan->split->pipe[1]; }
+
 int32_t harp_split_error_word(const harp_plan *plan) {
     int32_t w = 0;
     if (plan->split)

@@ -13,7 +13,7 @@ from harp_testlib import TOL, gpu_apply, host_rows, promote
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("radices", [(8, 8, 16), (8, 8, 3, 16), (8, 8, 7, 5, 3), (8, 8, 8, 8, 2), (8, 8, 8, 8, 7), (16, 16, 7, 5),
+@pytest.mark.parametrize("radices", [(8, 8, 16), (8, 8, 8, 8), (8, 8, 3, 16), (8, 8, 7, 5, 3), (8, 8, 8, 8, 2), (8, 8, 8, 8, 7), (16, 16, 7, 5),
                                      (16, 16, 43), (16, 16, 47), (8, 8, 8, 19)])
 @pytest.mark.parametrize("n_rows", [8, 9, 16, 17, 31, 33, 65, 131, 2049, 6001])
 def test_matches_the_oracle(radices, n_rows):
