@@ -64,8 +64,11 @@ struct PhaseDesc {
     int32_t B;                 // 8 or 16
     int32_t lane_step;         // element offset between the slots of lanes q and q+1
     int32_t j_off[4];          // element offsets of a lane's slots
+};
+
+struct ClusterPhase {          // cluster variant
     int32_t lm, jr[4];         // local index of slot j of lane q is lm * q + jr[j]
-    int32_t order;             // cluster variant: offset of the item order inside ctab
+    int32_t order;             // offset of the item order inside ctab
 };
 
 struct FastParams {
@@ -81,12 +84,13 @@ struct FastParams {
     // phases whose block fragments a CTA keeps in tensor memory for all its tiles (bit p = phase p):
     // warp w reads the fragments of its own items w and w + 16 from its 32 lanes, 32 columns per item
     uint32_t tm_mask;
+    PhaseDesc ph[kMaxPhases];
     // cluster variant: chunk numbers of a row in the order of the CTA that loads / stores them, item numbers of every phase in
     // the order of the CTA that runs them, and the phases after which the results move to another CTA (bit p = phase p)
     const int32_t *ctab;
     int32_t ctab_len, order_in, order_out;
     uint32_t xchg_mask;
-    PhaseDesc ph[kMaxPhases];
+    ClusterPhase cl[kMaxPhases];
 };
 
 // Per-section cycle counters of the whole-row kernel (build with -DHARP_FAST_TIMING): thread 0 of every CTA
@@ -159,12 +163,12 @@ __device__ __forceinline__ void st_cluster128(uint32_t addr, uint32_t rank, cons
     asm volatile("st.shared::cluster.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(remote), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 template <int NJ>
-__device__ __forceinline__ void store_to_owner(const TileCtx &c, const PhaseDesc &ph, int it, const uint4 (&raw)[NJ][2], int cs) {
+__device__ __forceinline__ void store_to_owner(const TileCtx &c, const PhaseDesc &ph, const ClusterPhase &cl, int it, const uint4 (&raw)[NJ][2], int cs) {
     const uint32_t a0 = c.sbase + 2u * (uint32_t)(c.g * c.pitch + c.q * ph.lane_step + c.tab[ph.items_off + it]);
     const uint32_t a1 = a0 + 2u * (uint32_t)(8 * c.pitch);
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
-        const uint32_t rank = (uint32_t)((ph.lm * c.q + ph.jr[j]) * cs / ph.B);
+        const uint32_t rank = (uint32_t)((cl.lm * c.q + cl.jr[j]) * cs / ph.B);
         st_cluster128(a0 + 2u * ph.j_off[j], rank, raw[j][0]);
         st_cluster128(a1 + 2u * ph.j_off[j], rank, raw[j][1]);
     }
@@ -311,7 +315,7 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
             const PhaseDesc &ph = P.ph[p];
             // items [0, n) of the phase, or this CTA's share of them in its order
             const int n = CL ? ph.n_items / cs : ph.n_items;
-            const int32_t *item = ord + ph.order + rank * n;
+            const int32_t *item = ord + (CL ? P.cl[p].order : 0) + rank * n;
             const bool xchg = CL && ((P.xchg_mask >> p) & 1u);
             const int tm_slot = !CL && ((P.tm_mask >> p) & 1u) ? __popc(P.tm_mask & ((1u << p) - 1u)) : -1;
             if ((MODES & bit(MODE_CC)) && ph.mode == MODE_CC) {
@@ -355,7 +359,7 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                     const int it = CL ? item[k] : k;
                     ss16_load(c, ph, it, raw, bf, tm_slot);
                     octet_mma16<true>(raw, bf, unused);
-                    if (xchg) store_to_owner<4>(c, ph, it, raw, cs);
+                    if (xchg) store_to_owner<4>(c, ph, P.cl[p], it, raw, cs);
                     else ss16_store(c, ph, it, raw);
                 }
             } else if ((MODES & bit(MODE_SS)) && ph.mode == MODE_SS) {
@@ -375,7 +379,7 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                     }
                     octet_mma8(raw, bf);
                     if (xchg) {
-                        store_to_owner<2>(c, ph, it, raw, cs);
+                        store_to_owner<2>(c, ph, P.cl[p], it, raw, cs);
                         continue;
                     }
 #pragma unroll
@@ -973,9 +977,9 @@ harp_status_t harp_fast_build(harp_plan *plan) {
             const Layout &L = src_side ? Lsrc : Lnat;
             const int lm = (mode == MODE_GS || mode == MODE_CG || mode == MODE_CC || mode == MODE_PO)
                                ? 1 : L.lm[(size_t)p];   // table-indexed slots use the plain map
-            D.lm = lm;
+            P.cl[k].lm = lm;
             const int *jo = B == 16 ? (lm == 1 ? joff1_16 : lm == 2 ? joff2_16 : joff4_16) : (lm == 1 ? joff1_8 : joff2_8);
-            for (int j = 0; j < 4; ++j) D.jr[j] = jo[j];
+            for (int j = 0; j < 4; ++j) P.cl[k].jr[j] = jo[j];
             if (mode == MODE_GS || mode == MODE_CG) {    // these index the item table by slot
                 D.lane_step = lm;
                 for (int j = 0; j < 4; ++j) D.j_off[j] = jo[j];
@@ -1083,7 +1087,7 @@ harp_status_t harp_fast_build(harp_plan *plan) {
                 }
                 if (!ok) { st = HARP_ERR_UNSUPPORTED; break; }
             }
-            if (clustered) D.order = by_digit(item_owner);
+            if (clustered) P.cl[k].order = by_digit(item_owner);
             D.items_off = (int32_t)tables.size();
             tables.insert(tables.end(), items.begin(), items.end());
             // fragments: B[k-slot][n-slot] = G[local index of the k-slot][local index of the n-slot]
