@@ -248,9 +248,9 @@ int64_t harp_two_sided_static_capacity_bytes(void);
  *   grad       DEVICE float[harp_plan_n_params(plan)], laid out like the blocks given to
  *              harp_plan_create (stage after stage, [D_t][b_t][b_t]); overwritten, or added to
  *              if accumulate != 0
- * Any schedule is accepted.  Sums over rows are taken in fp64 by one thread per entry (no
+ * Any schedule is accepted.  Sums over rows are taken in fp64, in an order that the shapes fix (no
  * atomics: the result does not depend on scheduling).  The call allocates and frees scratch
- * on the stream (at most ~256 MB, from a memory pool of the library's own that keeps what it has
+ * on the stream (about 200 MB of states and the partial sums of one wave of CTAs, from a memory pool of the library's own that keeps what it has
  * been given until the process ends); HARP_ERR_ALLOC if that fails.  Asynchronous on stream. */
 harp_status_t harp_grad_blocks(const harp_plan_t *plan, const void *x, const void *gy, int64_t n_rows,
                                harp_dtype_t dtype, float *grad, int accumulate, void *stream);
