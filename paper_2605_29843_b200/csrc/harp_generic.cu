@@ -341,6 +341,10 @@ __device__ __forceinline__ void stage_blocks_t(float *v, int n_rg, int R4, int d
 }
 
 
+// The kernel is launched with the programmatic stream-serialisation attribute: what stands above this call reads plan data only and runs
+// while the kernel before it in the stream is still busy on other SMs; the rows are touched once that has completed.
+__device__ __forceinline__ void rows_ready() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- the two ends of the stage list done on the way in / out of the transposed tile ----------------
 // Stage 0 of the table (stride 1, radix 4): a thread that copies the quad of coordinates 4m .. 4m+3 of
 // four rows between global memory and the tile owns block m of that stage, so the stage is applied in
@@ -361,6 +365,7 @@ __device__ __forceinline__ void copy_in_with_stage0(const T *xt, float *v, int r
         int pos[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) pos[j] = tpos(4 * m + j) * R4;
+        rows_ready();
         float e[4][4], nx[4][4];
 #pragma unroll
         for (int rr = 0; rr < 4; ++rr) {
@@ -478,6 +483,7 @@ __device__ __forceinline__ void stage_from_global(const T *xt, float *v, int row
         for (int i = 0; i < B; ++i)
 #pragma unroll
             for (int j = 0; j < B; ++j) K[i][j] = __ldg(Kt + (size_t)(j * B + i) * nblk + c);
+        rows_ready();
 #pragma unroll 2
         for (int rg = 0; rg < n_rg; ++rg) {
             float4 in[B];
@@ -515,6 +521,8 @@ harp_rowvec_kernel(T *__restrict__ x, int64_t n_rows, int d, int rows_per_cta, i
     // fuse_lo / fuse_hi (host: no permutation, aligned rows): stage 0 and the top stage run on the way
     // in and out of the tile
     const int top = st.m - 1;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (transpose ? !fuse_hi : !fuse_lo) rows_ready();
     // a1-a3: load, sign, gather (forward) -- or plain load (transpose)
     if (!transpose && fuse_lo) {
         copy_in_with_stage0<T>(xt, v, rows, n_rg, R4, d, blocks + st.off[0], signs, tid, nthr);
@@ -552,6 +560,7 @@ harp_rowvec_kernel(T *__restrict__ x, int64_t n_rows, int d, int rows_per_cta, i
             *reinterpret_cast<float4 *>(v + tpos(i) * R4 + 4 * rg) = make_float4(e[0], e[1], e[2], e[3]);
         }
     }
+    rows_ready();                                        // (threads that had nothing to load)
     __syncthreads();
     for (int k = 0; k < st.m; ++k) {
         const int t = transpose ? st.m - 1 - k : k;
@@ -636,8 +645,20 @@ harp_status_t launch_rowvec(const harp_plan *plan, const StageTable &st, const f
     const bool ends_ok = !plan->d_perm && d % 4 == 0 && (reinterpret_cast<uintptr_t>(x) % (4 * sizeof(T))) == 0 && st.m >= 3;
     const int fuse_lo = ends_ok && st.b[0] == 4 && st.s[0] == 1;
     const int fuse_hi = ends_ok && st.b[st.m - 1] <= 4 && st.s[st.m - 1] >= 32;
-    kern<<<(unsigned)grid, NT, (size_t)d * 16 * g_pad, stream>>>((T *)x, n_rows, (int)d, (int)r, (int)(4 * g_pad), st, blocks,
-                                                              plan->d_perm, plan->d_signs, transpose, fuse_lo, fuse_hi);
+    // (4096 rows of d = 2048, one after the other on a stream: 24.8 us without the attribute, 23.6 with it)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = (size_t)d * 16 * g_pad;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kern, (T *)x, n_rows, (int)d, (int)r, (int)(4 * g_pad), st, blocks, (const int32_t *)plan->d_perm,
+                           (const int8_t *)plan->d_signs, transpose, fuse_lo, fuse_hi) != cudaSuccess)
+        return HARP_ERR_CUDA;
     g_harp_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? HARP_OK : HARP_ERR_CUDA;
 }

@@ -468,6 +468,7 @@ harp_gather_rows_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int32_t d
     const uint32_t buf_bytes = (uint32_t)R * row_bytes;
     const int chunks = d >> 3;                                      // 16-byte chunks per row
     for (int c = threadIdx.x; c < chunks; c += kGatherThreads) cp_async16(tab_s + 16u * c, table + 8 * c);
+    rows_ready_barrier();
     const int64_t n_groups = (n_rows + R - 1) / R;
     auto copy_in = [&](int64_t grp, uint32_t dst) {
         const int64_t row0 = grp * R;
@@ -916,10 +917,10 @@ cudaError_t launch_pass(void (*kern)(__nv_bfloat16 *, int64_t, int64_t, PassT), 
     return cudaLaunchKernelEx(&cfg, kern, x, r0, r1, P);
 }
 
-// (measured over 96 .. 8192 rows, d = 5120 .. 28672: with the attribute a call gains 3-5 us up to about this many elements --
-// passes of some 20 us --, e.g. 512 rows of d = 8192 20.5 -> 18.5 us, and loses 1-4 % on larger batches, where CTAs that
-// wait for the kernel before them hold shared memory its last CTAs could use)
-constexpr int64_t kOverlapMaxElems = (int64_t)16 << 20;
+// (measured over 512 .. 32768 rows, d = 5120 .. 28672: with the attribute a call gains 2-5 us while the batch fits L2 -- 1024 rows of
+// d = 28672 55.4 -> 49.6 us, 4096 of d = 14336 81.4 -> 79.1 -- and loses 2-20 % beyond, 32768 of d = 28672 1380 -> 1680 us: CTAs
+// that start early take the bandwidth in an order of their own)
+constexpr int64_t kOverlapMaxElems = (int64_t)64 << 20;
 // (400 rows of d = 14336: 21.1 us with the mma.sync slab pass, 18.6 with the tensor-memory one; at 256 rows its 128-row tiles
 // leave a third of the SMs idle and it is the slower one)
 constexpr int64_t kTmSlabMinRows = 384;
@@ -944,10 +945,19 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
     auto gather = [&](int dir) -> harp_status_t {
         const int64_t n_groups = (n_rows + sp->gather_rows - 1) / sp->gather_rows;
         const unsigned grid = (unsigned)std::min<int64_t>(n_groups, sp->sms);
-        harp_gather_rows_kernel<<<grid, kGatherThreads, sp->gather_smem, stream>>>(xb, n_rows, (int32_t)plan->d, sp->gather_rows,
-                                                                                   sp->gather[dir]);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(kGatherThreads);
+        cfg.dynamicSmemBytes = sp->gather_smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = overlap ? 1 : 0;
+        const cudaError_t err = cudaLaunchKernelEx(&cfg, harp_gather_rows_kernel, xb, n_rows, (int32_t)plan->d, (int32_t)sp->gather_rows, sp->gather[dir]);
         g_harp_launches.fetch_add(1, std::memory_order_relaxed);
-        return cudaGetLastError() == cudaSuccess ? HARP_OK : HARP_ERR_CUDA;
+        return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? HARP_OK : HARP_ERR_CUDA;
     };
     if (sp->gather[0] && !transpose) {
         const harp_status_t gs = gather(0);
