@@ -184,14 +184,14 @@ harp_col_kernel(__nv_bfloat16 *__restrict__ W, int64_t ld, int64_t n_cols, ColPa
 // ---------------------------------------------------------------------------------------
 // The same passes fed by bulk tensor copies, for slabs of boxes of C positions (C = 64: phases of eight and eight inside a box, C = 16: one
 // of sixteen) with one phase across the boxes, and upper passes of one phase.  The kernel above spends most of a tile's time
-// issuing its copies; here sixteen warps multiply one of three buffers in place while the copy engine stores and refills the others.
+// issuing its copies; here 32 warps multiply one of three buffers in place while the copy engine stores and refills the others.
 // A tile is [row][64 columns], 128-byte rows, 128-byte swizzle: chunk c of row r lies at c ^ (r % 8).  The eight rows of an
 // ldmatrix have to differ in that value.  Neighbouring rows do; a slab's boxes lie one row apart beyond their size, so rows of
 // different boxes do; an upper tile is [position][place].  For the second phase inside a box of 64 (rows eight apart) the first
 // writes chunk c to c ^ ((r + position / 8) % 8), and the phase across the boxes goes back to what the copy engine expects:
 // a warp takes a block through all its chunks, so a row is read whole before it is written.
 // (8192 x 28672 processed on both sides: 922 -> 765 us; 4096 x 11008: 189 -> 149; 2048 x 2048: 25 -> 21)
-constexpr int kColPipeThreads = 512, kColPipeBufs = 3, kColPipeSmem = 226 * 1024;
+constexpr int kColPipeThreads = 1024, kColPipeBufs = 3, kColPipeSmem = 226 * 1024;
 constexpr uint32_t kColSpin = 1u << 22;       // limit of every wait for a bulk copy
 
 struct ColPipePass {
