@@ -6,9 +6,9 @@ import pytest
 import torch
 
 import paper_2605_29843_b200 as harp
-from oracle import harp_oracle as orc
+from oracle import c_oracle, harp_oracle as orc
 from paper_2605_29843_b200 import workloads as wl
-from harp_testlib import TOL, gpu_apply, host_rows, promote
+from harp_testlib import TOL, gpu_apply, host_rows, promote, to_device, to_host_f64
 
 pytestmark = pytest.mark.gpu
 
@@ -26,3 +26,21 @@ def test_matches_the_oracle(radices, n_rows):
         got, guards = gpu_apply(plan, xh, "bf16", tr, harp.KERNEL_SPLIT)
         assert guards and harp.harp_plan_error_word(plan) == 0
         assert orc.rel_err_rows(got[rows], fn(oplan, promote(xh[rows], "bf16"))) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("out_radices", [(16, 16, 8), (16, 8), (8, 8, 7, 16), (8, 8, 8, 5, 2), (8, 8, 5, 4)])
+@pytest.mark.parametrize("in_radices", [(8,), (9, 8), (8, 8, 5), (8, 8, 8, 8, 3)])
+def test_columns_match_the_oracle(out_radices, in_radices):
+    """The column side: slabs of three shapes, upper passes of one phase, 8 to 12288 columns (tiles of 64, the last one ragged)."""
+    p_out = wl.make_plan(83, int(np.prod(out_radices)), out_radices, "qr", perm="identity", signs=True)
+    p_in = wl.make_plan(84, int(np.prod(in_radices)), in_radices, "qr", perm="identity", signs=True)
+    plan = harp.plan_from_spec(p_out)
+    wh = host_rows(np.random.default_rng(85).standard_normal((p_out.d, p_in.d)), "bf16")
+    wd = to_device(wh, "bf16")
+    harp.two_sided_(wd, plan, harp.plan_from_spec(p_in))
+    torch.cuda.synchronize()
+    assert harp.harp_plan_error_word(plan) == 0
+    want = c_oracle.two_sided(c_oracle.CPlan(p_out), c_oracle.CPlan(p_in), promote(wh, "bf16"))
+    # an entry against the smaller norm of its row and column: one bound of the rows' test per side
+    scale = np.minimum(np.linalg.norm(want, axis=1, keepdims=True), np.linalg.norm(want, axis=0, keepdims=True))
+    assert np.max(np.abs(to_host_f64(wd) - want) / scale) <= 2 * TOL["bf16"]
