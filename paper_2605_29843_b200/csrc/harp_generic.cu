@@ -627,14 +627,19 @@ harp_status_t launch_rowvec(const harp_plan *plan, const StageTable &st, const f
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t d = plan->d;
-    // groups of four rows per CTA: an odd number (bank spread), as many as shared memory holds,
-    // but no more than one wave of CTAs needs
+    // groups of four rows per CTA: at most what shared memory holds (padded to an odd number: bank spread);
     // MINB CTAs share an SM (and its shared memory): while one multiplies, another copies
     int64_t g_max = (226 * 1024 / MINB) / (d * 16);
     if (g_max % 2 == 0) --g_max;
     if (g_max < 1) return HARP_ERR_UNSUPPORTED;
-    int64_t g = ((n_rows + (int64_t)sms * MINB - 1) / ((int64_t)sms * MINB) + 3) / 4;
-    g = std::max<int64_t>(1, std::min<int64_t>(g, std::min<int64_t>(g_max, 15)));
+    // the size for which waves of CTAs times a CTA's time -- its rows and about one group's worth for the block kernels it
+    // fetches -- is least (2048 rows of d = 4096: 171 CTAs of 12 rows 108 us, 256 of 8 rows 80; 10000 rows of d = 2048,
+    // 28 rows 67 us, 24 rows 61)
+    int64_t g = 1, best = INT64_MAX;
+    for (int64_t c = std::min<int64_t>(g_max, 15); c >= 1; --c) {
+        const int64_t ctas = (n_rows + 4 * c - 1) / (4 * c), cost = (ctas + (int64_t)sms * MINB - 1) / ((int64_t)sms * MINB) * (c + 1);
+        if (cost < best) { best = cost; g = c; }
+    }
     const int64_t g_pad = g | 1;                     // g_pad <= g_max because g_max is odd
     const int64_t r = 4 * g;
     const int64_t grid = (n_rows + r - 1) / r;
