@@ -20,11 +20,11 @@
 //   upper pass  [half of the rows][row][outer digit][inner digit][column of 32 or 64 bytes], 32- or 64-byte swizzle.  The inner digit's
 //               radix is odd (or there is one digit), so a step of either digit is an odd number of columns; the two rows of a
 //               quarter-warp come from the two halves, whose distance moves the top bit of the swizzle by one.
-// Columns of 64 bytes double the fragments of a column group and halve the number of groups.  Sixteen-wide blocks take them (d = 8192,
+// Columns of 64 bytes double the fragments of a column group and halve the number of groups.  One phase of sixteen takes them (d = 8192,
 // 16384 rows: 223 -> 218 us; 16 groups instead of 32 also fill 144 SMs instead of 128), and so do two phases of eight for
 // batches that fill the SMs, with the fragments in registers so that three buffers fit (d = 14336, 32768 rows: 750 -> 667 us;
 // d = 28672, 4096 rows: 190 -> 175 us; with the fragments in shared memory and one buffer per team it was slower than columns of 32).
-// One phase of eight takes them too (d = 4096, radix 8, 16384 rows: 119 -> 111 us).
+// So does one phase of eight (d = 4096, radix 8, 16384 rows: 119 -> 111 us).
 // A slab's first two phases stay with one warp (its box, fragments in registers, no barrier between them).
 #include <algorithm>
 #include <new>
@@ -94,7 +94,7 @@ __device__ __forceinline__ uint32_t local_off(const PipePhase &ph, int r) {
 //   lower8, upper8, upper8One   three teams of eight warps, at most 85 registers; lower8: a warp per box of 64 coordinates in the first two phases
 //                    (upper8One: one phase, columns of 64 bytes)
 //   upper8Wide       one team of sixteen warps, two phases, a warp's two octets of each with their fragments in registers
-//   upper16          sixteen-wide blocks need 128 registers: two teams of eight warps
+//   upper16          one phase of sixteen-wide blocks, 128 registers: two teams of eight warps
 //   dense32, dense48 all upper stages as one block of up to 32 or 48: a warp holds sixteen rows of eight positions, the two
 //                    octets of a tile make a team of two warps; three teams
 enum Kind { kLower8, kUpper8, kUpper8One, kUpper8Wide, kUpper16, kDense32, kDense48 };
@@ -389,7 +389,7 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
                             else box_octet(fb, box, g, q);
                         }
                     }
-                } else if (B16 && ph.B == 16) {
+                } else if constexpr (B16) {
                     uint32_t so[4];
                     bool ok[4];
 #pragma unroll
@@ -578,7 +578,9 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
     PipePlan pl;
     pl.kind = lower ? kLower8 : widest == 8 ? (wide ? kUpper8Wide : np == 1 && S_mid % 32 == 0 ? kUpper8One : kUpper8) : widest == 16 ? kUpper16 : widest == 32 ? kDense32 : kDense48;
     const int ks = pl.kind >= kDense32 ? widest / 16 : 0, Lw = is_wide(pl.kind) ? 32 : 16;
-    if (wide && (pl.kind != kUpper8Wide || np != 2)) return HARP_ERR_UNSUPPORTED;
+    // Tiles of 32 positions read the fragments of two groups of sixteen as they lie in the plan, phases within groups: what the
+    // kernel's item numbers mean for one phase only (kUpper8Wide finds them by group)
+    if (wide ? pl.kind != kUpper8Wide || np != 2 : is_wide(pl.kind) && np != 1) return HARP_ERR_UNSUPPORTED;
     P.n_phases = lower ? np - 1 : np;
     if (lower) {
         if (np < 2 || S_mid > 512 || phs[0].B_real != 8 || phs[1].B_real != 8) return HARP_ERR_UNSUPPORTED;

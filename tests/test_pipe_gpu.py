@@ -17,6 +17,17 @@ pytestmark = pytest.mark.gpu
                                      (16, 16, 43), (16, 16, 47), (8, 8, 8, 19)])
 @pytest.mark.parametrize("n_rows", [8, 9, 16, 17, 31, 33, 65, 131, 2049, 6001])
 def test_matches_the_oracle(radices, n_rows):
+    check_rows(radices, n_rows)
+
+
+@pytest.mark.parametrize("radices", [(8, 8, 8, 9, 2), (8, 8, 8, 10, 3), (8, 8, 8, 13, 2), (16, 16, 9, 2)])
+@pytest.mark.parametrize("n_rows", [16, 17, 700])
+def test_two_upper_phases_with_a_block_wider_than_eight(radices, n_rows):
+    """Tiles of 32 positions read the fragments of two neighbouring groups of sixteen, which lie phase by phase within each group."""
+    check_rows(radices, n_rows)
+
+
+def check_rows(radices, n_rows):
     spec = wl.make_plan(81, int(np.prod(radices)), radices, "qr", perm="identity", signs=True)
     plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
     xh = host_rows(np.random.default_rng(82).standard_normal((n_rows, spec.d)), "bf16")
