@@ -864,9 +864,10 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
     const int n = (int)steps.size(), n_g = std::min(n - 1, 2), ring = std::max(1, n_g);
     const bool permuted = plan->d_perm != nullptr;
     // chunk of rows whose forward states, gradient states and permuted rows fit about 200 MB; the partial sums of a wave of
-    // CTAs come on top
+    // CTAs come on top.  The forward kernels (none where one step is all) take kFwdRows rows per CTA along grid.y.
     const int64_t per_row = std::max<int64_t>(1, d * (4 * (int64_t)(n - 1 + n_g) + (permuted ? (int64_t)sizeof(T) : 0)));
-    const int64_t most = std::max<int64_t>(16, (200ll << 20) / per_row), n_chunks = (n_rows + most - 1) / most;
+    const int64_t fit = std::max<int64_t>(16, (200ll << 20) / per_row), most = n > 1 ? std::min<int64_t>(fit, 65535ll * kFwdRows) : fit;
+    const int64_t n_chunks = (n_rows + most - 1) / most;
     const int64_t chunk = (n_rows + n_chunks - 1) / n_chunks;
     int sms = 148;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device);

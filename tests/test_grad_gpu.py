@@ -67,6 +67,18 @@ def test_rows_spanning_several_slices(radices):
     assert np.array_equal(got, again)                       # fixed summation order
 
 
+@pytest.mark.parametrize("radices", [(4, 2), (2, 2, 2)])
+def test_more_rows_of_a_narrow_plan_than_one_grid_holds(radices):
+    """The forward kernels take 32 rows per CTA along grid.y (at most 65535): 2097120 rows in one launch."""
+    spec = wl.tiny_plan(37, radices, kind="qr", perm="identity", signs=True)
+    plan = harp.plan_from_spec(spec)
+    oplan = orc.OraclePlan.from_spec(spec)
+    xh, gh = _rows(38, 2097120 + 45, spec.d, "bf16")
+    got, _, _ = _gpu_grad(plan, xh, gh, "bf16")
+    want = _flat(orc.grad_blocks(oplan, promote(xh, "bf16"), promote(gh, "bf16")))
+    assert np.max(np.abs(got - want)) <= 2e-5 * np.max(np.abs(want))
+
+
 def test_accumulate_and_row_chunks_add_up():
     spec = wl.tiny_plan(33, (4, 4, 2), kind="qr", perm="random", signs=True)
     plan = harp.plan_from_spec(spec)
