@@ -22,6 +22,7 @@
 #include <new>
 
 #include "harp_internal.h"
+#include "harp_ring.h"
 #include "harp_tm_ptx.cuh"
 
 namespace {
@@ -499,6 +500,9 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
             }
         }
     };
+    [[maybe_unused]] BulkRing ring;
+    auto try_phase = [&](int k, uint32_t phase) { return harp_tm::mbar_try(smem_u32(&full_bar[k]), phase); };
+    auto stopped = [&] { return *(volatile int *)&dead != 0; };
     // ROWS, COLS: one thread, as few bulk copies as cover the tile (each one costs some 200 cycles to issue), completion on the buffer's mbarrier.  RUNS: every thread its chunks.
     auto copy_in = [&](int c, int r, int b) {
         float *tile = smem + b * P.tile_floats;
@@ -509,7 +513,8 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
 #pragma unroll 4
                 for (int q = 4 * lane; q < n_c; q += 128) cp_async16(tile + row * pitch + q, src + (int64_t)row * ld + tabs[q]);
             asm volatile("cp.async.commit_group;" ::: "memory");
-        } else if (threadIdx.x == 0) {
+        } else if (threadIdx.x == 0 && !stopped()) {
+            ring.issued(b);
             const uint32_t bar = smem_u32(&full_bar[b]), dst = smem_u32(tile), box_bytes = 4u * (uint32_t)(n_c / P.n_box * R);
             harp_tm::mbar_expect_tx(bar, box_bytes * (uint32_t)P.n_box);   // past the end of the batch the engine fills zeros
             for (int a = 0; a < P.n_box; ++a) {
@@ -533,7 +538,7 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
                     for (int k = 0; k < 4; ++k)
                         if (q0 + 128 * k < n_c) *reinterpret_cast<float4 *>(dst + (int64_t)row * ld + tabs[q0 + 128 * k]) = v[k];
                 }
-        } else if (threadIdx.x == 0) {
+        } else if (threadIdx.x == 0 && !stopped()) {
             const uint32_t src = smem_u32(tile), box_bytes = 4u * (uint32_t)(n_c / P.n_box * R);
             for (int a = 0; a < P.n_box; ++a) {
                 if constexpr (MODE == ROWS) harp_tm::tma_store_3d(&tmap, 0, r * R, (int)(group_base(c) >> 5) + a * P.box_e, src + a * box_bytes);
@@ -544,7 +549,6 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
     };
 
     int cur_cg = cg, cg_in = cg, rt_in = rt, buf = 0, buf_in = 0;
-    uint32_t parity = 0;                                       // bit b: phase of buffer b's barrier
     if (n_my > 0) load_kernels(cg);
     // plan data only up to here: may run under the kernel before this one
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -566,16 +570,10 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
             asm volatile("cp.async.wait_all;" ::: "memory");
         } else {
             if (fresh) asm volatile("cp.async.wait_all;" ::: "memory");
-            const uint32_t bar = smem_u32(&full_bar[buf]), par = (parity >> buf) & 1u;
-            uint32_t it = 0;
-            while (!harp_tm::mbar_try(bar, par)) {
-                if (++it > kF32Spin || ((it & 63) == 63 && *(volatile int *)&dead)) {
-                    dead = 1;
-                    atomicExch(err, 101);
-                    break;
-                }
+            if (!ring.wait(buf, kF32Spin, try_phase, stopped)) {
+                *(volatile int *)&dead = 1;                    // from here on nothing is copied any more
+                atomicExch(err, 101);
             }
-            parity ^= 1u << buf;
         }
         __syncthreads();
         if (MODE == RUNS && n_buf == 2 && t + 1 < n_my) {      // under the arithmetic of this tile
@@ -620,7 +618,10 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
         }
         buf = buf + 1 == n_buf ? 0 : buf + 1;
     }
-    if (MODE != RUNS && threadIdx.x == 0) harp_tm::bulk_wait0();
+    if (MODE != RUNS && threadIdx.x == 0) {
+        harp_tm::bulk_wait0();
+        ring.drain(n_buf, kF32Spin, try_phase);                // (after a wait that gave up: a late load must not land in the next CTA's memory)
+    }
 }
 
 // Fixed permutation and signs of fp32 rows, in place, whole rows through shared memory.  Forward: row gathered,
