@@ -86,6 +86,7 @@ extern "C" harp_status_t harp_plan_create(harp_plan_t **out, int64_t d, int32_t 
     if (!p) return HARP_ERR_ALLOC;
     p->d = d;
     p->opt_no_rowvec = getenv("HARP_NO_ROWVEC") != nullptr;
+    p->opt_no_maps = getenv("HARP_NO_TENSOR_MAPS") != nullptr;
     p->st.m = n_stages;
     int64_t s = 1, off = 0;
     for (int t = 0; t < n_stages; ++t) {

@@ -366,6 +366,7 @@ struct ColPlan {
     size_t pipe_smem[2] = {0, 0};
     int64_t S_mid = 1, U = 1;
     int32_t *d_err = nullptr;
+    void *encode = nullptr;    // null: no tensor maps
     int n_pass = 0;
     std::vector<void *> dev_allocs;
     int sms = 148;
@@ -585,7 +586,7 @@ harp_status_t launch_col_pipe(const ColPlan *cp, int which, void *W, int64_t n_c
     // a position group per CTA keeps its fragments; where that leaves more than a tenth of the SMs without work, equal shares
     P.n_parts = (int32_t)std::min<int64_t>(P.n_tiles, std::max<int64_t>(1, cp->sms / P.n_cg));
     if (P.n_cg > cp->sms || cp->sms % P.n_cg * 10 > cp->sms) P.n_parts = 0;
-    const auto enc = reinterpret_cast<EncodeTiled>(harp_tensor_map_encoder());
+    const auto enc = reinterpret_cast<EncodeTiled>(cp->encode);
     CUtensorMap tmap = {};
     const cuuint32_t ones[3] = {1, 1, 1};
     // slab: (column, position); upper: (column, place, position below the slab's size)
@@ -644,7 +645,8 @@ harp_status_t harp_col_build(harp_plan *plan) {
     }
     cp->S_mid = S_mid;
     cp->U = U;
-    if (st == HARP_OK && harp_tensor_map_encoder()) {
+    cp->encode = harp_tensor_map_encoder(plan);
+    if (st == HARP_OK && cp->encode) {
         cp->d_err = upload_c(cp, std::vector<int32_t>(1, 0), st);
         for (int s = 0; s < cp->n_pass && st == HARP_OK; ++s) st = build_col_pipe(cp, s, s == 0 ? lower : upper, s == 0, S_mid, U);
         if (st == HARP_OK && cudaFuncSetAttribute(harp_col_pipe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kColPipeSmem) != cudaSuccess)

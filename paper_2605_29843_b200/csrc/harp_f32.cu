@@ -667,9 +667,12 @@ struct F32Plan {
     int permute_rows = 0;              // rows per tile of the permutation kernel (0: identity)
     int sms = 148;
     int32_t *d_err = nullptr;          // device word, set when a wait gave up
+    void *encode = nullptr;            // encoder of tensor maps
 };
 
 namespace {
+
+constexpr int64_t kMaxF32Vectors = (int64_t)1 << 30;      // rows or columns of a call: coordinates of a bulk copy are 32-bit
 
 const StageTable &f32_table(const harp_plan *p) { return p->fused.m > 0 && p->d_fused_blocks ? p->fused : p->st; }
 const float *f32_blocks(const harp_plan *p) { return p->fused.m > 0 && p->d_fused_blocks ? p->d_fused_blocks : p->d_blocks; }
@@ -783,14 +786,12 @@ cudaError_t launch_f32(const F32Plan *fp, const F32Pass &P, float *x, int64_t n,
     const cudaError_t ae = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (ae != cudaSuccess) return ae;
     const int64_t n_row_tiles = (n + 32 * RT - 1) / (32 * RT);
-    if (n_row_tiles > 0x7fffffff) return cudaErrorInvalidValue;
     const int64_t n_tiles = n_row_tiles * P.n_cg;
     // row-mode runs below a 128-byte line: see the kernel's tile order (it keeps parts * n_cg of the SMs busy)
     const int n_parts = MODE == RUNS && P.L < 32 && P.n_cg <= fp->sms ? (int)std::min<int64_t>(n_row_tiles, fp->sms / P.n_cg) : 0;
     CUtensorMap tmap = {};
     if (MODE != RUNS) {
-        const auto enc = reinterpret_cast<EncodeTiled>(harp_tensor_map_encoder());
-        if (!enc || n > ((int64_t)1 << 30)) return cudaErrorNotSupported;
+        const auto enc = reinterpret_cast<EncodeTiled>(fp->encode);
         const cuuint32_t ones[3] = {1, 1, 1};
         CUresult r;
         if (MODE == ROWS) {
@@ -879,12 +880,13 @@ harp_status_t permute_rows(const harp_plan *plan, float *x, int64_t n, int trans
 harp_status_t harp_f32_build(harp_plan *plan) {
     const StageTable &st = f32_table(plan);
     const int64_t d = plan->d;
-    if (d > 32768) return HARP_ERR_UNSUPPORTED;
+    if (d > 32768 || !harp_tensor_map_encoder(plan)) return HARP_ERR_UNSUPPORTED;
     for (int t = 0; t < st.m; ++t)
         if (st.b[t] > kMaxF32Radix) return HARP_ERR_UNSUPPORTED;
     F32Plan *fp = new (std::nothrow) F32Plan();
     if (!fp) return HARP_ERR_ALLOC;
     plan->f32 = fp;
+    fp->encode = harp_tensor_map_encoder(plan);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -912,7 +914,7 @@ int32_t harp_f32_error_word(const harp_plan *plan) {
 
 harp_status_t harp_f32_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose, cudaStream_t stream) {
     const F32Plan *fp = plan->f32;
-    if (!fp || dtype != HARP_F32 || fp->n_pass[0] == 0 || (reinterpret_cast<uintptr_t>(x) & 15u) != 0) return HARP_ERR_UNSUPPORTED;
+    if (!fp || dtype != HARP_F32 || fp->n_pass[0] == 0 || n_rows > kMaxF32Vectors || (reinterpret_cast<uintptr_t>(x) & 15u) != 0) return HARP_ERR_UNSUPPORTED;
     float *xf = static_cast<float *>(x);
     harp_status_t rc = HARP_OK;
     if (fp->permute_rows && !transpose) rc = permute_rows(plan, xf, n_rows, 0, stream);
@@ -924,7 +926,7 @@ harp_status_t harp_f32_apply(const harp_plan *plan, void *x, int64_t n_rows, har
 // Forward apply down the columns of W (dim(plan) x n_cols, row-major, leading dimension ld).
 harp_status_t harp_f32_col_apply(const harp_plan *plan, void *W, int64_t n_cols, int64_t ld, harp_dtype_t dtype, cudaStream_t stream) {
     const F32Plan *fp = plan->f32;
-    if (!fp || dtype != HARP_F32 || fp->n_pass[1] == 0) return HARP_ERR_UNSUPPORTED;
+    if (!fp || dtype != HARP_F32 || fp->n_pass[1] == 0 || n_cols > kMaxF32Vectors) return HARP_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(W) & 15u) != 0 || n_cols % 4 != 0 || ld % 4 != 0) return HARP_ERR_UNSUPPORTED;
     return run_passes<true>(plan, static_cast<float *>(W), n_cols, ld, 0, stream);
 }

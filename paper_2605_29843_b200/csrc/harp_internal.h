@@ -52,9 +52,9 @@ struct harp_plan {
     ColPlan *col = nullptr;
     TmPlan *tm = nullptr;
     F32Plan *f32 = nullptr;
-    // test-only switch, read from the environment once, when the plan is built (HARP_NO_ROWVEC=1: the
-    // CUDA-core kernels keep their tile row-major)
-    bool opt_no_rowvec = false;
+    // test-only switches, read from the environment once, when the plan is built (HARP_NO_ROWVEC=1: the
+    // CUDA-core kernels keep their tile row-major; HARP_NO_TENSOR_MAPS=1: as on a driver that cannot encode tensor maps)
+    bool opt_no_rowvec = false, opt_no_maps = false;
     // staging owned by harp_apply_host
     static constexpr int kStages = 4;
     void *stage_buf[kStages] = {nullptr, nullptr, nullptr, nullptr};
@@ -91,8 +91,8 @@ harp_status_t harp_tm_build(harp_plan *plan);
 void harp_tm_destroy(harp_plan *plan);
 harp_status_t harp_tm_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype,
                             int transpose, cudaStream_t stream);
-// cuTensorMapEncodeTiled of the driver (null if it has none)
-void *harp_tensor_map_encoder();
+// cuTensorMapEncodeTiled of the driver (null if it has none, or for a plan built without: HARP_NO_TENSOR_MAPS)
+void *harp_tensor_map_encoder(const harp_plan *plan);
 int32_t harp_tm_error_word(const harp_plan *plan);
 // the stages below stride 256 alone (lower pass of the two-pass paths); 0 stages = not available
 int harp_tm_slab_stages(const harp_plan *plan);

@@ -533,6 +533,7 @@ struct PipePlan {
     size_t smem = 0;
     int sms = 148;
     int32_t *d_err = nullptr;
+    EncodeTiled encode = nullptr;
     std::vector<void *> dev_allocs;
 };
 
@@ -567,7 +568,7 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
                               PipePlan **out) {
     *out = nullptr;
     const int np = (int)phs.size(), pair = lower ? 2 : 0;     // lower: the first two phases count as one
-    if (np < 1 || np > kMaxPipePhases || !harp_tensor_map_encoder()) return HARP_ERR_UNSUPPORTED;
+    if (np < 1 || np > kMaxPipePhases || !harp_tensor_map_encoder(plan)) return HARP_ERR_UNSUPPORTED;
     int widest = 8;
     for (const GPhase &gp : phs) widest = std::max(widest, gp.B);
     PipePass P{};
@@ -622,6 +623,7 @@ harp_status_t harp_pipe_build(const harp_plan *plan, const std::vector<GPhase> &
         if (P.MT == 1) return HARP_ERR_UNSUPPORTED;
     }
     pl.d = plan->d;
+    pl.encode = reinterpret_cast<EncodeTiled>(harp_tensor_map_encoder(plan));
     pl.S_mid = S_mid;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -718,7 +720,7 @@ harp_status_t harp_pipe_apply(const PipePlan *pp, void *x, int64_t n_rows, int t
     P.n_parts = (int32_t)std::min<int64_t>(P.n_tiles, std::max<int64_t>(1, slots / P.n_cg));
     if (pp->kind == kLower8 && (P.n_cg > slots || slots % P.n_cg * 10 > slots)) P.n_parts = 0;
     const unsigned grid = (unsigned)(P.n_parts > 0 ? (int64_t)P.n_parts * P.n_cg : std::min<int64_t>((int64_t)P.n_tiles * P.n_cg, slots));
-    const auto enc = reinterpret_cast<EncodeTiled>(harp_tensor_map_encoder());
+    const EncodeTiled enc = pp->encode;
     CUtensorMap tmap = {};
     const cuuint32_t ones[4] = {1, 1, 1, 1};
     const cuuint64_t n = (cuuint64_t)n_rows, pitch = (cuuint64_t)pp->d * 2;

@@ -614,7 +614,7 @@ void harp_tm_destroy(harp_plan *plan) {
 harp_status_t harp_tm_build(harp_plan *plan) {
     const int64_t d = plan->d;
     if (d % 256 != 0) return HARP_ERR_UNSUPPORTED;
-    if (!encode_fn()) return HARP_ERR_UNSUPPORTED;
+    if (!harp_tensor_map_encoder(plan)) return HARP_ERR_UNSUPPORTED;
     const bool whole = d == 256 || d == 4096;        // the whole processor as passes of this path
     const int n_dig = d == 256 ? 2 : 3;
     // group the stages into phases whose radices multiply to 16 (all of them, or the two below stride 256)
@@ -742,7 +742,7 @@ namespace {
 
 }  // namespace
 
-void *harp_tensor_map_encoder() { return reinterpret_cast<void *>(encode_fn()); }
+void *harp_tensor_map_encoder(const harp_plan *plan) { return plan->opt_no_maps ? nullptr : reinterpret_cast<void *>(encode_fn()); }
 
 namespace {
 

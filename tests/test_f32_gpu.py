@@ -50,3 +50,25 @@ def test_two_sided_fp32(r_out, r_in):
     scale = np.minimum(np.linalg.norm(want, axis=1, keepdims=True), np.linalg.norm(want, axis=0, keepdims=True))
     assert np.max(err / scale) <= 2 * TOL["f32"]
     assert harp.harp_plan_error_word(plan_out) == 0
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_a_driver_without_tensor_maps(monkeypatch, dtype):
+    """Plans whose passes cannot be fed by bulk copies keep the kernels that need none: rows, permuted rows and both sides of a matrix."""
+    monkeypatch.setenv("HARP_NO_TENSOR_MAPS", "1")
+    for radices, perm in (((16, 16, 8), "random"), ((8, 8, 8, 8, 2), "identity"), ((16, 16, 43), "identity")):
+        spec = wl.tiny_plan(66, radices, kind="qr", perm=perm, signs=True)
+        plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
+        xh = host_rows(np.random.default_rng(67).standard_normal((70, spec.d)), dtype)
+        for tr, fn in ((False, orc.forward), (True, orc.transpose)):
+            got, guards = gpu_apply(plan, xh, dtype, tr)
+            assert guards and orc.rel_err_rows(got, fn(oplan, promote(xh, dtype))) <= TOL[dtype]
+    p_out = wl.tiny_plan(68, (8, 8, 8), kind="qr", perm="identity", signs=True)
+    p_in = wl.tiny_plan(69, (8, 8), kind="qr", perm="identity", signs=True)
+    wh = host_rows(np.random.default_rng(70).standard_normal((p_out.d, p_in.d)), dtype)
+    wd = to_device(wh, dtype)
+    harp.two_sided_(wd, harp.plan_from_spec(p_out), harp.plan_from_spec(p_in))
+    torch.cuda.synchronize()
+    want = orc.two_sided(orc.OraclePlan.from_spec(p_out), orc.OraclePlan.from_spec(p_in), promote(wh, dtype))
+    scale = np.minimum(np.linalg.norm(want, axis=1, keepdims=True), np.linalg.norm(want, axis=0, keepdims=True))
+    assert np.max(np.abs(to_host_f64(wd) - want) / scale) <= 2 * TOL[dtype]
