@@ -379,13 +379,13 @@ _current_device = _raw_stream = _apply_ex = None
 def _bind_torch() -> None:
     global _current_device, _raw_stream, _apply_ex
     import torch
-    _dtype_codes.update({torch.float32: HARP_F32, torch.bfloat16: HARP_BF16})
-    _apply_ex = lib().harp_apply_ex
     torch.cuda.init()
+    _dtype_codes.update({torch.float32: HARP_F32, torch.bfloat16: HARP_BF16})
     if hasattr(torch._C, "_cuda_getCurrentRawStream"):
         _current_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
     else:
         _current_device, _raw_stream = torch.cuda.current_device, lambda dev: torch.cuda.current_stream(dev).cuda_stream
+    _apply_ex = lib().harp_apply_ex        # last: what the callers test, also those on other threads
 
 
 def _torch_dtype_code(t) -> int:
