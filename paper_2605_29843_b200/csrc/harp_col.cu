@@ -234,12 +234,9 @@ harp_col_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, con
     }
     __syncthreads();
 
-    BulkRing ring;
-    auto try_phase = [&](int k, uint32_t phase) { return harp_tm::mbar_try(smem_u32(&full_bar[k]), phase); };
     // columns past the last arrive as zeros and are not written
     auto load = [&](int cg, int tile, int b) {
         const uint32_t bar = smem_u32(&full_bar[b]), dst = bufs + (uint32_t)(b * P.tile_bytes);
-        ring.issued(b);
         harp_tm::mbar_expect_tx(bar, (uint32_t)(P.n_box * P.box_rows * 128));
         if (P.Lr) harp_tm::tma_load_3d(dst, &tmap, 64 * tile, 0, cg * P.Lr, bar);
         else
@@ -258,6 +255,7 @@ harp_col_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, con
         at = blockIdx.x * per + min((int64_t)blockIdx.x, extra);
         end = at + per + ((int64_t)blockIdx.x < extra ? 1 : 0);
     }
+    uint32_t parity = 0;
     bool waited = false;
     while (at < end) {
         int cg, first, step, count;
@@ -288,11 +286,18 @@ harp_col_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, con
         __syncthreads();
         int b = 0;
         for (int t = 0; t < count; ++t, b = b + 1 == NB ? 0 : b + 1) {
-            const uint32_t sbase = bufs + (uint32_t)(b * P.tile_bytes);
-            if (!ring.wait(b, kColSpin, try_phase, [&] { return *(volatile int *)&dead != 0; })) {
-                *(volatile int *)&dead = 1;           // from here on nothing is copied any more
-                atomicExch(err, 302);
+            const uint32_t bar = smem_u32(&full_bar[b]), sbase = bufs + (uint32_t)(b * P.tile_bytes);
+            uint32_t it = 0;
+            bool got = true;
+            while (!harp_tm::mbar_try(bar, (parity >> b) & 1u)) {
+                if (++it > kColSpin || ((it & 63) == 63 && *(volatile int *)&dead)) {
+                    *(volatile int *)&dead = 1;       // from here on nothing is copied any more
+                    atomicExch(err, 302);
+                    got = false;
+                    break;
+                }
             }
+            if (got) parity ^= 1u << b;
             for (int p = 0; p < P.n_phases; ++p) {
                 const ColPhase &ph = P.ph[p];
                 if (p > 0) __syncthreads();
@@ -353,7 +358,7 @@ harp_col_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, con
     }
     if (tid == 0) {
         harp_tm::bulk_wait0();
-        ring.drain(NB, kColSpin, try_phase);        // (after a wait that gave up: a late load must not land in the next CTA's memory)
+        if (*(volatile int *)&dead) ring_drain(parity, NB, kColSpin, [&](int k, uint32_t phase) { return harp_tm::mbar_try(smem_u32(&full_bar[k]), phase); });
     }
 }
 

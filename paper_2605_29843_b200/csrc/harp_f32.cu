@@ -500,8 +500,6 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
             }
         }
     };
-    [[maybe_unused]] BulkRing ring;
-    auto try_phase = [&](int k, uint32_t phase) { return harp_tm::mbar_try(smem_u32(&full_bar[k]), phase); };
     auto stopped = [&] { return *(volatile int *)&dead != 0; };
     // ROWS, COLS: one thread, as few bulk copies as cover the tile (each one costs some 200 cycles to issue), completion on the buffer's mbarrier.  RUNS: every thread its chunks.
     auto copy_in = [&](int c, int r, int b) {
@@ -514,7 +512,6 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
                 for (int q = 4 * lane; q < n_c; q += 128) cp_async16(tile + row * pitch + q, src + (int64_t)row * ld + tabs[q]);
             asm volatile("cp.async.commit_group;" ::: "memory");
         } else if (threadIdx.x == 0 && !stopped()) {
-            ring.issued(b);
             const uint32_t bar = smem_u32(&full_bar[b]), dst = smem_u32(tile), box_bytes = 4u * (uint32_t)(n_c / P.n_box * R);
             harp_tm::mbar_expect_tx(bar, box_bytes * (uint32_t)P.n_box);   // past the end of the batch the engine fills zeros
             for (int a = 0; a < P.n_box; ++a) {
@@ -549,6 +546,7 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
     };
 
     int cur_cg = cg, cg_in = cg, rt_in = rt, buf = 0, buf_in = 0;
+    [[maybe_unused]] uint32_t parity = 0;                      // bit b: phase of buffer b's barrier
     if (n_my > 0) load_kernels(cg);
     // plan data only up to here: may run under the kernel before this one
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -570,10 +568,18 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
             asm volatile("cp.async.wait_all;" ::: "memory");
         } else {
             if (fresh) asm volatile("cp.async.wait_all;" ::: "memory");
-            if (!ring.wait(buf, kF32Spin, try_phase, stopped)) {
-                *(volatile int *)&dead = 1;                    // from here on nothing is copied any more
-                atomicExch(err, 101);
+            const uint32_t bar = smem_u32(&full_bar[buf]), par = (parity >> buf) & 1u;
+            uint32_t it = 0;
+            bool got = true;
+            while (!harp_tm::mbar_try(bar, par)) {
+                if (++it > kF32Spin || ((it & 63) == 63 && stopped())) {
+                    *(volatile int *)&dead = 1;                // from here on nothing is copied any more
+                    atomicExch(err, 101);
+                    got = false;
+                    break;
+                }
             }
+            if (got) parity ^= 1u << buf;
         }
         __syncthreads();
         if (MODE == RUNS && n_buf == 2 && t + 1 < n_my) {      // under the arithmetic of this tile
@@ -620,7 +626,7 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
     }
     if (MODE != RUNS && threadIdx.x == 0) {
         harp_tm::bulk_wait0();
-        ring.drain(n_buf, kF32Spin, try_phase);                // (after a wait that gave up: a late load must not land in the next CTA's memory)
+        if (stopped()) ring_drain(parity, n_buf, kF32Spin, [&](int k, uint32_t phase) { return harp_tm::mbar_try(smem_u32(&full_bar[k]), phase); });
     }
 }
 

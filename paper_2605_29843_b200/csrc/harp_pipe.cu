@@ -236,12 +236,9 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
     const uint32_t row8_off = LOWER ? 1024u : 4u * (uint32_t)P.row_bytes;
     const uint32_t mt_step = LOWER ? 2048u : 8u * (uint32_t)P.row_bytes;
 
-    BulkRing ring;
-    auto try_phase = [&](int k, uint32_t phase) { return mbar_try(smem_u32(&full_bar[team * kMaxPipeBufs + k]), phase); };
     // Rows past the end of the batch arrive as zeros and are not written.
     auto load = [&](int cg, int tile, int b) {
         const uint32_t bar = smem_u32(&full_bar[team * kMaxPipeBufs + b]), dst = bufs + (uint32_t)(b * P.tile_bytes);
-        ring.issued(b);
         mbar_expect_tx(bar, (uint32_t)(P.n_box * P.box_bytes));
         for (int k = 0; k < P.n_box; ++k) {
             if constexpr (LOWER) harp_tm::tma_load_2d(dst + (uint32_t)(k * P.box_pitch), &tmap, 64 * (cg * P.n_box + k), tile * 16 * P.MT, bar);
@@ -265,6 +262,7 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
         at = blockIdx.x * per + min((int64_t)blockIdx.x, extra);
         end = at + per + ((int64_t)blockIdx.x < extra ? 1 : 0);
     }
+    uint32_t parity = 0;
     bool waited = false;
     while (at < end) {
         int cg, first, step, count;
@@ -320,11 +318,18 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
         __syncthreads();
         int b = 0;
         for (int t = team; t < count; t += TEAMS, b = b + 1 == NB ? 0 : b + 1) {
-            const uint32_t sbase = bufs + (uint32_t)(b * P.tile_bytes);
-            if (!ring.wait(b, kPipeSpin, try_phase, [&] { return *(volatile int *)&dead != 0; })) {
-                *(volatile int *)&dead = 1;           // from here on nothing is copied any more
-                atomicExch(err, 301);
+            const uint32_t bar = smem_u32(&full_bar[team * kMaxPipeBufs + b]), sbase = bufs + (uint32_t)(b * P.tile_bytes);
+            uint32_t it = 0;
+            bool got = true;
+            while (!mbar_try(bar, (parity >> b) & 1u)) {
+                if (++it > kPipeSpin || ((it & 63) == 63 && *(volatile int *)&dead)) {
+                    *(volatile int *)&dead = 1;       // from here on nothing is copied any more
+                    atomicExch(err, 301);
+                    got = false;
+                    break;
+                }
             }
+            if (got) parity ^= 1u << b;
             // the store of the tile before has had a phase's time to be read: refill its buffer
             auto refill = [&]() {
                 if (tid == 0 && t > team && t + (NB - 1) * TEAMS < count && !*(volatile int *)&dead) {
@@ -465,7 +470,8 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
     }
     if (tid == 0) {
         harp_tm::bulk_wait0();
-        ring.drain(NB, kPipeSpin, try_phase);        // (after a wait that gave up: a late load must not land in the next CTA's memory)
+        if (*(volatile int *)&dead)
+            ring_drain(parity, NB, kPipeSpin, [&](int k, uint32_t phase) { return mbar_try(smem_u32(&full_bar[team * kMaxPipeBufs + k]), phase); });
     }
 }
 
