@@ -531,6 +531,7 @@ struct SplitPlan {
     int gather_rows = 1;       // rows per buffer of the gather kernel
     size_t gather_smem = 0;
     PipePlan *pipe[3] = {nullptr, nullptr, nullptr};   // the passes fed by the copy engine (harp_pipe.cu), where the shape allows them; [2] upper, large batches
+    int64_t pipe_min_rows[3] = {0, 0, 0};              // smallest batches that take them
     // dense upper pass (replaces pass[1] when set)
     bool dense_upper = false;
     UpperPass up_fwd{}, up_bwd{};
@@ -841,6 +842,14 @@ harp_status_t harp_split_build(harp_plan *plan) {
         if (st == HARP_ERR_UNSUPPORTED) st = HARP_OK;
     }
     if (st == HARP_OK && want_dense && !sp->pipe[1]) st = build_dense_upper(plan, sp, lower.back().t1, S_mid, U);
+    for (int s = 0; s < 3; ++s)
+        if (sp->pipe[s]) sp->pipe_min_rows[s] = harp_pipe_min_rows(sp->pipe[s]);
+    // A slab pass fed by the copy engine fills the SMs' shared memory, so that the mma.sync upper pass behind it cannot fetch its
+    // fragments under it; with eight-wide upper blocks that costs a small batch more than the faster copies give (slabs of 512:
+    // 32 rows 11.9 us without, 15.2 with, 96 rows 20.6 and 20.4, 112 rows 20.6 and 17.9; of 384: 64 rows 13.3 and 16.3, 112 rows
+    // 20.6 and 17.6; of 256: 160 rows 20.6 and 22.1, 200 rows 20.6 and 19.0)
+    if (sp->pipe[0] && !sp->pipe[1] && sp->pass[1].present && !sp->pass[1].has16)
+        sp->pipe_min_rows[0] = std::max(sp->pipe_min_rows[0], 43008 / S_mid);
     if (st == HARP_OK &&
         (cudaFuncSetAttribute(harp_split_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024) != cudaSuccess ||
          cudaFuncSetAttribute(harp_split_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024) != cudaSuccess ||
@@ -974,8 +983,8 @@ harp_status_t harp_split_apply(const harp_plan *plan, void *x, int64_t n_rows, h
                 if (ts == HARP_OK) continue;
                 if (ts != HARP_ERR_UNSUPPORTED) return ts;
             }
-            if (sp->pipe[pi] && r1 - r0 >= harp_pipe_min_rows(sp->pipe[pi])) {
-                const bool wide = pi == 1 && sp->pipe[2] && r1 - r0 >= harp_pipe_min_rows(sp->pipe[2]);
+            if (sp->pipe[pi] && r1 - r0 >= sp->pipe_min_rows[pi]) {
+                const bool wide = pi == 1 && sp->pipe[2] && r1 - r0 >= sp->pipe_min_rows[2];
                 const harp_status_t ps = harp_pipe_apply(wide ? sp->pipe[2] : sp->pipe[pi], xb + r0 * plan->d, r1 - r0, transpose, overlap, stream);
                 if (ps != HARP_OK) return ps;
                 continue;

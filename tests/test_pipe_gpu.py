@@ -27,6 +27,11 @@ def test_two_upper_phases_with_a_block_wider_than_eight(radices, n_rows):
     check_rows(radices, n_rows)
 
 
+@pytest.mark.parametrize("radices,n_rows", [((8, 8, 8, 8, 8), 83), ((8, 8, 8, 8, 8), 84), ((8, 8, 6, 8, 8), 111), ((8, 8, 6, 8, 8), 112), ((8, 8, 4, 8, 8), 168)])
+def test_slab_pass_in_front_of_an_upper_pass_of_even_radices(radices, n_rows):
+    check_rows(radices, n_rows)
+
+
 def check_rows(radices, n_rows):
     spec = wl.make_plan(81, int(np.prod(radices)), radices, "qr", perm="identity", signs=True)
     plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
