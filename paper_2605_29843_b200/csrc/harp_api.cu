@@ -87,6 +87,7 @@ extern "C" harp_status_t harp_plan_create(harp_plan_t **out, int64_t d, int32_t 
     p->d = d;
     p->opt_no_rowvec = getenv("HARP_NO_ROWVEC") != nullptr;
     p->opt_no_maps = getenv("HARP_NO_TENSOR_MAPS") != nullptr;
+    p->opt_f32_passes = getenv("HARP_F32_PASSES") != nullptr;
     p->st.m = n_stages;
     int64_t s = 1, off = 0;
     for (int t = 0; t < n_stages; ++t) {
@@ -239,7 +240,8 @@ extern "C" harp_status_t harp_apply_ex(const harp_plan_t *plan, void *x, int64_t
     if (st != HARP_ERR_UNSUPPORTED) return st;
     // fp32 rows: up to d = 4096 the whole-row CUDA-core kernels of radices up to 8 hold enough rows of a tile to be the faster
     // ones (4096 rows of d = 4096, radix 8: 100 us against 128); beyond, and for larger radices, passes over column groups
-    if (dtype == HARP_F32 && (plan->d > 4096 || harp_generic_max_radix(plan) > 8)) {
+    // where the batch makes up for their two or three launches and the block kernels that each CTA fetches
+    if (dtype == HARP_F32 && (plan->d > 4096 || harp_generic_max_radix(plan) > 8) && harp_f32_preferred(plan, n_rows)) {
         st = harp_f32_apply(plan, x, n_rows, dtype, transpose, s);
         if (st != HARP_ERR_UNSUPPORTED) return st;
     }

@@ -785,6 +785,11 @@ typedef CUresult (*EncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, 
                                 const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// row-mode runs below a 128-byte line: see the kernel's tile order (it keeps parts * n_cg of the SMs busy)
+int pass_parts(const F32Plan *fp, const F32Pass &P, int64_t n_row_tiles) {
+    return P.mode == RUNS && P.L < 32 && P.n_cg <= fp->sms ? (int)std::min<int64_t>(n_row_tiles, fp->sms / P.n_cg) : 0;
+}
+
 template <int RT, int MODE, bool BIG>
 cudaError_t launch_f32(const F32Plan *fp, const F32Pass &P, float *x, int64_t n, int64_t ld, const float *blocks, const int8_t *signs,
                        int transpose, int sign_at, cudaStream_t stream) {
@@ -793,8 +798,7 @@ cudaError_t launch_f32(const F32Plan *fp, const F32Pass &P, float *x, int64_t n,
     if (ae != cudaSuccess) return ae;
     const int64_t n_row_tiles = (n + 32 * RT - 1) / (32 * RT);
     const int64_t n_tiles = n_row_tiles * P.n_cg;
-    // row-mode runs below a 128-byte line: see the kernel's tile order (it keeps parts * n_cg of the SMs busy)
-    const int n_parts = MODE == RUNS && P.L < 32 && P.n_cg <= fp->sms ? (int)std::min<int64_t>(n_row_tiles, fp->sms / P.n_cg) : 0;
+    const int n_parts = pass_parts(fp, P, n_row_tiles);
     CUtensorMap tmap = {};
     if (MODE != RUNS) {
         const auto enc = reinterpret_cast<EncodeTiled>(fp->encode);
@@ -916,6 +920,32 @@ int32_t harp_f32_error_word(const harp_plan *plan) {
     if (!plan->f32 || !plan->f32->d_err) return 0;
     int32_t v = 0;
     return cudaMemcpy(&v, plan->f32->d_err, sizeof(v), cudaMemcpyDeviceToHost) == cudaSuccess ? v : -1;
+}
+
+// The passes cost two or three launches, the block kernels of a column group in every CTA, and tiles of 32 rows; the whole-row kernels
+// a wave of CTAs, whatever the batch leaves of it idle.  Radices (16, 16, 4), whole rows against passes: 128 rows 14 us and 25,
+// 256 rows 25 and 25, 512 rows 45 and 28; (16, 16), one pass: 128 rows 6 and 13, 4096 rows 62 and 13; d = 8192 in radix 8 (four rows
+// a CTA, waves of 592): 128 rows 40 and 25, 512 rows 41 and 50, 768 rows 78 and 63; with a random permutation 59 and 39, 61 and 68, 116 and 83.
+bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows) {
+    const F32Plan *fp = plan->f32;
+    if (!fp || fp->n_pass[0] == 0) return false;
+    if (plan->opt_f32_passes || harp_generic_supported(plan, HARP_F32) != HARP_OK) return true;
+    const double elems = (double)n_rows * (double)plan->d;
+    double us = 0.0;
+    for (int p = 0; p < fp->n_pass[0]; ++p) {
+        const F32Pass &P = fp->pass[0][p];
+        const int64_t tiles = (n_rows + 32 * P.RT - 1) / (32 * P.RT), n_c = (int64_t)P.E * P.L;
+        const int64_t n_parts = pass_parts(fp, P, tiles), per = n_parts > 0 ? (tiles + n_parts - 1) / n_parts : (tiles * P.n_cg + fp->sms - 1) / fp->sms;
+        const int64_t groups = n_parts > 0 ? 1 : 1 + (per - 1) / tiles;      // whose block kernels a CTA fetches
+        double radices = 0.0;
+        for (int k = 0; k < P.n_ph; ++k) radices += P.ph[k].b;
+        us += 5.1 + 3.3e-4 * (double)(P.w_floats * groups) + 4.06e-4 * (double)(per * n_c * P.RT) * radices + 2.6e-6 * elems;
+    }
+    if (fp->permute_rows) {
+        const int64_t waves = ((n_rows + fp->permute_rows - 1) / fp->permute_rows + fp->sms - 1) / fp->sms;
+        us += 5.6 + 2.1e-4 * (double)(waves * std::min<int64_t>(fp->permute_rows, n_rows) * plan->d);
+    }
+    return us < harp_generic_estimate(plan, n_rows, fp->sms);
 }
 
 harp_status_t harp_f32_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose, cudaStream_t stream) {

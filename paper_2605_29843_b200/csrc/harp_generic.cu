@@ -261,6 +261,14 @@ harp_blockowner_kernel(T *__restrict__ x, int64_t n_rows, int d, int rows_per_ct
     }
 }
 
+// rows per CTA of the block-owner kernel: what shared memory holds, one wave when the batch allows it
+int64_t blockowner_rows(int64_t d, int64_t n_rows, int sms) {
+    int64_t r = (227 * 1024 - 1024) / (d * (int64_t)sizeof(float));
+    if (r < 1) r = (227 * 1024) / (d * (int64_t)sizeof(float));
+    r = std::min<int64_t>(r, (n_rows + sms - 1) / sms);
+    return std::max<int64_t>(1, std::min<int64_t>(r, 64));
+}
+
 template <typename T, int NT, bool BIG, bool SWZ>
 harp_status_t launch_blockowner_swz(const harp_plan *plan, const StageTable &st, const float *blocks, void *x, int64_t n_rows,
                                     int transpose, cudaStream_t stream) {
@@ -271,11 +279,7 @@ harp_status_t launch_blockowner_swz(const harp_plan *plan, const StageTable &st,
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t d = plan->d;
-    const int per_sm = 1;                                               // CTAs per SM (see __launch_bounds__)
-    int64_t r = ((227 * 1024) / per_sm - 1024) / (d * (int64_t)sizeof(float));   // what shared memory holds
-    if (r < 1) r = (227 * 1024) / (d * (int64_t)sizeof(float));
-    r = std::min<int64_t>(r, (n_rows + (int64_t)sms * per_sm - 1) / ((int64_t)sms * per_sm));   // one wave when the batch allows it
-    r = std::max<int64_t>(1, std::min<int64_t>(r, 64));
+    const int64_t r = blockowner_rows(d, n_rows, sms);
     const int64_t grid = (n_rows + r - 1) / r;
     if (grid > 0x7fffffffLL) return HARP_ERR_BAD_DIM;
     kern<<<(unsigned)grid, NT, (size_t)r * d * sizeof(float), stream>>>((T *)x, n_rows, (int)d, (int)r, st,
@@ -617,6 +621,19 @@ harp_rowvec_kernel(T *__restrict__ x, int64_t n_rows, int d, int rows_per_cta, i
     }
 }
 
+// Groups of four rows per CTA: the size for which waves of CTAs times a CTA's time -- its rows and about one group's worth for the
+// block kernels it fetches -- is least (2048 rows of d = 4096: 171 CTAs of 12 rows 108 us, 256 of 8 rows 80; 10000 rows of
+// d = 2048, 28 rows 67 us, 24 rows 61)
+struct RowvecGroups { int64_t g, cost; };
+RowvecGroups rowvec_groups(int64_t n_rows, int64_t g_max, int64_t slots) {
+    RowvecGroups best{1, INT64_MAX};
+    for (int64_t c = std::min<int64_t>(g_max, 15); c >= 1; --c) {
+        const int64_t ctas = (n_rows + 4 * c - 1) / (4 * c), cost = (ctas + slots - 1) / slots * (c + 1);
+        if (cost < best.cost) best = {c, cost};
+    }
+    return best;
+}
+
 template <typename T, int NT, bool BIG, int MINB = 1>
 harp_status_t launch_rowvec(const harp_plan *plan, const StageTable &st, const float *blocks, void *x, int64_t n_rows,
                             int transpose, cudaStream_t stream) {
@@ -632,14 +649,7 @@ harp_status_t launch_rowvec(const harp_plan *plan, const StageTable &st, const f
     int64_t g_max = (226 * 1024 / MINB) / (d * 16);
     if (g_max % 2 == 0) --g_max;
     if (g_max < 1) return HARP_ERR_UNSUPPORTED;
-    // the size for which waves of CTAs times a CTA's time -- its rows and about one group's worth for the block kernels it
-    // fetches -- is least (2048 rows of d = 4096: 171 CTAs of 12 rows 108 us, 256 of 8 rows 80; 10000 rows of d = 2048,
-    // 28 rows 67 us, 24 rows 61)
-    int64_t g = 1, best = INT64_MAX;
-    for (int64_t c = std::min<int64_t>(g_max, 15); c >= 1; --c) {
-        const int64_t ctas = (n_rows + 4 * c - 1) / (4 * c), cost = (ctas + (int64_t)sms * MINB - 1) / ((int64_t)sms * MINB) * (c + 1);
-        if (cost < best) { best = cost; g = c; }
-    }
+    const int64_t g = rowvec_groups(n_rows, g_max, (int64_t)sms * MINB).g;
     const int64_t g_pad = g | 1;                     // g_pad <= g_max because g_max is odd
     const int64_t r = 4 * g;
     const int64_t grid = (n_rows + r - 1) / r;
@@ -759,6 +769,42 @@ harp_status_t harp_generic_build(harp_plan *plan) {
     return max_fb <= 8 ? upload_element_major(ft, fb.data()) : HARP_OK;
 }
 
+namespace {
+
+// rows per CTA of the kernel with a thread per element: as many as registers (kMaxItems) and shared memory allow, at most 8, but at
+// least ~2 CTAs per SM in flight when the batch is small
+int element_rows(int64_t d, int64_t n_rows) {
+    int r = (int)std::min<int64_t>(std::min<int64_t>((int64_t)kThreads * kMaxItems / d, (227 * 1024) / (d * (int64_t)sizeof(float))), 8);
+    while (r > 1 && (n_rows + r - 1) / r < 296) --r;
+    return std::max(r, 1);
+}
+
+}  // namespace
+
+double harp_generic_estimate(const harp_plan *plan, int64_t n_rows, int sms) {
+    const int64_t d = plan->d;
+    const StageTable &st = plan->fused.m > 0 && plan->d_fused_blocks ? plan->fused : plan->st;
+    const int mx = harp_generic_max_radix(plan);
+    const bool perm = plan->d_perm != nullptr;
+    const double dm = 1e-4 * (double)d * st.m;                       // coordinates x stages
+    if (mx > 8) {                                                    // a thread per element, radices as given
+        const int64_t r = element_rows(d, n_rows), waves = ((n_rows + r - 1) / r + sms - 1) / sms;
+        int64_t sum = 0;
+        for (int t = 0; t < plan->st.m; ++t) sum += plan->st.b[t];
+        // (a tenth below the fit: near the crossing one launch is the safer choice)
+        return 0.9 * (5.8 + (double)waves * (0.83 + 1e-5 * (double)(r * d) * (15.4 * (double)sum + 98.0 * plan->st.m)));
+    }
+    if (d % 32 == 0 && d * 16 <= 226 * 1024 && !plan->opt_no_rowvec) {
+        int64_t g_max = 226 * 1024 / (d * 16);
+        if (g_max % 2 == 0) --g_max;
+        const double units = (double)rowvec_groups(n_rows, g_max, sms).cost;
+        return units * (mx <= 4 ? 2.3 * dm + (perm ? 8.7e-4 * (double)d : 0.0) : 5.0 * dm + (perm ? 10.4e-4 * (double)d : 0.0));
+    }
+    const int64_t r = blockowner_rows(d, n_rows, sms), waves = ((n_rows + r - 1) / r + sms - 1) / sms;
+    return (double)waves * (mx <= 4 ? (2.2 + 0.72 * (double)r) * dm + (perm ? 5.8e-4 * (double)(r * d) : 0.0)
+                                    : (6.7 + 0.78 * (double)r) * dm + (perm ? 10.6e-4 * (double)(r * d) : 0.0));
+}
+
 int harp_generic_max_radix(const harp_plan *plan) {
     const StageTable &st = plan->fused.m > 0 && plan->d_fused_blocks ? plan->fused : plan->st;
     int b = 0;
@@ -801,14 +847,7 @@ harp_status_t harp_generic_apply(const harp_plan *plan, void *x, int64_t n_rows,
         return dtype == HARP_F32 ? launch_blockowner<float, 256, true>(plan, bst, bblk, x, n_rows, transpose, stream)
                                  : launch_blockowner<__nv_bfloat16, 256, true>(plan, bst, bblk, x, n_rows, transpose, stream);
     }
-    // rows per CTA: as many as registers (kMaxItems) and shared memory allow, at most 8,
-    // but keep at least ~2 CTAs per SM in flight when the batch is small.
-    int r = (int)((int64_t)kThreads * kMaxItems / d);
-    const int r_smem = (int)((227 * 1024) / (d * (int64_t)sizeof(float)));
-    if (r > r_smem) r = r_smem;
-    if (r > 8) r = 8;
-    while (r > 1 && (n_rows + r - 1) / r < 296) --r;
-    if (r < 1) r = 1;
+    const int r = element_rows(d, n_rows);
     const int64_t items = ((int64_t)r * d + kThreads - 1) / kThreads;
 #define HARP_GEN_DISPATCH(T)                                                                  \
     if (items <= 4) return launch<T, 4>(plan, x, n_rows, r, transpose, stream);               \

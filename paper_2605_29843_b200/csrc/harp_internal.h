@@ -53,8 +53,9 @@ struct harp_plan {
     TmPlan *tm = nullptr;
     F32Plan *f32 = nullptr;
     // test-only switches, read from the environment once, when the plan is built (HARP_NO_ROWVEC=1: the
-    // CUDA-core kernels keep their tile row-major; HARP_NO_TENSOR_MAPS=1: as on a driver that cannot encode tensor maps)
-    bool opt_no_rowvec = false, opt_no_maps = false;
+    // CUDA-core kernels keep their tile row-major; HARP_NO_TENSOR_MAPS=1: as on a driver that cannot encode tensor maps;
+    // HARP_F32_PASSES=1: fp32 rows take the passes over column groups whatever the batch)
+    bool opt_no_rowvec = false, opt_no_maps = false, opt_f32_passes = false;
     // staging owned by harp_apply_host
     static constexpr int kStages = 4;
     void *stage_buf[kStages] = {nullptr, nullptr, nullptr, nullptr};
@@ -67,6 +68,10 @@ extern std::atomic<int64_t> g_harp_launches;
 // generic CUDA-core path (harp_generic.cu)
 harp_status_t harp_generic_build(harp_plan *plan);   // fused stage table for the block-owner kernel
 int harp_generic_max_radix(const harp_plan *plan);   // of the stage table its kernels run
+// Estimated microseconds of an fp32 batch on these kernels (harp_f32_preferred: on the passes over column groups), for the choice between
+// them: waves of CTAs times a CTA's time.  The constants are fitted to 1235 batches measured on both (d = 72 .. 32768, radices 2 .. 43,
+// 1 .. 4096 rows, identity and random permutation): standard deviation 12 % for the passes, 4 to 8 % here up to radix 8, 23 % above it.
+double harp_generic_estimate(const harp_plan *plan, int64_t n_rows, int sms);
 harp_status_t harp_generic_supported(const harp_plan *plan, harp_dtype_t dtype);
 harp_status_t harp_generic_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype,
                                  int transpose, cudaStream_t stream);
@@ -111,6 +116,7 @@ harp_status_t harp_col_apply(const harp_plan *plan, void *W, int64_t n_cols, int
 harp_status_t harp_f32_build(harp_plan *plan);
 void harp_f32_destroy(harp_plan *plan);
 int32_t harp_f32_error_word(const harp_plan *plan);
+bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows);      // faster than the whole-row kernels, by the estimates
 harp_status_t harp_f32_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose,
                              cudaStream_t stream);
 harp_status_t harp_f32_col_apply(const harp_plan *plan, void *W, int64_t n_cols, int64_t ld, harp_dtype_t dtype,

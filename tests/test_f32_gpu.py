@@ -34,6 +34,28 @@ def test_rows_match_the_oracle(radices, perm, n_rows):
     assert harp.harp_plan_error_word(plan) == 0
 
 
+@pytest.mark.parametrize("radices,perm", [((16, 16, 8), "identity"), ((16, 16, 8), "random"), ((2, 16, 9, 4), "identity"), ((16, 16), "identity"),
+                                          ((4, 4, 4, 43), "identity"), ((8, 8, 8, 8, 2), "identity"), ((8, 8, 5, 3, 11), "identity"),
+                                          ((4, 4, 4, 4, 4, 4, 2), "identity")])
+@pytest.mark.parametrize("n_rows", [1, 33, 64, 127])
+def test_passes_match_the_oracle(monkeypatch, radices, perm, n_rows):
+    """The same batches with the passes for all of them: by themselves the smaller ones take the whole-row kernels."""
+    monkeypatch.setenv("HARP_F32_PASSES", "1")
+    test_rows_match_the_oracle(radices, perm, n_rows)
+
+
+@pytest.mark.parametrize("radices,few,many", [((16, 16, 4), 64, 1024), ((8, 8, 8, 8, 2), 500, 128)])
+def test_small_batches_take_one_launch(radices, few, many):
+    """`few` rows are one wave of the whole-row kernels, `many` are faster in two passes."""
+    plan = harp.plan_from_spec(wl.tiny_plan(71, radices, kind="qr", perm="identity", signs=True))
+    for n_rows, launches in ((few, 1), (many, 2)):
+        x = torch.zeros((n_rows, plan.d), device="cuda")
+        before = harp.harp_launch_count()
+        harp.apply_(plan, x)
+        torch.cuda.synchronize()
+        assert harp.harp_launch_count() - before == launches
+
+
 @pytest.mark.parametrize("r_out,r_in", [((8, 8, 8), (4, 3, 5)), ((16, 16, 2), (7, 4)), ((2, 2, 2, 2, 3), (4, 4, 4, 4, 4)),
                                         ((43, 4), (4, 17)), ((64,), (2, 2)), ((8, 8, 8, 8), (8, 9))])
 def test_two_sided_fp32(r_out, r_in):
