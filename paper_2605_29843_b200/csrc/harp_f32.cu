@@ -631,7 +631,9 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
 }
 
 // Fixed permutation and signs of fp32 rows, in place, whole rows through shared memory.  Forward: row gathered,
-// out[i] = s[perm[i]] * in[perm[i]]; transpose: scattered, out[perm[i]] = s[perm[i]] * in[i].
+// out[i] = s[perm[i]] * in[perm[i]]; transpose: scattered, out[perm[i]] = s[perm[i]] * in[i].  The bank is mixed
+// with higher bits of the index: the coordinates that a warp gathers under a digit reversal are powers of two apart.
+__device__ __forceinline__ int permute_at(int i) { return i ^ (((i >> 5) ^ (i >> 10)) & 31); }
 __global__ void __launch_bounds__(512, 1)
 harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, const int32_t *__restrict__ perm,
                         const int8_t *__restrict__ signs, int transpose) {
@@ -643,12 +645,12 @@ harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, const in
         float *xr = x + row0 * d;
         if (!transpose) {
 #pragma unroll 4
-            for (int i = threadIdx.x; i < rows * d; i += 512) smem[i] = xr[i];
+            for (int i = threadIdx.x; i < rows * d; i += 512) smem[permute_at(i)] = xr[i];
         } else {
 #pragma unroll 2
             for (int i = threadIdx.x; i < d; i += 512) {
                 const int to = perm[i];
-                for (int r = 0; r < rows; ++r) smem[r * d + to] = xr[(int64_t)r * d + i];
+                for (int r = 0; r < rows; ++r) smem[permute_at(r * d + to)] = xr[(int64_t)r * d + i];
             }
         }
         __syncthreads();
@@ -657,7 +659,7 @@ harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, const in
             const int from = transpose ? i : perm[i];
             const bool neg = signs && signs[from] < 0;
             for (int r = 0; r < rows; ++r) {
-                const float v = smem[r * d + from];
+                const float v = smem[permute_at(r * d + from)];
                 xr[(int64_t)r * d + i] = neg ? -v : v;
             }
         }
@@ -865,7 +867,7 @@ harp_status_t run_passes(const harp_plan *plan, float *x, int64_t n, int64_t ld,
 harp_status_t permute_rows(const harp_plan *plan, float *x, int64_t n, int transpose, cudaStream_t stream) {
     const F32Plan *fp = plan->f32;
     const int R = fp->permute_rows;
-    const size_t smem = (size_t)R * plan->d * sizeof(float);
+    const size_t smem = (size_t)(R * plan->d + 31) / 32 * 32 * sizeof(float);
     if (cudaFuncSetAttribute(harp_f32_permute_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess)
         return HARP_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};

@@ -789,10 +789,10 @@ double harp_generic_estimate(const harp_plan *plan, int64_t n_rows, int sms) {
     const double dm = 1e-4 * (double)d * st.m;                       // coordinates x stages
     if (mx > 8) {                                                    // a thread per element, radices as given
         const int64_t r = element_rows(d, n_rows), waves = ((n_rows + r - 1) / r + sms - 1) / sms;
-        int64_t sum = 0;
-        for (int t = 0; t < plan->st.m; ++t) sum += plan->st.b[t];
+        double stages = 0.0;
+        for (int t = 0; t < plan->st.m; ++t) stages += 15.4 * plan->st.b[t] + (plan->st.b[t] == 2 ? 35.0 : 98.0);
         // (a tenth below the fit: near the crossing one launch is the safer choice)
-        return 0.9 * (5.8 + (double)waves * (0.83 + 1e-5 * (double)(r * d) * (15.4 * (double)sum + 98.0 * plan->st.m)));
+        return 0.9 * (5.8 + (double)waves * (0.83 + 1e-5 * (double)(r * d) * stages));
     }
     if (d % 32 == 0 && d * 16 <= 226 * 1024 && !plan->opt_no_rowvec) {
         int64_t g_max = 226 * 1024 / (d * 16);
