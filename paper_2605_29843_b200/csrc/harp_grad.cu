@@ -19,6 +19,7 @@
 // own some of the results (forward) or some of the rows of the gradient block (backward).  The first step reads x and the
 // last dL/dy in their own type.  Radices with no such kernel use the plain one-thread-per-element kernels.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 #include <map>
 #include <mutex>
@@ -786,7 +787,12 @@ Shape bwd_shape(const harp_plan *plan, const Step &sp) {
 int slice_rows(const harp_plan *plan, const Step &sp, int64_t rows, int sms) {
     const Shape sh = bwd_shape(plan, sp);
     const int64_t y = std::max<int64_t>(1, sms * (int64_t)sh.per_sm / sh.x);
-    return (int)std::max<int64_t>(8, (rows + y - 1) / y);
+    // Narrow plans, whose wave has hundreds of slices: a slice's rows are a serial chain of the backward kernel, shared by `subs` warps, and
+    // the slices one of the reduction, shared by eight; near the root of the rows the two last equally long (8192 rows of
+    // d = 2: 592 slices 23.9 us, 158 slices 9.7)
+    const int b = plan->st.b[sp.t], subs = sp.n == 2 ? kSubs : b == 16 ? 1 : b == 7 || b == 8 ? 2 : kSubs;
+    const int64_t even = (int64_t)(0.125 * subs * std::sqrt((double)rows));
+    return (int)std::max<int64_t>(std::max<int64_t>(8, even), (rows + y - 1) / y);
 }
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 dim3 grid2(int64_t x, int per_x, int64_t rows, int per_y) { return dim3((unsigned)((x + per_x - 1) / per_x), (unsigned)((rows + per_y - 1) / per_y)); }
