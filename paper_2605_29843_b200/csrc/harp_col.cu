@@ -566,6 +566,9 @@ harp_status_t build_col_pipe(ColPlan *cp, int which, const std::vector<GPhase> &
             for (int64_t hi = 0; hi < S_mid; hi += gp.S * gp.B_real)
                 for (int64_t lo = 0; lo < gp.S; ++lo) add((hi + lo) / C * (C + 1) + (hi + lo) % C);
         D.n_items = (int32_t)tab.size() - D.items_off;
+        // Blocks for half of the warps at least.  Smaller tiles are faster in the kernel above: slabs of 16 x 4 (d = 3840 x 8192, both
+        // sides, 179 us there, 220 here), of 16 x 8 (5120 x 3840: 108 and 116), two positions of an upper group (1232 x 4096: 83 and 108)
+        if (2 * D.n_items < kColPipeThreads / 32) return HARP_OK;
         for (int i = D.items_off; i < (int)tab.size(); ++i)
             if (tab[(size_t)i] < 0 || 128 * (tab[(size_t)i] + (gp.B_real - 1) * D.wr + 1) > P.tile_bytes) return HARP_OK;
     }
