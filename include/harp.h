@@ -199,9 +199,12 @@ harp_status_t harp_apply_passes(const harp_plan_t *const *plans, int32_t n_passe
  *   W        DEVICE d_out x d_in row-major, d_out = dim(plan_out), d_in = dim(plan_in)
  *   scratch  DEVICE buffer of harp_two_sided_scratch_bytes(...) bytes, 256-byte aligned,
  *            or NULL to let the call allocate and free it on the stream
- *            (cudaMallocAsync/cudaFreeAsync).  It is used only when the column side has to go
- *            through a transposed copy of W (plan_out with a permutation, fp32, or d_in not a
- *            multiple of 8); otherwise the columns are processed in place and it is ignored.
+ *            (cudaMallocAsync/cudaFreeAsync).  It is used only when the column side goes through a
+ *            transposed copy of W: plan_out with a permutation, d_in not a multiple of 8 (bf16) or 4
+ *            (fp32), a W that is not 16-byte aligned, a plan_out that the column kernels have no pass
+ *            for (fp32: wider than 32768 or with a radix above 64), and fp32 matrices of a few columns
+ *            where plan_out has a radix above 8.  Otherwise the columns are processed in place and it
+ *            is ignored.
  * Both plans must live on the current device (else HARP_ERR_DIM_MISMATCH).
  * Asynchronous on stream. */
 harp_status_t harp_apply_two_sided(void *W, harp_dtype_t dtype, const harp_plan_t *plan_out,

@@ -924,6 +924,20 @@ int32_t harp_f32_error_word(const harp_plan *plan) {
     return cudaMemcpy(&v, plan->f32->d_err, sizeof(v), cudaMemcpyDeviceToHost) == cudaSuccess ? v : -1;
 }
 
+namespace {
+
+// microseconds of a pass over n vectors, see harp_generic_estimate
+double pass_estimate(const F32Plan *fp, const F32Pass &P, int64_t n) {
+    const int64_t tiles = (n + 32 * P.RT - 1) / (32 * P.RT), n_c = (int64_t)P.E * P.L;
+    const int64_t n_parts = pass_parts(fp, P, tiles), per = n_parts > 0 ? (tiles + n_parts - 1) / n_parts : (tiles * P.n_cg + fp->sms - 1) / fp->sms;
+    const int64_t groups = n_parts > 0 ? 1 : 1 + (per - 1) / tiles;          // whose block kernels a CTA fetches
+    double radices = 0.0;
+    for (int k = 0; k < P.n_ph; ++k) radices += P.ph[k].b;
+    return 5.1 + 3.3e-4 * (double)(P.w_floats * groups) + 4.06e-4 * (double)(per * n_c * P.RT) * radices + 2.6e-6 * (double)n * (double)P.d;
+}
+
+}  // namespace
+
 // The passes cost two or three launches, the block kernels of a column group in every CTA, and tiles of 32 rows; the whole-row kernels
 // a wave of CTAs, whatever the batch leaves of it idle.  Radices (16, 16, 4), whole rows against passes: 128 rows 14 us and 25,
 // 256 rows 25 and 25, 512 rows 45 and 28; (16, 16), one pass: 128 rows 6 and 13, 4096 rows 62 and 13; d = 8192 in radix 8 (four rows
@@ -932,17 +946,8 @@ bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows) {
     const F32Plan *fp = plan->f32;
     if (!fp || fp->n_pass[0] == 0) return false;
     if (plan->opt_f32_passes || harp_generic_supported(plan, HARP_F32) != HARP_OK) return true;
-    const double elems = (double)n_rows * (double)plan->d;
     double us = 0.0;
-    for (int p = 0; p < fp->n_pass[0]; ++p) {
-        const F32Pass &P = fp->pass[0][p];
-        const int64_t tiles = (n_rows + 32 * P.RT - 1) / (32 * P.RT), n_c = (int64_t)P.E * P.L;
-        const int64_t n_parts = pass_parts(fp, P, tiles), per = n_parts > 0 ? (tiles + n_parts - 1) / n_parts : (tiles * P.n_cg + fp->sms - 1) / fp->sms;
-        const int64_t groups = n_parts > 0 ? 1 : 1 + (per - 1) / tiles;      // whose block kernels a CTA fetches
-        double radices = 0.0;
-        for (int k = 0; k < P.n_ph; ++k) radices += P.ph[k].b;
-        us += 5.1 + 3.3e-4 * (double)(P.w_floats * groups) + 4.06e-4 * (double)(per * n_c * P.RT) * radices + 2.6e-6 * elems;
-    }
+    for (int p = 0; p < fp->n_pass[0]; ++p) us += pass_estimate(fp, fp->pass[0][p], n_rows);
     if (fp->permute_rows) {
         const int64_t waves = ((n_rows + fp->permute_rows - 1) / fp->permute_rows + fp->sms - 1) / fp->sms;
         us += 5.6 + 2.1e-4 * (double)(waves * std::min<int64_t>(fp->permute_rows, n_rows) * plan->d);
@@ -966,5 +971,12 @@ harp_status_t harp_f32_col_apply(const harp_plan *plan, void *W, int64_t n_cols,
     const F32Plan *fp = plan->f32;
     if (!fp || dtype != HARP_F32 || fp->n_pass[1] == 0 || n_cols > kMaxF32Vectors) return HARP_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(W) & 15u) != 0 || n_cols % 4 != 0 || ld % 4 != 0) return HARP_ERR_UNSUPPORTED;
+    // Few columns of a narrow plan with a radix above 8: as rows of the transposed matrix (two transposes, a launch and a trip each) where
+    // the whole-row kernel takes them in a wave (369 x 16, radices 41, 3, 3: 27 us, in place 38)
+    if (harp_generic_max_radix(plan) > 8 && harp_generic_supported(plan, HARP_F32) == HARP_OK && !plan->opt_f32_passes) {
+        double us = 0.0;
+        for (int p = 0; p < fp->n_pass[1]; ++p) us += pass_estimate(fp, fp->pass[1][p], n_cols);
+        if (us > 2.0 * (3.0 + 2.4e-6 * (double)n_cols * (double)plan->d) + harp_generic_estimate(plan, n_cols, fp->sms)) return HARP_ERR_UNSUPPORTED;
+    }
     return run_passes<true>(plan, static_cast<float *>(W), n_cols, ld, 0, stream);
 }

@@ -74,6 +74,13 @@ def test_two_sided_fp32(r_out, r_in):
     assert harp.harp_plan_error_word(plan_out) == 0
 
 
+@pytest.mark.parametrize("r_out,r_in", [((2, 2, 2, 2, 3), (4, 3, 5)), ((43, 4), (4, 17)), ((41, 3, 3), (4, 4)), ((64,), (2, 2)), ((8, 8, 8), (8, 9))])
+def test_two_sided_fp32_in_place(monkeypatch, r_out, r_in):
+    """Column passes for small matrices too, which by themselves go through the transposed copy."""
+    monkeypatch.setenv("HARP_F32_PASSES", "1")
+    test_two_sided_fp32(r_out, r_in)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_a_driver_without_tensor_maps(monkeypatch, dtype):
     """Plans whose passes cannot be fed by bulk copies keep the kernels that need none: rows, permuted rows and both sides of a matrix."""
