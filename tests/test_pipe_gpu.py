@@ -60,3 +60,15 @@ def test_columns_match_the_oracle(out_radices, in_radices):
     # an entry against the smaller norm of its row and column: one bound of the rows' test per side
     scale = np.minimum(np.linalg.norm(want, axis=1, keepdims=True), np.linalg.norm(want, axis=0, keepdims=True))
     assert np.max(np.abs(to_host_f64(wd) - want) / scale) <= 2 * TOL["bf16"]
+
+
+@pytest.mark.parametrize("radices", [(16, 16, 8, 7), (8, 8, 8, 8, 7), (8, 8, 8, 8, 2), (8, 8, 8, 8, 8), (16, 16, 43), (8, 8, 8, 8)])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_a_row_has_the_same_bits_in_every_batch(radices, transpose):
+    """The kernels that take over at 9, 17, 384 rows and from the wide tiles on round where the others round, and sum in their order."""
+    plan = harp.plan_from_spec(wl.make_plan(86, int(np.prod(radices)), radices, "qr", perm="identity", signs=True))
+    x = torch.randn((4099, plan.d), generator=torch.Generator(device="cuda").manual_seed(87), device="cuda").to(torch.bfloat16)
+    want = harp.apply_(plan, x.clone(), transpose, harp.KERNEL_SPLIT)
+    for n_rows in (1, 8, 9, 16, 17, 100, 383, 384, 700):
+        got = harp.apply_(plan, x[:n_rows].clone(), transpose, harp.KERNEL_SPLIT)
+        assert torch.equal(got.view(torch.int16), want[:n_rows].view(torch.int16)), n_rows
