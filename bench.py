@@ -42,7 +42,7 @@ N_BUF = 4
 # proportion to the rows, so a full launch is scaled by n_rows / R.  Write-back that is still in L2
 # when a kernel ends is not in these figures (cfg1 and cfg2 read below their algorithmic bytes for
 # that reason).
-NCU_TRAFFIC = {1: (4096, 33.8e6), 2: (16384, 209.8e6), 3: (4096, 259.1e6), 4: (4096, 364.2e6), 5: (4096, 833.3e6)}
+NCU_TRAFFIC = {1: (4096, 33.8e6), 2: (16384, 209.8e6), 3: (4096, 250.2e6), 4: (4096, 356.1e6), 5: (4096, 831.1e6)}
 
 
 def ncu_traffic(cfg: int, n_rows: int):

@@ -253,7 +253,7 @@ int64_t harp_two_sided_static_capacity_bytes(void);
  *              if accumulate != 0
  * Any schedule is accepted.  Sums over rows are taken in fp64, in an order that the shapes fix (no
  * atomics: the result does not depend on scheduling).  The call allocates and frees scratch
- * on the stream (about 200 MB of states and the partial sums of one wave of CTAs, from a memory pool of the library's own that keeps what it has
+ * on the stream (states of about 200 MB of rows, of sixteen rows at least, and the partial sums of one wave of CTAs, from a memory pool of the library's own that keeps what it has
  * been given until the process ends); HARP_ERR_ALLOC if that fails.  Asynchronous on stream. */
 harp_status_t harp_grad_blocks(const harp_plan_t *plan, const void *x, const void *gy, int64_t n_rows,
                                harp_dtype_t dtype, float *grad, int accumulate, void *stream);
@@ -304,10 +304,11 @@ harp_status_t harp_diag_weighted_error(const void *Wt, const void *Wq, int64_t d
 harp_status_t harp_apply_host(harp_plan_t *plan, void *x_host, int64_t n_rows,
                               harp_dtype_t dtype, int transpose);
 
-/* Device-side wait status of the plan's HARP_KERNEL_TMEM kernels.  Every wait inside those kernels
+/* Device-side wait status of the plan's kernels that are fed by bulk copies (HARP_KERNEL_TMEM, the
+ * two-pass rows, the columns of two-sided products, the fp32 passes).  Every wait inside those kernels
  * (on a bulk copy, on the tensor core, on another warp) has an iteration limit; a wait that runs out
- * sets a device word, the kernel releases its tensor memory and returns, and the rows it was working
- * on are left undefined.  Returns 0 if no wait has given up since the plan was built, a positive
+ * sets a device word, the kernel copies nothing more, waits as long again for its loads in flight,
+ * releases its tensor memory and returns, and the rows it was working on are left undefined.  Returns 0 if no wait has given up since the plan was built, a positive
  * code naming the wait otherwise, -1 for NULL or a failed copy.  Synchronises with the device. */
 int32_t harp_plan_error_word(const harp_plan_t *plan);
 

@@ -16,8 +16,8 @@
 //         two-sided product of an fp32 matrix needs neither a transposed copy nor scratch.
 // ROWS and COLS tiles move by bulk copies over three buffers: one SM moves about 30 bytes per cycle to and from L2, and
 // a warp that issues loads and stores is held at that rate with every shared-memory access behind it (the arithmetic of a
-// tile took four times as long with the copies done by extra warps through the load/store unit).  The runs of RUNS are too
-// short for the copy engine (about five cycles a run); there cp.async fetches the next tile.
+// tile took four times as long with the copies done by extra warps through the load/store unit).  RUNS tiles (runs of
+// 16 to 128 bytes) move by cp.async, the next tile under the arithmetic of this one.
 #include <algorithm>
 #include <new>
 

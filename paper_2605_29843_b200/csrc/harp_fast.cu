@@ -1206,7 +1206,8 @@ void harp_fast_destroy(harp_plan *plan) {
     plan->fast = nullptr;
 }
 
-// Batches that the two-pass path takes from this kernel.  With four phases (radix 8, d = 4096) a whole-row tile costs more than two
+// Batches that the two-pass path takes from this kernel.  With four phases (groups of 8 or 16 in rows of at least 4096 that fit shared
+// memory leave one such shape, d = 4096 as 8 x 8 x 8 x 8) a whole-row tile costs more than two
 // passes at copy rate, unless its batch is less than the clusters of eight hold (128 rows 7.7 us against 7.8) or nearly one full
 // wave of tiles (1800 to 2300 rows 17 us against 18 to 19); 256 rows 10.0 -> 8.4 us, 1024 14.8 -> 12.3, 2500 30.9 -> 20.3,
 // 16384 123 -> 111.  With three phases of sixteen (97 against 91 us, 65536 rows 366 against 396) it keeps them.

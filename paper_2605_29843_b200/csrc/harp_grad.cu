@@ -911,8 +911,8 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
         if (permuted) {
             using Bits = std::conditional_t<sizeof(T) == 2, uint16_t, uint32_t>;
             const size_t row_smem = (size_t)((d + 2 * (d >> 6) + 2) / 2 * 2) * sizeof(T);
-            // four rows per CTA (the kernel counts on at most that) where they leave two CTAs for every SM (8 rows of d = 3375: 11 us with four, 5.5
-            // with one).  Shared memory is taken from the L1 that the one-thread-per-element kernels behind this one live on (radices 6, 54,
+            // four rows per CTA (the kernel counts on at most that) where they leave two CTAs for every SM (8 rows of d = 3375: the call 45.0 us
+            // with four, 41.8 with one).  Shared memory is taken from the L1 that the one-thread-per-element kernels behind this one live on (radices 6, 54,
             // 20, 1024 rows: 3160 us behind 53 KB a CTA, 1750 behind 26; 7, 49, 8, 2051 rows in fp32: 2240 behind 44 KB, 1310 behind 11).
             const size_t cap = red.m == tab.m ? 100 * 1024 : 12 * 1024;
             int R = 4;

@@ -882,10 +882,10 @@ harp_status_t harp_split_build(harp_plan *plan) {
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms > 0) sp->sms = sms;
-        // Rows per chunk.  A chunk that fits L2 lets the second pass read what the first wrote
-        // without going to HBM, but every chunk costs two launches and two partial waves; with
-        // the present kernels (bound by instruction issue, not by HBM) large chunks are faster,
-        // so the default is one chunk of up to 8 GiB.  HARP_SPLIT_CHUNK_MB overrides it.
+        // Rows per chunk.  A chunk that fits L2 lets the second pass read what the first wrote without going to HBM, but
+        // every chunk costs two launches and two partial waves, and these cost more (us in one chunk, in chunks of 117 MB, of
+        // 48 MB: 32768 rows of d = 14336 667, 695, 805; 65536 of d = 28672 2869, 3077, 3879; 16384 of d = 11008 272, 293, 355;
+        // 16384 of d = 8192 210, 241, 258).  So the default is one chunk of up to 8 GiB; HARP_SPLIT_CHUNK_MB overrides it.
         const char *e = getenv("HARP_SPLIT_CHUNK_MB");
         const int64_t chunk_bytes = (int64_t)(e ? atoi(e) : 8192) << 20;
         sp->chunk_rows = std::max<int64_t>(64, chunk_bytes / (d * 2) / 64 * 64);
