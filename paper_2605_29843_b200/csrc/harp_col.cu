@@ -288,16 +288,15 @@ harp_col_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, con
         for (int t = 0; t < count; ++t, b = b + 1 == NB ? 0 : b + 1) {
             const uint32_t bar = smem_u32(&full_bar[b]), sbase = bufs + (uint32_t)(b * P.tile_bytes);
             uint32_t it = 0;
-            bool got = true;
             while (!harp_tm::mbar_try(bar, (parity >> b) & 1u)) {
                 if (++it > kColSpin || ((it & 63) == 63 && *(volatile int *)&dead)) {
                     *(volatile int *)&dead = 1;       // from here on nothing is copied any more
                     atomicExch(err, 302);
-                    got = false;
+                    parity ^= 1u << b;        // (undone below: the phase is still awaited)
                     break;
                 }
             }
-            if (got) parity ^= 1u << b;
+            parity ^= 1u << b;
             for (int p = 0; p < P.n_phases; ++p) {
                 const ColPhase &ph = P.ph[p];
                 if (p > 0) __syncthreads();

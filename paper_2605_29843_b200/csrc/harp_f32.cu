@@ -570,16 +570,15 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
             if (fresh) asm volatile("cp.async.wait_all;" ::: "memory");
             const uint32_t bar = smem_u32(&full_bar[buf]), par = (parity >> buf) & 1u;
             uint32_t it = 0;
-            bool got = true;
             while (!harp_tm::mbar_try(bar, par)) {
                 if (++it > kF32Spin || ((it & 63) == 63 && stopped())) {
                     *(volatile int *)&dead = 1;                // from here on nothing is copied any more
                     atomicExch(err, 101);
-                    got = false;
+                    parity ^= 1u << buf;        // (undone below: the phase is still awaited)
                     break;
                 }
             }
-            if (got) parity ^= 1u << buf;
+            parity ^= 1u << buf;
         }
         __syncthreads();
         if (MODE == RUNS && n_buf == 2 && t + 1 < n_my) {      // under the arithmetic of this tile

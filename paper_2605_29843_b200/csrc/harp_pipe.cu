@@ -320,16 +320,15 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
         for (int t = team; t < count; t += TEAMS, b = b + 1 == NB ? 0 : b + 1) {
             const uint32_t bar = smem_u32(&full_bar[team * kMaxPipeBufs + b]), sbase = bufs + (uint32_t)(b * P.tile_bytes);
             uint32_t it = 0;
-            bool got = true;
             while (!mbar_try(bar, (parity >> b) & 1u)) {
                 if (++it > kPipeSpin || ((it & 63) == 63 && *(volatile int *)&dead)) {
                     *(volatile int *)&dead = 1;       // from here on nothing is copied any more
                     atomicExch(err, 301);
-                    got = false;
+                    parity ^= 1u << b;        // (undone below: the phase is still awaited)
                     break;
                 }
             }
-            if (got) parity ^= 1u << b;
+            parity ^= 1u << b;
             // the store of the tile before has had a phase's time to be read: refill its buffer
             auto refill = [&]() {
                 if (tid == 0 && t > team && t + (NB - 1) * TEAMS < count && !*(volatile int *)&dead) {

@@ -38,14 +38,13 @@ int main(int argc, char **argv) {
     };
     for (int k = 0; k < kBuf && k < kTiles; ++k) load(k, k);
     for (int t = 0, b = 0; t < kTiles; ++t, b = b + 1 == kBuf ? 0 : b + 1) {
-        bool got = true;
         for (uint32_t it = 0; !try_phase(b, (parity >> b) & 1u);)
             if (++it > kLimit || ((it & 63) == 63 && dead)) {
                 dead = true;
-                got = false;
+                parity ^= 1u << b;
                 break;
             }
-        if (got) parity ^= 1u << b;
+        parity ^= 1u << b;
         if (t > 0 && t + kBuf - 1 < kTiles && !dead) load(t + kBuf - 1, b == 0 ? kBuf - 1 : b - 1);
         if (!dead) { wrong += held[b] != t || due[b] >= 0; ++stored; }
     }
