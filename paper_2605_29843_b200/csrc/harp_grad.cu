@@ -137,7 +137,7 @@ fwd_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int vec,
 }
 
 // CTAs per SM of the backward kernels (registers: 168 per thread from radix 5 to 8, else 128)
-constexpr int k44PerSm = 3;
+constexpr int k44PerSm = 3, kFwd44PerSm = 6;
 __host__ __device__ constexpr int bwd_per_sm(int b, int bi, int subs) { return (b >= 5 && b <= 6 ? 12 : 16) / (((b + bi - 1) / bi) * subs); }
 
 // sums of the warps that split the rows, added in the order of the warps; sum k of a lane goes to dst(k)
@@ -249,7 +249,7 @@ struct Pair44 {
         q = S1 ? lane & 3 : lane >> 3;
         const int64_t u = first_unit + (S1 ? lane >> 2 : lane & 7);
         have = u < d / 16;
-        const int64_t uu = have ? u : 0, alpha = uu / s, beta = uu - alpha * s;
+        const int64_t uu = have ? u : S1 ? 0 : min((int64_t)(lane & 7), d / 16 - 1), alpha = uu / s, beta = uu - alpha * s;     // past the end: any units, neighbours too
         base = alpha * 16 * s + beta;
         c1 = (4 * alpha + q) * s + beta;
         c2 = alpha * 4 * s + beta + q * s;
@@ -289,11 +289,61 @@ __device__ __forceinline__ void mul4t(const float (&x)[4], const float (&k)[4][4
     }
 }
 
-template <bool S1, typename TI>
-__global__ void __launch_bounds__(kOwnThreads)
-fwd44_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int vec, float *__restrict__ out, int64_t rows, int64_t d, int64_t s,
+// Rows on their way to the lanes of a Pair44.  A row's coordinates of a warp come by asynchronous copies of 8 or 16 bytes a lane into a
+// ring of the warp's own in shared memory, several rows ahead of the one being multiplied: a step reads little per row and thread (16
+// bytes a state), so that with loads one row ahead the rows in flight, 12 KB an SM, bounded it at 1.8 TB/s.  S1: a unit's sixteen values
+// in a row, 20 words apart in fp32 (both orders of reading then hit 32 banks); otherwise sixteen runs of the eight neighbouring units, four runs and 32 bytes of padding.
+template <bool S1, typename T>
+struct Rows44 {
+    static constexpr int kBytes = sizeof(T) == 2 ? 256 : 640;
+    static __device__ __forceinline__ void issue(unsigned char *dst, const T *row, const Pair44<S1> &u, int64_t s) {
+        const int lane = threadIdx.x & 31;
+        uint32_t to = (uint32_t)__cvta_generic_to_shared(dst);
+        if constexpr (S1) {
+            const T *src = row + u.base + 4 * u.q;
+            if constexpr (sizeof(T) == 2) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to + 8 * lane), "l"(src) : "memory");
+            else asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + (lane >> 2) * 80 + u.q * 16), "l"(src) : "memory");
+        } else if constexpr (sizeof(T) == 2) {
+            const T *src = row + (u.base - (lane & 7)) + (lane & 15) * s;
+            if (lane < 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * lane), "l"(src) : "memory");
+        } else {
+            const int run = lane >> 1;
+            const T *src = row + (u.base - (lane & 7)) + run * s + (lane & 1) * 4;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * lane + (run >> 2) * 32), "l"(src) : "memory");
+        }
+    }
+    // first stage's order: coordinates base + (4 q + i) s
+    static __device__ __forceinline__ void first(const unsigned char *from, const Pair44<S1> &u, float (&v)[4]) {
+        const int lane = threadIdx.x & 31;
+        if constexpr (S1) load_block<4, T>(reinterpret_cast<const T *>(from + (sizeof(T) == 2 ? 8 * lane : (lane >> 2) * 80 + u.q * 16)), 1, true, v);
+        else if constexpr (sizeof(T) == 2) load_block<4, T>(reinterpret_cast<const T *>(from) + 32 * u.q + (lane & 7), 8, false, v);
+        else load_block<4, T>(reinterpret_cast<const T *>(from) + 40 * u.q + (lane & 7), 8, false, v);
+    }
+    // second stage's: base + (q + 4 j) s
+    static __device__ __forceinline__ void second(const unsigned char *from, const Pair44<S1> &u, float (&v)[4]) {
+        const int lane = threadIdx.x & 31;
+        if constexpr (S1) load_block<4, T>(reinterpret_cast<const T *>(from + (lane >> 2) * (sizeof(T) == 2 ? 32 : 80)) + u.q, 4, false, v);
+        else if constexpr (sizeof(T) == 2) load_block<4, T>(reinterpret_cast<const T *>(from) + 8 * u.q + (lane & 7), 32, false, v);
+        else load_block<4, T>(reinterpret_cast<const T *>(from) + 8 * u.q + (lane & 7), 40, false, v);
+    }
+};
+constexpr int kRing = 8;               // rows in a warp's ring
+__device__ __forceinline__ void ring_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// the oldest row of the ring has arrived, for the whole warp
+__device__ __forceinline__ void ring_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 1) : "memory");
+    __syncwarp();
+}
+
+// RING: rows by asynchronous copies (16-byte boundaries: see ring44)
+template <bool S1, bool RING, typename TI>
+__global__ void __launch_bounds__(kOwnThreads, kFwd44PerSm)
+fwd44_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int vec, float *__restrict__ out, int64_t rows, int64_t d, int64_t s, int slice,
              const float *__restrict__ em1, const float *__restrict__ em2) {
-    const Pair44<S1> u(d, s, ((int64_t)blockIdx.x * (kOwnThreads / 32) + (threadIdx.x >> 5)) * 8);
+    using Rows = Rows44<S1, TI>;
+    __shared__ __align__(16) unsigned char ring[RING ? kOwnThreads / 32 : 1][RING ? kRing : 1][RING ? Rows::kBytes : 16];
+    const int w = threadIdx.x >> 5;
+    const Pair44<S1> u(d, s, ((int64_t)blockIdx.x * (kOwnThreads / 32) + w) * 8);
     const int64_t nblk = d / 4, in0 = u.base + 4 * u.q * s, out0 = S1 ? in0 : u.base + u.q * s, os = S1 ? 1 : 4 * s;
     float k1[4][4], k2[4][4];
 #pragma unroll
@@ -306,69 +356,78 @@ fwd44_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int ve
         }
     }
     prior_kernel_done();
-    const int64_t r0 = (int64_t)blockIdx.y * kFwdRows, r1 = min(rows, r0 + kFwdRows);
-    const TI *p = in + r0 * d + in0;
-    float *w = out + r0 * d + out0;
-    float x[4][4];
-    for (int64_t r = r0; r < r1; r += 4, p += 4 * d, w += 4 * d) {
+    const int64_t r0 = (int64_t)blockIdx.y * slice, r1 = min(rows, r0 + slice);
+    float *to = out + r0 * d + out0;
+    auto row = [&](const float (&x)[4]) {
+        float y[4], z[4];
+        mul4(x, k1, y);
+        u.transpose(y);
+        mul4(y, k2, z);
+        if (S1) u.transpose(z);
+        if (u.have) store_block<4>(to, os, S1, z);
+        to += d;
+    };
+    if constexpr (RING) {
+        const TI *src = in + r0 * d;
+#pragma unroll 1
+        for (int k = 0; k < kRing; ++k, src += d) {
+            if (r0 + k < r1) Rows::issue(ring[w][k], src, u, s);
+            ring_commit();
+        }
+        for (int64_t r = r0; r < r1; ++r, src += d) {
+            unsigned char *slot = ring[w][(int)(r - r0) & (kRing - 1)];
+            float x[4];
+            ring_wait();
+            Rows::first(slot, u, x);
+            __syncwarp();
+            if (r + kRing < r1) Rows::issue(slot, src, u, s);
+            ring_commit();
+            row(x);
+        }
+    } else {
+        const TI *p = in + r0 * d + in0;
+        float x[4][4];
+        for (int64_t r = r0; r < r1; r += 4, p += 4 * d) {
 #pragma unroll
-        for (int n = 0; n < 4; ++n)
-            if (r + n < r1) load_block<4, TI>(p + n * d, s, vec, x[n]);
+            for (int n = 0; n < 4; ++n)
+                if (r + n < r1) load_block<4, TI>(p + n * d, s, vec, x[n]);
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            if (r + n >= r1) break;
-            float y[4], z[4];
-            mul4(x[n], k1, y);
-            u.transpose(y);
-            mul4(y, k2, z);
-            if (S1) u.transpose(z);
-            if (u.have) store_block<4>(w + n * d, os, S1, z);
+            for (int n = 0; n < 4; ++n)
+                if (r + n < r1) row(x[n]);
         }
     }
 }
 
-template <bool S1, typename TV, typename TG>
+template <bool S1, bool RING, typename TV, typename TG>
 __global__ void __launch_bounds__(32 * kSubs, k44PerSm)
 bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v, const TG *__restrict__ g, int vec_g, float *__restrict__ g_out,
              int64_t rows, int64_t d, int64_t s, int slice, int add, const float *__restrict__ em1, const float *__restrict__ em2, double *__restrict__ part1,
              double *__restrict__ part2) {
-    __shared__ double sh[32][kSubs][32];
+    using RowsV = Rows44<S1, TV>;
+    using RowsG = Rows44<S1, TG>;
+    constexpr int kSums = 32 * kSubs * 32 * 8, kRings = kSubs * kRing * (RowsV::kBytes + RowsG::kBytes);
+    __shared__ __align__(16) unsigned char smem[RING && kRings > kSums ? kRings : kSums];        // the rings, then the warps' sums
     const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
     const Pair44<S1> u(d, s, (int64_t)blockIdx.x * 8);
     const int64_t nblk = d / 4, first = u.base + 4 * u.q * s, second = S1 ? first : u.base + u.q * s, gs = S1 ? 1 : 4 * s;
-    float k1[4][4], k2[4][4], sg[4];
+    float k1[4][4], k2[4][4], sg[4];           // k1 with the signs of the step's coordinates
     double acc[32];                            // first stage's sums, second stage's
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         sg[i] = sign_of(signs, first + i * s);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            k1[i][j] = em1[(int64_t)(i * 4 + j) * nblk + u.c1];
+            k1[i][j] = sg[i] * em1[(int64_t)(i * 4 + j) * nblk + u.c1];
             k2[i][j] = em2[(int64_t)(i * 4 + j) * nblk + u.c2];
             acc[i * 4 + j] = acc[16 + i * 4 + j] = 0.0;
         }
     }
     prior_kernel_done();
     const int64_t r0 = (int64_t)blockIdx.y * slice + sub, r1 = min(rows, (int64_t)(blockIdx.y + 1) * slice);
-    const TV *pv = v + r0 * d + first;
-    const TG *pg = g + r0 * d + second;
     float *w = g_out ? g_out + r0 * d + first : nullptr;
-    float nv[4], ng[4];
-    if (r0 < r1) {
-        load_block<4, TV>(pv, s, vec_v, nv);
-        load_block<4, TG>(pg, gs, vec_g, ng);
-    }
-    for (int64_t r = r0; r < r1; r += kSubs) {
-        float x[4], y[4], gy[4], h[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { x[i] = sg[i] * nv[i]; gy[i] = ng[i]; }
-        pv += kSubs * d;
-        pg += kSubs * d;
-        if (r + kSubs < r1) {                  // the next row's values are on their way
-            load_block<4, TV>(pv, s, vec_v, nv);
-            load_block<4, TG>(pg, gs, vec_g, ng);
-        }
-        if (S1) u.transpose(gy);
+    // x: first stage's order, gy: second stage's
+    auto row = [&](const float (&x)[4], const float (&gy)[4]) {
+        float y[4], h[4];
         mul4(x, k1, y);
         u.transpose(y);
         {
@@ -395,16 +454,247 @@ bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
                 for (int j = 0; j < 4; ++j) acc[i * 4 + j] += vd * gd[j];
             }
         }
-        if (w) {
+        if (w) {                               // (a step with signs is the first one and has no gradient state behind it)
             float o[4];
             mul4t(h, k1, o);
             if (u.have) store_block<4>(w, s, S1, o);
             w += kSubs * d;
         }
+    };
+    if constexpr (RING) {
+        unsigned char *ring_v = smem + sub * kRing * RowsV::kBytes, *ring_g = smem + kSubs * kRing * RowsV::kBytes + sub * kRing * RowsG::kBytes;
+        const TV *pv = v + r0 * d;
+        const TG *pg = g + r0 * d;
+#pragma unroll 1
+        for (int k = 0; k < kRing; ++k, pv += kSubs * d, pg += kSubs * d) {
+            if (r0 + k * kSubs < r1) {
+                RowsV::issue(ring_v + k * RowsV::kBytes, pv, u, s);
+                RowsG::issue(ring_g + k * RowsG::kBytes, pg, u, s);
+            }
+            ring_commit();
+        }
+        int k = 0;
+        for (int64_t r = r0; r < r1; r += kSubs, pv += kSubs * d, pg += kSubs * d, k = (k + 1) & (kRing - 1)) {
+            float x[4], gy[4];
+            ring_wait();
+            RowsV::first(ring_v + k * RowsV::kBytes, u, x);
+            RowsG::second(ring_g + k * RowsG::kBytes, u, gy);
+            __syncwarp();
+            if (r + kRing * kSubs < r1) {
+                RowsV::issue(ring_v + k * RowsV::kBytes, pv, u, s);
+                RowsG::issue(ring_g + k * RowsG::kBytes, pg, u, s);
+            }
+            ring_commit();
+            row(x, gy);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+    } else {
+        const TV *pv = v + r0 * d + first;
+        const TG *pg = g + r0 * d + second;
+        float nv[4], ng[4];
+        if (r0 < r1) {
+            load_block<4, TV>(pv, s, vec_v, nv);
+            load_block<4, TG>(pg, gs, vec_g, ng);
+        }
+        for (int64_t r = r0; r < r1; r += kSubs) {
+            float x[4], gy[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { x[i] = nv[i]; gy[i] = ng[i]; }
+            pv += kSubs * d;
+            pg += kSubs * d;
+            if (r + kSubs < r1) {              // the next row's values are on their way
+                load_block<4, TV>(pv, s, vec_v, nv);
+                load_block<4, TG>(pg, gs, vec_g, ng);
+            }
+            if (S1) u.transpose(gy);
+            row(x, gy);
+        }
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i * 4 + j] = sg[i] < 0.f ? -acc[i * 4 + j] : acc[i * 4 + j];
     double *d1 = part1 + (int64_t)blockIdx.y * 16 * nblk + u.c1, *d2 = part2 + (int64_t)blockIdx.y * 16 * nblk + u.c2;
-    combine<32, kSubs>(acc, sh, sub, lane, add, [&](int e) -> double * {
+    combine<32, kSubs>(acc, reinterpret_cast<double (*)[kSubs][32]>(smem), sub, lane, add, [&](int e) -> double * {
         return !u.have ? nullptr : e < 16 ? d1 + (int64_t)e * nblk : d2 + (int64_t)(e - 16) * nblk;
+    });
+}
+
+// ---- four radix-2 stages of strides s, 2 s, 4 s and 8 s on the same units: a thread holds two stages' blocks in the first order (coordinate
+// i of four: pairs i, i ^ 1, then i, i ^ 2) and the other two stages' in the second.  As much register space for kernels and sums as two
+// radix-4 stages, and half the state traffic of two radix-2 stages a step.
+template <bool S1>
+struct Quad2222 : Pair44<S1> {
+    int64_t c[4][2];                   // block numbers of this thread: stage, block
+    __device__ __forceinline__ Quad2222(int64_t d, int64_t s, int64_t first_unit) : Pair44<S1>(d, s, first_unit) {
+        const int64_t alpha = this->base / (16 * s), beta = this->base - alpha * 16 * s;
+        const int q = this->q;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            c[0][b] = (8 * alpha + 2 * q + b) * s + beta;
+            c[1][b] = (4 * alpha + q) * 2 * s + b * s + beta;
+            c[2][b] = (2 * alpha + b) * 4 * s + q * s + beta;
+            c[3][b] = 8 * alpha * s + (q + 4 * b) * s + beta;
+        }
+    }
+};
+// stage of pairs (0, 1), (2, 3) (HI = 0) or (0, 2), (1, 3) (HI = 1) with kernels k[block][i][j]; T: transposed kernels
+template <int HI, bool T>
+__device__ __forceinline__ void mul22(const float (&x)[4], const float (&k)[2][2][2], float (&y)[4]) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int at0 = HI ? b : 2 * b, st = HI ? 2 : 1;
+            y[at0 + j * st] = fmaf(x[at0 + st], T ? k[b][j][1] : k[b][1][j], fmaf(x[at0], T ? k[b][j][0] : k[b][0][j], 0.f));
+        }
+}
+template <int HI>
+__device__ __forceinline__ void outer22(const double (&x)[4], const double (&g)[4], double *acc) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int at0 = HI ? b : 2 * b, st = HI ? 2 : 1;
+                acc[b * 4 + i * 2 + j] += x[at0 + i * st] * g[at0 + j * st];
+            }
+}
+__device__ __forceinline__ void widen(const float (&x)[4], double (&y)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) y[i] = (double)x[i];
+}
+struct Blocks4 { const float *em[4]; };
+struct Sums4 { double *part[4]; };
+
+template <bool S1, typename TI>
+__global__ void __launch_bounds__(kOwnThreads, kFwd44PerSm)
+fwd2222_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, float *__restrict__ out, int64_t rows, int64_t d, int64_t s, int slice, const Blocks4 em) {
+    using Rows = Rows44<S1, TI>;
+    __shared__ __align__(16) unsigned char ring[kOwnThreads / 32][kRing][Rows::kBytes];
+    const int w = threadIdx.x >> 5;
+    const Quad2222<S1> u(d, s, ((int64_t)blockIdx.x * (kOwnThreads / 32) + w) * 8);
+    const int64_t nblk = d / 2, in0 = u.base + 4 * u.q * s, out0 = S1 ? in0 : u.base + u.q * s, os = S1 ? 1 : 4 * s;
+    float k[4][2][2][2];
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int ij = 0; ij < 4; ++ij)
+                k[t][b][ij >> 1][ij & 1] = (t == 0 ? sign_of(signs, in0 + (2 * b + (ij >> 1)) * s) : 1.f) * em.em[t][(int64_t)ij * nblk + u.c[t][b]];
+    prior_kernel_done();
+    const int64_t r0 = (int64_t)blockIdx.y * slice, r1 = min(rows, r0 + slice);
+    const TI *src = in + r0 * d;
+    float *to = out + r0 * d + out0;
+#pragma unroll 1
+    for (int n = 0; n < kRing; ++n, src += d) {
+        if (r0 + n < r1) Rows::issue(ring[w][n], src, u, s);
+        ring_commit();
+    }
+    for (int64_t r = r0; r < r1; ++r, src += d, to += d) {
+        unsigned char *slot = ring[w][(int)(r - r0) & (kRing - 1)];
+        float x[4], y[4];
+        ring_wait();
+        Rows::first(slot, u, x);
+        __syncwarp();
+        if (r + kRing < r1) Rows::issue(slot, src, u, s);
+        ring_commit();
+        mul22<0, false>(x, k[0], y);
+        mul22<1, false>(y, k[1], x);
+        u.transpose(x);
+        mul22<0, false>(x, k[2], y);
+        mul22<1, false>(y, k[3], x);
+        if (S1) u.transpose(x);
+        if (u.have) store_block<4>(to, os, S1, x);
+    }
+}
+
+template <bool S1, typename TV, typename TG>
+__global__ void __launch_bounds__(32 * kSubs, k44PerSm)
+bwd2222_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const TG *__restrict__ g, float *__restrict__ g_out, int64_t rows, int64_t d, int64_t s,
+               int slice, int add, const Blocks4 em, const Sums4 part) {
+    using RowsV = Rows44<S1, TV>;
+    using RowsG = Rows44<S1, TG>;
+    constexpr int kSums = 32 * kSubs * 32 * 8, kRings = kSubs * kRing * (RowsV::kBytes + RowsG::kBytes);
+    __shared__ __align__(16) unsigned char smem[kRings > kSums ? kRings : kSums];               // the rings, then the warps' sums
+    const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
+    const Quad2222<S1> u(d, s, (int64_t)blockIdx.x * 8);
+    const int64_t nblk = d / 2, first = u.base + 4 * u.q * s;
+    float k[4][2][2][2], sg[4];                // k[0] with the signs of the step's coordinates
+    double acc[32];                            // [stage][block][i][j]
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sg[i] = sign_of(signs, first + i * s);
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int ij = 0; ij < 4; ++ij) {
+                k[t][b][ij >> 1][ij & 1] = (t == 0 ? sg[2 * b + (ij >> 1)] : 1.f) * em.em[t][(int64_t)ij * nblk + u.c[t][b]];
+                acc[t * 8 + b * 4 + ij] = 0.0;
+            }
+    prior_kernel_done();
+    const int64_t r0 = (int64_t)blockIdx.y * slice + sub, r1 = min(rows, (int64_t)(blockIdx.y + 1) * slice);
+    unsigned char *ring_v = smem + sub * kRing * RowsV::kBytes, *ring_g = smem + kSubs * kRing * RowsV::kBytes + sub * kRing * RowsG::kBytes;
+    const TV *pv = v + r0 * d;
+    const TG *pg = g + r0 * d;
+    float *w = g_out ? g_out + r0 * d + first : nullptr;
+#pragma unroll 1
+    for (int n = 0; n < kRing; ++n, pv += kSubs * d, pg += kSubs * d) {
+        if (r0 + n * kSubs < r1) {
+            RowsV::issue(ring_v + n * RowsV::kBytes, pv, u, s);
+            RowsG::issue(ring_g + n * RowsG::kBytes, pg, u, s);
+        }
+        ring_commit();
+    }
+    int n = 0;
+    for (int64_t r = r0; r < r1; r += kSubs, pv += kSubs * d, pg += kSubs * d, n = (n + 1) & (kRing - 1)) {
+        float x[4], gy[4], y[4], z[4], h[4];
+        double a[4], b[4];
+        ring_wait();
+        RowsV::first(ring_v + n * RowsV::kBytes, u, x);
+        RowsG::second(ring_g + n * RowsG::kBytes, u, gy);
+        __syncwarp();
+        if (r + kRing * kSubs < r1) {
+            RowsV::issue(ring_v + n * RowsV::kBytes, pv, u, s);
+            RowsG::issue(ring_g + n * RowsG::kBytes, pg, u, s);
+        }
+        ring_commit();
+        mul22<0, false>(x, k[0], y);           // x, y: states in front of the first and the second stage
+        mul22<1, false>(y, k[1], z);
+        u.transpose(z);                        // in front of the third
+        mul22<0, false>(z, k[2], h);           // in front of the fourth
+        widen(h, a);
+        widen(gy, b);
+        outer22<1>(a, b, acc + 24);
+        mul22<1, true>(gy, k[3], h);           // gradient behind the third
+        widen(z, a);
+        widen(h, b);
+        outer22<0>(a, b, acc + 16);
+        mul22<0, true>(h, k[2], gy);
+        u.transpose(gy);                       // behind the second
+        widen(y, a);
+        widen(gy, b);
+        outer22<1>(a, b, acc + 8);
+        mul22<1, true>(gy, k[1], h);           // behind the first
+        widen(x, a);
+        widen(h, b);
+        outer22<0>(a, b, acc);
+        if (w) {
+            mul22<0, true>(h, k[0], gy);
+            if (u.have) store_block<4>(w, s, S1, gy);
+            w += kSubs * d;
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = sg[e >> 1] < 0.f ? -acc[e] : acc[e];        // [block][i][j]: coordinate 2 block + i
+    combine<32, kSubs>(acc, reinterpret_cast<double (*)[kSubs][32]>(smem), sub, lane, add, [&](int e) -> double * {
+        return !u.have ? nullptr : part.part[e >> 3] + ((int64_t)blockIdx.y * 4 + (e & 3)) * nblk + u.c[e >> 3][(e >> 2) & 1];
     });
 }
 
@@ -544,6 +834,265 @@ bwd22_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
         const int b = (e >> 2) & 1, ij = e & 3;
         return e < 8 ? d1 + (int64_t)ij * nblk + u.c1[b] : d2 + (int64_t)ij * nblk + u.c2[b];
     });
+}
+
+// ---- one stage of radix 7, 8 or 16 on tiles in shared memory.  A CTA keeps NB neighbouring blocks and walks over tiles of eight rows that
+// asynchronous copies bring into a ring of buffers; every value is fetched once, where threads that own entries of a block fetch all
+// of the block's values.  Backward, the outer products of a block are a product of the fp64 tensor core (mma.m8n8k4, the rows as the
+// contraction; radix 7 in an 8 x 8 tile): a lane converts one value of v and one of g where entry owners convert
+// seventeen for two of theirs, and the sums take 2 registers an entry for 32 lanes together.
+template <int B, bool S1, typename T>
+struct Wide {
+    static constexpr int NB = B <= 8 ? 32 : 16, NBW = NB / 4;          // blocks of a CTA, of a warp
+    static constexpr int E = 16 / (int)sizeof(T);                      // elements of a copy
+    static constexpr int kRows = 8;
+    static constexpr int ST = S1 ? 1 : sizeof(T) == 4 ? NB + 4 : NB;   // from one value of a block to the next
+    static constexpr int BP = !S1 ? 1 : sizeof(T) == 4 && B % 4 == 0 ? B + 4 : B;      // from one block to the next
+    // rows apart: in fp32 eight banks (16-byte loads of four blocks for two values and four rows, 4-byte loads of eight values for four rows)
+    static constexpr int pitch() {
+        int rs = ((S1 ? NB * BP : B * ST) + E - 1) / E * E;
+        if (sizeof(T) == 4) while (rs % 32 != 8) rs += 4;
+        else rs += E;
+        return rs;
+    }
+    static constexpr int RS = pitch(), kElems = kRows * RS;
+    static constexpr int kPer = NB * B / E;                            // copies of a row; the CTA's threads are kGroup of them in kStep rows
+    static constexpr int kGroup = kPer > 32 ? 64 : 32, kStep = kOwnThreads / kGroup;
+    int64_t off;                       // of this thread's copies in a row, -1: none
+    int to;
+    __device__ __forceinline__ Wide(int64_t d, int64_t s) {
+        const int k = (int)threadIdx.x % kGroup;
+        const int64_t b0 = (int64_t)blockIdx.x * NB;
+        off = -1;
+        to = 0;
+        if (k >= kPer) return;
+        if constexpr (S1) {
+            const int e = k * E;
+            off = b0 * B + e;
+            if (off >= d) off = -1;
+            to = BP == B ? e : e / B * BP + e % B;
+        } else {
+            const int i = k / (NB / E), j = k % (NB / E) * E;
+            const int64_t c = b0 + j, alpha = c / s;
+            if (c < d / B) off = alpha * B * s + (c - alpha * s) + i * s;
+            to = i * ST + j;
+        }
+    }
+    // rows [r, r + 8) of the slice that ends at r1, zeros behind it
+    __device__ __forceinline__ void issue(T *buf, const T *x, int64_t d, int64_t r, int64_t r1) const {
+        if (off < 0) return;
+        const int first = (int)threadIdx.x / kGroup;
+#pragma unroll
+        for (int n = 0; n < kRows; n += kStep) {
+            const int64_t row = r + first + n;
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(buf + (first + n) * RS + to);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(x + (row < r1 ? row : r1 - 1) * d + off), "r"(row < r1 ? 16 : 0) : "memory");
+        }
+    }
+    // value i of four neighbouring blocks
+    static __device__ __forceinline__ void four(const T *row, int i, int blk, float (&v)[4]) {
+        if constexpr (S1) {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) v[b] = to_f32<T>(row[(blk + b) * BP + i]);
+        } else {
+            load_block<4, T>(row + i * ST + blk, 1, true, v);
+        }
+    }
+    // all values of a block
+    static __device__ __forceinline__ void block(const T *row, int blk, float (&v)[B]) {
+        load_block<B, T>(row + blk * BP, ST, S1 && (sizeof(T) == 2 || BP != B), v);
+    }
+};
+// products of a block with IPL of its kernel's columns (forward) or rows (backward): lane -> block, results i0.. and rows first, first + step, ..
+template <int B>
+struct WideLane {
+    static constexpr int IPL = 4;
+    int blk, i0, first;
+    static constexpr int step = 2;
+    __device__ __forceinline__ WideLane() {
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        if (B <= 8) { blk = 8 * w + (lane & 7); i0 = 4 * ((lane >> 3) & 1); first = lane >> 4; }
+        else { blk = 8 * (w & 1) + (lane & 7); i0 = 4 * (lane >> 3); first = w >> 1; }
+    }
+};
+template <int B, bool S1, typename T>
+__device__ __forceinline__ void wide_products(const T *tile, const WideLane<B> &l, const float (&k)[4][B], float *out, int64_t d, int64_t s, int rows) {
+#pragma unroll (B <= 8 ? 2 : 1)
+    for (int n = 0; n < 4; ++n) {
+        const int r = l.first + 2 * n;
+        float v[B], o[4];
+        Wide<B, S1, T>::block(tile + r * Wide<B, S1, T>::RS, l.blk, v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float a = 0.f;
+#pragma unroll
+            for (int j = 0; j < B; ++j) a = fmaf(v[j], k[i][j], a);
+            o[i] = a;
+        }
+        if (out && r < rows) {
+            float *p = out + (int64_t)r * d;
+            if (S1 && B % 4 == 0) {
+                *reinterpret_cast<float4 *>(p) = make_float4(o[0], o[1], o[2], o[3]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (l.i0 + i < B) p[i * s] = o[i];
+            }
+        }
+    }
+}
+constexpr int kWideFwdPerSm = 4, kWideBwdPerSm = 3, kWideStages = 3;
+
+template <int B, bool S1, typename TI>
+__global__ void __launch_bounds__(kOwnThreads, kWideFwdPerSm)
+wide_fwd_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, float *__restrict__ out, int64_t rows, int64_t d, int64_t s, int slice,
+                const float *__restrict__ em) {
+    using W = Wide<B, S1, TI>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TI *buf = reinterpret_cast<TI *>(smem_raw);
+    const W w(d, s);
+    const WideLane<B> l;
+    const int64_t nblk = d / B, c = (int64_t)blockIdx.x * W::NB + l.blk, cc = min(c, nblk - 1), alpha = cc / s, base = alpha * B * s + (cc - alpha * s);
+    float k[4][B];
+#pragma unroll
+    for (int j = 0; j < B; ++j) {
+        const float sg = sign_of(signs, base + j * s);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) k[i][j] = l.i0 + i < B ? sg * em[(int64_t)(j * B + l.i0 + i) * nblk + cc] : 0.f;
+    }
+    prior_kernel_done();
+    const int64_t r0 = (int64_t)blockIdx.y * slice, r1 = min(rows, r0 + slice);
+    float *to = c < nblk ? out + base + l.i0 * s : nullptr;
+    for (int n = 0; n < kWideStages - 1; ++n) {
+        if (r0 + n * W::kRows < r1) w.issue(buf + n * W::kElems, in, d, r0 + n * W::kRows, r1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    int at = 0;
+    for (int64_t r = r0; r < r1; r += W::kRows, at = at + 1 == kWideStages ? 0 : at + 1) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kWideStages - 2) : "memory");
+        __syncthreads();
+        const int next = at == 0 ? kWideStages - 1 : at - 1;
+        const int64_t rn = r + (kWideStages - 1) * W::kRows;
+        if (rn < r1) w.issue(buf + next * W::kElems, in, d, rn, r1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        wide_products<B, S1, TI>(buf + at * W::kElems, l, k, to ? to + r * d : nullptr, d, s, (int)min((int64_t)W::kRows, r1 - r));
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
+}
+
+template <int B, bool S1, typename TV, typename TG>
+__global__ void __launch_bounds__(kOwnThreads, kWideBwdPerSm)
+wide_bwd_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const TG *__restrict__ g, float *__restrict__ g_out, int64_t rows, int64_t d,
+                int64_t s, int slice, int add, const float *__restrict__ em, double *__restrict__ part) {
+    using WV = Wide<B, S1, TV>;
+    using WG = Wide<B, S1, TG>;
+    constexpr int H = B <= 8 ? 1 : 2, Q = WV::NBW / 4, NB = WV::NB;    // 8 x 8 tiles of a block along either side; groups of four blocks of a warp
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TV *buf_v = reinterpret_cast<TV *>(smem_raw);
+    TG *buf_g = reinterpret_cast<TG *>(smem_raw + kWideStages * WV::kElems * sizeof(TV));
+    const WV wv(d, s);
+    const WG wg(d, s);
+    const WideLane<B> l;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kr = lane & 3, mi = lane >> 2;
+    const int64_t nblk = d / B, c = (int64_t)blockIdx.x * NB + l.blk, cc = min(c, nblk - 1), alpha = cc / s, base = alpha * B * s + (cc - alpha * s);
+    float k[4][B];
+    if (!S1) {                             // (the gradient state in front of the first stage is not needed)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < B; ++j) k[i][j] = l.i0 + i < B ? em[(int64_t)((l.i0 + i) * B + j) * nblk + cc] : 0.f;
+    }
+    double acc[Q][4][H][H][2] = {};
+    prior_kernel_done();
+    const int64_t r0 = (int64_t)blockIdx.y * slice, r1 = min(rows, r0 + slice);
+    float *to = !S1 && g_out && c < nblk ? g_out + base + l.i0 * s : nullptr;
+    for (int n = 0; n < kWideStages - 1; ++n) {
+        if (r0 + n * 8 < r1) {
+            wv.issue(buf_v + n * WV::kElems, v, d, r0 + n * 8, r1);
+            wg.issue(buf_g + n * WG::kElems, g, d, r0 + n * 8, r1);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    int at = 0;
+    for (int64_t r = r0; r < r1; r += 8, at = at + 1 == kWideStages ? 0 : at + 1) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kWideStages - 2) : "memory");
+        __syncthreads();
+        const int next = at == 0 ? kWideStages - 1 : at - 1;
+        const int64_t rn = r + (kWideStages - 1) * 8;
+        if (rn < r1) {
+            wv.issue(buf_v + next * WV::kElems, v, d, rn, r1);
+            wg.issue(buf_g + next * WG::kElems, g, d, rn, r1);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const TV *tv = buf_v + at * WV::kElems;
+        const TG *tg = buf_g + at * WG::kElems;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int b0 = warp * WV::NBW + 4 * q;
+#pragma unroll
+            for (int n = 0; n < 8; n += 4) {
+                float a[H][4], b[H][4];
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const int i = min(8 * h + mi, B - 1);          // past the end of a radix of 7: entries that are not kept
+                    WV::four(tv + (n + kr) * WV::RS, i, b0, a[h]);
+                    WG::four(tg + (n + kr) * WG::RS, i, b0, b[h]);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    double bd[H];
+#pragma unroll
+                    for (int h = 0; h < H; ++h) bd[h] = (double)b[h][e];
+#pragma unroll
+                    for (int hi = 0; hi < H; ++hi) {
+                        const double ad = (double)a[hi][e];
+#pragma unroll
+                        for (int hj = 0; hj < H; ++hj) dmma(acc[q][e][hi][hj], ad, bd[hj]);
+                    }
+                }
+            }
+        }
+        if (!S1 && g_out) wide_products<B, S1, TG>(tg, l, k, to ? to + r * d : nullptr, d, s, (int)min((int64_t)8, r1 - r));
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // by way of shared memory, [entry][block]: neighbouring threads add to neighbouring sums
+    double *sums = reinterpret_cast<double *>(smem_raw);
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int bl = warp * WV::NBW + 4 * q + e;
+            const int64_t ce = min((int64_t)blockIdx.x * NB + bl, nblk - 1), al = ce / s, be = al * B * s + (ce - al * s);
+#pragma unroll
+            for (int hi = 0; hi < H; ++hi) {
+                const int i = 8 * hi + mi;
+                if (i >= B) continue;
+                const bool neg = signs && signs[be + i * s] < 0;
+#pragma unroll
+                for (int hj = 0; hj < H; ++hj)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int j = 8 * hj + 2 * kr + h;
+                        if (j < B) sums[(i * B + j) * (NB + 1) + bl] = neg ? -acc[q][e][hi][hj][h] : acc[q][e][hi][hj][h];
+                    }
+            }
+        }
+    __syncthreads();
+    double *dst = part + (int64_t)blockIdx.y * (B * B) * nblk + (int64_t)blockIdx.x * NB;
+    const int nb = (int)min((int64_t)NB, nblk - (int64_t)blockIdx.x * NB);
+#pragma unroll 4
+    for (int n = threadIdx.x; n < B * B * NB; n += kOwnThreads) {
+        const int ij = n / NB, bl = n % NB;
+        if (bl >= nb) continue;
+        double *p = dst + (int64_t)ij * nblk + bl;
+        const double x = sums[ij * (NB + 1) + bl];
+        *p = add ? *p + x : x;
+    }
 }
 
 // ---- sums over slices of all stages that keep partial sums: grad[c][i][j] (+)= sum over slices of part[slice][i b + j][c],
@@ -753,15 +1302,31 @@ dim3 column_grid(int64_t d, int64_t rows) {
 
 // ---- steps of a plan
 
-struct Step { int t, n; };             // stages [t, t + n): one stage, or two of radix 4 or of radix 2
+struct Step { int t, n; bool wide; };  // stages [t, t + n): one stage, two of radix 4 or of radix 2, or four of radix 2; wide: one, on tiles in shared memory
 
-std::vector<Step> make_steps(const StageTable &st) {
+// rows by asynchronous copies: eight neighbouring units are whole 16-byte pieces, the unit's sixteen coordinates make d a multiple of sixteen
+bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+bool ring44(int64_t s, const void *p) { return (s == 1 || s % 8 == 0) && aligned16(p); }
+
+// stages on tiles in shared memory: whole 16-byte pieces of neighbouring blocks
+bool wide_stage(const StageTable &st, int64_t d, int t, size_t es, const void *p) {
+    const int b = st.b[t];
+    const int64_t e = 16 / (int64_t)es;
+    return (b == 7 || b == 8 || b == 16) && (t == 0 ? d % e == 0 : st.s[t] % e == 0) && aligned16(p);
+}
+
+// in, gy: the call's rows (the states of other steps start on 16-byte boundaries)
+std::vector<Step> make_steps(const StageTable &st, int64_t d, size_t es, const void *in, const void *gy) {
     std::vector<Step> steps;
     for (int t = 0; t < st.m;) {
         const int b = st.b[t];
-        const bool two = t + 1 < st.m && st.b[t + 1] == b && (b == 4 || b == 2);
-        steps.push_back({t, two ? 2 : 1});
-        t += two ? 2 : 1;
+        int n = 1;
+        while (n < 4 && t + n < st.m && st.b[t + n] == b) ++n;
+        if (b == 2 && n == 4 && ring44(st.s[t], t == 0 ? in : nullptr) && aligned16(t + n == st.m ? gy : nullptr)) n = 4;
+        else n = n >= 2 && (b == 4 || b == 2) ? 2 : 1;
+        const bool first = t == 0, last = t + n == st.m;
+        steps.push_back({t, n, n == 1 && wide_stage(st, d, t, first ? es : 4, first ? in : nullptr) && wide_stage(st, d, t, last ? es : 4, last ? gy : nullptr)});
+        t += n;
     }
     return steps;
 }
@@ -773,7 +1338,8 @@ struct Shape { int64_t x; int per_sm; };
 Shape bwd_shape(const harp_plan *plan, const Step &sp) {
     const int64_t d = plan->d;
     const int b = plan->st.b[sp.t];
-    if (sp.n == 2) return b == 4 ? Shape{(d / 16 + 7) / 8, k44PerSm} : Shape{(d / 4 + 31) / 32, 4};
+    if (sp.wide) return {(d / b + (b <= 8 ? 31 : 15)) / (b <= 8 ? 32 : 16), kWideBwdPerSm};
+    if (sp.n > 1) return b == 4 || sp.n == 4 ? Shape{(d / 16 + 7) / 8, k44PerSm} : Shape{(d / 4 + 31) / 32, 4};
     const int64_t x = (d / b + 31) / 32;
     switch (b) {
         case 7: return {x, bwd_per_sm(7, 4, 2)};
@@ -790,29 +1356,58 @@ int slice_rows(const harp_plan *plan, const Step &sp, int64_t rows, int sms) {
     // Narrow plans, whose wave has hundreds of slices: a slice's rows are a serial chain of the backward kernel, shared by `subs` warps, and
     // the slices one of the reduction, shared by eight; near the root of the rows the two last equally long (8192 rows of
     // d = 2: 592 slices 23.9 us, 158 slices 9.7)
-    const int b = plan->st.b[sp.t], subs = sp.n == 2 ? kSubs : b == 16 ? 1 : b == 7 || b == 8 ? 2 : kSubs;
+    const int b = plan->st.b[sp.t], subs = sp.n > 1 || sp.wide ? kSubs : b == 16 ? 1 : b == 7 || b == 8 ? 2 : kSubs;
     const int64_t even = (int64_t)(0.125 * subs * std::sqrt((double)rows));
-    return (int)std::max<int64_t>(std::max<int64_t>(8, even), (rows + y - 1) / y);
+    const int64_t n = std::max<int64_t>(std::max<int64_t>(8, even), (rows + y - 1) / y);
+    return (int)(sp.wide ? (n + 7) / 8 * 8 : n);
 }
-bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 dim3 grid2(int64_t x, int per_x, int64_t rows, int per_y) { return dim3((unsigned)((x + per_x - 1) / per_x), (unsigned)((rows + per_y - 1) / per_y)); }
 
 // one step forward: out = in through the step's stages
 template <typename TI>
-void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int8_t *signs, float *out, int64_t rows, cudaStream_t st) {
+void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int8_t *signs, float *out, int64_t rows, int sms, cudaStream_t st) {
     const int64_t d = plan->d, s = plan->st.s[sp.t];
     const int b = plan->st.b[sp.t];
     const float *em = plan->d_blocks_em + plan->st.off[sp.t];
     const float *em2 = sp.n == 2 ? plan->d_blocks_em + plan->st.off[sp.t + 1] : nullptr;
     const int vec = s == 1 && d % 4 == 0 && aligned16(in);
-    if (sp.n == 2 && b == 4) {
-        const dim3 grid = grid2(d / 16, 8 * (kOwnThreads / 32), rows, kFwdRows);
-        if (s == 1) launch_dep(fwd44_kernel<true, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, em, em2);
-        else launch_dep(fwd44_kernel<false, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, em, em2);
+    if (sp.n == 4 || (sp.n == 2 && b == 4)) {
+        // one wave of CTAs, like the backward kernels
+        const int64_t x = (d / 16 + 8 * (kOwnThreads / 32) - 1) / (8 * (kOwnThreads / 32)), y = std::max<int64_t>(1, sms * (int64_t)kFwd44PerSm / x);
+        const int slice = (int)std::max<int64_t>(kFwdRows / 2, (rows + y - 1) / y);
+        const dim3 grid = grid2(d / 16, 8 * (kOwnThreads / 32), rows, slice);
+        if (sp.n == 4) {
+            Blocks4 k;
+            for (int t = 0; t < 4; ++t) k.em[t] = plan->d_blocks_em + plan->st.off[sp.t + t];
+            if (s == 1) launch_dep(fwd2222_kernel<true, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, out, rows, d, s, slice, k);
+            else launch_dep(fwd2222_kernel<false, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, out, rows, d, s, slice, k);
+            return;
+        }
+        auto go = [&](auto s1, auto ring) {
+            launch_dep(fwd44_kernel<decltype(s1)::value, decltype(ring)::value, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, slice, em, em2);
+        };
+        using std::true_type; using std::false_type;
+        if (ring44(s, in)) s == 1 ? go(true_type(), true_type()) : go(false_type(), true_type());
+        else s == 1 ? go(true_type(), false_type()) : go(false_type(), false_type());
         return;
     }
     if (sp.n == 2) {
         launch_dep(fwd22_kernel<TI>, grid2(d / 4, kOwnThreads, rows, kFwdRows), dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, em, em2);
+        return;
+    }
+    if (wide_stage(plan->st, d, sp.t, sizeof(TI), in)) {
+        auto go = [&](auto bc, auto s1) {
+            constexpr int B = decltype(bc)::value;
+            using W = Wide<B, decltype(s1)::value, TI>;
+            const int64_t x = (d / B + W::NB - 1) / W::NB, y = std::max<int64_t>(1, sms * (int64_t)kWideFwdPerSm / x);
+            const int slice = (int)((std::max<int64_t>(1, (rows + y - 1) / y) + 7) / 8 * 8);
+            launch_dep(wide_fwd_kernel<B, decltype(s1)::value, TI>, dim3((unsigned)x, (unsigned)((rows + slice - 1) / slice)), dim3(kOwnThreads),
+                       kWideStages * W::kElems * sizeof(TI), st, in, signs, out, rows, d, s, slice, em);
+        };
+        using std::true_type; using std::false_type;
+        if (b == 7) s == 1 ? go(std::integral_constant<int, 7>(), true_type()) : go(std::integral_constant<int, 7>(), false_type());
+        else if (b == 8) s == 1 ? go(std::integral_constant<int, 8>(), true_type()) : go(std::integral_constant<int, 8>(), false_type());
+        else s == 1 ? go(std::integral_constant<int, 16>(), true_type()) : go(std::integral_constant<int, 16>(), false_type());
         return;
     }
 #define HARP_FWD(B, OUT) case B: launch_dep(fwd_kernel<B, OUT, TI>, grid2(d / B, kOwnThreads / (B / OUT), rows, kFwdRows), dim3(kOwnThreads), 0, st, in, signs, vec, out, rows, d, s, em); return
@@ -829,21 +1424,53 @@ void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int
 // one step backward: g_out (unless null) from g, sums of the step's outer products into part (or, radices without owner
 // kernels, into grad)
 template <typename TV, typename TG>
-int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8_t *signs, const TG *g, float *g_out, int64_t rows, double *part, double *part2,
+int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8_t *signs, const TG *g, float *g_out, int64_t rows, double *all_parts, const int64_t *part_off,
                   int slice, int add, float *grad, int acc, cudaStream_t st) {
     const int64_t d = plan->d, s = plan->st.s[sp.t];
     const int b = plan->st.b[sp.t];
     const float *em = plan->d_blocks_em + plan->st.off[sp.t];
     const float *em2 = sp.n == 2 ? plan->d_blocks_em + plan->st.off[sp.t + 1] : nullptr;
     const int vec_v = s == 1 && d % 4 == 0 && aligned16(v), vec_g = s == 1 && d % 4 == 0 && aligned16(g);
+    double *part = all_parts + part_off[sp.t], *part2 = sp.n == 2 ? all_parts + part_off[sp.t + 1] : nullptr;
+    if (sp.n == 4) {
+        const dim3 grid = grid2(d / 16, 8, rows, slice);
+        Blocks4 k;
+        Sums4 sums;
+        for (int t = 0; t < 4; ++t) { k.em[t] = plan->d_blocks_em + plan->st.off[sp.t + t]; sums.part[t] = all_parts + part_off[sp.t + t]; }
+        if (s == 1) launch_dep(bwd2222_kernel<true, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, g, g_out, rows, d, s, slice, add, k, sums);
+        else launch_dep(bwd2222_kernel<false, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, g, g_out, rows, d, s, slice, add, k, sums);
+        return 1;
+    }
     if (sp.n == 2 && b == 4) {
         const dim3 grid = grid2(d / 16, 8, rows, slice);
-        if (s == 1) launch_dep(bwd44_kernel<true, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, em2, part, part2);
-        else launch_dep(bwd44_kernel<false, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, em2, part, part2);
+        auto go = [&](auto s1, auto ring) {
+            launch_dep(bwd44_kernel<decltype(s1)::value, decltype(ring)::value, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, em2, part, part2);
+        };
+        using std::true_type; using std::false_type;
+        if (ring44(s, v) && ring44(s, g)) s == 1 ? go(true_type(), true_type()) : go(false_type(), true_type());
+        else s == 1 ? go(true_type(), false_type()) : go(false_type(), false_type());
         return 1;
     }
     if (sp.n == 2) {
         launch_dep(bwd22_kernel<TV, TG>, grid2(d / 4, 32, rows, slice), dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, em2, part, part2);
+        return 1;
+    }
+    if (sp.wide) {
+        auto go = [&](auto bc, auto s1) {
+            constexpr int B = decltype(bc)::value;
+            using WV = Wide<B, decltype(s1)::value, TV>;
+            using WG = Wide<B, decltype(s1)::value, TG>;
+            const auto kern = wide_bwd_kernel<B, decltype(s1)::value, TV, TG>;
+            const size_t smem = std::max(kWideStages * (WV::kElems * sizeof(TV) + WG::kElems * sizeof(TG)), sizeof(double) * B * B * (WV::NB + 1));      // the ring, then the sums
+            // per call: the attribute belongs to the current device's copy of the kernel
+            if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            launch_dep(kern, dim3((unsigned)((d / B + WV::NB - 1) / WV::NB), (unsigned)((rows + slice - 1) / slice)), dim3(kOwnThreads), smem, st,
+                       v, signs, g, g_out, rows, d, s, slice, add, em, part);
+        };
+        using std::true_type; using std::false_type;
+        if (b == 7) s == 1 ? go(std::integral_constant<int, 7>(), true_type()) : go(std::integral_constant<int, 7>(), false_type());
+        else if (b == 8) s == 1 ? go(std::integral_constant<int, 8>(), true_type()) : go(std::integral_constant<int, 8>(), false_type());
+        else s == 1 ? go(std::integral_constant<int, 16>(), true_type()) : go(std::integral_constant<int, 16>(), false_type());
         return 1;
     }
 #define HARP_BWD(B, BI, SUBS) case B: launch_dep(bwd_kernel<B, BI, SUBS, TV, TG>, grid2(d / B, 32, rows, slice), dim3(32 * ((B + BI - 1) / BI) * SUBS), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, part); return 1
@@ -866,7 +1493,7 @@ template <typename T>
 harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_t n_rows, float *grad, int accumulate, cudaStream_t st) {
     const int64_t d = plan->d;
     const StageTable &tab = plan->st;
-    const std::vector<Step> steps = make_steps(tab);
+    const std::vector<Step> steps = make_steps(tab, d, sizeof(T), plan->d_perm ? nullptr : x, gy);
     const int n = (int)steps.size(), n_g = std::min(n - 1, 2), ring = std::max(1, n_g);
     const bool permuted = plan->d_perm != nullptr;
     // chunk of rows whose forward states, gradient states and permuted rows fit about 200 MB; the partial sums of a wave of
@@ -927,19 +1554,18 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
             ++launches;
         }
         for (int k = 0; k + 1 < n; ++k, ++launches) {
-            if (k == 0) step_forward<T>(plan, steps[0], xc, signs, vp, rows, st);
-            else step_forward<float>(plan, steps[(size_t)k], vp + (k - 1) * plane, nullptr, vp + k * plane, rows, st);
+            if (k == 0) step_forward<T>(plan, steps[0], xc, signs, vp, rows, sms, st);
+            else step_forward<float>(plan, steps[(size_t)k], vp + (k - 1) * plane, nullptr, vp + k * plane, rows, sms, st);
         }
         for (int k = n - 1; k >= 0; --k) {
             const Step &sp = steps[(size_t)k];
             const float *v_in = vp + (k - 1) * plane, *g_in = gp + ((k + 1) % ring) * plane;
             float *out = k > 0 ? gp + (k % ring) * plane : nullptr;
             const int slice = slice_rows(plan, sp, chunk, sms);
-            double *p1 = part + part_off[sp.t], *p2 = sp.n == 2 ? part + part_off[sp.t + 1] : nullptr;
-            if (k == 0 && k == n - 1) launches += step_backward<T, T>(plan, sp, xc, signs, gc, out, rows, p1, p2, slice, r0 > 0, grad, acc, st);
-            else if (k == n - 1) launches += step_backward<float, T>(plan, sp, v_in, nullptr, gc, out, rows, p1, p2, slice, r0 > 0, grad, acc, st);
-            else if (k == 0) launches += step_backward<T, float>(plan, sp, xc, signs, g_in, out, rows, p1, p2, slice, r0 > 0, grad, acc, st);
-            else launches += step_backward<float, float>(plan, sp, v_in, nullptr, g_in, out, rows, p1, p2, slice, r0 > 0, grad, acc, st);
+            if (k == 0 && k == n - 1) launches += step_backward<T, T>(plan, sp, xc, signs, gc, out, rows, part, part_off, slice, r0 > 0, grad, acc, st);
+            else if (k == n - 1) launches += step_backward<float, T>(plan, sp, v_in, nullptr, gc, out, rows, part, part_off, slice, r0 > 0, grad, acc, st);
+            else if (k == 0) launches += step_backward<T, float>(plan, sp, xc, signs, g_in, out, rows, part, part_off, slice, r0 > 0, grad, acc, st);
+            else launches += step_backward<float, float>(plan, sp, v_in, nullptr, g_in, out, rows, part, part_off, slice, r0 > 0, grad, acc, st);
         }
         if (red.m > 0 && r0 + chunk >= n_rows) {
             for (int k = 0; k < red.m; ++k) red.st[k].n_slices = (int32_t)((chunk + red.st[k].rows - 1) / red.st[k].rows);

@@ -220,3 +220,38 @@ def test_parameter_gradient_of_a_plan_built_from_theta():
             # the loss is smooth; blocks are rounded to fp32 inside loss(), hence the loose step and bound
             fd = (loss(tp) - loss(tm)) / (2 * h)
             assert abs(g_theta[c, k] - fd) <= 2e-3 * max(1.0, abs(fd)), (t, c, k, g_theta[c, k], fd)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("n_rows", [1, 9, 75])
+@pytest.mark.parametrize("radices", [(2, 2, 2, 2), (2,) * 9, (2, 2, 2, 2, 4, 4), (3, 4, 4), (4, 4, 3, 4, 4), (8, 16, 7), (16, 16), (8, 8, 2), (7, 4, 8), (4, 8, 3, 16)])
+def test_steps_fed_by_asynchronous_copies(dtype, n_rows, radices):
+    """Four radix-2 stages a step and two radix-4 ones (at stride one, at multiples of eight, and at a stride of three, whose rows take
+    plain loads), stages of radix 7, 8 and 16 on tiles of eight rows (whole and in part, blocks in a row and strided)."""
+    spec = wl.tiny_plan(39, radices, kind="qr", perm="identity", signs=True)
+    plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
+    xh, gh = _rows(40, n_rows, spec.d, dtype)
+    got, _, _ = _gpu_grad(plan, xh, gh, dtype)
+    want = _flat(orc.grad_blocks(oplan, promote(xh, dtype), promote(gh, dtype)))
+    assert np.max(np.abs(got - want)) <= 2e-5 * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("radices", [(2, 2, 2, 2), (4, 4, 4, 4), (8, 8), (16, 7)])
+def test_rows_off_sixteen_byte_boundaries(dtype, radices):
+    """Rows that start one element behind a 16-byte boundary take the kernels with plain loads; both sums are the same."""
+    spec = wl.tiny_plan(41, radices, kind="qr", perm="identity", signs=True)
+    plan = harp.plan_from_spec(spec)
+    xh, gh = _rows(42, 21, spec.d, dtype)
+    got, x_d, g_d = _gpu_grad(plan, xh, gh, dtype)
+    for shift_x, shift_g in ((1, 0), (0, 1), (1, 1)):
+        bufs = []
+        for t, shift in ((x_d, shift_x), (g_d, shift_g)):
+            b = torch.empty(t.numel() + 8, dtype=t.dtype, device="cuda")
+            b[shift:shift + t.numel()] = t.reshape(-1)
+            bufs.append((b, b.data_ptr() + shift * t.element_size()))
+        out = torch.zeros(harp.harp_plan_n_params(plan), dtype=torch.float32, device="cuda")
+        harp.harp_grad_blocks(plan, bufs[0][1], bufs[1][1], 21, DT[dtype], out.data_ptr(), False, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        # the same fp32 states and fp64 sums in another order: a rounding of the result
+        assert np.max(np.abs(out.cpu().numpy() - got)) <= 1e-6 * np.max(np.abs(got))
