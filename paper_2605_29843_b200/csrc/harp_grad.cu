@@ -190,7 +190,7 @@ bwd_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec_v
     const int64_t r0 = (int64_t)blockIdx.y * slice, r1 = min(rows, r0 + slice);
     constexpr bool kWhole = B % BI == 0;
     const bool vec_o = s == 1 && kWhole;
-#pragma unroll (B >= 7 ? 1 : 2)
+#pragma unroll (B >= 7 ? 1 : B <= 3 ? 4 : 2)
     for (int64_t r = r0 + sub; r < r1; r += SUBS) {
         float vv[BI], gg[B];
         if constexpr (kWhole) {
@@ -254,20 +254,16 @@ struct Pair44 {
         c1 = (4 * alpha + q) * s + beta;
         c2 = alpha * 4 * s + beta + q * s;
     }
-    // x[i] of thread q becomes x[q] of thread i
-    __device__ __forceinline__ void transpose(float (&x)[4]) const {
-        constexpr int M1 = S1 ? 1 : 8, M2 = S1 ? 2 : 16;
-        const bool b0 = q & 1, b1 = q & 2;
+    // x[i] of thread q becomes x[q] of thread i, by way of kSwap words of the warp's own (a 16-byte store and four loads, free of bank
+    // conflicts; two rounds of shuffles and selects are twenty instructions).  The warp synchronises before the words are written again.
+    static constexpr int kSwap = 160;
+    __device__ __forceinline__ void transpose(float *words, float (&x)[4]) const {
+        const int lane = threadIdx.x & 31;
+        float *w = words + (S1 ? lane >> 2 : lane & 7) * 20;
+        *reinterpret_cast<float4 *>(w + 4 * q) = make_float4(x[0], x[1], x[2], x[3]);
+        __syncwarp();
 #pragma unroll
-        for (int h = 0; h < 4; h += 2) {
-            const float r = __shfl_xor_sync(0xffffffffu, b0 ? x[h] : x[h + 1], M1);
-            if (b0) x[h] = r; else x[h + 1] = r;
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float r = __shfl_xor_sync(0xffffffffu, b1 ? x[h] : x[h + 2], M2);
-            if (b1) x[h] = r; else x[h + 2] = r;
-        }
+        for (int i = 0; i < 4; ++i) x[i] = w[4 * i + q];
     }
 };
 __device__ __forceinline__ void mul4(const float (&x)[4], const float (&k)[4][4], float (&y)[4]) {        // y_j = sum_i x_i k[i][j]
@@ -342,6 +338,7 @@ fwd44_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int ve
              const float *__restrict__ em1, const float *__restrict__ em2) {
     using Rows = Rows44<S1, TI>;
     __shared__ __align__(16) unsigned char ring[RING ? kOwnThreads / 32 : 1][RING ? kRing : 1][RING ? Rows::kBytes : 16];
+    __shared__ __align__(16) float words[kOwnThreads / 32][S1 ? 2 : 1][Pair44<S1>::kSwap];
     const int w = threadIdx.x >> 5;
     const Pair44<S1> u(d, s, ((int64_t)blockIdx.x * (kOwnThreads / 32) + w) * 8);
     const int64_t nblk = d / 4, in0 = u.base + 4 * u.q * s, out0 = S1 ? in0 : u.base + u.q * s, os = S1 ? 1 : 4 * s;
@@ -361,11 +358,12 @@ fwd44_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, int ve
     auto row = [&](const float (&x)[4]) {
         float y[4], z[4];
         mul4(x, k1, y);
-        u.transpose(y);
+        u.transpose(words[w][0], y);
         mul4(y, k2, z);
-        if (S1) u.transpose(z);
+        if (S1) u.transpose(words[w][S1 ? 1 : 0], z);
         if (u.have) store_block<4>(to, os, S1, z);
         to += d;
+        if (!RING) __syncwarp();
     };
     if constexpr (RING) {
         const TI *src = in + r0 * d;
@@ -407,6 +405,7 @@ bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
     using RowsG = Rows44<S1, TG>;
     constexpr int kSums = 32 * kSubs * 32 * 8, kRings = kSubs * kRing * (RowsV::kBytes + RowsG::kBytes);
     __shared__ __align__(16) unsigned char smem[RING && kRings > kSums ? kRings : kSums];        // the rings, then the warps' sums
+    __shared__ __align__(16) float words[kSubs][2][Pair44<S1>::kSwap];
     const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
     const Pair44<S1> u(d, s, (int64_t)blockIdx.x * 8);
     const int64_t nblk = d / 4, first = u.base + 4 * u.q * s, second = S1 ? first : u.base + u.q * s, gs = S1 ? 1 : 4 * s;
@@ -429,7 +428,9 @@ bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
     auto row = [&](const float (&x)[4], const float (&gy)[4]) {
         float y[4], h[4];
         mul4(x, k1, y);
-        u.transpose(y);
+        mul4t(gy, k2, h);
+        u.transpose(words[sub][0], y);
+        u.transpose(words[sub][1], h);
         {
             double gd[4];
 #pragma unroll
@@ -441,8 +442,6 @@ bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
                 for (int j = 0; j < 4; ++j) acc[16 + i * 4 + j] += vd * gd[j];
             }
         }
-        mul4t(gy, k2, h);
-        u.transpose(h);
         {
             double gd[4];
 #pragma unroll
@@ -507,8 +506,12 @@ bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
                 load_block<4, TV>(pv, s, vec_v, nv);
                 load_block<4, TG>(pg, gs, vec_g, ng);
             }
-            if (S1) u.transpose(gy);
+            if (S1) {
+                u.transpose(words[sub][0], gy);
+                __syncwarp();
+            }
             row(x, gy);
+            __syncwarp();
         }
     }
 #pragma unroll
@@ -521,7 +524,7 @@ bwd44_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
     });
 }
 
-// ---- four radix-2 stages of strides s, 2 s, 4 s and 8 s on the same units: a thread holds two stages' blocks in the first order (coordinate
+// ---- four radix-2 stages of strides s, 2 s, 4 s and 8 s (NS = 3: the first three of them) on the same units: a thread holds two stages' blocks in the first order (coordinate
 // i of four: pairs i, i ^ 1, then i, i ^ 2) and the other two stages' in the second.  As much register space for kernels and sums as two
 // radix-4 stages, and half the state traffic of two radix-2 stages a step.
 template <bool S1>
@@ -569,17 +572,18 @@ __device__ __forceinline__ void widen(const float (&x)[4], double (&y)[4]) {
 struct Blocks4 { const float *em[4]; };
 struct Sums4 { double *part[4]; };
 
-template <bool S1, typename TI>
+template <int NS, bool S1, typename TI>
 __global__ void __launch_bounds__(kOwnThreads, kFwd44PerSm)
 fwd2222_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, float *__restrict__ out, int64_t rows, int64_t d, int64_t s, int slice, const Blocks4 em) {
     using Rows = Rows44<S1, TI>;
     __shared__ __align__(16) unsigned char ring[kOwnThreads / 32][kRing][Rows::kBytes];
+    __shared__ __align__(16) float words[kOwnThreads / 32][S1 ? 2 : 1][Pair44<S1>::kSwap];
     const int w = threadIdx.x >> 5;
     const Quad2222<S1> u(d, s, ((int64_t)blockIdx.x * (kOwnThreads / 32) + w) * 8);
     const int64_t nblk = d / 2, in0 = u.base + 4 * u.q * s, out0 = S1 ? in0 : u.base + u.q * s, os = S1 ? 1 : 4 * s;
-    float k[4][2][2][2];
+    float k[NS][2][2][2];
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
+    for (int t = 0; t < NS; ++t)
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
@@ -604,31 +608,37 @@ fwd2222_kernel(const TI *__restrict__ in, const int8_t *__restrict__ signs, floa
         ring_commit();
         mul22<0, false>(x, k[0], y);
         mul22<1, false>(y, k[1], x);
-        u.transpose(x);
+        u.transpose(words[w][0], x);
         mul22<0, false>(x, k[2], y);
-        mul22<1, false>(y, k[3], x);
-        if (S1) u.transpose(x);
+        if constexpr (NS == 4) {
+            mul22<1, false>(y, k[3], x);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] = y[i];
+        }
+        if (S1) u.transpose(words[w][S1 ? 1 : 0], x);
         if (u.have) store_block<4>(to, os, S1, x);
     }
 }
 
-template <bool S1, typename TV, typename TG>
+template <int NS, bool S1, typename TV, typename TG>
 __global__ void __launch_bounds__(32 * kSubs, k44PerSm)
 bwd2222_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const TG *__restrict__ g, float *__restrict__ g_out, int64_t rows, int64_t d, int64_t s,
                int slice, int add, const Blocks4 em, const Sums4 part) {
     using RowsV = Rows44<S1, TV>;
     using RowsG = Rows44<S1, TG>;
-    constexpr int kSums = 32 * kSubs * 32 * 8, kRings = kSubs * kRing * (RowsV::kBytes + RowsG::kBytes);
+    constexpr int kSums = 8 * NS * kSubs * 32 * 8, kRings = kSubs * kRing * (RowsV::kBytes + RowsG::kBytes);
     __shared__ __align__(16) unsigned char smem[kRings > kSums ? kRings : kSums];               // the rings, then the warps' sums
+    __shared__ __align__(16) float words[kSubs][2][Pair44<S1>::kSwap];
     const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
     const Quad2222<S1> u(d, s, (int64_t)blockIdx.x * 8);
     const int64_t nblk = d / 2, first = u.base + 4 * u.q * s;
-    float k[4][2][2][2], sg[4];                // k[0] with the signs of the step's coordinates
-    double acc[32];                            // [stage][block][i][j]
+    float k[NS][2][2][2], sg[4];                // k[0] with the signs of the step's coordinates
+    double acc[8 * NS];                        // [stage][block][i][j]
 #pragma unroll
     for (int i = 0; i < 4; ++i) sg[i] = sign_of(signs, first + i * s);
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
+    for (int t = 0; t < NS; ++t)
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
@@ -665,17 +675,22 @@ bwd2222_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const
         ring_commit();
         mul22<0, false>(x, k[0], y);           // x, y: states in front of the first and the second stage
         mul22<1, false>(y, k[1], z);
-        u.transpose(z);                        // in front of the third
-        mul22<0, false>(z, k[2], h);           // in front of the fourth
-        widen(h, a);
-        widen(gy, b);
-        outer22<1>(a, b, acc + 24);
-        mul22<1, true>(gy, k[3], h);           // gradient behind the third
+        u.transpose(words[sub][0], z);         // in front of the third
+        if constexpr (NS == 4) {
+            mul22<0, false>(z, k[2], h);       // in front of the fourth
+            widen(h, a);
+            widen(gy, b);
+            outer22<1>(a, b, acc + 24);
+            mul22<1, true>(gy, k[3], h);       // gradient behind the third
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) h[i] = gy[i];
+        }
         widen(z, a);
         widen(h, b);
         outer22<0>(a, b, acc + 16);
         mul22<0, true>(h, k[2], gy);
-        u.transpose(gy);                       // behind the second
+        u.transpose(words[sub][1], gy);        // behind the second
         widen(y, a);
         widen(gy, b);
         outer22<1>(a, b, acc + 8);
@@ -693,7 +708,7 @@ bwd2222_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = sg[e >> 1] < 0.f ? -acc[e] : acc[e];        // [block][i][j]: coordinate 2 block + i
-    combine<32, kSubs>(acc, reinterpret_cast<double (*)[kSubs][32]>(smem), sub, lane, add, [&](int e) -> double * {
+    combine<8 * NS, kSubs>(acc, reinterpret_cast<double (*)[kSubs][32]>(smem), sub, lane, add, [&](int e) -> double * {
         return !u.have ? nullptr : part.part[e >> 3] + ((int64_t)blockIdx.y * 4 + (e & 3)) * nblk + u.c[e >> 3][(e >> 2) & 1];
     });
 }
@@ -1302,7 +1317,7 @@ dim3 column_grid(int64_t d, int64_t rows) {
 
 // ---- steps of a plan
 
-struct Step { int t, n; bool wide; };  // stages [t, t + n): one stage, two of radix 4 or of radix 2, or four of radix 2; wide: one, on tiles in shared memory
+struct Step { int t, n; bool wide; };  // stages [t, t + n): one stage, two of radix 4 or of radix 2, or three or four of radix 2; wide: one, on tiles in shared memory
 
 // rows by asynchronous copies: eight neighbouring units are whole 16-byte pieces, the unit's sixteen coordinates make d a multiple of sixteen
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -1321,9 +1336,11 @@ std::vector<Step> make_steps(const StageTable &st, int64_t d, size_t es, const v
     for (int t = 0; t < st.m;) {
         const int b = st.b[t];
         int n = 1;
-        while (n < 4 && t + n < st.m && st.b[t + n] == b) ++n;
-        if (b == 2 && n == 4 && ring44(st.s[t], t == 0 ? in : nullptr) && aligned16(t + n == st.m ? gy : nullptr)) n = 4;
-        else n = n >= 2 && (b == 4 || b == 2) ? 2 : 1;
+        while (t + n < st.m && st.b[t + n] == b) ++n;
+        // radix 2: threes in front so that fours are left over (d = 2048: 3 + 4 + 4; a three leaves a stride that is a multiple of eight behind it)
+        const int k = n % 4 == 0 ? 4 : 3;
+        const bool ring = b == 2 && n >= 3 && d % (16 * (int64_t)st.s[t]) == 0 && ring44(st.s[t], t == 0 ? in : nullptr) && aligned16(t + k == st.m ? gy : nullptr);
+        n = ring ? k : n >= 2 && (b == 4 || b == 2) ? 2 : 1;
         const bool first = t == 0, last = t + n == st.m;
         steps.push_back({t, n, n == 1 && wide_stage(st, d, t, first ? es : 4, first ? in : nullptr) && wide_stage(st, d, t, last ? es : 4, last ? gy : nullptr)});
         t += n;
@@ -1339,7 +1356,7 @@ Shape bwd_shape(const harp_plan *plan, const Step &sp) {
     const int64_t d = plan->d;
     const int b = plan->st.b[sp.t];
     if (sp.wide) return {(d / b + (b <= 8 ? 31 : 15)) / (b <= 8 ? 32 : 16), kWideBwdPerSm};
-    if (sp.n > 1) return b == 4 || sp.n == 4 ? Shape{(d / 16 + 7) / 8, k44PerSm} : Shape{(d / 4 + 31) / 32, 4};
+    if (sp.n > 1) return b == 4 || sp.n > 2 ? Shape{(d / 16 + 7) / 8, k44PerSm} : Shape{(d / 4 + 31) / 32, 4};
     const int64_t x = (d / b + 31) / 32;
     switch (b) {
         case 7: return {x, bwd_per_sm(7, 4, 2)};
@@ -1371,16 +1388,21 @@ void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int
     const float *em = plan->d_blocks_em + plan->st.off[sp.t];
     const float *em2 = sp.n == 2 ? plan->d_blocks_em + plan->st.off[sp.t + 1] : nullptr;
     const int vec = s == 1 && d % 4 == 0 && aligned16(in);
-    if (sp.n == 4 || (sp.n == 2 && b == 4)) {
+    if (sp.n > 2 || (sp.n == 2 && b == 4)) {
         // one wave of CTAs, like the backward kernels
         const int64_t x = (d / 16 + 8 * (kOwnThreads / 32) - 1) / (8 * (kOwnThreads / 32)), y = std::max<int64_t>(1, sms * (int64_t)kFwd44PerSm / x);
         const int slice = (int)std::max<int64_t>(kFwdRows / 2, (rows + y - 1) / y);
         const dim3 grid = grid2(d / 16, 8 * (kOwnThreads / 32), rows, slice);
-        if (sp.n == 4) {
-            Blocks4 k;
-            for (int t = 0; t < 4; ++t) k.em[t] = plan->d_blocks_em + plan->st.off[sp.t + t];
-            if (s == 1) launch_dep(fwd2222_kernel<true, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, out, rows, d, s, slice, k);
-            else launch_dep(fwd2222_kernel<false, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, out, rows, d, s, slice, k);
+        if (sp.n > 2) {
+            Blocks4 k{};
+            for (int t = 0; t < sp.n; ++t) k.em[t] = plan->d_blocks_em + plan->st.off[sp.t + t];
+            auto go = [&](auto ns, auto s1) {
+                launch_dep(fwd2222_kernel<decltype(ns)::value, decltype(s1)::value, TI>, grid, dim3(kOwnThreads), 0, st, in, signs, out, rows, d, s, slice, k);
+            };
+            using Three = std::integral_constant<int, 3>;
+            using Four = std::integral_constant<int, 4>;
+            if (sp.n == 4) s == 1 ? go(Four(), std::true_type()) : go(Four(), std::false_type());
+            else s == 1 ? go(Three(), std::true_type()) : go(Three(), std::false_type());
             return;
         }
         auto go = [&](auto s1, auto ring) {
@@ -1432,13 +1454,18 @@ int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8
     const float *em2 = sp.n == 2 ? plan->d_blocks_em + plan->st.off[sp.t + 1] : nullptr;
     const int vec_v = s == 1 && d % 4 == 0 && aligned16(v), vec_g = s == 1 && d % 4 == 0 && aligned16(g);
     double *part = all_parts + part_off[sp.t], *part2 = sp.n == 2 ? all_parts + part_off[sp.t + 1] : nullptr;
-    if (sp.n == 4) {
+    if (sp.n > 2) {
         const dim3 grid = grid2(d / 16, 8, rows, slice);
-        Blocks4 k;
-        Sums4 sums;
-        for (int t = 0; t < 4; ++t) { k.em[t] = plan->d_blocks_em + plan->st.off[sp.t + t]; sums.part[t] = all_parts + part_off[sp.t + t]; }
-        if (s == 1) launch_dep(bwd2222_kernel<true, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, g, g_out, rows, d, s, slice, add, k, sums);
-        else launch_dep(bwd2222_kernel<false, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, g, g_out, rows, d, s, slice, add, k, sums);
+        Blocks4 k{};
+        Sums4 sums{};
+        for (int t = 0; t < sp.n; ++t) { k.em[t] = plan->d_blocks_em + plan->st.off[sp.t + t]; sums.part[t] = all_parts + part_off[sp.t + t]; }
+        auto go = [&](auto ns, auto s1) {
+            launch_dep(bwd2222_kernel<decltype(ns)::value, decltype(s1)::value, TV, TG>, grid, dim3(32 * kSubs), 0, st, v, signs, g, g_out, rows, d, s, slice, add, k, sums);
+        };
+        using Three = std::integral_constant<int, 3>;
+        using Four = std::integral_constant<int, 4>;
+        if (sp.n == 4) s == 1 ? go(Four(), std::true_type()) : go(Four(), std::false_type());
+        else s == 1 ? go(Three(), std::true_type()) : go(Three(), std::false_type());
         return 1;
     }
     if (sp.n == 2 && b == 4) {
