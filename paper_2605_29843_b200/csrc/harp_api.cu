@@ -238,10 +238,8 @@ extern "C" harp_status_t harp_apply_ex(const harp_plan_t *plan, void *x, int64_t
     if (st != HARP_ERR_UNSUPPORTED) return st;
     st = harp_split_apply(plan, x, n_rows, dtype, transpose, s);
     if (st != HARP_ERR_UNSUPPORTED) return st;
-    // fp32 rows: up to d = 4096 the whole-row CUDA-core kernels of radices up to 8 hold enough rows of a tile to be the faster
-    // ones (4096 rows of d = 4096, radix 8: 100 us against 128); beyond, and for larger radices, passes over column groups
-    // where the batch makes up for their two or three launches and the block kernels that each CTA fetches
-    if (dtype == HARP_F32 && (plan->d > 4096 || harp_generic_max_radix(plan) > 8) && harp_f32_preferred(plan, n_rows)) {
+    // fp32 rows: passes over column groups where the batch makes up for their launches and the block kernels that each CTA fetches
+    if (dtype == HARP_F32 && harp_f32_preferred(plan, n_rows)) {
         st = harp_f32_apply(plan, x, n_rows, dtype, transpose, s);
         if (st != HARP_ERR_UNSUPPORTED) return st;
     }

@@ -22,6 +22,7 @@
 #include <new>
 
 #include "harp_internal.h"
+#include "harp_regs.h"
 #include "harp_ring.h"
 #include "harp_tm_ptx.cuh"
 
@@ -61,6 +62,7 @@ struct F32Pass {
     int32_t n_box, box_e;      // bulk copies of a tile; places (COLS) or runs of 32 coordinates (ROWS) one of them covers
     int64_t S, d;
     F32Phase ph[kMaxF32Phases];
+    RegPass reg;               // shape > 0: the pass is one of harp_regs.cu or harp_big.cu and nothing above counts
 };
 
 __device__ __forceinline__ void cp_async4(float *dst, const float *src) {
@@ -629,41 +631,64 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
     }
 }
 
-// Fixed permutation and signs of fp32 rows, in place, whole rows through shared memory.  Forward: row gathered,
-// out[i] = s[perm[i]] * in[perm[i]]; transpose: scattered, out[perm[i]] = s[perm[i]] * in[i].  The bank is mixed
-// with higher bits of the index: the coordinates that a warp gathers under a digit reversal are powers of two apart.
-__device__ __forceinline__ int permute_at(int i) { return i ^ (((i >> 5) ^ (i >> 10)) & 31); }
-__global__ void __launch_bounds__(512, 1)
-harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, const int32_t *__restrict__ perm,
-                        const int8_t *__restrict__ signs, int transpose) {
+// Fixed permutation and signs of fp32 rows, in place, whole rows through shared memory: out[i] = +-in[table[i]], table: the source of every
+// coordinate (the permutation forward, its inverse for the transpose) with the sign in the top bit.  Groups of R rows come by asynchronous 16-byte
+// copies, the next one (n_buf = 2) while this one is gathered; an entry of the table is read once for the rows of a group.  The
+// pieces of a row are exchanged within 128 bytes by higher bits of the index: under a digit reversal the coordinates that a warp gathers are
+// powers of two apart (4-way conflicts instead of 16-way; finer exchanges would split the pieces).
+__device__ __forceinline__ int permute_piece(int c) { return c ^ ((c >> 4) & 7); }
+constexpr int kPermuteThreads = 512;
+__global__ void __launch_bounds__(kPermuteThreads, 2)
+harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, int n_buf, const int32_t *__restrict__ table) {
     extern __shared__ __align__(16) float smem[];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    for (int64_t row0 = (int64_t)blockIdx.x * R; row0 < n; row0 += (int64_t)gridDim.x * R) {
-        const int rows = (int)min((int64_t)R, n - row0);
-        float *xr = x + row0 * d;
-        if (!transpose) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");        // (whoever comes next waits for this grid's end before it touches a row)
+    const int pieces = d / 4;
+    const int64_t groups = (n + R - 1) / R;
+    auto copy_in = [&](int64_t g, float *buf) {
+        if (g < groups) {
+            const int rows = (int)min((int64_t)R, n - g * R);
+            const float *src = x + g * R * d;
+            for (int r = 0; r < rows; ++r)
 #pragma unroll 4
-            for (int i = threadIdx.x; i < rows * d; i += 512) smem[permute_at(i)] = xr[i];
+                for (int c = threadIdx.x; c < pieces; c += kPermuteThreads) cp_async16(buf + r * d + 4 * permute_piece(c), src + (int64_t)r * d + 4 * c);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    copy_in(blockIdx.x, smem);
+    int buf = 0;
+    for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
+        if (n_buf == 2) {
+            copy_in(g + gridDim.x, smem + (buf ^ 1) * R * d);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
-#pragma unroll 2
-            for (int i = threadIdx.x; i < d; i += 512) {
-                const int to = perm[i];
-                for (int r = 0; r < rows; ++r) smem[permute_at(r * d + to)] = xr[(int64_t)r * d + i];
-            }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
-#pragma unroll 2
-        for (int i = threadIdx.x; i < d; i += 512) {
-            const int from = transpose ? i : perm[i];
-            const bool neg = signs && signs[from] < 0;
+        const int rows = (int)min((int64_t)R, n - g * R);
+        const float *tile = smem + buf * R * d;
+        float *dst = x + g * R * d;
+        for (int c = threadIdx.x; c < pieces; c += kPermuteThreads) {
+            const int4 t = __ldg(reinterpret_cast<const int4 *>(table) + c);
+            const int src[4] = {t.x, t.y, t.z, t.w};
+            int at[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = src[k] & 0x7fffffff;
+                at[k] = 4 * permute_piece(i >> 2) + (i & 3);
+            }
             for (int r = 0; r < rows; ++r) {
-                const float v = smem[permute_at(r * d + from)];
-                xr[(int64_t)r * d + i] = neg ? -v : v;
+                float o[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) o[k] = __uint_as_float(__float_as_uint(tile[r * d + at[k]]) ^ ((uint32_t)src[k] & 0x80000000u));
+                *reinterpret_cast<float4 *>(dst + (int64_t)r * d + 4 * c) = make_float4(o[0], o[1], o[2], o[3]);
             }
         }
-        __syncthreads();
+        __syncthreads();                                       // the buffer is free
+        if (n_buf == 2) buf ^= 1;
+        else copy_in(g + gridDim.x, smem);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 }  // namespace
@@ -671,7 +696,9 @@ harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, const in
 struct F32Plan {
     int n_pass[2] = {0, 0};            // [0] rows, [1] columns
     F32Pass pass[2][kMaxF32Passes];
-    int permute_rows = 0;              // rows per tile of the permutation kernel (0: identity)
+    int permute_rows = 0;              // most rows of a group of the permutation kernel (0: identity), its buffers, and tables per direction
+    int permute_bufs = 0;
+    int32_t *d_table[2] = {nullptr, nullptr};
     int sms = 148;
     int32_t *d_err = nullptr;          // device word, set when a wait gave up
     void *encode = nullptr;            // encoder of tensor maps
@@ -745,10 +772,12 @@ bool make_pass(const StageTable &st, int64_t d, int t0, int t1, int L, int H, in
     return true;
 }
 
+constexpr double kPassCost = 1.6;      // against a pass of harp_regs.cu
+
 // Cost of a pass relative to one trip of the rows through HBM.  What moves it: 16- and 32-byte runs of the row-mode
 // copies, one row per lane (every kernel load serves half as much arithmetic), phases with fewer blocks than warps.
 double pass_cost(const F32Pass &P, bool col) {
-    double c = 1.0, mac = 0.0;
+    double c = kPassCost, mac = 0.0;
     for (int p = 0; p < P.n_ph; ++p) mac += P.ph[p].b;
     if (!col && P.S > 1) c += P.L == 4 ? 1.0 : P.L == 8 ? 0.1 : 0.0;
     if (P.RT == 1) c += 0.02 * mac;
@@ -761,12 +790,26 @@ double pass_cost(const F32Pass &P, bool col) {
 }
 
 // cheapest cover of the stages by passes (dynamic program over the stage boundaries)
-int plan_passes(const StageTable &st, int64_t d, bool col, F32Pass *out) {
+int plan_passes(const StageTable &st, const StageTable &orig, int64_t d, bool col, F32Pass *out) {
     struct Best { double cost; int from; F32Pass pass; int n; };
     std::vector<Best> best((size_t)st.m + 1, Best{1e30, -1, F32Pass{}, 0});
     best[0].cost = 0.0;
     for (int t0 = 0; t0 < st.m; ++t0) {
         if (best[(size_t)t0].cost > 1e29) continue;
+        // passes of harp_regs.cu run the plan's own stages (its small radices are fused in st, which rounds their products)
+        for (int t1 = t0 + 1; t1 <= st.m; ++t1) {
+            auto stage_at = [&](int64_t stride) {
+                int o = 0;
+                while (o < orig.m && orig.s[o] < stride) ++o;
+                return o == orig.m || orig.s[o] == stride ? o : -1;
+            };
+            const int o0 = stage_at(st.s[t0]), o1 = t1 < st.m ? stage_at(st.s[t1]) : orig.m;
+            F32Pass P{};
+            if (o0 < 0 || o1 < 0 || o1 - o0 > 11) continue;
+            if (!harp_regs_pass(orig, d, o0, o1, col, P.reg) && (col || o1 != o0 + 1 || !harp_big_pass(orig, d, o0, P.reg))) continue;
+            const double c = best[(size_t)t0].cost + 1.0;
+            if (c < best[(size_t)t1].cost) best[(size_t)t1] = Best{c, t0, P, best[(size_t)t0].n + 1};
+        }
         for (int t1 = t0 + 1; t1 <= st.m; ++t1)
             for (int RT = 1; RT <= 2; ++RT)
                 for (int L = 1, H = 1; L <= 32; L *= 2, H = st.s[t0] == 1 ? L : 1) {
@@ -844,6 +887,12 @@ harp_status_t run_passes(const harp_plan *plan, float *x, int64_t n, int64_t ld,
         // the permutation kernel carries the signs of a permuted plan
         const int sign_at = p == 0 && plan->d_signs && !plan->d_perm ? (transpose ? 2 : 1) : 0;
         cudaError_t err = cudaErrorInvalidValue;
+        if (P.reg.shape > 0) {
+            err = P.reg.shape > kBigShape ? harp_big_launch(fp->encode, P.reg, fp->sms, x, n, ld, plan->d_blocks, transpose, fp->d_err, stream) : harp_regs_launch(fp->encode, P.reg, fp->sms, x, n, ld, COL ? plan->d_blocks : plan->d_blocks_em, sign_at ? plan->d_signs : nullptr, transpose, fp->d_err, stream);
+            g_harp_launches.fetch_add(1, std::memory_order_relaxed);
+            if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return HARP_ERR_CUDA;
+            continue;
+        }
 #define HARP_F32_LAUNCH(M, BIG)                                                                                          \
     err = P.RT == 2 ? launch_f32<2, M, BIG>(fp, P, x, n, ld, blocks, plan->d_signs, transpose, sign_at, stream)          \
                     : launch_f32<1, M, BIG>(fp, P, x, n, ld, blocks, plan->d_signs, transpose, sign_at, stream)
@@ -865,13 +914,16 @@ harp_status_t run_passes(const harp_plan *plan, float *x, int64_t n, int64_t ld,
 
 harp_status_t permute_rows(const harp_plan *plan, float *x, int64_t n, int transpose, cudaStream_t stream) {
     const F32Plan *fp = plan->f32;
-    const int R = fp->permute_rows;
-    const size_t smem = (size_t)(R * plan->d + 31) / 32 * 32 * sizeof(float);
+    // two CTAs an SM where two groups' buffers leave room; a small batch is spread over the SMs row by row
+    int R = fp->permute_rows;
+    while (R > 1 && n < (int64_t)R * 2 * fp->sms) --R;
+    const size_t smem = (size_t)fp->permute_bufs * R * plan->d * sizeof(float);
+    const int per_sm = smem <= 113 * 1024 ? 2 : 1;
     if (cudaFuncSetAttribute(harp_f32_permute_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess)
         return HARP_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<int64_t>((n + R - 1) / R, fp->sms));
-    cfg.blockDim = dim3(512);
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>((n + R - 1) / R, (int64_t)per_sm * fp->sms));
+    cfg.blockDim = dim3(kPermuteThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -879,15 +931,14 @@ harp_status_t permute_rows(const harp_plan *plan, float *x, int64_t n, int trans
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, harp_f32_permute_kernel, x, n, (int)plan->d, R, (const int32_t *)plan->d_perm,
-                                               (const int8_t *)plan->d_signs, transpose);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, harp_f32_permute_kernel, x, n, (int)plan->d, R, fp->permute_bufs, (const int32_t *)fp->d_table[transpose]);
     g_harp_launches.fetch_add(1, std::memory_order_relaxed);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? HARP_OK : HARP_ERR_CUDA;
 }
 
 }  // namespace
 
-// Host arrays and an error word only: the kernels read the block kernels the plan already keeps.
+// Host arrays, an error word and the tables of a permutation: the kernels read the block kernels the plan already keeps.
 harp_status_t harp_f32_build(harp_plan *plan) {
     const StageTable &st = f32_table(plan);
     const int64_t d = plan->d;
@@ -904,15 +955,35 @@ harp_status_t harp_f32_build(harp_plan *plan) {
     if (sms > 0) fp->sms = sms;
     if (cudaMalloc(&fp->d_err, sizeof(int32_t)) != cudaSuccess) return HARP_ERR_ALLOC;
     if (cudaMemset(fp->d_err, 0, sizeof(int32_t)) != cudaSuccess) return HARP_ERR_CUDA;
-    if (d % 4 == 0) fp->n_pass[0] = plan_passes(st, d, false, fp->pass[0]);
-    if (plan->h_perm.empty()) fp->n_pass[1] = plan_passes(st, d, true, fp->pass[1]);
-    else fp->permute_rows = (int)std::max<int64_t>(1, std::min<int64_t>(8, (200 * 1024) / (d * 4)));
+    if (d % 4 == 0) fp->n_pass[0] = plan_passes(st, plan->st, d, false, fp->pass[0]);
+    if (plan->h_perm.empty()) fp->n_pass[1] = plan_passes(st, plan->st, d, true, fp->pass[1]);
+    else if (d % 4 == 0) {
+        fp->permute_bufs = 2 * d * 4 <= kSmemMax ? 2 : 1;
+        fp->permute_rows = (int)std::max<int64_t>(1, std::min<int64_t>(4, (112 * 1024) / (fp->permute_bufs * d * 4)));
+        std::vector<int32_t> table[2];
+        try {
+            for (auto &t : table) t.resize((size_t)d);
+        } catch (const std::bad_alloc &) {
+            return HARP_ERR_ALLOC;
+        }
+        for (int64_t i = 0; i < d; ++i) {
+            const int32_t from = plan->h_perm[(size_t)i], flip = !plan->h_signs.empty() && plan->h_signs[(size_t)from] < 0 ? INT32_MIN : 0;
+            table[0][(size_t)i] = from | flip;
+            table[1][(size_t)from] = (int32_t)i | flip;
+        }
+        for (int k = 0; k < 2; ++k) {
+            if (cudaMalloc(&fp->d_table[k], sizeof(int32_t) * (size_t)d) != cudaSuccess) return HARP_ERR_ALLOC;
+            if (cudaMemcpy(fp->d_table[k], table[k].data(), sizeof(int32_t) * (size_t)d, cudaMemcpyHostToDevice) != cudaSuccess) return HARP_ERR_CUDA;
+        }
+    }
     return HARP_OK;
 }
 
 void harp_f32_destroy(harp_plan *plan) {
     if (!plan->f32) return;
     if (plan->f32->d_err) cudaFree(plan->f32->d_err);
+    for (int32_t *t : plan->f32->d_table)
+        if (t) cudaFree(t);
     delete plan->f32;
     plan->f32 = nullptr;
 }
@@ -927,6 +998,8 @@ namespace {
 
 // microseconds of a pass over n vectors, see harp_generic_estimate
 double pass_estimate(const F32Plan *fp, const F32Pass &P, int64_t n) {
+    if (P.reg.shape > kBigShape) return 6.0 + 2.5e-6 * (double)n * (double)P.reg.d;
+    if (P.reg.shape > 0) return 3.2 + 1.3e-6 * (double)n * (double)P.reg.d;
     const int64_t tiles = (n + 32 * P.RT - 1) / (32 * P.RT), n_c = (int64_t)P.E * P.L;
     const int64_t n_parts = pass_parts(fp, P, tiles), per = n_parts > 0 ? (tiles + n_parts - 1) / n_parts : (tiles * P.n_cg + fp->sms - 1) / fp->sms;
     const int64_t groups = n_parts > 0 ? 1 : 1 + (per - 1) / tiles;          // whose block kernels a CTA fetches
@@ -945,13 +1018,20 @@ bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows) {
     const F32Plan *fp = plan->f32;
     if (!fp || fp->n_pass[0] == 0) return false;
     if (plan->opt_f32_passes || harp_generic_supported(plan, HARP_F32) != HARP_OK) return true;
+    // (whole-row kernels of four rows a CTA keep a batch that fills one wave to the most part: one launch)
+    if (plan->d >= 8192 && plan->d <= 226 * 64 && plan->d_perm == nullptr && harp_generic_max_radix(plan) <= 8 && n_rows > 2 * fp->sms && n_rows <= 4 * fp->sms) return false;
     double us = 0.0;
-    for (int p = 0; p < fp->n_pass[0]; ++p) us += pass_estimate(fp, fp->pass[0][p], n_rows);
-    if (fp->permute_rows) {
-        const int64_t waves = ((n_rows + fp->permute_rows - 1) / fp->permute_rows + fp->sms - 1) / fp->sms;
-        us += 5.6 + 2.1e-4 * (double)(waves * std::min<int64_t>(fp->permute_rows, n_rows) * plan->d);
+    // up to d = 4096 the whole-row CUDA-core kernels of radices up to 8 hold enough rows of a tile to beat passes other than those of harp_regs.cu
+    const bool whole = plan->d <= 4096 && harp_generic_max_radix(plan) <= 8;
+    for (int p = 0; p < fp->n_pass[0]; ++p) {
+        if (whole && fp->pass[0][p].reg.shape == 0) return false;
+        us += pass_estimate(fp, fp->pass[0][p], n_rows);
     }
-    return us < harp_generic_estimate(plan, n_rows, fp->sms);
+    if (fp->permute_rows) {
+        us += 3.5 + 1.3e-6 * (double)n_rows * (double)plan->d;
+    }
+    // (under a digit reversal the whole-row kernels take 1.4 times their estimate: 512 rows of d = 4096 27 us)
+    return us < (fp->permute_rows ? 1.3 : 1.0) * harp_generic_estimate(plan, n_rows, fp->sms);
 }
 
 harp_status_t harp_f32_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose, cudaStream_t stream) {
