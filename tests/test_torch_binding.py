@@ -1,4 +1,5 @@
 """The torch conveniences look torch and the library's function up once (no GPU needed: CUDA initialisation is replaced)."""
+import numpy as np
 import pytest
 import torch
 
@@ -32,3 +33,15 @@ def test_a_failed_initialisation_is_tried_again(unbound, monkeypatch):
     monkeypatch.setattr(torch.cuda, "init", lambda: None)
     harp._bind_torch()
     assert harp._apply_ex is not None
+
+
+def test_the_call_without_ctypes_takes_what_ctypes_took(unbound, monkeypatch):
+    """None for a null pointer, anything with __index__ for an integer; floats and a wrong number of arguments are refused."""
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    harp._bind_torch()
+    null, bad_dtype = 1, harp.lib().harp_apply_ex(1, 1, 1, 7, 0, 0, None)
+    assert harp._apply_ex(None, 1 << 63, np.int64(1), 0, 0, np.int32(0), None) == null
+    assert harp._apply_ex(1, 1, 1, 7, 0, 0, 0) == bad_dtype != null
+    for args in ((None, 0, 1.0, 0, 0, 0, 0), (None, 0, 1, 0, 0, 0), (None, 0, 1, 0, 0, "0", 0)):
+        with pytest.raises(TypeError):
+            harp._apply_ex(*args)
