@@ -988,6 +988,8 @@ void harp_f32_destroy(harp_plan *plan) {
     plan->f32 = nullptr;
 }
 
+const int32_t *harp_f32_source_table(const harp_plan *plan) { return plan->f32 ? plan->f32->d_table[0] : nullptr; }
+
 int32_t harp_f32_error_word(const harp_plan *plan) {
     if (!plan->f32 || !plan->f32->d_err) return 0;
     int32_t v = 0;

@@ -851,6 +851,54 @@ bwd22_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, int vec
     });
 }
 
+// ---- one radix-2 stage at a stride that is a multiple of four, backward: a thread owns four neighbouring blocks, so that a row is two 16-byte loads
+// of either state where single blocks take 4-byte ones (1024 rows of d = 8192 behind four radix-8 stages: 30 us at 2.2 TB/s)
+template <typename TV, typename TG>
+__global__ void __launch_bounds__(32 * kSubs, 4)
+bwd2x4_kernel(const TV *__restrict__ v, const TG *__restrict__ g, float *__restrict__ g_out, int64_t rows, int64_t d, int64_t s, int slice, int add,
+              const float *__restrict__ em, double *__restrict__ part) {
+    __shared__ double sh[16][kSubs][32];
+    const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
+    const int64_t nblk = d / 2, cc = ((int64_t)blockIdx.x * 32 + lane) * 4;
+    const bool have = cc < nblk;
+    const int64_t c = have ? cc : 0, alpha = c / s, base = alpha * 2 * s + (c - alpha * s);
+    float k[2][2][4];
+    double acc[16] = {};                       // [i][j][block]
+#pragma unroll
+    for (int ij = 0; ij < 4; ++ij) load_block<4, float>(em + ij * nblk + c, 1, true, k[ij >> 1][ij & 1]);
+    prior_kernel_done();
+    const int64_t r0 = (int64_t)blockIdx.y * slice, r1 = min(rows, r0 + slice);
+#pragma unroll 2
+    for (int64_t r = r0 + sub; r < r1; r += kSubs) {
+        float x[2][4], y[2][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            load_block<4, TV>(v + r * d + base + i * s, 1, true, x[i]);
+            load_block<4, TG>(g + r * d + base + i * s, 1, true, y[i]);
+        }
+        double xd[2][4], yd[2][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) { xd[i][b] = (double)x[i][b]; yd[i][b] = (double)y[i][b]; }
+#pragma unroll
+        for (int ij = 0; ij < 4; ++ij)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[ij * 4 + b] += xd[ij >> 1][b] * yd[ij & 1][b];
+        if (g_out && have) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                float o[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) o[b] = fmaf(y[1][b], k[i][1][b], fmaf(y[0][b], k[i][0][b], 0.f));
+                store_block<4>(g_out + r * d + base + i * s, 1, true, o);
+            }
+        }
+    }
+    double *dst = part + (int64_t)blockIdx.y * 4 * nblk + c;
+    combine<16, kSubs>(acc, sh, sub, lane, add, [&](int e) -> double * { return have ? dst + (int64_t)(e >> 2) * nblk + (e & 3) : nullptr; });
+}
+
 // ---- one stage of radix 7, 8 or 16 on tiles in shared memory.  A CTA keeps NB neighbouring blocks and walks over tiles of eight rows that
 // asynchronous copies bring into a ring of buffers; every value is fetched once, where threads that own entries of a block fetch all
 // of the block's values.  Backward, the outer products of a block are a product of the fp64 tensor core (mma.m8n8k4, the rows as the
@@ -1213,6 +1261,63 @@ permute_kernel(const T *__restrict__ x, int vec, T *__restrict__ out, int64_t ro
     }
 }
 
+// The same for aligned rows: groups of R rows by asynchronous 16-byte copies, the next group on its way while this one is gathered, and one table
+// with the sign in its top bit in place of an index and the sign behind it.  Pieces are exchanged within 128 bytes by higher bits of the
+// index (a digit reversal: 4-way conflicts).
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 3)
+permute_ring_kernel(const T *__restrict__ x, T *__restrict__ out, int64_t rows, int d, const int32_t *__restrict__ table, int R) {
+    constexpr int V = 16 / (int)sizeof(T), kLog = sizeof(T) == 2 ? 3 : 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *smem = reinterpret_cast<T *>(smem_raw);
+    auto piece = [](int c) { return c ^ ((c >> (sizeof(T) == 2 ? 3 : 4)) & 7); };
+    const int pieces = d / V;
+    const int64_t groups = (rows + R - 1) / R;
+    auto copy_in = [&](int64_t g, T *buf) {
+        if (g < groups) {
+            const int nr = (int)min((int64_t)R, rows - g * R);
+            const T *src = x + g * R * d;
+            for (int r = 0; r < nr; ++r)
+#pragma unroll 2
+                for (int c = threadIdx.x; c < pieces; c += kThreads)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(buf + r * d + V * piece(c))), "l"(src + (int64_t)r * d + V * c) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    prior_kernel_done();
+    copy_in(blockIdx.x, smem);
+    int buf = 0;
+    for (int64_t g = blockIdx.x; g < groups; g += gridDim.x, buf ^= 1) {
+        copy_in(g + gridDim.x, smem + (buf ^ 1) * R * d);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        const int nr = (int)min((int64_t)R, rows - g * R);
+        const T *tile = smem + buf * R * d;
+        for (int i = (int)threadIdx.x * 4; i < d; i += kThreads * 4) {
+            const int4 t = __ldg(reinterpret_cast<const int4 *>(table + i));
+            const int src[4] = {t.x, t.y, t.z, t.w};
+            int at[4];
+            T flip[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int e = src[k] & 0x7fffffff;
+                at[k] = V * piece(e >> kLog) + (e & (V - 1));
+                flip[k] = src[k] < 0 ? (T)((T)1 << (8 * sizeof(T) - 1)) : (T)0;
+            }
+            T *to = out + g * R * d + i;
+            for (int r = 0; r < nr; ++r, to += d) {
+                T o[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) o[k] = tile[r * d + at[k]] ^ flip[k];
+                if constexpr (sizeof(T) == 2) *reinterpret_cast<uint2 *>(to) = make_uint2(o[0] | (uint32_t)o[1] << 16, o[2] | (uint32_t)o[3] << 16);
+                else *reinterpret_cast<uint4 *>(to) = make_uint4(o[0], o[1], o[2], o[3]);
+            }
+        }
+        __syncthreads();                                       // the buffer is free
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // one stage on a chunk: out[r][base + j s] = sum_i in[r][base + i s] * K[c][i][j]   (transpose: K[c][j][i]).
 // Neighbouring lanes hold neighbouring positions: inside one block when s is small, in neighbouring
 // blocks otherwise -- so K is read block-major (entry k of block c at c b^2 + k) for s < 8 and
@@ -1308,6 +1413,8 @@ cudaMemPool_t scratch_pool(int device) {
     return pool;
 }
 
+constexpr int64_t kMostScratch = 1280ll << 20, kLeastScratch = 160ll << 20;     // bytes of states of a chunk
+
 // grid of the kernels in which a thread keeps its coordinate and walks over rows
 dim3 column_grid(int64_t d, int64_t rows) {
     const int64_t gx = (d + kThreads - 1) / kThreads;
@@ -1317,7 +1424,7 @@ dim3 column_grid(int64_t d, int64_t rows) {
 
 // ---- steps of a plan
 
-struct Step { int t, n; bool wide; };  // stages [t, t + n): one stage, two of radix 4 or of radix 2, or three or four of radix 2; wide: one, on tiles in shared memory
+struct Step { int t, n; bool wide; };  // stages [t, t + n): one stage, two of radix 4 or of radix 2, or three or four of radix 2; wide: one, on tiles in shared memory or by fours of blocks
 
 // rows by asynchronous copies: eight neighbouring units are whole 16-byte pieces, the unit's sixteen coordinates make d a multiple of sixteen
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -1329,6 +1436,9 @@ bool wide_stage(const StageTable &st, int64_t d, int t, size_t es, const void *p
     const int64_t e = 16 / (int64_t)es;
     return (b == 7 || b == 8 || b == 16) && (t == 0 ? d % e == 0 : st.s[t] % e == 0) && aligned16(p);
 }
+
+// a radix-2 stage alone, by fours of neighbouring blocks (the first stage, which carries the signs, has stride one)
+bool fours_stage(const StageTable &st, int t, const void *p) { return st.b[t] == 2 && t > 0 && st.s[t] % 4 == 0 && aligned16(p); }
 
 // in, gy: the call's rows (the states of other steps start on 16-byte boundaries)
 std::vector<Step> make_steps(const StageTable &st, int64_t d, size_t es, const void *in, const void *gy) {
@@ -1342,7 +1452,8 @@ std::vector<Step> make_steps(const StageTable &st, int64_t d, size_t es, const v
         const bool ring = b == 2 && n >= 3 && d % (16 * (int64_t)st.s[t]) == 0 && ring44(st.s[t], t == 0 ? in : nullptr) && aligned16(t + k == st.m ? gy : nullptr);
         n = ring ? k : n >= 2 && (b == 4 || b == 2) ? 2 : 1;
         const bool first = t == 0, last = t + n == st.m;
-        steps.push_back({t, n, n == 1 && wide_stage(st, d, t, first ? es : 4, first ? in : nullptr) && wide_stage(st, d, t, last ? es : 4, last ? gy : nullptr)});
+        const bool wide = wide_stage(st, d, t, first ? es : 4, first ? in : nullptr) && wide_stage(st, d, t, last ? es : 4, last ? gy : nullptr);
+        steps.push_back({t, n, n == 1 && (wide || fours_stage(st, t, last ? gy : nullptr))});
         t += n;
     }
     return steps;
@@ -1355,6 +1466,7 @@ struct Shape { int64_t x; int per_sm; };
 Shape bwd_shape(const harp_plan *plan, const Step &sp) {
     const int64_t d = plan->d;
     const int b = plan->st.b[sp.t];
+    if (sp.wide && b == 2) return {(d / 2 + 127) / 128, 4};
     if (sp.wide) return {(d / b + (b <= 8 ? 31 : 15)) / (b <= 8 ? 32 : 16), kWideBwdPerSm};
     if (sp.n > 1) return b == 4 || sp.n > 2 ? Shape{(d / 16 + 7) / 8, k44PerSm} : Shape{(d / 4 + 31) / 32, 4};
     const int64_t x = (d / b + 31) / 32;
@@ -1482,6 +1594,10 @@ int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8
         launch_dep(bwd22_kernel<TV, TG>, grid2(d / 4, 32, rows, slice), dim3(32 * kSubs), 0, st, v, signs, vec_v, g, vec_g, g_out, rows, d, s, slice, add, em, em2, part, part2);
         return 1;
     }
+    if (sp.wide && b == 2) {
+        launch_dep(bwd2x4_kernel<TV, TG>, grid2(d / 2, 128, rows, slice), dim3(32 * kSubs), 0, st, v, g, g_out, rows, d, s, slice, add, em, part);
+        return 1;
+    }
     if (sp.wide) {
         auto go = [&](auto bc, auto s1) {
             constexpr int B = decltype(bc)::value;
@@ -1523,35 +1639,40 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
     const std::vector<Step> steps = make_steps(tab, d, sizeof(T), plan->d_perm ? nullptr : x, gy);
     const int n = (int)steps.size(), n_g = std::min(n - 1, 2), ring = std::max(1, n_g);
     const bool permuted = plan->d_perm != nullptr;
-    // chunk of rows whose forward states, gradient states and permuted rows fit about 200 MB; the partial sums of a wave of
-    // CTAs come on top.  The forward kernels (none where one step is all) take kFwdRows rows per CTA along grid.y.
+    // Chunk of rows whose forward states, gradient states and permuted rows fit the budget; the partial sums of a wave of CTAs come on top.  The
+    // forward kernels (none where one step is all) take kFwdRows rows per CTA along grid.y.  Chunks that stay near L2 are not worth their launches
+    // and partial waves (16384 rows of d = 4096, chunks of 110 MB 1083 us, 200 MB 863, 640 MB 751, one of 1200 MB 719); a device without room for it takes the smaller ones.
     const int64_t per_row = std::max<int64_t>(1, d * (4 * (int64_t)(n - 1 + n_g) + (permuted ? (int64_t)sizeof(T) : 0)));
-    const int64_t fit = std::max<int64_t>(16, (200ll << 20) / per_row), most = n > 1 ? std::min<int64_t>(fit, 65535ll * kFwdRows) : fit;
-    const int64_t n_chunks = (n_rows + most - 1) / most;
-    const int64_t chunk = (n_rows + n_chunks - 1) / n_chunks;
     int sms = 148;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device);
-    int64_t part_len = 0, part_off[HARP_MAX_STAGES] = {};
+    int64_t chunk = 0, plane = 0, part_len = 0, part_off[HARP_MAX_STAGES] = {};
     ReduceTable red{};
-    for (const Step &sp : steps) {
-        const int b = tab.b[sp.t];
-        if (!owner_radix(b)) continue;
-        const int slice = slice_rows(plan, sp, chunk, sms);
-        for (int t = sp.t; t < sp.t + sp.n; ++t) {
-            part_off[t] = part_len;
-            red.st[red.m++] = ReduceStage{tab.off[t], part_len, d / b, d * b, b * b, slice, 0};
-            red.total += d * b;
-            part_len += ((chunk + slice - 1) / slice) * d * b;
-        }
-    }
-    const int64_t plane = (chunk * d + 3) / 4 * 4;
-    const size_t bytes = (size_t)(part_len * 8 + 16 + plane * 4 * (n - 1 + n_g) + (permuted ? plane * (int64_t)sizeof(T) : 0));
     double *part = nullptr;
     cudaMemPool_t pool = scratch_pool(plan->device);
-    const cudaError_t ae = pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&part), bytes, pool, st) : cudaMallocAsync(reinterpret_cast<void **>(&part), bytes, st);
-    if (ae != cudaSuccess) {
-        cudaGetLastError();
-        return HARP_ERR_ALLOC;
+    for (int64_t budget = kMostScratch; !part; budget /= 2) {
+        if (budget < kLeastScratch) return HARP_ERR_ALLOC;
+        const int64_t fit = std::max<int64_t>(16, budget / per_row), most = n > 1 ? std::min<int64_t>(fit, 65535ll * kFwdRows) : fit;
+        const int64_t n_chunks = (n_rows + most - 1) / most;
+        chunk = (n_rows + n_chunks - 1) / n_chunks;
+        part_len = 0;
+        red = ReduceTable{};
+        for (const Step &sp : steps) {
+            const int b = tab.b[sp.t];
+            if (!owner_radix(b)) continue;
+            const int slice = slice_rows(plan, sp, chunk, sms);
+            for (int t = sp.t; t < sp.t + sp.n; ++t) {
+                part_off[t] = part_len;
+                red.st[red.m++] = ReduceStage{tab.off[t], part_len, d / b, d * b, b * b, slice, 0};
+                red.total += d * b;
+                part_len += ((chunk + slice - 1) / slice) * d * b;
+            }
+        }
+        plane = (chunk * d + 3) / 4 * 4;
+        const size_t bytes = (size_t)(part_len * 8 + 16 + plane * 4 * (n - 1 + n_g) + (permuted ? plane * (int64_t)sizeof(T) : 0));
+        if ((pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&part), bytes, pool, st) : cudaMallocAsync(reinterpret_cast<void **>(&part), bytes, st)) != cudaSuccess) {
+            cudaGetLastError();
+            part = nullptr;
+        }
     }
     float *vp = reinterpret_cast<float *>(part + (part_len + 1) / 2 * 2), *gp = vp + (n - 1) * plane;      // state planes on 16-byte boundaries
     T *xp = reinterpret_cast<T *>(gp + n_g * plane);
@@ -1575,8 +1696,18 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
             // per call: the attribute belongs to the current device's copy of the kernel
             const int staged = smem <= 48 * 1024 || (smem <= 200 * 1024 && cudaFuncSetAttribute(permute_kernel<Bits>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess);
             if (!staged) smem = 0;
-            launch_dep(permute_kernel<Bits>, dim3((unsigned)std::min<int64_t>((rows + R - 1) / R, 148 * 8)), dim3(kThreads), smem, st, reinterpret_cast<const Bits *>(xc), (int)(aligned16(xc) && d % (16 / (int64_t)sizeof(T)) == 0), reinterpret_cast<Bits *>(xp),
+            const int32_t *table = harp_f32_source_table(plan);
+            const int64_t ring_rows = std::min<int64_t>(4, 36 * 1024 / (d * (int64_t)sizeof(T)));
+            if (table && red.m == tab.m && ring_rows > 0 && aligned16(xc) && d % (16 / (int64_t)sizeof(T)) == 0) {
+                const int r = (int)std::max<int64_t>(1, std::min<int64_t>(ring_rows, rows / (3 * sms)));
+                const size_t bytes = (size_t)(2 * r * d) * sizeof(T);
+                if (bytes > 48 * 1024) cudaFuncSetAttribute(permute_ring_kernel<Bits>, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
+                launch_dep(permute_ring_kernel<Bits>, dim3((unsigned)std::min<int64_t>((rows + r - 1) / r, 3 * sms)), dim3(kThreads), bytes, st, reinterpret_cast<const Bits *>(xc),
+                           reinterpret_cast<Bits *>(xp), rows, (int)d, table, r);
+            } else {
+                launch_dep(permute_kernel<Bits>, dim3((unsigned)std::min<int64_t>((rows + R - 1) / R, 148 * 8)), dim3(kThreads), smem, st, reinterpret_cast<const Bits *>(xc), (int)(aligned16(xc) && d % (16 / (int64_t)sizeof(T)) == 0), reinterpret_cast<Bits *>(xp),
                        rows, (int)d, plan->d_perm, plan->d_signs, staged, R);
+            }
             xc = xp;
             ++launches;
         }

@@ -116,6 +116,8 @@ harp_status_t harp_col_apply(const harp_plan *plan, void *W, int64_t n_cols, int
 harp_status_t harp_f32_build(harp_plan *plan);
 void harp_f32_destroy(harp_plan *plan);
 int32_t harp_f32_error_word(const harp_plan *plan);
+// source of every coordinate under the plan's permutation, its sign in the top bit (device; null: none, or a plan without fp32 passes)
+const int32_t *harp_f32_source_table(const harp_plan *plan);
 bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows);      // faster than the whole-row kernels, by the estimates
 harp_status_t harp_f32_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose,
                              cudaStream_t stream);
