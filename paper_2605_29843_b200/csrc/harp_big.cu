@@ -8,8 +8,8 @@
 // are on different banks, for the operands as for the results.
 //
 // What bounds it: the products (43 of 48 results kept) and the copy engine (a run of 32 bytes in and out takes 3.3 cycles), about equally.
-// All positions of some rows are worked on at the same time, a CTA to eight of them, for the sake of DRAM pages (CTAs in pairs on 64 bytes of a
-// row, an equal share of the whole list for every SM: 12 k cycles a tile of 40 rows).
+// All positions of some rows are worked on at the same time, a CTA to eight of them, for the sake of DRAM pages (an equal share of the whole list of
+// tiles for each of 148 SMs instead of 128: 287 us for both passes of 4096 rows of d = 11008, 186 this way).
 #include <algorithm>
 
 #include "harp_internal.h"
@@ -21,7 +21,7 @@ namespace {
 
 using harp_tm::smem_u32;
 
-constexpr int kBigThreads = 256;
+constexpr int kBigWarps = 8, kBigThreads = 32 * (kBigWarps + 1);       // the last warp copies
 constexpr uint32_t kBigSpin = 1u << 22;        // limit of every wait for a bulk copy
 constexpr int kBigSmem = 226 * 1024, kBigBufs = 3;
 
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kBigThreads, 1)
 harp_big_kernel(const float *__restrict__ blocks, int32_t *err, const __grid_constant__ CUtensorMap tmap, const BigArgs P) {
     constexpr int R = 8 * RT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[kBigBufs];
+    __shared__ __align__(8) uint64_t full_bar[kBigBufs], done_bar[kBigBufs];       // the tile has arrived; the warps have stored its results
     __shared__ int dead;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");        // (whoever comes next waits for this grid's end before it touches a row)
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, tile_bytes = (uint32_t)P.b * R * 32u;
@@ -45,7 +45,7 @@ harp_big_kernel(const float *__restrict__ blocks, int32_t *err, const __grid_con
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rl = lane & 7, l = 4 * (warp >> 2) + (lane >> 3), j0 = (warp & 3) * JT;
     const int b = P.b, pitch = P.pitch;
     if (threadIdx.x == 0) {
-        for (int k = 0; k < kBigBufs; ++k) harp_tm::mbar_init(smem_u32(&full_bar[k]), 1);
+        for (int k = 0; k < kBigBufs; ++k) { harp_tm::mbar_init(smem_u32(&full_bar[k]), 1); harp_tm::mbar_init(smem_u32(&done_bar[k]), kBigWarps); }
         dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -59,41 +59,52 @@ harp_big_kernel(const float *__restrict__ blocks, int32_t *err, const __grid_con
                 for (int j = lane; j < b; j += 32)
                     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(wts + (k * b + (TR ? j : i)) * pitch + (TR ? i : j))), "l"(src + (k * b + i) * b + j) : "memory");
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
     auto stopped = [&] { return *(volatile int *)&dead != 0; };
-    auto copy = [&](bool in, int n, int k) {                   // thread 0: this CTA's n-th tile
-        const int tile = t0 + n * P.n_parts;
-        if (in) {
-            const uint32_t bar = smem_u32(&full_bar[k]);
-            harp_tm::mbar_expect_tx(bar, tile_bytes);          // past the last row the engine fills zeros
-            harp_tm::tma_load_3d(base + k * tile_bytes, &tmap, lo * 8, tile * R, hi * b, bar);
-        } else {
-            harp_tm::tma_store_3d(&tmap, lo * 8, tile * R, hi * b, base + k * tile_bytes);
-            harp_tm::bulk_commit();
-        }
+    // whether the phase of a barrier completed before the limit; after one that did not nothing is copied any more
+    auto wait = [&](uint64_t *bar, uint32_t parity) {
+        for (uint32_t it = 0; !harp_tm::mbar_try(smem_u32(bar), parity);)
+            if (++it > kBigSpin || ((it & 63) == 63 && stopped())) {
+                *(volatile int *)&dead = 1;
+                atomicExch(err, 103);
+                return;
+            }
     };
-    int buf = 0;
-    uint32_t parity = 0;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
     // plan data only up to here: may run under the kernel before this one
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int k = 0; k < kBigBufs - 1 && k < n_my; ++k)
-        if (threadIdx.x == 0) copy(true, k, k);
-    // byte offset of (position l, row lane % 8) in a place of the tile: 16-byte halves exchanged in every second group of four rows
-    const uint32_t at0 = (uint32_t)(rl * 32 + ((l * 4) ^ (((rl >> 2) & 1) << 4)));
-    for (int n = 0; n < n_my; ++n, buf = buf + 1 == kBigBufs ? 0 : buf + 1) {
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        const uint32_t bar = smem_u32(&full_bar[buf]), par = (parity >> buf) & 1u;
-        uint32_t it = 0;
-        while (!harp_tm::mbar_try(bar, par)) {
-            if (++it > kBigSpin || ((it & 63) == 63 && stopped())) {
-                *(volatile int *)&dead = 1;                    // from here on nothing is copied any more
-                atomicExch(err, 103);
-                parity ^= 1u << buf;                           // (undone below: the phase is still awaited)
-                break;
+
+    if (warp == kBigWarps) {                                   // copies; tile n in buffer n mod kBigBufs
+        if (lane != 0) return;
+        uint32_t loaded = ~0u;                                 // bit per buffer: phase of its last load
+        auto load = [&](int n) {
+            const int k = n % kBigBufs;
+            harp_tm::mbar_expect_tx(smem_u32(&full_bar[k]), tile_bytes);       // past the last row the engine fills zeros
+            harp_tm::tma_load_3d(base + k * tile_bytes, &tmap, lo * 8, (t0 + n * P.n_parts) * R, hi * b, smem_u32(&full_bar[k]));
+            loaded ^= 1u << k;
+        };
+        for (int n = 0; n < kBigBufs && n < n_my; ++n) load(n);
+        for (int n = 0; n < n_my && !stopped(); ++n) {
+            const int k = n % kBigBufs;
+            wait(&done_bar[k], (uint32_t)(n / kBigBufs) & 1u);
+            if (stopped()) break;
+            harp_tm::tma_store_3d(&tmap, lo * 8, (t0 + n * P.n_parts) * R, hi * b, base + k * tile_bytes);
+            harp_tm::bulk_commit();
+            if (n + kBigBufs < n_my) {
+                harp_tm::bulk_wait_read0();
+                load(n + kBigBufs);
             }
         }
-        parity ^= 1u << buf;
-        __syncthreads();
+        harp_tm::bulk_wait0();
+        if (stopped()) ring_drain(loaded, kBigBufs, kBigSpin, [&](int k, uint32_t phase) { return harp_tm::mbar_try(smem_u32(&full_bar[k]), phase); });
+        return;
+    }
+
+    // byte offset of (position l, row lane % 8) in a place of the tile: 16-byte halves exchanged in every second group of four rows
+    const uint32_t at0 = (uint32_t)(rl * 32 + ((l * 4) ^ (((rl >> 2) & 1) << 4)));
+    for (int n = 0; n < n_my; ++n) {
+        const int buf = n % kBigBufs;
+        wait(&full_bar[buf], (uint32_t)(n / kBigBufs) & 1u);
         const uint32_t tile = base + buf * tile_bytes + at0;
         const float *w = wts + (size_t)l * b * pitch + j0;
         float acc[JT][RT] = {};
@@ -101,7 +112,7 @@ harp_big_kernel(const float *__restrict__ blocks, int32_t *err, const __grid_con
         struct Operand { float x[RT]; float4 k[JT / 4]; } oa, ob;
         auto fetch = [&](Operand &o, int i) {
 #pragma unroll
-            for (int k = 0; k < RT; ++k) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(o.x[k]) : "r"(tile + (uint32_t)i * (R * 32) + k * 256));
+            for (int k = 0; k < RT; ++k) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(o.x[k]) : "r"(tile + (uint32_t)i * (R * 32) + k * 256) : "memory");
 #pragma unroll
             for (int j = 0; j < JT / 4; ++j) o.k[j] = *reinterpret_cast<const float4 *>(w + i * pitch + 4 * j);
         };
@@ -115,23 +126,15 @@ harp_big_kernel(const float *__restrict__ blocks, int32_t *err, const __grid_con
             }
         };
         fetch(oa, 0);
-        auto products = [&](int i0, int i1) {                  // an even number of operands
-            for (int i = i0; i < i1; i += 2) {
-                fetch(ob, i + 1);
-                multiply(oa);
-                fetch(oa, min(i + 2, b - 1));
-                multiply(ob);
-            }
-        };
-        const int mid = b / 4 * 2, even = b / 2 * 2;
-        products(0, mid);
-        if (threadIdx.x == 0 && n + kBigBufs - 1 < n_my && !stopped()) {
-            harp_tm::bulk_wait_read0();                        // the store of the tile before this one, issued half a tile ago
-            copy(true, n + kBigBufs - 1, buf == 0 ? kBigBufs - 1 : buf - 1);
+        for (int i = 0; i + 1 < b; i += 2) {
+            fetch(ob, i + 1);
+            multiply(oa);
+            fetch(oa, min(i + 2, b - 1));
+            multiply(ob);
         }
-        products(mid, even);
-        if (even < b) multiply(oa);
-        __syncthreads();                                       // nobody stores before everybody has read
+        if (b & 1) multiply(oa);
+        // nobody stores before everybody has read: the four warps that share these positions
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp >> 2)) : "memory");
 #pragma unroll
         for (int j = 0; j < JT; ++j)
             if (j0 + j < b) {
@@ -140,13 +143,8 @@ harp_big_kernel(const float *__restrict__ blocks, int32_t *err, const __grid_con
                     asm volatile("st.shared.f32 [%0], %1;" ::"r"(tile + (uint32_t)(j0 + j) * (R * 32) + k * 256), "f"(acc[j][k]) : "memory");
             }
         harp_tm::fence_async_smem();                           // results before the copy engine reads them
-        __syncthreads();
-        if (threadIdx.x == 0 && !stopped()) copy(false, n, buf);
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (threadIdx.x == 0) {
-        harp_tm::bulk_wait0();
-        if (stopped()) ring_drain(parity, kBigBufs, kBigSpin, [&](int k, uint32_t phase) { return harp_tm::mbar_try(smem_u32(&full_bar[k]), phase); });
+        __syncwarp();
+        if (lane == 0) harp_tm::mbar_arrive(smem_u32(&done_bar[buf]));
     }
 }
 
