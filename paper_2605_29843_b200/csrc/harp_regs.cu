@@ -143,8 +143,9 @@ __device__ __forceinline__ float lds1(uint32_t a) {
 }
 __device__ __forceinline__ void sts1(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
 
-// byte offset of tile coordinate c in a vector's tile (rows)
-__device__ __forceinline__ uint32_t place(int c) { return (uint32_t)(((c & ~31) | ((((c >> 2) ^ (c >> 5)) & 7) << 2) | (c & 3)) * 4); }
+// byte offset of tile coordinate c in a vector's tile (rows).  A unit's first coordinate and the offsets of its other values have no bits in
+// common, so place(first + offset) = place(first) ^ place(offset), and the latter is a constant.
+__host__ __device__ constexpr uint32_t place(int c) { return (uint32_t)(((c & ~31) | ((((c >> 2) ^ (c >> 5)) & 7) << 2) | (c & 3)) * 4); }
 
 // one phase on the G vectors of a tile of rows, in place
 template <class P, class Ge, int G, uint32_t kVec, bool TR>
@@ -155,8 +156,11 @@ __device__ __forceinline__ void rows_phase(uint32_t tile, const float (&w)[Ge::k
     if (!Ge::have(threadIdx.x)) return;
     uint32_t a[nA];
 #pragma unroll
-    for (int i = 0; i < nA; ++i) a[i] = tile + place(Ge::coord(threadIdx.x, kRun ? 4 * i : i));
-#pragma unroll 1
+    for (int i = 0; i < nA; ++i) {
+        const int e = kRun ? 4 * i : i;
+        a[i] = tile + (place(Ge::coord(threadIdx.x, e / Ge::N * Ge::N)) ^ place(e % Ge::N * Ge::T));
+    }
+#pragma unroll
     for (int r = 0; r < G; r += U) {
         float v[U][Ge::V][1];
 #pragma unroll
@@ -165,10 +169,10 @@ __device__ __forceinline__ void rows_phase(uint32_t tile, const float (&w)[Ge::k
             for (int i = 0; i < nA; ++i) {
                 if constexpr (kRun) {
                     float q[4];
-                    lds4(q, a[i] + u * kVec);
+                    lds4(q, a[i] + (r + u) * kVec);
                     v[u][4 * i][0] = q[0]; v[u][4 * i + 1][0] = q[1]; v[u][4 * i + 2][0] = q[2]; v[u][4 * i + 3][0] = q[3];
                 } else {
-                    v[u][i][0] = lds1(a[i] + u * kVec);
+                    v[u][i][0] = lds1(a[i] + (r + u) * kVec);
                 }
             }
 #pragma unroll
@@ -179,13 +183,11 @@ __device__ __forceinline__ void rows_phase(uint32_t tile, const float (&w)[Ge::k
             for (int i = 0; i < nA; ++i) {
                 if constexpr (kRun) {
                     const float q[4] = {v[u][4 * i][0], v[u][4 * i + 1][0], v[u][4 * i + 2][0], v[u][4 * i + 3][0]};
-                    sts4(a[i] + u * kVec, q);
+                    sts4(a[i] + (r + u) * kVec, q);
                 } else {
-                    sts1(a[i] + u * kVec, v[u][i][0]);
+                    sts1(a[i] + (r + u) * kVec, v[u][i][0]);
                 }
             }
-#pragma unroll
-        for (int i = 0; i < nA; ++i) a[i] += U * kVec;
     }
 }
 
