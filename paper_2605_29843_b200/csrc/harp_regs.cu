@@ -17,6 +17,7 @@
 // the products of two radix-8 phases 1.1 k.
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "harp_internal.h"
 #include "harp_regs.h"
@@ -38,6 +39,8 @@ struct Ph {
     static constexpr int kStages = 1 + (B > 1) + (C > 1);
     static constexpr int kRadices = A + (B > 1 ? B : 0) + (C > 1 ? C : 0);     // kernel entries per value
 };
+// one stage of radix 16, its units' results shared by four threads: 64 kernel entries and four results each, all values read by each
+struct Ph16 { static constexpr int A = 16, B = 1, C = 1, N = 16, kStages = 1, kRadices = 16; };
 struct None { static constexpr int A = 1, B = 1, C = 1, N = 1, kStages = 0, kRadices = 0; };
 
 // geometry of a phase: tile stride T, units dealt to U owners, `kSets` each
@@ -51,6 +54,16 @@ struct Geo {
     static __device__ __forceinline__ int coord(int owner, int i) {
         const int u = unit(owner, i / N);
         return (u / T) * (T * N) + (i % N) * T + u % T;
+    }
+};
+
+template <int NC, int T_, int U>
+struct Geo<Ph16, NC, T_, U> {
+    static constexpr int T = T_, N = 16, kUnits = NC / N, kSets = 1, V = 4, kW = 64;
+    static_assert(4 * kUnits == U, "four owners a unit");
+    static __device__ __forceinline__ int coord(int owner, int i) {
+        const int u = owner >> 2;
+        return (u / T) * (T * N) + i * T + u % T;
     }
 };
 
@@ -94,6 +107,22 @@ __device__ __forceinline__ void load_stage(float *w, const float *blocks, int n_
 // pos: plan coordinate of the first value of set n of this owner
 template <class P, class G, bool TR, bool EM, typename Pos>
 __device__ __forceinline__ void load_phase(float (&w)[G::kW], const float *blocks, const int64_t *off, int d, int Sp, const int8_t *signs, const Pos &pos) {
+    if constexpr (std::is_same_v<P, Ph16>) {                   // w[operand][result of this owner's four]
+        const int p = pos(0), r = p % Sp, org = p - r, n_blk = d / 16, j0 = 4 * ((int)threadIdx.x & 3);
+        const float *k = blocks + off[0] + org / 16 + r;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) w[4 * i + j] = __ldg(k + (TR ? (j0 + j) * 16 + i : i * 16 + j0 + j) * n_blk);
+        if (signs) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (signs[p + (TR ? j0 + j : i) * Sp] < 0) w[4 * i + j] *= -1.f;
+        }
+        return;
+    } else
 #pragma unroll
     for (int n = 0; n < G::kSets; ++n) {
         const int p = pos(n), r = p % Sp, org = p - r;
@@ -188,6 +217,39 @@ __device__ __forceinline__ void rows_phase(uint32_t tile, const float (&w)[Ge::k
                     sts1(a[i] + (r + u) * kVec, v[u][i][0]);
                 }
             }
+    }
+}
+
+// the same for units shared by four threads: nobody stores before everybody has read
+template <class Ge, int G, uint32_t kVec>
+__device__ __forceinline__ void rows_phase_shared(uint32_t tile, const float (&w)[Ge::kW]) {
+    constexpr bool kRun = Ge::T == 1;
+    const uint32_t p0 = place(Ge::coord(threadIdx.x, 0));
+    const int j0 = 4 * ((int)threadIdx.x & 3);
+    float o[G][4];
+#pragma unroll
+    for (int r = 0; r < G; ++r) {
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; i += kRun ? 4 : 1) {
+            const uint32_t a = tile + (p0 ^ place(i * Ge::T)) + r * kVec;
+            if constexpr (kRun) lds4(v + i, a);
+            else v[i] = lds1(a);
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[r][j] = i == 0 ? v[0] * w[j] : fmaf(v[i], w[4 * i + j], o[r][j]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < G; ++r) {
+        if constexpr (kRun) {
+            sts4(tile + place(Ge::coord(threadIdx.x, j0)) + r * kVec, o[r]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sts1(tile + place(Ge::coord(threadIdx.x, j0 + j)) + r * kVec, o[r][j]);
+        }
     }
 }
 
@@ -323,6 +385,7 @@ harp_regs_kernel(const float *__restrict__ blocks, const int8_t *__restrict__ si
                     else return w3;
                 }();
                 if constexpr (C::COL) cols_phase<Pp, Gp, C::TR>(tile, w, warp, lane);
+                else if constexpr (std::is_same_v<Pp, Ph16>) rows_phase_shared<Gp, C::G, C::kVec>(tile, w);
                 else rows_phase<Pp, Gp, C::G, C::kVec, C::TR>(tile, w);
             }
         };
@@ -416,6 +479,7 @@ const Shape kShapes[] = {
     {false, 512, 64, 0, 8, {2, 2, 2, 2, 2, 2, 2, 2}},
     {false, 512, 64, 0, 3, {8, 8, 8}},
     {false, 512, 64, 0, 3, {4, 4, 4}},
+    {false, 512, 128, 0, 2, {16, 16}},
     {false, 512, 64, 64, 1, {8}},
     {false, 512, 64, 32, 2, {8, 2}},
     {false, 2048, 256, 32, 2, {8, 8}},
@@ -445,6 +509,8 @@ bool harp_regs_pass(const StageTable &st, int64_t d, int t0, int t1, bool col, R
         const int64_t S = st.s[t0];
         int64_t E = 1;
         for (int t = t0; t < t1; ++t) E *= st.b[t];
+        // radix 16 in narrow rows: the whole-row kernels take small batches in one launch
+        if (sh.b[0] == 16 && d <= 4096) continue;
         // all of a row's coordinates in a row of memory (whole rows of d up to NC: several to a tile), or runs of L below the stride
         if (sh.l == 0 ? S != 1 || d % 32 != 0 || (d < sh.nc && (sh.nc % d != 0 || E != d)) : S % sh.l != 0) continue;
         P = RegPass{};
@@ -488,19 +554,20 @@ cudaError_t harp_regs_launch(void *encode, const RegPass &P, int sms, float *x, 
         HARP_REGS_ROWS(4, 512, 64, 0, P222, P222, P22);
         HARP_REGS_ROWS(5, 512, 64, 0, P8, P8, P8);
         HARP_REGS_ROWS(6, 512, 64, 0, P4, P4, P4);
-        HARP_REGS_ROWS(7, 512, 64, 64, P8);
-        HARP_REGS_ROWS(8, 512, 64, 32, P8, P2);
-        HARP_REGS_ROWS(9, 2048, 256, 32, P8, P8);
-        HARP_REGS_ROWS(10, 2048, 256, 32, P4, P4, P4);
-        HARP_REGS_ROWS(11, 1792, 256, 32, P8, Ph<7>);
-        HARP_REGS_ROWS(12, 1280, 128, 128, Ph<5, 2>);
-        HARP_REGS_COLS(13, 64, 1, P8, P8);
-        HARP_REGS_COLS(14, 64, 8, P8);
-        HARP_REGS_COLS(15, 64, 4, P8, P2);
-        HARP_REGS_COLS(16, 64, 1, P222, P222);
-        HARP_REGS_COLS(17, 64, 2, P222, P22);
-        HARP_REGS_COLS(18, 64, 1, P4, P4, P4);
-        HARP_REGS_COLS(19, 80, 8, Ph<5, 2>);
+        HARP_REGS_ROWS(7, 512, 128, 0, Ph16, Ph16);
+        HARP_REGS_ROWS(8, 512, 64, 64, P8);
+        HARP_REGS_ROWS(9, 512, 64, 32, P8, P2);
+        HARP_REGS_ROWS(10, 2048, 256, 32, P8, P8);
+        HARP_REGS_ROWS(11, 2048, 256, 32, P4, P4, P4);
+        HARP_REGS_ROWS(12, 1792, 256, 32, P8, Ph<7>);
+        HARP_REGS_ROWS(13, 1280, 128, 128, Ph<5, 2>);
+        HARP_REGS_COLS(14, 64, 1, P8, P8);
+        HARP_REGS_COLS(15, 64, 8, P8);
+        HARP_REGS_COLS(16, 64, 4, P8, P2);
+        HARP_REGS_COLS(17, 64, 1, P222, P222);
+        HARP_REGS_COLS(18, 64, 2, P222, P22);
+        HARP_REGS_COLS(19, 64, 1, P4, P4, P4);
+        HARP_REGS_COLS(20, 80, 8, Ph<5, 2>);
         default: return cudaErrorInvalidValue;
     }
 #undef HARP_REGS_COLS

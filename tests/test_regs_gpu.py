@@ -32,6 +32,7 @@ def _rows_match(radices, perm, n_rows):
     ((2,) * 8 + (11,), "identity"),       # a group of three quarters of a tile
     ((8, 8, 8, 8, 7), "identity"),        # 224 of 256 threads own a unit of eight
     ((8, 8, 8, 8, 8), "identity"),
+    ((16, 16, 8, 7), "identity"), ((16, 16, 43), "random"),    # units of sixteen shared by four threads
 ])
 def test_passes_in_registers(monkeypatch, radices, perm, n_rows):
     monkeypatch.setenv("HARP_F32_PASSES", "1")
