@@ -1386,9 +1386,11 @@ outer_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const T
     }
 }
 
+constexpr int64_t kMostScratch = 1280ll << 20, kLeastScratch = 160ll << 20;     // bytes of states of a chunk
+
 // Scratch comes from a memory pool of the library's own (one per device, created on first use)
-// whose release threshold is unlimited: the default pool hands its memory back at every
-// synchronisation, and mapping 256 MB anew costs more than the kernels of a call.  Returns null
+// that keeps one call's worth: the default pool hands its memory back at every
+// synchronisation, and mapping 256 MB anew costs more than the kernels of a call.  What calls on several streams take beyond it goes back at a synchronisation.  Returns null
 // if the pool cannot be created; the caller then allocates from the device's default pool.
 cudaMemPool_t scratch_pool(int device) {
     static std::mutex mu;
@@ -1406,14 +1408,12 @@ cudaMemPool_t scratch_pool(int device) {
         cudaGetLastError();
         pool = nullptr;
     } else {
-        uint64_t keep = ~0ull;
+        uint64_t keep = (uint64_t)kMostScratch + (256ull << 20);      // a call's states and partial sums
         cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
     pools[device] = pool;
     return pool;
 }
-
-constexpr int64_t kMostScratch = 1280ll << 20, kLeastScratch = 160ll << 20;     // bytes of states of a chunk
 
 // grid of the kernels in which a thread keeps its coordinate and walks over rows
 dim3 column_grid(int64_t d, int64_t rows) {
