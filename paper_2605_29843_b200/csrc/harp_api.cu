@@ -46,7 +46,8 @@ extern "C" const char *harp_status_string(harp_status_t s) {
 
 extern "C" int32_t harp_plan_error_word(const harp_plan_t *plan) {
     if (!plan) return -1;
-    const int32_t w = harp_tm_error_word(plan);
+    int32_t w = harp_tm_error_word(plan);
+    if (w == 0) w = harp_fast_error_word(plan);
     if (w != 0) return w;
     const int32_t s = harp_split_error_word(plan), c = harp_col_error_word(plan);
     return s != 0 ? s : c != 0 ? c : harp_f32_error_word(plan);

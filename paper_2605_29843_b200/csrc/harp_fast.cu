@@ -45,6 +45,10 @@
 namespace {
 
 constexpr int kMaxPhases = 8;
+// Threads of the kernels for clusters of eight and sixteen CTAs: a CTA has two to eight items of eight blocks a phase, and 255 registers
+// hold the next ones' fragments (16 rows of d = 4096 in radix 16 5.4 -> 4.7 us with 512 threads and with 256, in radix 8 5.9 -> 5.5).
+constexpr int kCountedThreads = 256;
+constexpr uint32_t kExchangeSpin = 1u << 22;   // limit of a wait for the bytes of an exchange
 constexpr int kTileRows = 16;
 constexpr int kThreads = 512;
 
@@ -90,6 +94,7 @@ struct FastParams {
     const int32_t *ctab;
     int32_t ctab_len, order_in, order_out;
     uint32_t xchg_mask;
+    int32_t *err;              // set when a wait for an exchange gave up
     ClusterPhase cl[kMaxPhases];
 };
 
@@ -135,11 +140,11 @@ __device__ __forceinline__ uint32_t tm_item(const TileCtx &c, int slot, int it) 
 
 // ---- MODE_SS, B = 16: load / store of one item's operands
 __device__ __forceinline__ void ss16_load(const TileCtx &c, const PhaseDesc &ph, int it, uint4 (&raw)[4][2], uint4 (&bf)[8],
-                                          int tm_slot) {
+                                          int tm_slot, bool have_frag = false) {
     const uint32_t a0 = c.sbase + 2u * (uint32_t)(c.g * c.pitch + c.q * ph.lane_step + c.tab[ph.items_off + it]);
     const uint32_t a1 = a0 + 2u * (uint32_t)(8 * c.pitch);
     const uint4 *bp = ph.bfrag + (size_t)it * 256 + c.lane;
-    load_frag8(bf, bp, tm_slot >= 0, tm_item(c, tm_slot, it));
+    if (!have_frag) load_frag8(bf, bp, tm_slot >= 0, tm_item(c, tm_slot, it));
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         raw[j][0] = lds128(a0 + 2u * ph.j_off[j]);
@@ -156,26 +161,49 @@ __device__ __forceinline__ void ss16_store(const TileCtx &c, const PhaseDesc &ph
     }
 }
 // The same store in the cluster variant after an exchange phase: slot j of lane q goes to the CTA that owns the phase's local
-// index of that slot from here on, at the same place of its tile.
+// index of that slot from here on, at the same place of its tile, and counts on that CTA's barrier of the phase.
+__device__ __forceinline__ void st_async128(uint32_t addr, uint32_t bar, uint32_t rank, const uint4 &v) {
+    uint32_t remote, remote_bar;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote_bar) : "r"(bar), "r"(rank));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1,%2,%3,%4}, [%5];"
+                 ::"r"(remote), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(remote_bar) : "memory");
+}
 __device__ __forceinline__ void st_cluster128(uint32_t addr, uint32_t rank, const uint4 &v) {
     uint32_t remote;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
     asm volatile("st.shared::cluster.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(remote), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-template <int NJ>
-__device__ __forceinline__ void store_to_owner(const TileCtx &c, const PhaseDesc &ph, const ClusterPhase &cl, int it, const uint4 (&raw)[NJ][2], int cs) {
+template <int NJ, bool COUNTED>
+__device__ __forceinline__ void store_to_owner(const TileCtx &c, const PhaseDesc &ph, const ClusterPhase &cl, int it, const uint4 (&raw)[NJ][2],
+                                               int lg, uint32_t bar) {
     const uint32_t a0 = c.sbase + 2u * (uint32_t)(c.g * c.pitch + c.q * ph.lane_step + c.tab[ph.items_off + it]);
     const uint32_t a1 = a0 + 2u * (uint32_t)(8 * c.pitch);
+    constexpr int kLgB = NJ == 4 ? 4 : 3;
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
-        const uint32_t rank = (uint32_t)((cl.lm * c.q + cl.jr[j]) * cs / ph.B);
-        st_cluster128(a0 + 2u * ph.j_off[j], rank, raw[j][0]);
-        st_cluster128(a1 + 2u * ph.j_off[j], rank, raw[j][1]);
+        const uint32_t rank = (uint32_t)(cl.lm * c.q + cl.jr[j]) >> (kLgB - lg);
+        if (COUNTED) {
+            if (c.okA) st_async128(a0 + 2u * ph.j_off[j], bar, rank, raw[j][0]);
+            if (c.okB) st_async128(a1 + 2u * ph.j_off[j], bar, rank, raw[j][1]);
+        } else {
+            st_cluster128(a0 + 2u * ph.j_off[j], rank, raw[j][0]);
+            st_cluster128(a1 + 2u * ph.j_off[j], rank, raw[j][1]);
+        }
     }
 }
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+// until all bytes of an exchange are here; gives up, and says so, after a bounded number of tries
+__device__ __forceinline__ void wait_exchange(uint32_t bar, int32_t *err) {
+    for (uint32_t tries = 0; tries < kExchangeSpin; ++tries) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar) : "memory");
+        if (ok) return;
+    }
+    *err = 1;
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // ---- MODE_GS: operands from global memory
 __device__ __forceinline__ void gs_load(const TileCtx &c, const PhaseDesc &ph, int it, uint4 (&raw)[4][2], uint4 (&bf)[8],
                                         int tm_slot) {
@@ -205,15 +233,25 @@ constexpr uint32_t kModesGeneral = bit(MODE_CC) | bit(MODE_SS) | bit(MODE_GS) | 
 constexpr uint32_t kModesInPlace = bit(MODE_CC) | bit(MODE_SS);                 // identity permutation
 constexpr uint32_t kModesReorderOut = bit(MODE_SS) | bit(MODE_PO);   // the digit-reversal scheme, both directions
 
-// CL: a cluster of cs CTAs works on one tile (batches whose tiles would leave most SMs idle).  Every CTA keeps the tile's layout
+// KIND: a cluster of 2^lg CTAs works on one tile (batches whose tiles would leave most SMs idle).  Every CTA keeps the tile's layout
 // and holds the part of it that it owns: the blocks of a phase are dealt out by the value of a digit that the phase does
 // not mix, and where the next phase needs another digit the phase's results are written to their new owner through
 // distributed shared memory.  What bounds a lone tile is one SM fetching the block kernels of a whole row (393 KB at
-// d = 4096) and running their items one after the other; cs SMs share both.
-template <int NT, uint32_t MODES, bool CL>
+// d = 4096) and running their items one after the other; the SMs of a cluster share both.  What bounds a cluster is a chain of
+// latencies, so nothing that a shift can do is a division (16 rows of d = 4096: 6.5 -> 5.5 us), and rows that are not there are
+// neither copied nor exchanged (1 row 4.4 us).  CLUSTER_COUNTED (eight and sixteen CTAs): the exchange is st.async, every piece
+// counted on a barrier of its new owner, which waits for its own bytes alone; a cluster barrier after plain remote stores is a
+// release and an acquire of all memory (8.1 -> 7.7 us).  Nothing is overwritten early: a CTA stores to another only positions
+// that the other does not own in the phases before, and it stores after an exchange only once every CTA's items of
+// the phase before have arrived.  CLUSTER (two and four CTAs) keeps the barrier: 2048 pieces a CTA take st.async
+// longer than the barrier costs (256 rows 9.6 against 11.2 us).
+enum { ALONE = 0, CLUSTER = 1, CLUSTER_COUNTED = 2 };
+
+template <int NT, uint32_t MODES, int KIND>
 __global__ void __launch_bounds__(NT, 1)
-harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles, int stagger, int cs, FastParams P) {
+harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles, int stagger, int lg, FastParams P) {
     constexpr int NW = NT / 32;
+    constexpr bool CL = KIND != ALONE, COUNTED = KIND == CLUSTER_COUNTED;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileCtx c;
     c.sbase = smem_u32(smem_raw);
@@ -224,10 +262,25 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
     c.q = c.lane & 3;
     const int d = P.d, pitch = P.pitch;
     int32_t *tab_s = reinterpret_cast<int32_t *>(smem_raw + (size_t)kTileRows * pitch * 2);
+    // cluster variant: one barrier per exchange, behind the tables; every one of them completes once
+    const uint32_t bars = COUNTED ? (smem_u32(tab_s + P.tables_len + P.ctab_len) + 7u) & ~7u : 0;
+    if (CL) {
+        if (COUNTED && threadIdx.x == 0) {
+            const int64_t rows = min((int64_t)kTileRows, n_rows - (int64_t)(blockIdx.x >> lg) * kTileRows);
+            for (int p = 0; p < P.n_phases; ++p)
+                if ((P.xchg_mask >> p) & 1u) {
+                    harp_tm::mbar_init(bars + 8 * p, 1);
+                    harp_tm::mbar_expect_tx(bars + 8 * p, (uint32_t)(2 * rows * (P.d >> lg)));
+                }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        __syncwarp();
+        cluster_arrive();
+    }
     for (int i = threadIdx.x; i < P.tables_len; i += NT) tab_s[i] = __ldg(P.tables + i);
     c.tab = tab_s;
     // cluster variant: rank, and the chunk and item orders behind the tables
-    const int rank = CL ? (int)(blockIdx.x % (unsigned)cs) : 0;
+    const int rank = CL ? (int)(blockIdx.x & ((1u << lg) - 1u)) : 0;
     const int32_t *ord = tab_s + P.tables_len;
     if (CL)
         for (int i = threadIdx.x; i < P.ctab_len; i += NT) tab_s[P.tables_len + i] = __ldg(P.ctab + i);
@@ -259,6 +312,19 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
         harp_tm::tmem_wait_st();
     }
     const int warp = c.warp, lane = c.lane;
+    // Counted clusters: the fragments of a warp's first item of the next phase come to registers while the rows or the
+    // exchange are on their way
+    constexpr bool kAhead = COUNTED;
+    uint4 ahead[8];
+    auto fetch_ahead = [&](int p) {
+        if (p >= P.n_phases) return;
+        const PhaseDesc &ph = P.ph[p];
+        if (ph.B != 16 || ph.mode == MODE_CC || warp >= (ph.n_items >> lg)) return;
+        const uint4 *bp = ph.bfrag + (size_t)ord[P.cl[p].order + rank * (ph.n_items >> lg) + warp] * 256 + lane;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) ahead[e] = __ldg(bp + e * 32);
+    };
+    if (kAhead) fetch_ahead(0);
 
     // All CTAs have the same work, so without this they copy their tiles in step and share the
     // HBM bandwidth at those moments while it idles during the phases.  Three classes of CTAs
@@ -272,13 +338,13 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
     // attribute, a CTA gets here while the kernel before it in the stream is still running on other SMs
     // (tables, tensor-memory fill and the start delay then cost nothing); the rows are touched only after
     // that kernel has completed.  The kernel after this one may start its own preamble as SMs become free.
-    if (CL) cluster_sync();                        // every CTA of the cluster is running before anybody writes to its shared memory
+    if (CL) cluster_wait();                        // every CTA of the cluster is running, its barriers set, before anybody writes to its shared memory
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #ifdef HARP_FAST_TIMING
     long long tacc[16] = {0}, tlast = clock64();
 #endif
-    for (int64_t tile = CL ? blockIdx.x / (unsigned)cs : blockIdx.x; tile < n_tiles; tile += CL ? n_tiles : gridDim.x) {
+    for (int64_t tile = CL ? blockIdx.x >> lg : blockIdx.x; tile < n_tiles; tile += CL ? n_tiles : gridDim.x) {
         const int64_t row0 = tile * kTileRows;
 #ifdef HARP_FAST_TIMING
         if (threadIdx.x == 0) { tacc[0] += 1; tlast = clock64(); }
@@ -294,16 +360,17 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
             // a thread owns the same 16-byte chunks of every row; no index arithmetic per chunk
             const int32_t *cmap = tab_s + P.copy_in;
             const int chunks = d >> 3;
-            const int per_in = CL ? chunks / cs : chunks, first_in = CL ? rank * per_in : 0;
-            const int rsteps = CL ? max(1, NT / per_in) : 1, r_first = CL && rsteps > 1 ? threadIdx.x / per_in : 0;     // few chunks: threads share the rows
+            const int lg_in = CL ? 28 - __clz(d) - lg : 0, per_in = chunks >> (CL ? lg : 0), first_in = CL ? rank * per_in : 0;
+            const int rsteps = CL ? max(1, NT >> lg_in) : 1, r_first = CL && rsteps > 1 ? threadIdx.x >> lg_in : 0;     // (d is a power of two) few chunks: threads share the rows
             if (r_first < rsteps)
-            for (int cj = CL && rsteps > 1 ? threadIdx.x - r_first * per_in : threadIdx.x; cj < per_in; cj += NT) {
+            for (int cj = CL && rsteps > 1 ? threadIdx.x & (per_in - 1) : threadIdx.x; cj < per_in; cj += NT) {
                 const int ch = CL ? ord[P.order_in + first_in + cj] : cj;
                 const uint32_t dst = c.sbase + 2u * (uint32_t)cmap[ch];
                 const __nv_bfloat16 *src = x + row0 * d + 8 * ch;
                 const __nv_bfloat16 *last_src = x + last * d + 8 * ch;
+                const int r_end = COUNTED ? (int)min((int64_t)kTileRows, n_rows - row0) : kTileRows;     // (a cluster neither copies nor exchanges the rows that are not there)
 #pragma unroll 4
-                for (int r = r_first; r < kTileRows; r += rsteps)
+                for (int r = r_first; r < r_end; r += rsteps)
                     cp_async16(dst + 2u * (uint32_t)(r * pitch), row0 + r <= last ? src + (int64_t)r * d : last_src);
             }
             cp_async_wait_all();
@@ -314,14 +381,60 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
         for (int p = 0; p < P.n_phases; ++p) {
             const PhaseDesc &ph = P.ph[p];
             // items [0, n) of the phase, or this CTA's share of them in its order
-            const int n = CL ? ph.n_items / cs : ph.n_items;
+            const int n = CL ? ph.n_items >> lg : ph.n_items;
             const int32_t *item = ord + (CL ? P.cl[p].order : 0) + rank * n;
             const bool xchg = CL && ((P.xchg_mask >> p) & 1u);
+            const bool fetched = kAhead && (p == 0 || ((P.xchg_mask >> (p - 1)) & 1u));      // `ahead` holds the warp's first item
             const int tm_slot = !CL && ((P.tm_mask >> p) & 1u) ? __popc(P.tm_mask & ((1u << p) - 1u)) : -1;
             if ((MODES & bit(MODE_CC)) && ph.mode == MODE_CC) {
                 // lane -> (matrix row, 8-column half) of the 16x16 (or 16x8) operand tile
                 const int mrow = (lane & 7) + ((lane >> 3) & 1) * 8, mcol = (lane >> 4) * 8;
-                if (ph.B == 16) {
+                if (COUNTED) {
+                    // four items at a time: numbers, fragments and rows of all of them before the first product (one after the
+                    // other, each waits for its own fragment: 16 rows of d = 4096 in radix 8 5.9 -> 5.5 us)
+                    const bool wide = ph.B == 16;
+                    const uint32_t row_addr = c.sbase + 2u * (uint32_t)(wide ? mrow * pitch + mcol : (lane & 15) * pitch);
+                    for (int k0 = warp; k0 < n; k0 += 4 * NW) {
+                        int it[4];
+                        uint32_t addr[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) it[u] = item[min(k0 + u * NW, n - 1)];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) addr[u] = row_addr + 2u * (uint32_t)tab_s[ph.items_off + it[u]];
+                        if (wide) {
+                            uint4 bf[4];
+                            uint32_t a[4][4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) bf[u] = __ldg(ph.bfrag + (size_t)it[u] * 32 + lane);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (k0 + u * NW < n) ldmatrix_x4(a[u], addr[u]);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (k0 + u * NW < n) {
+                                    float c0[4], c1[4];
+                                    mma_k16(c0, a[u], bf[u].x, bf[u].y);
+                                    mma_k16(c1, a[u], bf[u].z, bf[u].w);
+                                    stmatrix_x4(addr[u], pack_bf16(c0[0], c0[1]), pack_bf16(c0[2], c0[3]), pack_bf16(c1[0], c1[1]), pack_bf16(c1[2], c1[3]));
+                                }
+                        } else {
+                            const uint32_t *bf8 = reinterpret_cast<const uint32_t *>(ph.bfrag);
+                            uint32_t bf[4], a[4][2];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) bf[u] = __ldg(bf8 + (size_t)it[u] * 32 + lane);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (k0 + u * NW < n) ldmatrix_x2(a[u], addr[u]);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (k0 + u * NW < n) {
+                                    float c0[4];
+                                    mma_k8(c0, a[u], bf[u]);
+                                    stmatrix_x2(addr[u], pack_bf16(c0[0], c0[1]), pack_bf16(c0[2], c0[3]));
+                                }
+                        }
+                    }
+                } else if (ph.B == 16) {
 #pragma unroll 4
                     for (int k = warp; k < n; k += NW) {
                         const int it = CL ? item[k] : k;
@@ -357,9 +470,14 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                 uint32_t unused[8][4];
                 for (int k = warp; k < n; k += NW) {
                     const int it = CL ? item[k] : k;
-                    ss16_load(c, ph, it, raw, bf, tm_slot);
+                    const bool have = fetched && k == warp;
+                    if (have) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) bf[e] = ahead[e];
+                    }
+                    ss16_load(c, ph, it, raw, bf, tm_slot, have);
                     octet_mma16<true>(raw, bf, unused);
-                    if (xchg) store_to_owner<4>(c, ph, P.cl[p], it, raw, cs);
+                    if (xchg) store_to_owner<4, COUNTED>(c, ph, P.cl[p], it, raw, lg, bars + 8 * p);
                     else ss16_store(c, ph, it, raw);
                 }
             } else if ((MODES & bit(MODE_SS)) && ph.mode == MODE_SS) {
@@ -379,7 +497,7 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                     }
                     octet_mma8(raw, bf);
                     if (xchg) {
-                        store_to_owner<2>(c, ph, P.cl[p], it, raw, cs);
+                        store_to_owner<2, COUNTED>(c, ph, P.cl[p], it, raw, lg, bars + 8 * p);
                         continue;
                     }
 #pragma unroll
@@ -405,7 +523,12 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                         const int it = CL ? item[k] : k;
                     const int32_t *tab = tab_s + ph.items_off + it * 24;
                     uint4 bf[8], out[4][2];
-                    load_frag8(bf, ph.bfrag + (size_t)it * 256 + lane, tm_slot >= 0, tm_item(c, tm_slot, it));
+                    if (fetched && k == warp) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) bf[e] = ahead[e];
+                    } else {
+                        load_frag8(bf, ph.bfrag + (size_t)it * 256 + lane, tm_slot >= 0, tm_item(c, tm_slot, it));
+                    }
 #pragma unroll
                     for (int w = 0; w < 4; ++w) {
                         float acc[2][2][4];
@@ -468,7 +591,9 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                     }
                 }
             }
-            if (xchg) cluster_sync();
+            if (kAhead && xchg) fetch_ahead(p + 1);
+            if (COUNTED && xchg) wait_exchange(bars + 8 * p, P.err);
+            else if (xchg) { cluster_arrive(); cluster_wait(); }
             else __syncthreads();
             FAST_MARK(2 + p);
         }
@@ -477,10 +602,10 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
             const int32_t *cmap = tab_s + P.copy_out;
             const int chunks = d >> 3;
             const int rows = (int)min((int64_t)kTileRows, n_rows - row0);
-            const int per_out = CL ? chunks / cs : chunks, first_out = CL ? rank * per_out : 0;
-            const int rsteps = CL ? max(1, NT / per_out) : 1, r_first = CL && rsteps > 1 ? threadIdx.x / per_out : 0;
+            const int lg_out = CL ? 28 - __clz(d) - lg : 0, per_out = chunks >> (CL ? lg : 0), first_out = CL ? rank * per_out : 0;
+            const int rsteps = CL ? max(1, NT >> lg_out) : 1, r_first = CL && rsteps > 1 ? threadIdx.x >> lg_out : 0;
             if (r_first < rsteps)
-            for (int cj = CL && rsteps > 1 ? threadIdx.x - r_first * per_out : threadIdx.x; cj < per_out; cj += NT) {
+            for (int cj = CL && rsteps > 1 ? threadIdx.x & (per_out - 1) : threadIdx.x; cj < per_out; cj += NT) {
                 const int ch = CL ? ord[P.order_out + first_out + cj] : cj;
                 const uint32_t src = c.sbase + 2u * (uint32_t)cmap[ch];
                 __nv_bfloat16 *dst = x + row0 * d + 8 * ch;
@@ -512,10 +637,11 @@ struct FastPlan {
     size_t smem_bytes = 0;
     int variant_fwd = 0, variant_bwd = 0;     // which compiled set of phase modes each direction needs
     std::vector<void *> dev_allocs;
+    int32_t *d_err = nullptr;
     int max_ctas = 0;
     int max_cluster = 1;                      // CTAs that may share a tile (1: no cluster variant)
     size_t cl_smem_bytes = 0;
-    int clusters[4] = {0, 0, 0, 0};           // clusters of 1, 2, 4, 8 CTAs the device holds at once
+    int clusters[5] = {0, 0, 0, 0, 0};        // clusters of 1, 2, 4, 8, 16 CTAs the device holds at once
 };
 
 namespace {
@@ -530,6 +656,15 @@ T *upload(FastPlan *fp, const std::vector<T> &v, harp_status_t &st) {
     fp->dev_allocs.push_back(p);
     if (!v.empty() && cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) st = HARP_ERR_CUDA;
     return static_cast<T *>(p);
+}
+
+int cluster_threads(int cs) { return cs >= 8 ? kCountedThreads : kThreads; }
+
+// f(kernel that runs clusters of cs CTAs)
+template <typename F>
+cudaError_t with_cluster_kernel(bool reorder, int cs, F f) {
+    if (cs < 8) return reorder ? f(harp_fast_kernel<kThreads, kModesReorderOut, CLUSTER>) : f(harp_fast_kernel<kThreads, kModesInPlace, CLUSTER>);
+    return reorder ? f(harp_fast_kernel<kCountedThreads, kModesReorderOut, CLUSTER_COUNTED>) : f(harp_fast_kernel<kCountedThreads, kModesInPlace, CLUSTER_COUNTED>);
 }
 
 }  // namespace
@@ -1141,15 +1276,18 @@ harp_status_t harp_fast_build(harp_plan *plan) {
         P.tables_len = (int32_t)tables.size();
         P.ctab = upload(fp, ctab, st);
         P.ctab_len = (int32_t)ctab.size();
-        fp->cl_smem_bytes = std::max(fp->cl_smem_bytes, tile_bytes + (tables.size() + ctab.size()) * sizeof(int32_t) + 16);
+        if (clustered && !fp->d_err) fp->d_err = upload(fp, std::vector<int32_t>{0}, st);
+        P.err = fp->d_err;
+        fp->cl_smem_bytes = std::max(fp->cl_smem_bytes, tile_bytes + (tables.size() + ctab.size()) * sizeof(int32_t) + 8 + 8 * kMaxPhases);
         fp->smem_bytes = std::max(fp->smem_bytes, tile_bytes + tables.size() * sizeof(int32_t) + 16);
     }
     if (st == HARP_OK && fp->smem_bytes > 227u * 1024u) st = HARP_ERR_UNSUPPORTED;
     if (st == HARP_OK) {
-        if (cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesGeneral, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-            cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesReorderOut, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-            cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesInPlace, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-            cudaFuncSetAttribute(harp_fast_kernel<kThreads, kModesReorderOut, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+        auto allow = [&](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess; };
+        if (!allow(harp_fast_kernel<kThreads, kModesGeneral, ALONE>) || !allow(harp_fast_kernel<kThreads, kModesReorderOut, ALONE>) ||
+            !allow(harp_fast_kernel<kThreads, kModesInPlace, CLUSTER>) || !allow(harp_fast_kernel<kThreads, kModesReorderOut, CLUSTER>) ||
+            !allow(harp_fast_kernel<kCountedThreads, kModesInPlace, CLUSTER_COUNTED>) ||
+            !allow(harp_fast_kernel<kCountedThreads, kModesReorderOut, CLUSTER_COUNTED>))
             st = HARP_ERR_CUDA;
         fp->variant_fwd = digitrev ? 1 : 0;
         fp->variant_bwd = digitrev ? 1 : 0;
@@ -1158,21 +1296,26 @@ harp_status_t harp_fast_build(harp_plan *plan) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         fp->max_ctas = sms > 0 ? sms : 148;
         if (clustered && fp->cl_smem_bytes <= 227u * 1024u) {
-            fp->max_cluster = std::min(phases[(size_t)(np - 1)].B, std::min(phases[(size_t)(np - 2)].B, phases[0].B)) >= 8 ? 8 : 1;
-            for (int lg = 1; lg < 4; ++lg) {
+            fp->max_cluster = std::min(phases[(size_t)(np - 1)].B, std::min(phases[(size_t)(np - 2)].B, phases[0].B));     // 8 or 16
+            auto wide = [&](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess; };
+            if (!wide(harp_fast_kernel<kCountedThreads, kModesInPlace, CLUSTER_COUNTED>) ||
+                !wide(harp_fast_kernel<kCountedThreads, kModesReorderOut, CLUSTER_COUNTED>)) {
+                cudaGetLastError();
+                fp->max_cluster = 8;
+            }
+            for (int lg = 1; lg < 5 && (1 << lg) <= fp->max_cluster; ++lg) {
                 cudaLaunchConfig_t cfg = {};
                 cudaLaunchAttribute at[1];
                 at[0].id = cudaLaunchAttributeClusterDimension;
                 at[0].val.clusterDim.x = 1u << lg;
                 at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
                 cfg.gridDim = dim3((unsigned)fp->max_ctas / (1u << lg) * (1u << lg));
-                cfg.blockDim = dim3(kThreads);
+                cfg.blockDim = dim3(cluster_threads(1 << lg));
                 cfg.dynamicSmemBytes = fp->cl_smem_bytes;
                 cfg.attrs = at;
                 cfg.numAttrs = 1;
                 int nc = 0;
-                const cudaError_t e = digitrev ? cudaOccupancyMaxActiveClusters(&nc, harp_fast_kernel<kThreads, kModesReorderOut, true>, &cfg)
-                                               : cudaOccupancyMaxActiveClusters(&nc, harp_fast_kernel<kThreads, kModesInPlace, true>, &cfg);
+                const cudaError_t e = with_cluster_kernel(digitrev, 1 << lg, [&](auto kernel) { return cudaOccupancyMaxActiveClusters(&nc, kernel, &cfg); });
                 if (e != cudaSuccess) { cudaGetLastError(); nc = 0; }
                 fp->clusters[lg] = nc;
             }
@@ -1197,6 +1340,13 @@ extern "C" int32_t harp_debug_fast_timing(int64_t *out, int32_t reset) {
         if (cudaMemcpyToSymbol(g_fast_timing, zero, sizeof(zero)) != cudaSuccess) return -1;
     }
     return 0;
+}
+
+// Non-zero if a kernel of this plan gave up on a wait since the plan was built (synchronises the device copy of the word; for tests).
+int32_t harp_fast_error_word(const harp_plan *plan) {
+    if (!plan->fast || !plan->fast->d_err) return 0;
+    int32_t v = 0;
+    return cudaMemcpy(&v, plan->fast->d_err, sizeof(v), cudaMemcpyDeviceToHost) == cudaSuccess ? v : -1;
 }
 
 void harp_fast_destroy(harp_plan *plan) {
@@ -1232,17 +1382,20 @@ harp_status_t harp_fast_apply(const harp_plan *plan, void *x, int64_t n_rows, ha
     // a quarter of a tile period, estimated from the measured 28 k cycles per tile of d = 4096 with
     // three phases (the gain is flat between half and the full value)
     const int stagger = n_tiles >= 4 * (int64_t)grid ? (int)(0.57 * (double)P.d * P.n_phases) : 0;
-    // Clusters while all tiles are in flight at once.  Measured (16 to 1100 rows, radices 8 and 16): eight CTAs gain from d = 2048 on
-    // (16 rows of d = 4096: 12.3 -> 7.8 us, radix 8 15.5 -> 6.9), four from 4096 on (500 rows: 12.7 -> 11.9, radix 8 15.8 ->
-    // 10.5), two only where four phases are run (1100 rows, radix 8: 15.9 -> 14.6; radix 16 13.0 -> 13.5)
+    // Clusters while all tiles are in flight at once.  Measured (1 to 1100 rows, radices 8 and 16): sixteen CTAs, for which every phase has
+    // to be 16 wide, gain where four to seven tiles are all the device holds that way (16 rows of d = 4096: eight CTAs 5.5 us, sixteen 5.0;
+    // 100 rows 6.5 and 6.1), eight from d = 2048 on (one CTA a tile 12.3 us, radix 8 15.5 against 5.5), four from 4096 on (500 rows: 12.7 -> 11.2,
+    // radix 8 15.8 -> 10.5), two only where four phases are run (1100 rows, radix 8: 15.9 -> 14.6; radix 16 13.0 -> 13.5)
     int cs = 1;
-    if (n_tiles <= fp->clusters[3] && P.d >= 2048) cs = 8;
+    if (n_tiles <= fp->clusters[4] && P.d >= 4096) cs = 16;
+    else if (n_tiles <= fp->clusters[3] && P.d >= 2048) cs = 8;
     else if (n_tiles <= fp->clusters[2] && P.d >= 4096) cs = 4;
     else if (n_tiles <= fp->clusters[1] && P.d >= 4096 && P.n_phases >= 4) cs = 2;
     if (cs > fp->max_cluster) cs = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(cs > 1 ? (int)n_tiles * cs : grid));
-    cfg.blockDim = dim3(kThreads);
+    const bool reorder = (transpose ? fp->variant_bwd : fp->variant_fwd) == 1;
+    cfg.blockDim = dim3(cs > 1 ? cluster_threads(cs) : kThreads);
     cfg.dynamicSmemBytes = cs > 1 ? fp->cl_smem_bytes : fp->smem_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -1254,11 +1407,10 @@ harp_status_t harp_fast_apply(const harp_plan *plan, void *x, int64_t n_rows, ha
     cfg.attrs = attr;
     cfg.numAttrs = cs > 1 ? 2 : 1;
     cudaError_t err;
-    const bool reorder = (transpose ? fp->variant_bwd : fp->variant_fwd) == 1;
-    if (cs > 1) err = reorder ? cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesReorderOut, true>, xb, n_rows, n_tiles, 0, cs, P)
-                              : cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesInPlace, true>, xb, n_rows, n_tiles, 0, cs, P);
-    else err = reorder ? cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesReorderOut, false>, xb, n_rows, n_tiles, stagger, cs, P)
-                       : cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesGeneral, false>, xb, n_rows, n_tiles, stagger, cs, P);
+    const int lg = cs == 16 ? 4 : cs == 8 ? 3 : cs == 4 ? 2 : cs == 2 ? 1 : 0;
+    if (cs > 1) err = with_cluster_kernel(reorder, cs, [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, xb, n_rows, n_tiles, 0, lg, P); });
+    else err = reorder ? cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesReorderOut, ALONE>, xb, n_rows, n_tiles, stagger, 0, P)
+                       : cudaLaunchKernelEx(&cfg, harp_fast_kernel<kThreads, kModesGeneral, ALONE>, xb, n_rows, n_tiles, stagger, 0, P);
     g_harp_launches.fetch_add(1, std::memory_order_relaxed);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? HARP_OK : HARP_ERR_CUDA;
 }

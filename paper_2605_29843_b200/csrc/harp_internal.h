@@ -79,6 +79,7 @@ harp_status_t harp_generic_apply(const harp_plan *plan, void *x, int64_t n_rows,
 // tensor-core path (harp_fast.cu)
 harp_status_t harp_fast_build(harp_plan *plan);     // HARP_OK or HARP_ERR_UNSUPPORTED (plan->fast stays null)
 void harp_fast_destroy(harp_plan *plan);
+int32_t harp_fast_error_word(const harp_plan *plan);
 bool harp_fast_yields(const harp_plan *plan, int64_t n_rows);   // the two-pass path is faster for this batch
 harp_status_t harp_fast_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype,
                               int transpose, cudaStream_t stream);

@@ -1,4 +1,4 @@
-"""The whole-row kernel with a cluster of two, four or eight CTAs per tile (small batches), against the oracle: every
+"""The whole-row kernel with a cluster of two to sixteen CTAs per tile (small batches), against the oracle: every
 position of the exchange between phases (before the last phase, after the first, both for a digit reversal), phases of width 8
 and 16, ragged tiles, and row counts on both sides of the cluster sizes' limits."""
 import numpy as np
@@ -37,3 +37,21 @@ def test_same_bits_as_one_cta_per_tile():
         harp.apply_(plan, big, transpose=tr, kernel=harp.KERNEL_FAST)
         harp.apply_(plan, small, transpose=tr, kernel=harp.KERNEL_FAST)
         assert torch.equal(big[:200], small)
+
+
+@pytest.mark.parametrize("radices,perm", [((4,) * 6, "digit_reversal"), ((16, 16, 16), "identity"), ((8, 8, 8, 8), "identity"),
+                                          ((2,) * 11, "identity")])
+def test_same_bits_at_every_cluster_size(radices, perm):
+    """One row to a few tiles (sixteen, eight, four CTAs a tile; a last tile of one row, of some, of all sixteen): the bits of one CTA per
+    tile, the row behind the batch untouched, and no wait given up."""
+    spec = wl.make_plan(74, int(np.prod(radices)), radices, "qr", perm=perm)
+    plan = harp.plan_from_spec(spec)
+    x = torch.randn((2400, spec.d), device="cuda").to(torch.bfloat16)
+    for tr in (False, True):
+        big = x.clone()
+        harp.apply_(plan, big, transpose=tr, kernel=harp.KERNEL_FAST)
+        for n in (1, 2, 8, 9, 15, 16, 17, 64, 97, 112, 113, 128, 129, 145, 250, 300):
+            small = x[:n + 1].clone()
+            harp.apply_(plan, small[:n], transpose=tr, kernel=harp.KERNEL_FAST)
+            assert torch.equal(small[:n], big[:n]) and torch.equal(small[n], x[n]), n
+    assert harp.harp_plan_error_word(plan) == 0
