@@ -283,11 +283,6 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
         __syncthreads();
         const uint32_t *src = P.bfrag + (size_t)cg * P.frag_stride;
         for (int i = threadIdx.x * 4; i < P.bfrag_words; i += TEAMS * kTeamThreads * 4) cp_async16(bf_s + 4u * i, src + P.smem_off + i);
-        if (!waited) {                               // the rows only once the kernel before has completed
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            waited = true;
-        }
         [[maybe_unused]] uint32_t fa[8], fb[8], wf[2][2][8];
         if constexpr (K == kUpper8Wide) {
             // the fragments of two neighbouring groups of sixteen positions: item = (block, octet of the 32 positions)
@@ -310,6 +305,11 @@ harp_pipe_kernel(const __grid_constant__ CUtensorMap tmap, int32_t *err, const _
             fb[4] = f1.x; fb[5] = f1.y; fb[6] = f1.z; fb[7] = f1.w;
 #pragma unroll
             for (int e = 0; e < 8; ++e) fa[e] = __ldg(src + P.pair_off[0] + (box * 8 + e) * 32 + lane);
+        }
+        if (!waited) {                               // the rows only once the kernel before has completed
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            waited = true;
         }
         if (tid == 0 && !*(volatile int *)&dead)
             for (int k = 0; k < NB; ++k)

@@ -133,7 +133,7 @@ harp_split_kernel(__nv_bfloat16 *__restrict__ x, int64_t row_begin, int64_t row_
     // whose occupancy is limited by shared memory rather than registers use one buffer instead.
     auto copy_in = [&](int64_t tile, uint32_t sb) {
         const int64_t row0 = row_begin + tile * tile_rows;
-        // rows past the end are computed on a copy of the last row and never stored
+        // (rows past the end: whatever the buffer holds goes through the products, and is never stored)
         if (copier) {
             if (row0 + tile_rows <= row_end && single_chunk) {
                 const __nv_bfloat16 *src = xg + (row0 + cp_r) * rs + goff[0];
@@ -143,17 +143,15 @@ harp_split_kernel(__nv_bfloat16 *__restrict__ x, int64_t row_begin, int64_t row_
 #pragma unroll 4
                 for (int r = cp_r; r < tile_rows; r += cp_rows, src += src_step, dst += dst_step) cp_async16(dst, src);
             } else {
-                const __nv_bfloat16 *last_row = xg + (row_end - 1) * rs;
                 const __nv_bfloat16 *src = xg + (row0 + cp_r) * rs;
                 uint32_t dst = sb + 2u * (uint32_t)(cp_r * pitch);
                 const int64_t src_step = (int64_t)cp_rows * rs;
                 const uint32_t dst_step = 2u * (uint32_t)(cp_rows * pitch);
                 int64_t row = row0 + cp_r;
-                for (int r = cp_r; r < tile_rows; r += cp_rows, src += src_step, dst += dst_step, row += cp_rows) {
-                    const __nv_bfloat16 *s0 = row < row_end ? src : last_row;
+                for (int r = cp_r; r < tile_rows && row < row_end; r += cp_rows, src += src_step, dst += dst_step, row += cp_rows) {
 #pragma unroll
                     for (int mth = 0; mth < 4; ++mth)
-                        if (goff[mth] >= 0) cp_async16(dst + soff[mth], s0 + goff[mth]);
+                        if (goff[mth] >= 0) cp_async16(dst + soff[mth], src + goff[mth]);
                 }
             }
         }
