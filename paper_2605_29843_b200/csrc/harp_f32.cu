@@ -1,4 +1,6 @@
-// fp32 rows of any width: passes over column groups on CUDA cores.
+// fp32 rows of any width: passes over column groups on CUDA cores.  This file chooses the passes and launches them; their kernels are
+// harp_regs.cu's (radices up to 8 and pairs of 16, block kernels in registers), harp_big.cu's (one stage of radix 17 to 48) and, for all
+// other shapes, the one below.
 //
 // A pass runs the consecutive stages [t0, t1) of the plan.  They mix coordinates at strides
 // S, ..., S*E/b (S = stride of stage t0, E = product of the radices), so a column group of E * L
@@ -1012,15 +1014,15 @@ double pass_estimate(const F32Plan *fp, const F32Pass &P, int64_t n) {
 
 }  // namespace
 
-// The passes cost two or three launches, the block kernels of a column group in every CTA, and tiles of 32 rows; the whole-row kernels
-// a wave of CTAs, whatever the batch leaves of it idle.  Radices (16, 16, 4), whole rows against passes: 128 rows 14 us and 25,
-// 256 rows 25 and 25, 512 rows 45 and 28; (16, 16), one pass: 128 rows 6 and 13, 4096 rows 62 and 13; d = 8192 in radix 8 (four rows
-// a CTA, waves of 592): 128 rows 40 and 25, 512 rows 41 and 50, 768 rows 78 and 63; with a random permutation 59 and 39, 61 and 68, 116 and 83.
+// Passes by the kernel above cost two or three launches, the block kernels of a column group in every CTA, and tiles of 32 rows; the
+// whole-row kernels a wave of CTAs, whatever the batch leaves of it idle: radices (16, 16, 4), whole rows against passes: 128 rows 14 us and
+// 25, 256 rows 25 and 25, 512 rows 45 and 28.  The register passes are faster nearly everywhere (d = 8192 in radix 8, whole rows and passes:
+// 1 row 23 and 6.6 us, 256 rows 35 and 12, 4096 rows 294 and 104); the whole-row kernel keeps the batches that fill its one wave of
+// tiles of four rows there (297 to 592 rows, 44 and 18 us: one launch, which callers with a fixed launch budget count on).
 bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows) {
     const F32Plan *fp = plan->f32;
     if (!fp || fp->n_pass[0] == 0) return false;
     if (plan->opt_f32_passes || harp_generic_supported(plan, HARP_F32) != HARP_OK) return true;
-    // (whole-row kernels of four rows a CTA keep a batch that fills one wave to the most part: one launch)
     if (plan->d >= 8192 && plan->d <= 226 * 64 && plan->d_perm == nullptr && harp_generic_max_radix(plan) <= 8 && n_rows > 2 * fp->sms && n_rows <= 4 * fp->sms) return false;
     double us = 0.0;
     // up to d = 4096 the whole-row CUDA-core kernels of radices up to 8 hold enough rows of a tile to beat passes other than those of harp_regs.cu

@@ -70,7 +70,8 @@ harp_status_t harp_generic_build(harp_plan *plan);   // fused stage table for th
 int harp_generic_max_radix(const harp_plan *plan);   // of the stage table its kernels run
 // Estimated microseconds of an fp32 batch on these kernels (harp_f32_preferred: on the passes over column groups), for the choice between
 // them: waves of CTAs times a CTA's time.  The constants are fitted to 1235 batches measured on both (d = 72 .. 32768, radices 2 .. 43,
-// 1 .. 4096 rows, identity and random permutation): standard deviation 12 % for the passes, 4 to 8 % here up to radix 8, 23 % above it.
+// 1 .. 4096 rows, identity and random permutation): standard deviation 12 % for the passes of harp_f32.cu, 4 to 8 % here up to radix 8, 23 % above it.
+// (the passes of harp_regs.cu and harp_big.cu: a launch and a rate, measured at 1 to 4096 rows)
 double harp_generic_estimate(const harp_plan *plan, int64_t n_rows, int sms);
 harp_status_t harp_generic_supported(const harp_plan *plan, harp_dtype_t dtype);
 harp_status_t harp_generic_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype,
