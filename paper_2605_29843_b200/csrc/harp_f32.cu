@@ -24,6 +24,7 @@
 #include <new>
 
 #include "harp_internal.h"
+#include "harp_permute.h"
 #include "harp_regs.h"
 #include "harp_ring.h"
 #include "harp_tm_ptx.cuh"
@@ -635,16 +636,14 @@ harp_f32_pass_kernel(float *__restrict__ x, int64_t n, int64_t ld, const float *
 
 // Fixed permutation and signs of fp32 rows, in place, whole rows through shared memory: out[i] = +-in[table[i]], table: the source of every
 // coordinate (the permutation forward, its inverse for the transpose) with the sign in the top bit.  Groups of R rows come by asynchronous 16-byte
-// copies, the next one (n_buf = 2) while this one is gathered; an entry of the table is read once for the rows of a group.  The
-// pieces of a row are exchanged within 128 bytes by higher bits of the index: under a digit reversal the coordinates that a warp gathers are
-// powers of two apart (4-way conflicts instead of 16-way; finer exchanges would split the pieces).
-__device__ __forceinline__ int permute_piece(int c) { return c ^ ((c >> 4) & 7); }
+// copies, the next one (n_buf = 2) while this one is gathered; an entry of the table is read once for the rows of a group.  harp_permute.h
+// says where the pieces of a row lie.
 constexpr int kPermuteThreads = 512;
 __global__ void __launch_bounds__(kPermuteThreads, 2)
 harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, int n_buf, const int32_t *__restrict__ table) {
     extern __shared__ __align__(16) float smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");        // (whoever comes next waits for this grid's end before it touches a row)
-    const int pieces = d / 4;
+    const int pieces = d / 4, pitch = permute_pitch<4>(d);
     const int64_t groups = (n + R - 1) / R;
     auto copy_in = [&](int64_t g, float *buf) {
         if (g < groups) {
@@ -652,7 +651,7 @@ harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, int n_bu
             const float *src = x + g * R * d;
             for (int r = 0; r < rows; ++r)
 #pragma unroll 4
-                for (int c = threadIdx.x; c < pieces; c += kPermuteThreads) cp_async16(buf + r * d + 4 * permute_piece(c), src + (int64_t)r * d + 4 * c);
+                for (int c = threadIdx.x; c < pieces; c += kPermuteThreads) cp_async16(buf + r * pitch + 4 * permute_piece<4>(c), src + (int64_t)r * d + 4 * c);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -661,28 +660,25 @@ harp_f32_permute_kernel(float *__restrict__ x, int64_t n, int d, int R, int n_bu
     int buf = 0;
     for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
         if (n_buf == 2) {
-            copy_in(g + gridDim.x, smem + (buf ^ 1) * R * d);
+            copy_in(g + gridDim.x, smem + (buf ^ 1) * R * pitch);
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
         const int rows = (int)min((int64_t)R, n - g * R);
-        const float *tile = smem + buf * R * d;
+        const float *tile = smem + buf * R * pitch;
         float *dst = x + g * R * d;
         for (int c = threadIdx.x; c < pieces; c += kPermuteThreads) {
             const int4 t = __ldg(reinterpret_cast<const int4 *>(table) + c);
             const int src[4] = {t.x, t.y, t.z, t.w};
             int at[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = src[k] & 0x7fffffff;
-                at[k] = 4 * permute_piece(i >> 2) + (i & 3);
-            }
+            for (int k = 0; k < 4; ++k) at[k] = permute_place<4>(src[k] & 0x7fffffff);
             for (int r = 0; r < rows; ++r) {
                 float o[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) o[k] = __uint_as_float(__float_as_uint(tile[r * d + at[k]]) ^ ((uint32_t)src[k] & 0x80000000u));
+                for (int k = 0; k < 4; ++k) o[k] = __uint_as_float(__float_as_uint(tile[r * pitch + at[k]]) ^ ((uint32_t)src[k] & 0x80000000u));
                 *reinterpret_cast<float4 *>(dst + (int64_t)r * d + 4 * c) = make_float4(o[0], o[1], o[2], o[3]);
             }
         }
@@ -919,7 +915,7 @@ harp_status_t permute_rows(const harp_plan *plan, float *x, int64_t n, int trans
     // two CTAs an SM where two groups' buffers leave room; a small batch is spread over the SMs row by row
     int R = fp->permute_rows;
     while (R > 1 && n < (int64_t)R * 2 * fp->sms) --R;
-    const size_t smem = (size_t)fp->permute_bufs * R * plan->d * sizeof(float);
+    const size_t smem = (size_t)fp->permute_bufs * R * permute_pitch<4>(plan->d) * sizeof(float);
     const int per_sm = smem <= 113 * 1024 ? 2 : 1;
     if (cudaFuncSetAttribute(harp_f32_permute_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess)
         return HARP_ERR_CUDA;
@@ -960,8 +956,9 @@ harp_status_t harp_f32_build(harp_plan *plan) {
     if (d % 4 == 0) fp->n_pass[0] = plan_passes(st, plan->st, d, false, fp->pass[0]);
     if (plan->h_perm.empty()) fp->n_pass[1] = plan_passes(st, plan->st, d, true, fp->pass[1]);
     else if (d % 4 == 0) {
-        fp->permute_bufs = 2 * d * 4 <= kSmemMax ? 2 : 1;
-        fp->permute_rows = (int)std::max<int64_t>(1, std::min<int64_t>(4, (112 * 1024) / (fp->permute_bufs * d * 4)));
+        const int64_t row_bytes = permute_pitch<4>(d) * 4;
+        fp->permute_bufs = 2 * row_bytes <= kSmemMax ? 2 : 1;
+        fp->permute_rows = (int)std::max<int64_t>(1, std::min<int64_t>(4, (112 * 1024) / (fp->permute_bufs * row_bytes)));
         std::vector<int32_t> table[2];
         try {
             for (auto &t : table) t.resize((size_t)d);

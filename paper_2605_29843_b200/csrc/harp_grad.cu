@@ -25,6 +25,7 @@
 #include <mutex>
 
 #include "harp_internal.h"
+#include "harp_permute.h"
 
 namespace {
 
@@ -1262,16 +1263,14 @@ permute_kernel(const T *__restrict__ x, int vec, T *__restrict__ out, int64_t ro
 }
 
 // The same for aligned rows: groups of R rows by asynchronous 16-byte copies, the next group on its way while this one is gathered, and one table
-// with the sign in its top bit in place of an index and the sign behind it.  Pieces are exchanged within 128 bytes by higher bits of the
-// index (a digit reversal: 4-way conflicts).
+// with the sign in its top bit in place of an index and the sign behind it.  harp_permute.h says where the pieces lie.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 3)
 permute_ring_kernel(const T *__restrict__ x, T *__restrict__ out, int64_t rows, int d, const int32_t *__restrict__ table, int R) {
-    constexpr int V = 16 / (int)sizeof(T), kLog = sizeof(T) == 2 ? 3 : 2;
+    constexpr int V = 16 / (int)sizeof(T);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *smem = reinterpret_cast<T *>(smem_raw);
-    auto piece = [](int c) { return c ^ ((c >> (sizeof(T) == 2 ? 3 : 4)) & 7); };
-    const int pieces = d / V;
+    const int pieces = d / V, pitch = permute_pitch<V>(d);
     const int64_t groups = (rows + R - 1) / R;
     auto copy_in = [&](int64_t g, T *buf) {
         if (g < groups) {
@@ -1280,7 +1279,7 @@ permute_ring_kernel(const T *__restrict__ x, T *__restrict__ out, int64_t rows, 
             for (int r = 0; r < nr; ++r)
 #pragma unroll 2
                 for (int c = threadIdx.x; c < pieces; c += kThreads)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(buf + r * d + V * piece(c))), "l"(src + (int64_t)r * d + V * c) : "memory");
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(buf + r * pitch + V * permute_piece<V>(c))), "l"(src + (int64_t)r * d + V * c) : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -1288,11 +1287,11 @@ permute_ring_kernel(const T *__restrict__ x, T *__restrict__ out, int64_t rows, 
     copy_in(blockIdx.x, smem);
     int buf = 0;
     for (int64_t g = blockIdx.x; g < groups; g += gridDim.x, buf ^= 1) {
-        copy_in(g + gridDim.x, smem + (buf ^ 1) * R * d);
+        copy_in(g + gridDim.x, smem + (buf ^ 1) * R * pitch);
         asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncthreads();
         const int nr = (int)min((int64_t)R, rows - g * R);
-        const T *tile = smem + buf * R * d;
+        const T *tile = smem + buf * R * pitch;
         for (int i = (int)threadIdx.x * 4; i < d; i += kThreads * 4) {
             const int4 t = __ldg(reinterpret_cast<const int4 *>(table + i));
             const int src[4] = {t.x, t.y, t.z, t.w};
@@ -1300,15 +1299,14 @@ permute_ring_kernel(const T *__restrict__ x, T *__restrict__ out, int64_t rows, 
             T flip[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int e = src[k] & 0x7fffffff;
-                at[k] = V * piece(e >> kLog) + (e & (V - 1));
+                at[k] = permute_place<V>(src[k] & 0x7fffffff);
                 flip[k] = src[k] < 0 ? (T)((T)1 << (8 * sizeof(T) - 1)) : (T)0;
             }
             T *to = out + g * R * d + i;
             for (int r = 0; r < nr; ++r, to += d) {
                 T o[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) o[k] = tile[r * d + at[k]] ^ flip[k];
+                for (int k = 0; k < 4; ++k) o[k] = tile[r * pitch + at[k]] ^ flip[k];
                 if constexpr (sizeof(T) == 2) *reinterpret_cast<uint2 *>(to) = make_uint2(o[0] | (uint32_t)o[1] << 16, o[2] | (uint32_t)o[3] << 16);
                 else *reinterpret_cast<uint4 *>(to) = make_uint4(o[0], o[1], o[2], o[3]);
             }
@@ -1697,10 +1695,11 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
             const int staged = smem <= 48 * 1024 || (smem <= 200 * 1024 && cudaFuncSetAttribute(permute_kernel<Bits>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess);
             if (!staged) smem = 0;
             const int32_t *table = harp_f32_source_table(plan);
-            const int64_t ring_rows = std::min<int64_t>(4, 36 * 1024 / (d * (int64_t)sizeof(T)));
-            if (table && red.m == tab.m && ring_rows > 0 && aligned16(xc) && d % (16 / (int64_t)sizeof(T)) == 0) {
+            constexpr int V = 16 / (int)sizeof(T);
+            const int64_t pitch_bytes = d % V == 0 ? permute_pitch<V>(d) * (int64_t)sizeof(T) : 0, ring_rows = pitch_bytes > 0 ? std::min<int64_t>(4, 36 * 1024 / pitch_bytes) : 0;
+            if (table && red.m == tab.m && ring_rows > 0 && aligned16(xc)) {
                 const int r = (int)std::max<int64_t>(1, std::min<int64_t>(ring_rows, rows / (3 * sms)));
-                const size_t bytes = (size_t)(2 * r * d) * sizeof(T);
+                const size_t bytes = (size_t)(2 * r * pitch_bytes);
                 if (bytes > 48 * 1024) cudaFuncSetAttribute(permute_ring_kernel<Bits>, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
                 launch_dep(permute_ring_kernel<Bits>, dim3((unsigned)std::min<int64_t>((rows + r - 1) / r, 3 * sms)), dim3(kThreads), bytes, st, reinterpret_cast<const Bits *>(xc),
                            reinterpret_cast<Bits *>(xp), rows, (int)d, table, r);

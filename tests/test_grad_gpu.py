@@ -255,3 +255,16 @@ def test_rows_off_sixteen_byte_boundaries(dtype, radices):
         torch.cuda.synchronize()
         # the same fp32 states and fp64 sums in another order: a rounding of the result
         assert np.max(np.abs(out.cpu().numpy() - got)) <= 1e-6 * np.max(np.abs(got))
+
+
+@pytest.mark.parametrize("n_rows", [445, 900, 2000])
+@pytest.mark.parametrize("radices,dtype", [((8, 5, 3), "bf16"), ((8, 5, 3), "f32"), ((3, 3, 8), "bf16"), ((5, 5, 4), "f32"), ((7, 7, 8), "bf16"), ((7, 7, 8), "f32"),
+                                           ((8, 5, 5, 5), "bf16"), ((8, 5, 5, 5), "f32"), ((4, 4, 5, 5, 5), "f32"), ((2,), "f32"), ((2, 2), "bf16"), ((2, 3), "bf16")])
+def test_permuted_rows_that_are_no_whole_groups_of_pieces(radices, dtype, n_rows):
+    """Widths of no multiple of 128 bytes behind a permutation, down to less than a piece of 16; more rows than one group of them a CTA."""
+    spec = wl.tiny_plan(43, radices, kind="qr", perm="random", signs=True)
+    plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
+    xh, gh = _rows(44, n_rows, spec.d, dtype)
+    got, _, _ = _gpu_grad(plan, xh, gh, dtype)
+    want = _flat(orc.grad_blocks(oplan, promote(xh, dtype), promote(gh, dtype)))
+    assert np.max(np.abs(got - want)) <= 2e-5 * np.max(np.abs(want))
