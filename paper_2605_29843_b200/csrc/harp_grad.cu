@@ -1490,6 +1490,12 @@ int slice_rows(const harp_plan *plan, const Step &sp, int64_t rows, int sms) {
 }
 dim3 grid2(int64_t x, int per_x, int64_t rows, int per_y) { return dim3((unsigned)((x + per_x - 1) / per_x), (unsigned)((rows + per_y - 1) / per_y)); }
 
+// The one-thread-per-element kernels read every state as often as a block has rows or columns, from L1 and L2.  An SM keeps the split of L1 and
+// shared memory that the kernel before asked for, and behind the wide stages' 113 to 190 KB that is the smallest L1 (1024 rows of radices 7, 39, 2, 8:
+// 1407 us, 720 this way); 32 KB hold eight CTAs of 2 KB.  Per call: the attribute belongs to the current device's copy of the kernel.
+template <typename Kernel>
+void prefer_l1(Kernel kernel) { cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 14); }
+
 // one step forward: out = in through the step's stages
 template <typename TI>
 void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int8_t *signs, float *out, int64_t rows, int sms, cudaStream_t st) {
@@ -1549,6 +1555,7 @@ void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int
     }
 #undef HARP_FWD
     const bool by_em = s >= 8;                     // see stage_kernel
+    prefer_l1(stage_kernel<TI>);
     launch_dep(stage_kernel<TI>, column_grid(d, rows), dim3(kThreads), 0, st, in, signs, out, rows, d, b, s, by_em ? em : plan->d_blocks + plan->st.off[sp.t],
                by_em ? 1 : (int64_t)b * b, by_em ? d / b : 1, 0);
 }
@@ -1622,9 +1629,11 @@ int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8
     }
 #undef HARP_BWD
     const bool by_em = s >= 8;
+    prefer_l1(outer_kernel<TV, TG>);
     launch_dep(outer_kernel<TV, TG>, dim3((unsigned)std::min<int64_t>((d * b + 31) / 32, 148 * 64)), dim3(kThreads), 0, st, v, signs, g, rows, d, b, s,
                grad + plan->st.off[sp.t], acc, by_em ? 0 : 1);
     if (!g_out) return 1;
+    prefer_l1(stage_kernel<TG>);
     launch_dep(stage_kernel<TG>, column_grid(d, rows), dim3(kThreads), 0, st, g, (const int8_t *)nullptr, g_out, rows, d, b, s,
                by_em ? em : plan->d_blocks + plan->st.off[sp.t], by_em ? 1 : (int64_t)b * b, by_em ? d / b : 1, 1);
     return 2;

@@ -268,3 +268,29 @@ def test_permuted_rows_that_are_no_whole_groups_of_pieces(radices, dtype, n_rows
     got, _, _ = _gpu_grad(plan, xh, gh, dtype)
     want = _flat(orc.grad_blocks(oplan, promote(xh, dtype), promote(gh, dtype)))
     assert np.max(np.abs(got - want)) <= 2e-5 * np.max(np.abs(want))
+
+
+def _back_to_back(radices, n_rows, dtype="f32"):
+    """Microseconds of a call among others, best of five."""
+    spec = wl.tiny_plan(45, radices, kind="qr", perm="identity", signs=True)
+    plan = harp.plan_from_spec(spec)
+    x = torch.randn((n_rows, spec.d), device="cuda")
+    g, out = torch.randn_like(x), torch.zeros(harp.harp_plan_n_params(plan), device="cuda")
+    best = float("inf")
+    for _ in range(6):
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ev[0].record()
+        for _ in range(10):
+            harp.harp_grad_blocks(plan, x.data_ptr(), g.data_ptr(), n_rows, DT[dtype], out.data_ptr(), False, torch.cuda.current_stream().cuda_stream)
+        ev[1].record()
+        torch.cuda.synchronize()
+        best = min(best, ev[0].elapsed_time(ev[1]) * 100)
+    return best
+
+
+def test_stages_on_tiles_leave_the_others_their_l1():
+    """A stage of radix 39, one thread an element, takes as long behind stages on tiles in shared memory as among its like, but for their
+    own time: 1.5 times as long a product (3.0 behind stages that leave it the smallest L1)."""
+    mixed, alike = (7, 39, 2, 8), (39, 11, 10)
+    per_product = [_back_to_back(r, 1024) / (np.prod(r) * sum(b for b in r if b > 8)) for r in (mixed, alike)]
+    assert per_product[0] <= 2.2 * per_product[1], per_product
