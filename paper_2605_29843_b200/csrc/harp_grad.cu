@@ -1385,6 +1385,9 @@ outer_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const T
 }
 
 constexpr int64_t kMostScratch = 1280ll << 20, kLeastScratch = 160ll << 20;     // bytes of states of a chunk
+// ... of a plan with one-thread-per-element kernels, which read a state once per row or column of a block: from L2, while two states fit it
+// (10000 rows of radices 7, 57, 4: chunks of 200 MB 3575 us, one of 1280 MB 6514; 2400 rows of 2^6, 45, 2 in bf16 1875 and 2407)
+constexpr int64_t kPlainScratch = 200ll << 20;
 
 // Scratch comes from a memory pool of the library's own (one per device, created on first use)
 // that keeps one call's worth: the default pool hands its memory back at every
@@ -1656,7 +1659,8 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
     ReduceTable red{};
     double *part = nullptr;
     cudaMemPool_t pool = scratch_pool(plan->device);
-    for (int64_t budget = kMostScratch; !part; budget /= 2) {
+    const bool plain = std::any_of(steps.begin(), steps.end(), [&](const Step &sp) { return !owner_radix(tab.b[sp.t]); });
+    for (int64_t budget = plain ? kPlainScratch : kMostScratch; !part; budget /= 2) {
         if (budget < kLeastScratch) return HARP_ERR_ALLOC;
         const int64_t fit = std::max<int64_t>(16, budget / per_row), most = n > 1 ? std::min<int64_t>(fit, 65535ll * kFwdRows) : fit;
         const int64_t n_chunks = (n_rows + most - 1) / most;

@@ -294,3 +294,24 @@ def test_stages_on_tiles_leave_the_others_their_l1():
     mixed, alike = (7, 39, 2, 8), (39, 11, 10)
     per_product = [_back_to_back(r, 1024) / (np.prod(r) * sum(b for b in r if b > 8)) for r in (mixed, alike)]
     assert per_product[0] <= 2.2 * per_product[1], per_product
+
+
+def _grad_launches(plan, x, g, out):
+    before = harp.harp_launch_count()
+    harp.harp_grad_blocks(plan, x.data_ptr(), g.data_ptr(), x.shape[0], harp.HARP_F32, out.data_ptr(), False, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    return harp.harp_launch_count() - before
+
+
+def test_states_of_one_thread_per_element_stages_stay_near_l2():
+    """200 MB of states a chunk where a radix has no owner kernel: 10000 rows of d = 1596 in two chunks (three stages, five planes less one)."""
+    spec = wl.tiny_plan(46, (7, 57, 4), kind="qr", perm="identity", signs=True)
+    plan = harp.plan_from_spec(spec)
+    x = torch.randn((10000, spec.d), device="cuda")
+    g = torch.randn_like(x)
+    outs = [torch.zeros(harp.harp_plan_n_params(plan), device="cuda") for _ in range(3)]
+    one = _grad_launches(plan, x[:5000], g[:5000], outs[0])
+    _grad_launches(plan, x[5000:], g[5000:], outs[1])
+    assert _grad_launches(plan, x, g, outs[2]) == 2 * one - 1         # the reduction once
+    # sums in fp64, rounded to fp32 once in the whole and once in either half
+    assert float((outs[0] + outs[1] - outs[2]).abs().max()) <= 1e-6 * float(outs[2].abs().max())
