@@ -770,12 +770,15 @@ bool make_pass(const StageTable &st, int64_t d, int t0, int t1, int L, int H, in
     return true;
 }
 
-constexpr double kPassCost = 1.6;      // against a pass of harp_regs.cu
+// A pass of harp_regs.cu or harp_big.cu against one of the kernel above, in trips.  Covers of 5528 batches of rows and 1627 matrices, d = 256 .. 32768,
+// against covers without those passes: with 0.75 0.3 % of them more than 4 or 5 % slower, rows on average 0.729 of the time and columns 0.939; with
+// 0.5 0.6 %, 0.731 and 0.939, with 0.9 0.3 %, 0.730 and 0.956.
+constexpr double kRegCost = 0.75;
 
 // Cost of a pass relative to one trip of the rows through HBM.  What moves it: 16- and 32-byte runs of the row-mode
 // copies, one row per lane (every kernel load serves half as much arithmetic), phases with fewer blocks than warps.
 double pass_cost(const F32Pass &P, bool col) {
-    double c = kPassCost, mac = 0.0;
+    double c = 1.0, mac = 0.0;
     for (int p = 0; p < P.n_ph; ++p) mac += P.ph[p].b;
     if (!col && P.S > 1) c += P.L == 4 ? 1.0 : P.L == 8 ? 0.1 : 0.0;
     if (P.RT == 1) c += 0.02 * mac;
@@ -805,7 +808,7 @@ int plan_passes(const StageTable &st, const StageTable &orig, int64_t d, bool co
             F32Pass P{};
             if (o0 < 0 || o1 < 0 || o1 - o0 > 11) continue;
             if (!harp_regs_pass(orig, d, o0, o1, col, P.reg) && (col || o1 != o0 + 1 || !harp_big_pass(orig, d, o0, P.reg))) continue;
-            const double c = best[(size_t)t0].cost + 1.0;
+            const double c = best[(size_t)t0].cost + kRegCost;
             if (c < best[(size_t)t1].cost) best[(size_t)t1] = Best{c, t0, P, best[(size_t)t0].n + 1};
         }
         for (int t1 = t0 + 1; t1 <= st.m; ++t1)

@@ -101,3 +101,22 @@ def test_a_driver_without_tensor_maps(monkeypatch, dtype):
     want = orc.two_sided(orc.OraclePlan.from_spec(p_out), orc.OraclePlan.from_spec(p_in), promote(wh, dtype))
     scale = np.minimum(np.linalg.norm(want, axis=1, keepdims=True), np.linalg.norm(want, axis=0, keepdims=True))
     assert np.max(np.abs(to_host_f64(wd) - want) / scale) <= 2 * TOL[dtype]
+
+
+def _launches(call):
+    before = harp.harp_launch_count()
+    call()
+    torch.cuda.synchronize()
+    return harp.harp_launch_count() - before
+
+
+def test_covers_with_and_without_register_passes():
+    """A third pass in place of a wide tile of one row a lane, where no pass with its block kernels in registers takes part: rows of
+    radices (8, 8, 15, 10) 31 and 38 us, columns of (2, 2, 2, 2, 48, 2, 2, 2)."""
+    plan = harp.plan_from_spec(wl.tiny_plan(72, (8, 8, 15, 10), kind="qr", perm="identity", signs=True))
+    x = torch.zeros((48, plan.d), device="cuda")
+    assert _launches(lambda: harp.apply_(plan, x)) == 3
+    p_out = harp.plan_from_spec(wl.tiny_plan(73, (2, 2, 2, 2, 48, 2, 2, 2), kind="qr", perm="identity", signs=True))
+    p_in = harp.plan_from_spec(wl.tiny_plan(74, (12, 11, 14, 2), kind="qr", perm="identity", signs=True))
+    w, rows = torch.zeros((p_out.d, p_in.d), device="cuda"), torch.zeros((p_out.d, p_in.d), device="cuda")
+    assert _launches(lambda: harp.two_sided_(w, p_out, p_in)) - _launches(lambda: harp.apply_(p_in, rows)) == 3
