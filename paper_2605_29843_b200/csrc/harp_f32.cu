@@ -1034,8 +1034,10 @@ bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows) {
     if (fp->permute_rows) {
         us += 3.5 + 1.3e-6 * (double)n_rows * (double)plan->d;
     }
-    // (under a digit reversal the whole-row kernels take 1.4 times their estimate: 512 rows of d = 4096 27 us)
-    return us < (fp->permute_rows ? 1.3 : 1.0) * harp_generic_estimate(plan, n_rows, fp->sms);
+    // A permutation: where register passes are all there is to choose, the whole-row kernels take more than their estimate (512 rows of d = 4096
+    // under a digit reversal 27 us, 1.4 times; 180 batches 0.534 of their time with 1.3, 0.548 with 1); for other plans it holds (256 rows
+    // of radices (4, 4, 15, 4) behind a random one 20.7 us, three passes 27.8)
+    return us < (fp->permute_rows && whole ? 1.3 : 1.0) * harp_generic_estimate(plan, n_rows, fp->sms);
 }
 
 harp_status_t harp_f32_apply(const harp_plan *plan, void *x, int64_t n_rows, harp_dtype_t dtype, int transpose, cudaStream_t stream) {

@@ -120,3 +120,10 @@ def test_covers_with_and_without_register_passes():
     p_in = harp.plan_from_spec(wl.tiny_plan(74, (12, 11, 14, 2), kind="qr", perm="identity", signs=True))
     w, rows = torch.zeros((p_out.d, p_in.d), device="cuda"), torch.zeros((p_out.d, p_in.d), device="cuda")
     assert _launches(lambda: harp.two_sided_(w, p_out, p_in)) - _launches(lambda: harp.apply_(p_in, rows)) == 3
+
+
+def test_permuted_rows_of_a_large_radix_take_the_faster_route():
+    """256 rows of radices (4, 4, 15, 4) behind a random permutation: the whole-row kernel (20.7 us) and not a permutation and two passes (27.8)."""
+    plan = harp.plan_from_spec(wl.tiny_plan(75, (4, 4, 15, 4), kind="qr", perm="random", signs=True))
+    x = torch.zeros((256, plan.d), device="cuda")
+    assert _launches(lambda: harp.apply_(plan, x)) == 1
