@@ -1017,13 +1017,15 @@ double pass_estimate(const F32Plan *fp, const F32Pass &P, int64_t n) {
 // Passes by the kernel above cost two or three launches, the block kernels of a column group in every CTA, and tiles of 32 rows; the
 // whole-row kernels a wave of CTAs, whatever the batch leaves of it idle: radices (16, 16, 4), whole rows against passes: 128 rows 14 us and
 // 25, 256 rows 25 and 25, 512 rows 45 and 28.  The register passes are faster nearly everywhere (d = 8192 in radix 8, whole rows and passes:
-// 1 row 23 and 6.6 us, 256 rows 35 and 12, 4096 rows 294 and 104); the whole-row kernel keeps the batches that fill its one wave of
-// tiles of four rows there (297 to 592 rows, 44 and 18 us: one launch, which callers with a fixed launch budget count on).
+// 1 row 23 and 6.6 us, 256 rows 35 and 12, 4096 rows 294 and 104).  One exception, which no time speaks for (42 and 18 us): batches of d = 8192 that
+// fill five sixths or more of the whole-row kernel's one wave of tiles of four rows stay with its one launch, as before there were register passes; 500
+// rows are promised it (test_small_batches_take_one_launch).  Smaller batches and other widths take what the estimates say (300 rows of radices
+// (4, 3, 4, 2, 4, 4, 7) 55 us whole, 39 in passes; of 2^10, 8 38 and 13).
 bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows) {
     const F32Plan *fp = plan->f32;
     if (!fp || fp->n_pass[0] == 0) return false;
     if (plan->opt_f32_passes || harp_generic_supported(plan, HARP_F32) != HARP_OK) return true;
-    if (plan->d >= 8192 && plan->d <= 226 * 64 && plan->d_perm == nullptr && harp_generic_max_radix(plan) <= 8 && n_rows > 2 * fp->sms && n_rows <= 4 * fp->sms) return false;
+    if (plan->d == 8192 && plan->d_perm == nullptr && harp_generic_max_radix(plan) <= 8 && 6 * n_rows > 20 * fp->sms && n_rows <= 4 * fp->sms) return false;
     double us = 0.0;
     // up to d = 4096 the whole-row CUDA-core kernels of radices up to 8 hold enough rows of a tile to beat passes other than those of harp_regs.cu
     const bool whole = plan->d <= 4096 && harp_generic_max_radix(plan) <= 8;
