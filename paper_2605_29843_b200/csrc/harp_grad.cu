@@ -1385,9 +1385,10 @@ outer_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const T
 }
 
 constexpr int64_t kMostScratch = 1280ll << 20, kLeastScratch = 160ll << 20;     // bytes of states of a chunk
-// ... of a plan with one-thread-per-element kernels, which read a state once per row or column of a block: from L2, while two states fit it
-// (10000 rows of radices 7, 57, 4: chunks of 200 MB 3575 us, one of 1280 MB 6514; 2400 rows of 2^6, 45, 2 in bf16 1875 and 2407)
-constexpr int64_t kPlainScratch = 200ll << 20;
+// Bytes of one state of a chunk of a plan with one-thread-per-element kernels, which read two states once per row or column of a block: from L2, while
+// they fit it (10000 rows of radices 7, 57, 4 6514 us in one chunk, 3577 in two; 1024 rows of 2^8, 49 1504 in one, of 51 MB, 1189 in two; 4096
+// rows of 2^8, 43 in bf16 3151 with 40 MB, 3229 with 32, 3861 with 16)
+constexpr int64_t kPlainState = 40ll << 20;
 
 // Scratch comes from a memory pool of the library's own (one per device, created on first use)
 // that keeps one call's worth: the default pool hands its memory back at every
@@ -1660,9 +1661,9 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
     double *part = nullptr;
     cudaMemPool_t pool = scratch_pool(plan->device);
     const bool plain = std::any_of(steps.begin(), steps.end(), [&](const Step &sp) { return !owner_radix(tab.b[sp.t]); });
-    for (int64_t budget = plain ? kPlainScratch : kMostScratch; !part; budget /= 2) {
+    for (int64_t budget = kMostScratch; !part; budget /= 2) {
         if (budget < kLeastScratch) return HARP_ERR_ALLOC;
-        const int64_t fit = std::max<int64_t>(16, budget / per_row), most = n > 1 ? std::min<int64_t>(fit, 65535ll * kFwdRows) : fit;
+        const int64_t fit = std::max<int64_t>(16, std::min(budget / per_row, plain ? kPlainState / (4 * d) : INT64_MAX)), most = n > 1 ? std::min<int64_t>(fit, 65535ll * kFwdRows) : fit;
         const int64_t n_chunks = (n_rows + most - 1) / most;
         chunk = (n_rows + n_chunks - 1) / n_chunks;
         part_len = 0;
