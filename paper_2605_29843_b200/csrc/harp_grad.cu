@@ -42,18 +42,24 @@ __device__ __forceinline__ void prior_kernel_done() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// An SM that has to change the split of L1 and shared memory is emptied first, which undoes that overlap and costs a small call more than its
+// kernels take.  split: percent of shared memory that every launch asks for, -1: what each kernel needs.
+struct Chain { cudaStream_t stream; int split; };
+
 template <typename... KArgs, typename... Args>
-void launch_dep(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
+void launch_dep(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, const Chain &chain, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cfg.stream = chain.stream;
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = (unsigned)std::max(0, chain.split);
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chain.split >= 0 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);     // errors are read with cudaGetLastError by the caller
 }
 
@@ -1496,13 +1502,13 @@ dim3 grid2(int64_t x, int per_x, int64_t rows, int per_y) { return dim3((unsigne
 
 // The one-thread-per-element kernels read every state as often as a block has rows or columns, from L1 and L2.  An SM keeps the split of L1 and
 // shared memory that the kernel before asked for, and behind the wide stages' 113 to 190 KB that is the smallest L1 (1024 rows of radices 7, 39, 2, 8:
-// 1407 us, 720 this way); 32 KB hold eight CTAs of 2 KB.  Per call: the attribute belongs to the current device's copy of the kernel.
-template <typename Kernel>
-void prefer_l1(Kernel kernel) { cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 14); }
+// 1447 us, 718 this way; 128 rows 145 and 124); 14 percent, 32 KB, hold eight CTAs of 2 KB.  A small launch leaves the split alone (two rows of 4, 32, 4, 7:
+// 53 us this way, 37).
+Chain plain_chain(const Chain &chain, int64_t rows, int64_t d) { return {chain.stream, rows * d >= 1 << 17 ? 14 : -1}; }
 
 // one step forward: out = in through the step's stages
 template <typename TI>
-void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int8_t *signs, float *out, int64_t rows, int sms, cudaStream_t st) {
+void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int8_t *signs, float *out, int64_t rows, int sms, const Chain &st) {
     const int64_t d = plan->d, s = plan->st.s[sp.t];
     const int b = plan->st.b[sp.t];
     const float *em = plan->d_blocks_em + plan->st.off[sp.t];
@@ -1559,8 +1565,7 @@ void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int
     }
 #undef HARP_FWD
     const bool by_em = s >= 8;                     // see stage_kernel
-    prefer_l1(stage_kernel<TI>);
-    launch_dep(stage_kernel<TI>, column_grid(d, rows), dim3(kThreads), 0, st, in, signs, out, rows, d, b, s, by_em ? em : plan->d_blocks + plan->st.off[sp.t],
+    launch_dep(stage_kernel<TI>, column_grid(d, rows), dim3(kThreads), 0, plain_chain(st, rows, d), in, signs, out, rows, d, b, s, by_em ? em : plan->d_blocks + plan->st.off[sp.t],
                by_em ? 1 : (int64_t)b * b, by_em ? d / b : 1, 0);
 }
 
@@ -1568,7 +1573,7 @@ void step_forward(const harp_plan *plan, const Step &sp, const TI *in, const int
 // kernels, into grad)
 template <typename TV, typename TG>
 int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8_t *signs, const TG *g, float *g_out, int64_t rows, double *all_parts, const int64_t *part_off,
-                  int slice, int add, float *grad, int acc, cudaStream_t st) {
+                  int slice, int add, float *grad, int acc, const Chain &st) {
     const int64_t d = plan->d, s = plan->st.s[sp.t];
     const int b = plan->st.b[sp.t];
     const float *em = plan->d_blocks_em + plan->st.off[sp.t];
@@ -1633,18 +1638,16 @@ int step_backward(const harp_plan *plan, const Step &sp, const TV *v, const int8
     }
 #undef HARP_BWD
     const bool by_em = s >= 8;
-    prefer_l1(outer_kernel<TV, TG>);
-    launch_dep(outer_kernel<TV, TG>, dim3((unsigned)std::min<int64_t>((d * b + 31) / 32, 148 * 64)), dim3(kThreads), 0, st, v, signs, g, rows, d, b, s,
+    launch_dep(outer_kernel<TV, TG>, dim3((unsigned)std::min<int64_t>((d * b + 31) / 32, 148 * 64)), dim3(kThreads), 0, plain_chain(st, rows, d), v, signs, g, rows, d, b, s,
                grad + plan->st.off[sp.t], acc, by_em ? 0 : 1);
     if (!g_out) return 1;
-    prefer_l1(stage_kernel<TG>);
-    launch_dep(stage_kernel<TG>, column_grid(d, rows), dim3(kThreads), 0, st, g, (const int8_t *)nullptr, g_out, rows, d, b, s,
+    launch_dep(stage_kernel<TG>, column_grid(d, rows), dim3(kThreads), 0, plain_chain(st, rows, d), g, (const int8_t *)nullptr, g_out, rows, d, b, s,
                by_em ? em : plan->d_blocks + plan->st.off[sp.t], by_em ? 1 : (int64_t)b * b, by_em ? d / b : 1, 1);
     return 2;
 }
 
 template <typename T>
-harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_t n_rows, float *grad, int accumulate, cudaStream_t st) {
+harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_t n_rows, float *grad, int accumulate, cudaStream_t stream) {
     const int64_t d = plan->d;
     const StageTable &tab = plan->st;
     const std::vector<Step> steps = make_steps(tab, d, sizeof(T), plan->d_perm ? nullptr : x, gy);
@@ -1681,7 +1684,7 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
         }
         plane = (chunk * d + 3) / 4 * 4;
         const size_t bytes = (size_t)(part_len * 8 + 16 + plane * 4 * (n - 1 + n_g) + (permuted ? plane * (int64_t)sizeof(T) : 0));
-        if ((pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&part), bytes, pool, st) : cudaMallocAsync(reinterpret_cast<void **>(&part), bytes, st)) != cudaSuccess) {
+        if ((pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&part), bytes, pool, stream) : cudaMallocAsync(reinterpret_cast<void **>(&part), bytes, stream)) != cudaSuccess) {
             cudaGetLastError();
             part = nullptr;
         }
@@ -1689,6 +1692,9 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
     float *vp = reinterpret_cast<float *>(part + (part_len + 1) / 2 * 2), *gp = vp + (n - 1) * plane;      // state planes on 16-byte boundaries
     T *xp = reinterpret_cast<T *>(gp + n_g * plane);
     const int8_t *signs = permuted ? nullptr : plan->d_signs;       // the permutation kernel carries the signs
+    // a small call's kernels share one split (2400 rows of radices 4, 4, 4 behind a permutation 31.6 us each with its own, 22.3 this way; 256 rows of 2^11
+    // 36.7 and 30.7); from some 2^22 values on it makes no difference or the larger L1 gains (16384 rows of d = 4096 708 and 716)
+    const Chain st{stream, !plain && chunk * d <= 1 << 22 ? 100 : -1};
     harp_status_t rc = HARP_OK;
     for (int64_t r0 = 0; r0 < n_rows && rc == HARP_OK; r0 += chunk) {
         const int64_t rows = std::min(chunk, n_rows - r0);
@@ -1746,7 +1752,7 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
         g_harp_launches.fetch_add(launches, std::memory_order_relaxed);
         if (cudaGetLastError() != cudaSuccess) rc = HARP_ERR_CUDA;
     }
-    cudaFreeAsync(part, st);
+    cudaFreeAsync(part, stream);
     return rc;
 }
 
