@@ -315,3 +315,15 @@ def test_states_of_one_thread_per_element_stages_stay_near_l2():
     assert _grad_launches(plan, x, g, outs[2]) == 2 * one - 1         # the reduction once
     # sums in fp64, rounded to fp32 once in the whole and once in either half
     assert float((outs[0] + outs[1] - outs[2]).abs().max()) <= 1e-6 * float(outs[2].abs().max())
+
+
+@pytest.mark.parametrize("n_rows", [1, 65, 700])
+@pytest.mark.parametrize("radices", [(2, 2, 2), (4, 4, 2), (4, 4, 2, 2, 2), (16, 8, 2), (4, 8, 8, 2)])
+def test_a_radix_two_stage_alone(radices, n_rows):
+    """Widths of 8 to 512: single blocks up to where fours of them fill a warp (d = 256), fours from there on."""
+    spec = wl.tiny_plan(47, radices, kind="qr", perm="identity", signs=True)
+    plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
+    xh, gh = _rows(48, n_rows, spec.d, "f32")
+    got, _, _ = _gpu_grad(plan, xh, gh, "f32")
+    want = _flat(orc.grad_blocks(oplan, promote(xh, "f32"), promote(gh, "f32")))
+    assert np.max(np.abs(got - want)) <= 2e-5 * np.max(np.abs(want))
