@@ -327,3 +327,16 @@ def test_a_radix_two_stage_alone(radices, n_rows):
     got, _, _ = _gpu_grad(plan, xh, gh, "f32")
     want = _flat(orc.grad_blocks(oplan, promote(xh, "f32"), promote(gh, "f32")))
     assert np.max(np.abs(got - want)) <= 2e-5 * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("n_rows", [1, 2, 3, 4, 8])
+@pytest.mark.parametrize("radices", [(16, 16), (8, 8, 7), (16, 8, 2)])
+def test_few_rows_of_wide_stages(dtype, n_rows, radices):
+    """One row (radix 16) and three (7 and 8) without tiles of eight, from there on with them."""
+    spec = wl.tiny_plan(49, radices, kind="qr", perm="random", signs=True)
+    plan, oplan = harp.plan_from_spec(spec), orc.OraclePlan.from_spec(spec)
+    xh, gh = _rows(50, n_rows, spec.d, dtype)
+    got, _, _ = _gpu_grad(plan, xh, gh, dtype)
+    want = _flat(orc.grad_blocks(oplan, promote(xh, dtype), promote(gh, dtype)))
+    assert np.max(np.abs(got - want)) <= 2e-5 * np.max(np.abs(want))
