@@ -1392,9 +1392,9 @@ outer_kernel(const TV *__restrict__ v, const int8_t *__restrict__ signs, const T
 
 constexpr int64_t kMostScratch = 1280ll << 20, kLeastScratch = 160ll << 20;     // bytes of states of a chunk
 // Bytes of one state of a chunk of a plan with one-thread-per-element kernels, which read two states once per row or column of a block: from L2, while
-// they fit it (10000 rows of radices 7, 57, 4 6514 us in one chunk, 3577 in two; 1024 rows of 2^8, 49 1504 in one, of 51 MB, 1189 in two; 4096
-// rows of 2^8, 43 in bf16 3151 with 40 MB, 3229 with 32, 3861 with 16)
-constexpr int64_t kPlainState = 40ll << 20;
+// they fit it (10000 rows of radices 7, 57, 4 6514 us in one chunk, 3577 in two; 1024 rows of 2^8, 49 1504 in one, of 51 MB, 1189 in two; 2048
+// rows of 8, 8, 40, 2 behind a permutation 1466 in one, of 40 MB, and 1260 in two; 4096 rows of 2^8, 43 in bf16 3151 with 40 MB, 3229 with 32, 3861 with 16)
+constexpr int64_t kPlainState = 32ll << 20;
 
 // Scratch comes from a memory pool of the library's own (one per device, created on first use)
 // that keeps one call's worth: the default pool hands its memory back at every

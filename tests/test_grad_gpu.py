@@ -304,7 +304,7 @@ def _grad_launches(plan, x, g, out):
 
 
 def test_states_of_one_thread_per_element_stages_stay_near_l2():
-    """40 MB a state of a chunk where a radix has no owner kernel: 10000 rows of d = 1596 in two chunks."""
+    """32 MB a state of a chunk where a radix has no owner kernel: 10000 rows of d = 1596 in two chunks."""
     spec = wl.tiny_plan(46, (7, 57, 4), kind="qr", perm="identity", signs=True)
     plan = harp.plan_from_spec(spec)
     x = torch.randn((10000, spec.d), device="cuda")
