@@ -305,11 +305,13 @@ harp_status_t harp_apply_host(harp_plan_t *plan, void *x_host, int64_t n_rows,
                               harp_dtype_t dtype, int transpose);
 
 /* Device-side wait status of the plan's kernels that are fed by bulk copies (HARP_KERNEL_TMEM, the
- * two-pass rows, the columns of two-sided products, the fp32 passes).  Every wait inside those kernels
- * (on a bulk copy, on the tensor core, on another warp) has an iteration limit; a wait that runs out
- * sets a device word, the kernel copies nothing more, waits as long again for its loads in flight,
- * releases its tensor memory and returns, and the rows it was working on are left undefined.  Returns 0 if no wait has given up since the plan was built, a positive
- * code naming the wait otherwise, -1 for NULL or a failed copy.  Synchronises with the device. */
+ * two-pass rows, the columns of two-sided products, the fp32 passes) or exchange rows within a
+ * cluster (small bf16 batches).  Every wait inside those kernels (on a bulk copy, on the tensor core,
+ * on another warp, on an exchange) has an iteration limit; a wait that runs out sets a device word,
+ * the kernel copies nothing more, waits as long again for its loads and exchanges in flight, releases
+ * its tensor memory and returns, and the rows it was working on are left undefined.  Returns 0 if no
+ * wait has given up since the plan was built, a positive code naming the wait otherwise, -1 for NULL
+ * or a failed copy.  Synchronises with the device. */
 int32_t harp_plan_error_word(const harp_plan_t *plan);
 
 /* Per-section cycle counters of the tensor-memory kernels and of the whole-row kernel, for profiling

@@ -39,6 +39,7 @@
 
 #include "harp_internal.h"
 #include "harp_mma.cuh"
+#include "harp_exchange.h"
 #include "harp_fuse.h"
 #include "harp_tm_ptx.cuh"
 
@@ -192,15 +193,11 @@ __device__ __forceinline__ void store_to_owner(const TileCtx &c, const PhaseDesc
         }
     }
 }
-// until all bytes of an exchange are here; gives up, and says so, after a bounded number of tries
-__device__ __forceinline__ void wait_exchange(uint32_t bar, int32_t *err) {
-    for (uint32_t tries = 0; tries < kExchangeSpin; ++tries) {
-        uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(bar) : "memory");
-        if (ok) return;
-    }
-    *err = 1;
+__device__ __forceinline__ bool exchange_arrived(uint32_t bar) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar) : "memory");
+    return ok != 0;
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -243,7 +240,7 @@ constexpr uint32_t kModesReorderOut = bit(MODE_SS) | bit(MODE_PO);   // the digi
 // counted on a barrier of its new owner, which waits for its own bytes alone; a cluster barrier after plain remote stores is a
 // release and an acquire of all memory (8.1 -> 7.7 us).  Nothing is overwritten early: a CTA stores to another only positions
 // that the other does not own in the phases before, and it stores after an exchange only once every CTA's items of
-// the phase before have arrived.  CLUSTER (two and four CTAs) keeps the barrier: 2048 pieces a CTA take st.async
+// the phase before have arrived; harp_exchange.h says what follows a wait that gave up.  CLUSTER (two and four CTAs) keeps the barrier: 2048 pieces a CTA take st.async
 // longer than the barrier costs (256 rows 9.6 against 11.2 us).
 enum { ALONE = 0, CLUSTER = 1, CLUSTER_COUNTED = 2 };
 
@@ -311,6 +308,7 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
         }
         harp_tm::tmem_wait_st();
     }
+    [[maybe_unused]] bool lost = false;        // counted clusters: a wait of this thread gave up
     const int warp = c.warp, lane = c.lane;
     // Counted clusters: the fragments of a warp's first item of the next phase come to registers while the rows or the
     // exchange are on their way
@@ -592,7 +590,13 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
                 }
             }
             if (kAhead && xchg) fetch_ahead(p + 1);
-            if (COUNTED && xchg) wait_exchange(bars + 8 * p, P.err);
+            if (COUNTED && xchg) {
+                if (!exchange_wait(kExchangeSpin, [&] { return exchange_arrived(bars + 8 * p); })) {
+                    *P.err = 1;
+                    lost = true;                   // this thread sends and stores nothing more
+                    c.okA = c.okB = false;
+                }
+            }
             else if (xchg) { cluster_arrive(); cluster_wait(); }
             else __syncthreads();
             FAST_MARK(2 + p);
@@ -601,7 +605,7 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
         if (P.copy_out >= 0) {
             const int32_t *cmap = tab_s + P.copy_out;
             const int chunks = d >> 3;
-            const int rows = (int)min((int64_t)kTileRows, n_rows - row0);
+            const int rows = COUNTED && lost ? 0 : (int)min((int64_t)kTileRows, n_rows - row0);
             const int lg_out = CL ? 28 - __clz(d) - lg : 0, per_out = chunks >> (CL ? lg : 0), first_out = CL ? rank * per_out : 0;
             const int rsteps = CL ? max(1, NT >> lg_out) : 1, r_first = CL && rsteps > 1 ? threadIdx.x >> lg_out : 0;
             if (r_first < rsteps)
@@ -621,6 +625,10 @@ harp_fast_kernel(__nv_bfloat16 *__restrict__ x, int64_t n_rows, int64_t n_tiles,
         for (int k = 0; k < 16; ++k)
             if (tacc[k]) atomicAdd((unsigned long long *)&g_fast_timing[k], (unsigned long long)tacc[k]);
 #endif
+    // (a thread of the cluster that has ended counts as one that is here)
+    if (COUNTED && lost)
+        exchange_leave(P.xchg_mask, kExchangeSpin, [] { asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory"); },
+                       [&](int p) { return exchange_arrived(bars + 8 * p); });
     if (!CL && P.tm_mask) {
         harp_tm::tc_fence_before();
         __syncthreads();
