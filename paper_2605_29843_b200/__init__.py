@@ -371,19 +371,24 @@ def shard_rows(n_rows: int, rank: int, world: int):
 #
 # A decode step spends as long in this call as on the GPU (a small apply: 7 us on the device, 5.3 us here before torch and
 # the library's function were looked up once instead of in every call), so the path below is flat, and the library is called through
-# _harpcall.so instead of ctypes (1.35 us less).
+# _harpcall.abi3.so instead of ctypes (1.35 us less) where that was built.
 
 _dtype_codes = {}                  # torch dtype -> harp_dtype_t
 _current_device = _raw_stream = _apply_ex = None
 
 
+def _without_ctypes(function):
+    """The same function behind a cheaper call; `function` itself in a tree built without CPython's headers."""
+    try:
+        from . import _harpcall
+    except ImportError:
+        return function
+    return _harpcall.function(ctypes.cast(function, ctypes.c_void_p).value)
+
+
 def _bind_torch() -> None:
     global _current_device, _raw_stream, _apply_ex
     import torch
-    try:
-        from . import _harpcall
-    except ImportError as e:
-        raise ImportError(f"{_HERE}/_harpcall.so: run `python -m paper_2605_29843_b200.build`") from e
     torch.cuda.init()
     _dtype_codes.update({torch.float32: HARP_F32, torch.bfloat16: HARP_BF16})
     if hasattr(torch._C, "_cuda_getCurrentRawStream"):
@@ -391,7 +396,7 @@ def _bind_torch() -> None:
     else:
         _current_device, _raw_stream = torch.cuda.current_device, lambda dev: torch.cuda.current_stream(dev).cuda_stream
     # last: what the callers test, also those on other threads
-    _apply_ex = _harpcall.function(ctypes.cast(lib().harp_apply_ex, ctypes.c_void_p).value)
+    _apply_ex = _without_ctypes(lib().harp_apply_ex)
 
 
 def _torch_dtype_code(t) -> int:

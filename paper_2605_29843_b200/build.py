@@ -1,5 +1,5 @@
 """Build step: compiles the CUDA sources under csrc/ into libharp.so (sm_100a only) and csrc/pycall.c into
-_harpcall.so (the call from Python), in-tree, next to this file.  ``python -m paper_2605_29843_b200.build`` or build()."""
+_harpcall.abi3.so (the call from Python; ctypes does without it), in-tree, next to this file.  ``python -m paper_2605_29843_b200.build`` or build()."""
 from __future__ import annotations
 
 import glob
@@ -11,7 +11,7 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libharp.so")
-CALL, CALL_SRC = os.path.join(HERE, "_harpcall.so"), os.path.join(HERE, "csrc", "pycall.c")
+CALL, CALL_SRC = os.path.join(HERE, "_harpcall.abi3.so"), os.path.join(HERE, "csrc", "pycall.c")
 
 
 def sources():
@@ -28,8 +28,9 @@ def _stale() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if force or not os.path.exists(CALL) or os.path.getmtime(CALL_SRC) > os.path.getmtime(CALL):
-        subprocess.check_call([os.environ.get("CC", "gcc"), "-shared", "-fPIC", "-O2", "-I", sysconfig.get_paths()["include"], CALL_SRC, "-o", CALL])
+    headers = sysconfig.get_paths()["include"]
+    if (force or not os.path.exists(CALL) or os.path.getmtime(CALL_SRC) > os.path.getmtime(CALL)) and os.path.exists(os.path.join(headers, "Python.h")):
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-shared", "-fPIC", "-O2", "-I", headers, CALL_SRC, "-o", CALL])
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -1,7 +1,9 @@
 // A call of the library from Python without ctypes: function(address) returns a callable for a function of harp_apply_ex's
 // signature at that address.  ctypes converts seven arguments in 1.7 us (0.3 us here, argument checks included), a
-// fifth of a decode step's call.  Plain C beside CPython's headers; it does not link to the library.
+// fifth of a decode step's call.  Plain C beside CPython's headers, of the stable interface since 3.10, so that one build serves every
+// later interpreter; it does not link to the library.
 #define PY_SSIZE_T_CLEAN
+#define Py_LIMITED_API 0x030a0000
 #include <Python.h>
 #include <stdint.h>
 

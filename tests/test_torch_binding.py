@@ -1,4 +1,7 @@
 """The torch conveniences look torch and the library's function up once (no GPU needed: CUDA initialisation is replaced)."""
+import os
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -45,3 +48,20 @@ def test_the_call_without_ctypes_takes_what_ctypes_took(unbound, monkeypatch):
     for args in ((None, 0, 1.0, 0, 0, 0, 0), (None, 0, 1, 0, 0, 0), (None, 0, 1, 0, 0, "0", 0)):
         with pytest.raises(TypeError):
             harp._apply_ex(*args)
+
+
+def test_a_tree_with_the_library_alone_calls_through_ctypes(unbound, monkeypatch):
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    monkeypatch.setitem(sys.modules, harp.__name__ + "._harpcall", None)       # as if it were not there
+    monkeypatch.delattr(harp, "_harpcall", raising=False)
+    harp._bind_torch()
+    assert harp._apply_ex is harp.lib().harp_apply_ex
+    assert harp._apply_ex(None, 0, 1, 0, 0, 0, None) == 1
+
+
+def test_the_call_is_built_for_every_interpreter():
+    """The stable interface, and a name that no other interpreter's build has."""
+    harp_build.build()
+    assert os.path.basename(harp_build.CALL) == "_harpcall.abi3.so" and os.path.exists(harp_build.CALL)
+    assert harp._without_ctypes(harp.lib().harp_apply_ex)(None, 0, 1, 0, 0, 0, None) == 1
+    assert "Py_LIMITED_API" in open(harp_build.CALL_SRC).read()
