@@ -9,9 +9,9 @@
 
 typedef int (*apply_fn)(const void *plan, void *x, int64_t n_rows, int dtype, int transpose, int kernel, void *stream);
 
-// integers, None for a null pointer; whatever has __index__ counts as an integer, and pointers and codes wrap, as with ctypes
-static int to_u64(PyObject *o, uint64_t *out) {
-    if (o == Py_None) { *out = 0; return 1; }
+// integers, None for a null pointer alone; whatever has __index__ counts as an integer, and pointers and codes wrap, as with ctypes
+static int to_u64(PyObject *o, int pointer, uint64_t *out) {
+    if (pointer && o == Py_None) { *out = 0; return 1; }
     PyObject *i = PyNumber_Index(o);
     if (!i) return 0;
     *out = PyLong_AsUnsignedLongLongMask(i);
@@ -26,7 +26,7 @@ static PyObject *call(PyObject *self, PyObject *const *args, Py_ssize_t n) {
         return NULL;
     }
     for (int k = 0; k < 7; ++k)
-        if (!to_u64(args[k], &a[k])) return NULL;
+        if (!to_u64(args[k], k < 2 || k == 6, &a[k])) return NULL;
     const apply_fn fn = (apply_fn)PyLong_AsVoidPtr(self);
     int st;
     Py_BEGIN_ALLOW_THREADS

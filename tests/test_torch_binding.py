@@ -1,4 +1,5 @@
 """The torch conveniences look torch and the library's function up once (no GPU needed: CUDA initialisation is replaced)."""
+import ctypes
 import os
 import sys
 
@@ -65,3 +66,14 @@ def test_the_call_is_built_for_every_interpreter():
     assert os.path.basename(harp_build.CALL) == "_harpcall.abi3.so" and os.path.exists(harp_build.CALL)
     assert harp._without_ctypes(harp.lib().harp_apply_ex)(None, 0, 1, 0, 0, 0, None) == 1
     assert "Py_LIMITED_API" in open(harp_build.CALL_SRC).read()
+
+
+@pytest.mark.parametrize("at", [2, 3, 4, 5])
+def test_none_is_no_number(unbound, monkeypatch, at):
+    """Rows, codes and the direction, as ctypes refuses them; the plan, the rows' address and the stream are pointers."""
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    harp._bind_torch()
+    args = [None, None, 1, 0, 0, 0, None]
+    args[at] = None
+    with pytest.raises((TypeError, ctypes.ArgumentError)):
+        harp._apply_ex(*args)
