@@ -251,10 +251,17 @@ int64_t harp_two_sided_static_capacity_bytes(void);
  *   grad       DEVICE float[harp_plan_n_params(plan)], laid out like the blocks given to
  *              harp_plan_create (stage after stage, [D_t][b_t][b_t]); overwritten, or added to
  *              if accumulate != 0
- * Any schedule is accepted.  Sums over rows are taken in fp64, in an order that the shapes fix (no
- * atomics: the result does not depend on scheduling).  The call allocates and frees scratch
- * on the stream (states of about 200 MB of rows, of sixteen rows at least, and the partial sums of one wave of CTAs, from a memory pool of the library's own that keeps what it has
- * been given until the process ends); HARP_ERR_ALLOC if that fails.  Asynchronous on stream. */
+ * Any schedule is accepted.  Sums over rows are taken in fp64, in an order that the shapes and the
+ * size of a chunk of rows fix (no atomics: the result does not depend on scheduling).
+ * Scratch.  The call allocates and frees it on the stream: the states of a chunk of rows, sixteen rows
+ * at least, and the partial sums of one wave of CTAs.  A chunk's states take up to 1280 MB (a batch
+ * that needs less takes less; plans with a radix from 9 to 15 or above 16 take up to 32 MB a state).
+ * Where that cannot be allocated the call asks for 640, 320 and 160 MB before it returns
+ * HARP_ERR_ALLOC; HARP_GRAD_SCRATCH_MB in the environment when the plan is built passes over the sizes
+ * above that many MB.  The memory comes from a pool of the library's own, one a device, which keeps up to
+ * 1536 MB of what it was given until the process ends (for the next call: mapping it anew costs more than the
+ * kernels of a call) and hands back what calls on several streams took beyond that at a synchronisation.
+ * Asynchronous on stream. */
 harp_status_t harp_grad_blocks(const harp_plan_t *plan, const void *x, const void *gy, int64_t n_rows,
                                harp_dtype_t dtype, float *grad, int accumulate, void *stream);
 

@@ -89,6 +89,7 @@ extern "C" harp_status_t harp_plan_create(harp_plan_t **out, int64_t d, int32_t 
     p->opt_no_rowvec = getenv("HARP_NO_ROWVEC") != nullptr;
     p->opt_no_maps = getenv("HARP_NO_TENSOR_MAPS") != nullptr;
     p->opt_f32_passes = getenv("HARP_F32_PASSES") != nullptr;
+    if (const char *e = getenv("HARP_GRAD_SCRATCH_MB")) p->opt_grad_scratch = (int64_t)std::max(0, atoi(e)) << 20;
     p->st.m = n_stages;
     int64_t s = 1, off = 0;
     for (int t = 0; t < n_stages; ++t) {

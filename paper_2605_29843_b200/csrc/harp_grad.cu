@@ -1657,7 +1657,7 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
     const bool permuted = plan->d_perm != nullptr;
     // Chunk of rows whose forward states, gradient states and permuted rows fit the budget; the partial sums of a wave of CTAs come on top.  The
     // forward kernels (none where one step is all) take kFwdRows rows per CTA along grid.y.  Chunks that stay near L2 are not worth their launches
-    // and partial waves (16384 rows of d = 4096, chunks of 110 MB 1083 us, 200 MB 863, 640 MB 751, one of 1200 MB 719); a device without room for it takes the smaller ones.
+    // and partial waves (16384 rows of d = 4096, call after call on the same rows: chunks of 110 MB 1083 us, 200 MB 863, 640 MB 751, one of 1200 MB 719; on others each time 777); a device without room for it takes the smaller ones.
     const int64_t per_row = std::max<int64_t>(1, d * (4 * (int64_t)(n - 1 + n_g) + (permuted ? (int64_t)sizeof(T) : 0)));
     int sms = 148;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device);
@@ -1685,7 +1685,9 @@ harp_status_t grad_blocks(const harp_plan *plan, const T *x, const T *gy, int64_
             }
         }
         plane = (chunk * d + 3) / 4 * 4;
-        const size_t bytes = (size_t)(part_len * 8 + 16 + plane * 4 * (n - 1 + n_g) + (permuted ? plane * (int64_t)sizeof(T) : 0));
+        const int64_t states = plane * 4 * (n - 1 + n_g) + (permuted ? plane * (int64_t)sizeof(T) : 0);
+        if (states > plan->opt_grad_scratch) continue;
+        const size_t bytes = (size_t)(part_len * 8 + 16 + states);
         if ((pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&part), bytes, pool, stream) : cudaMallocAsync(reinterpret_cast<void **>(&part), bytes, stream)) != cudaSuccess) {
             cudaGetLastError();
             part = nullptr;

@@ -56,6 +56,8 @@ struct harp_plan {
     // CUDA-core kernels keep their tile row-major; HARP_NO_TENSOR_MAPS=1: as on a driver that cannot encode tensor maps;
     // HARP_F32_PASSES=1: fp32 rows take the passes over column groups whatever the batch)
     bool opt_no_rowvec = false, opt_no_maps = false, opt_f32_passes = false;
+    // most bytes of states that a gradient asks for (HARP_GRAD_SCRATCH_MB, read then too)
+    int64_t opt_grad_scratch = INT64_MAX;
     // staging owned by harp_apply_host
     static constexpr int kStages = 4;
     void *stage_buf[kStages] = {nullptr, nullptr, nullptr, nullptr};

@@ -340,3 +340,26 @@ def test_few_rows_of_wide_stages(dtype, n_rows, radices):
     got, _, _ = _gpu_grad(plan, xh, gh, dtype)
     want = _flat(orc.grad_blocks(oplan, promote(xh, dtype), promote(gh, dtype)))
     assert np.max(np.abs(got - want)) <= 2e-5 * np.max(np.abs(want))
+
+
+def test_smaller_chunks_where_the_largest_is_not_to_be_had(monkeypatch):
+    """Five steps of d = 8192 in fp32: 6000 rows are 1125 MB of states, in two chunks of up to 640 MB, four of 320 and eight of 160; below that
+    the call says that it has no memory and writes nothing."""
+    spec = wl.tiny_plan(51, (8, 8, 8, 8, 2), kind="qr", perm="identity", signs=True)
+    x = torch.randn((6000, spec.d), device="cuda")
+    g = torch.randn_like(x)
+    n_par = harp.harp_plan_n_params(harp.plan_from_spec(spec))
+    want = torch.zeros(n_par, device="cuda")
+    launches = _grad_launches(harp.plan_from_spec(spec), x, g, want)
+    for limit, chunks in ((1280, 1), (1000, 2), (400, 4), (160, 8)):
+        monkeypatch.setenv("HARP_GRAD_SCRATCH_MB", str(limit))
+        out = torch.zeros(n_par, device="cuda")
+        assert _grad_launches(harp.plan_from_spec(spec), x, g, out) == chunks * (launches - 1) + 1          # one reduction
+        # the same fp32 states and fp64 sums in another order: a rounding of the result
+        assert float((out - want).abs().max()) <= 1e-6 * float(want.abs().max())
+    monkeypatch.setenv("HARP_GRAD_SCRATCH_MB", "100")
+    plan, out = harp.plan_from_spec(spec), torch.full((n_par,), 3.0, device="cuda")
+    with pytest.raises(harp.HarpError) as e:
+        _grad_launches(plan, x, g, out)
+    torch.cuda.synchronize()
+    assert e.value.status == 9 and bool((out == 3.0).all())
