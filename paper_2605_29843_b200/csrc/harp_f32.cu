@@ -1018,8 +1018,8 @@ double pass_estimate(const F32Plan *fp, const F32Pass &P, int64_t n) {
 // whole-row kernels a wave of CTAs, whatever the batch leaves of it idle: radices (16, 16, 4), whole rows against passes: 128 rows 14 us and
 // 25, 256 rows 25 and 25, 512 rows 45 and 28.  The register passes are faster nearly everywhere (d = 8192 in radix 8, whole rows and passes:
 // 1 row 23 and 6.6 us, 256 rows 35 and 12, 4096 rows 294 and 104).  One exception, which no time speaks for (42 and 18 us): batches of d = 8192 that
-// fill five sixths or more of the whole-row kernel's one wave of tiles of four rows stay with its one launch, as before there were register passes; 500
-// rows are promised it (test_small_batches_take_one_launch).  Smaller batches and other widths take what the estimates say (300 rows of radices
+// fill five sixths or more of the whole-row kernel's one wave of tiles of four rows stay with its one launch, to which
+// test_small_batches_take_one_launch holds 500 rows.  Smaller batches and other widths take what the estimates say (300 rows of radices
 // (4, 3, 4, 2, 4, 4, 7) 55 us whole, 39 in passes; of 2^10, 8 38 and 13).
 bool harp_f32_preferred(const harp_plan *plan, int64_t n_rows) {
     const F32Plan *fp = plan->f32;
